@@ -122,9 +122,10 @@ struct PushArgs {
   float* momlo;                 // low FP32 parts of the crossing pass's moments [ns][nt][8]
   const float4* tetdf;          // contract form: low FP32 parts of grad lambda_1..3, [nt][4] float4
   unsigned long long* stats;    // [0] crossings, [1] frozen, [2] staging wait timeouts
-  CrossRec* xrec;               // mixed form: crossing records, 256-slot region per tile
-  CrossRec64* xrec64;           // FP64 form: the same, FP64 records
-  int32_t* xcount;              // mixed form: records per tile
+  CrossRec* xrec;               // mixed forms: crossing records, one region per common-path CTA
+  CrossRec64* xrec64;           // FP64 form: FP64 records, 256-slot region per tile
+  int32_t* xcount;              // records per region
+  int64_t xcap;                 // mixed forms: slots of a CTA's region (its tiles times 256)
   unsigned long long wait_ns;   // limit of each bounded wait of the staged kernel
   int32_t stall_cta;            // test support: this CTA waits on a barrier nothing completes (-1: none)
 };
@@ -976,7 +977,7 @@ struct LaneOut {
 };
 
 struct CrossList {
-  int32_t total;     // records of the current tile
+  int32_t total;     // records this CTA has written
   long long sums[kThreads / 32][32 * 6];   // per warp: run sums of the deposit, by head lane
   int32_t keys[kThreads / 32][32];         // per warp: run keys, by head lane
 };
@@ -1110,6 +1111,11 @@ __device__ __forceinline__ void mixed_particle(const PushArgs& A, int64_t p, int
   o.shome = s;
 }
 
+// Record regions of the mixed common path: each CTA appends the particles
+// that leave their tets to a region of its own (its tiles' records back to
+// back), and the crossing pass runs one CTA per region.
+__device__ __forceinline__ CrossRec* xregion(const PushArgs& A) { return A.xrec + blockIdx.x * A.xcap; }
+
 // Warp epilogue (all 32 lanes): append the queued lanes to the CTA's
 // crossing list (one shared-memory atomic per warp), reduce the one-segment
 // deposits over runs of equal (tet, species) keys (particles are sorted by
@@ -1127,7 +1133,7 @@ __device__ __forceinline__ void mixed_warp_epilogue(const PushArgs& A, int64_t p
     if (lane == 0) base = atomicAdd(&cl.total, __popc(qmask));
     base = __shfl_sync(full, base, 0);
     if (o.queue) {
-      CrossRec& r = A.xrec[(p & ~(int64_t)(kThreads - 1)) + base + __popc(qmask & ((1u << lane) - 1u))];
+      CrossRec& r = xregion(A)[base + __popc(qmask & ((1u << lane) - 1u))];
       r.a[0] = o.a[0];
       r.a[1] = o.a[1];
       r.a[2] = o.a[2];
@@ -1225,46 +1231,52 @@ __device__ __forceinline__ void mixed_warp_epilogue(const PushArgs& A, int64_t p
   if (lane == 0 && nf) atomicAdd(A.stats + 1, (unsigned long long)nf);
 }
 
-// End of a tile (all threads, after the tile's epilogues): publish the tile's
-// record count for the crossing kernel and reset the counter.
-__device__ __forceinline__ void publish_tile(const PushArgs& A, CrossList& cl, int64_t tile) {
+// End of a CTA's work (all threads): its region's record count.
+__device__ __forceinline__ void publish_region(const PushArgs& A, const CrossList& cl) {
   __syncthreads();
-  if (threadIdx.x == 0) {
-    A.xcount[tile] = cl.total;
-    cl.total = 0;
-  }
+  if (threadIdx.x == 0) A.xcount[blockIdx.x] = cl.total;
 }
 
-// Common path, one particle per thread, state read straight from global
-// memory.  Used when the particle arrays are not 16-byte aligned (so bulk
-// copies cannot stage them) and for a ragged last tile.
+// One tile's particle of this thread, state read straight from global memory.
+__device__ __forceinline__ void load_plain(const PushArgs& A, int64_t p, int32_t& T, double r[3], float v[3]) {
+  T = p < A.n ? A.tet[p] : -1;
+  if (T < 0) return;
+  r[0] = A.x[p];
+  r[1] = A.y[p];
+  r[2] = A.z[p];
+  v[0] = static_cast<const float*>(A.vx)[p];
+  v[1] = static_cast<const float*>(A.vy)[p];
+  v[2] = static_cast<const float*>(A.vz)[p];
+}
+
+// Common path for particle arrays that are not 16-byte aligned (bulk copies
+// cannot stage them) and for sets below one tile: CTAs walk the tiles, each
+// thread reads its particle from global memory.
 template <bool Q24>
-__global__ void __launch_bounds__(kThreads) k_push_mixed(PushArgs A, int64_t p0) {
+__global__ void __launch_bounds__(kThreads, 4) k_push_mixed(PushArgs A, int64_t ntiles) {
   __shared__ CrossList cl;
-  const int64_t p = p0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int lane = threadIdx.x & 31;
   if (threadIdx.x == 0) cl.total = 0;
   __syncthreads();
-  LaneOut o;
-  lane_init(o, lane);
-  if (p < A.n) {
-    const int32_t T = A.tet[p];
-    if (T >= 0) {
-      const float* vx = static_cast<const float*>(A.vx);
-      const float* vy = static_cast<const float*>(A.vy);
-      const float* vz = static_cast<const float*>(A.vz);
-      mixed_particle<Q24>(A, p, T, A.x[p], A.y[p], A.z[p], vx[p], vy[p], vz[p], o);
-    } else {
-      mixed_particle<Q24>(A, p, T, 0.0, 0.0, 0.0, 0.f, 0.f, 0.f, o);
-    }
+  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const int64_t p = tile * kThreads + threadIdx.x;
+    LaneOut o;
+    lane_init(o, lane);
+    int32_t T;
+    double r[3] = {0.0, 0.0, 0.0};
+    float v[3] = {0.f, 0.f, 0.f};
+    load_plain(A, p, T, r, v);
+    mixed_particle<Q24>(A, p, T, r[0], r[1], r[2], v[0], v[1], v[2], o);
+    mixed_warp_epilogue<Q24>(A, p, lane, o, cl);
   }
-  mixed_warp_epilogue<Q24>(A, p, lane, o, cl);
-  publish_tile(A, cl, (p0 >> 8) + blockIdx.x);
+  publish_region(A, cl);
 }
 
 // ------------------------------------------------- staged common path (TMA)
-// Persistent CTAs walk full 256-particle tiles.  Each tile's slices of the
-// seven particle arrays (x, y, z f64; vx, vy, vz f32; tet i32; 10 KB) are
+// Persistent CTAs walk the 256-particle tiles (the last one, if ragged, is
+// read straight from global memory by the CTA whose turn it is: a launch of
+// its own for it cost 5 us, a 100k-particle step 73 -> 55 us).  Each full
+// tile's slices of the seven particle arrays (x, y, z f64; vx, vy, vz f32; tet i32; 10 KB) are
 // brought into shared memory by cp.async.bulk copies completing on an
 // mbarrier, in a ring of three stages filled two tiles ahead, so HBM latency
 // overlaps the arithmetic.  A stage is refilled only after the iteration
@@ -1347,7 +1359,7 @@ __device__ __forceinline__ void stage_tile(const PushArgs& A, unsigned char* sta
 #define FEMPIC_TMA_MIN_BLOCKS 4
 #endif
 template <bool Q24>
-__global__ void __launch_bounds__(kThreads, FEMPIC_TMA_MIN_BLOCKS) k_push_mixed_tma(PushArgs A, int64_t ntiles) {
+__global__ void __launch_bounds__(kThreads, FEMPIC_TMA_MIN_BLOCKS) k_push_mixed_tma(PushArgs A, int64_t nfull) {
   __shared__ __align__(128) unsigned char smem[kStages][kStageBytes];
   // bar[kStages] is test support: a barrier no copy ever completes, for the
   // CTA that fempic_debug_stall names
@@ -1362,9 +1374,10 @@ __global__ void __launch_bounds__(kThreads, FEMPIC_TMA_MIN_BLOCKS) k_push_mixed_
   __syncthreads();
   const int64_t stride = gridDim.x;
   const int64_t t0 = blockIdx.x;
+  const int64_t ntiles = nfull + (A.n > nfull * kTile ? 1 : 0);
   if (tid == 0)
     for (int k = 0; k < kStages; k++)
-      if (t0 + k * stride < ntiles) stage_tile(A, smem[k], t0 + k * stride, &bar[k]);
+      if (t0 + k * stride < nfull) stage_tile(A, smem[k], t0 + k * stride, &bar[k]);
   uint32_t phase = 0u;   // bit k = parity of the next wait on stage k
   int st = 0;
   for (int64_t it = 0, tile = t0; tile < ntiles; tile += stride, it++) {
@@ -1372,17 +1385,17 @@ __global__ void __launch_bounds__(kThreads, FEMPIC_TMA_MIN_BLOCKS) k_push_mixed_
     // this barrier; the proxy fence orders those shared-memory reads before
     // the bulk copy that refills that stage below.
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    bool ok = mbar_wait_bounded(&bar[st], (phase >> st) & 1u, A.wait_ns);
+    bool ok = tile >= nfull || mbar_wait_bounded(&bar[st], (phase >> st) & 1u, A.wait_ns);
     if (it == 0 && (int)blockIdx.x == A.stall_cta) ok = ok && mbar_wait_bounded(&bar[kStages], 0u, A.wait_ns);
     if (__syncthreads_or(!ok)) {
       // give up: record it, wait (bounded) for this CTA's copies still in
       // flight (stages of tiles it .. it+kStages-1 not yet consumed), stop
       if (tid == 0) {
         atomicAdd(A.stats + 2, 1ull);
-        for (int64_t t = tile; t < ntiles; t += stride) A.xcount[t] = 0;   // no stale records
+        A.xcount[blockIdx.x] = cl.total;   // the records of the tiles done so far
         for (int k = 0; k < kStages; k++) {
           const int sk = (st + k) % kStages;
-          if (tile + k * stride < ntiles) mbar_wait_bounded(&bar[sk], (phase >> sk) & 1u, A.wait_ns);
+          if (tile + k * stride < nfull) mbar_wait_bounded(&bar[sk], (phase >> sk) & 1u, A.wait_ns);
         }
       }
       return;
@@ -1391,24 +1404,31 @@ __global__ void __launch_bounds__(kThreads, FEMPIC_TMA_MIN_BLOCKS) k_push_mixed_
     if (tid == 0 && it > 0) {
       const int prev = (st + kStages - 1) % kStages;
       const int64_t next = tile + (kStages - 1) * stride;
-      if (next < ntiles) stage_tile(A, smem[prev], next, &bar[prev]);
+      if (next < nfull) stage_tile(A, smem[prev], next, &bar[prev]);
     }
-    const unsigned char* S = smem[st];
-    const double ax = reinterpret_cast<const double*>(S)[tid];
-    const double ay = reinterpret_cast<const double*>(S + kTile * 8)[tid];
-    const double az = reinterpret_cast<const double*>(S + kTile * 16)[tid];
-    const float v0 = reinterpret_cast<const float*>(S + kTile * 24)[tid];
-    const float v1 = reinterpret_cast<const float*>(S + kTile * 28)[tid];
-    const float v2 = reinterpret_cast<const float*>(S + kTile * 32)[tid];
-    const int32_t T = reinterpret_cast<const int32_t*>(S + kTile * 36)[tid];
     const int64_t p = tile * kTile + tid;
+    int32_t T;
+    double r[3] = {0.0, 0.0, 0.0};
+    float v[3] = {0.f, 0.f, 0.f};
+    if (tile < nfull) {
+      const unsigned char* S = smem[st];
+      r[0] = reinterpret_cast<const double*>(S)[tid];
+      r[1] = reinterpret_cast<const double*>(S + kTile * 8)[tid];
+      r[2] = reinterpret_cast<const double*>(S + kTile * 16)[tid];
+      v[0] = reinterpret_cast<const float*>(S + kTile * 24)[tid];
+      v[1] = reinterpret_cast<const float*>(S + kTile * 28)[tid];
+      v[2] = reinterpret_cast<const float*>(S + kTile * 32)[tid];
+      T = reinterpret_cast<const int32_t*>(S + kTile * 36)[tid];
+    } else {
+      load_plain(A, p, T, r, v);
+    }
     LaneOut o;
     lane_init(o, lane);
-    mixed_particle<Q24>(A, p, T, ax, ay, az, v0, v1, v2, o);
+    mixed_particle<Q24>(A, p, T, r[0], r[1], r[2], v[0], v[1], v[2], o);
     mixed_warp_epilogue<Q24>(A, p, lane, o, cl);
-    publish_tile(A, cl, tile);
     st = (st + 1) % kStages;
   }
+  publish_region(A, cl);
 }
 
 // Crossing path of a particle that leaves its home tet, one face at a time.
@@ -1587,42 +1607,54 @@ __device__ __forceinline__ void cross_finish(const PushArgs& A, const CrossState
   ncr += (unsigned)c.nc;
 }
 
-// Crossing pass of the 24-bit form.  Each warp takes a stream of tile
-// regions of the record queue (tile, tile + warps, ...); each loop iteration
-// advances every busy lane by one face, and a lane whose particle is done
-// takes the stream's next record, so neither a particle that crosses many
-// faces (a fast beam particle) nor the end of a tile holds idle lanes.
-// Records of one tile come from neighbouring tets, so the warp's tet records
-// and deposit slots stay in cache.
+// Crossing passes of the mixed forms: one CTA per record region.  The CTA's
+// warps draw records from a shared cursor; each loop iteration advances every
+// busy lane by one face, and idle lanes take new records once kRefill of them
+// wait, so that the extra work of a fresh particle (its start's barycentrics)
+// runs for several lanes at once.  Bound by the latency of the dependent tet
+// records and by the reductions of the deposit (without any deposit a 24M
+// beam-plasma step takes 0.74 of 1.21 ms).  Drawing by CTA keeps warps level
+// where some tiles hold many long walks (a 10 keV beam leaves its tet every
+// step and crosses about eight faces).  Against a fixed stream of tiles per
+// warp with lanes refilled one by one: 1.30 -> 1.21 ms per step on that load,
+// 0.203 -> 0.185 on the 10M cavity; waiting for 1, 8, 12, 16 idle lanes:
+// 1.29, 1.24, 1.21, 1.22 ms.
+constexpr int kCrossThreadsDF = 192;    // contract pass: 4 CTAs per SM at 80 registers
+constexpr int kCrossThreadsQ24 = 256;   // 24-bit pass: 4 CTAs per SM at 64 registers
+constexpr int kRefill = 12;
 
-__global__ void __launch_bounds__(kThreads) k_cross_q24(PushArgs A, int64_t ntiles) {
+// Hands out the region's records to idle lanes: >= 0 for a lane that takes
+// that record, else -1.  `more` turns false when the region is used up.
+__device__ __forceinline__ int32_t draw_record(unsigned idle, int lane, bool have, int32_t cnt, int32_t* cursor,
+                                               bool& more) {
+  int32_t base = 0;
+  const int32_t want = __popc(idle);
+  if (lane == 0) base = atomicAdd(cursor, want);
+  base = __shfl_sync(0xffffffffu, base, 0);
+  more = base + want < cnt;
+  const int32_t k = base + __popc(idle & ((1u << lane) - 1u));
+  return !have && k < cnt ? k : -1;
+}
+
+__global__ void __launch_bounds__(kCrossThreadsQ24, 4) k_cross_q24(PushArgs A) {
+  __shared__ int32_t cursor;
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
-  const unsigned lt = (1u << lane) - 1u;
+  const CrossRec* rec = xregion(A);
+  const int32_t cnt = A.xcount[blockIdx.x];
+  if (threadIdx.x == 0) cursor = 0;
+  __syncthreads();
   unsigned ncr = 0, nfrz = 0;
-  const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  int64_t tile = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  int32_t cnt = tile < ntiles ? A.xcount[tile] : 0, next = 0;
-  bool have = false, fresh = false;
+  bool have = false, fresh = false, more = cnt > 0;
   CrossState c;
   for (;;) {
-    unsigned idle = __ballot_sync(full, !have);
-    while (idle && tile < ntiles) {   // warp-uniform: assigns records or advances a tile
-      const int32_t avail = cnt - next;
-      const int32_t want = __popc(idle);
-      const int32_t take = avail < want ? avail : want;
-      const int r = __popc(idle & lt);
-      if (!have && r < take) {
-        cross_begin(A, A.xrec[tile * kThreads + next + r], c);
+    const unsigned idle = __ballot_sync(full, !have);
+    if (more && __popc(idle) >= kRefill) {
+      const int32_t k = draw_record(idle, lane, have, cnt, &cursor, more);
+      if (k >= 0) {
+        cross_begin(A, rec[k], c);
         have = true;
         fresh = true;
-      }
-      next += take;
-      idle = __ballot_sync(full, !have);
-      if (next == cnt) {
-        tile += warps;
-        cnt = tile < ntiles ? A.xcount[tile] : 0;
-        next = 0;
       }
     }
     if (!__any_sync(full, have)) break;
@@ -1886,42 +1918,25 @@ __device__ __forceinline__ void cross_finish_df(const PushArgs& A, const CrossSt
   ncr += (unsigned)c.nc;
 }
 
-// Each loop iteration advances every busy lane by one piece; idle lanes take
-// the next records of the warp's record stream, which runs on across its
-// tiles (tile, tile + warps, ...): a tile holds about 36 leaving particles
-// on the cavity, so a per-tile loop would leave most lanes idle at the end of
-// every tile (the stream measured 9 % faster).
-#ifndef FEMPIC_CROSS_MIN_BLOCKS
-#define FEMPIC_CROSS_MIN_BLOCKS 3
-#endif
-__global__ void __launch_bounds__(kThreads, FEMPIC_CROSS_MIN_BLOCKS) k_cross_df(PushArgs A, int64_t ntiles) {
+__global__ void __launch_bounds__(kCrossThreadsDF, 4) k_cross_df(PushArgs A) {
+  __shared__ int32_t cursor;
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
-  const unsigned lt = (1u << lane) - 1u;
+  const CrossRec* rec = xregion(A);
+  const int32_t cnt = A.xcount[blockIdx.x];
+  if (threadIdx.x == 0) cursor = 0;
+  __syncthreads();
   unsigned ncr = 0, nfrz = 0;
-  const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  int64_t tile = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  int32_t cnt = tile < ntiles ? A.xcount[tile] : 0, next = 0;
-  bool have = false, fresh = false;
+  bool have = false, fresh = false, more = cnt > 0;
   CrossStateDF c;
   for (;;) {
-    unsigned idle = __ballot_sync(full, !have);
-    while (idle && tile < ntiles) {   // warp-uniform: assigns records or advances a tile
-      const int32_t avail = cnt - next;
-      const int32_t want = __popc(idle);
-      const int32_t take = avail < want ? avail : want;
-      const int r = __popc(idle & lt);
-      if (!have && r < take) {
-        cross_begin_df(A, A.xrec[tile * kThreads + next + r], c);
+    const unsigned idle = __ballot_sync(full, !have);
+    if (more && __popc(idle) >= kRefill) {
+      const int32_t k = draw_record(idle, lane, have, cnt, &cursor, more);
+      if (k >= 0) {
+        cross_begin_df(A, rec[k], c);
         have = true;
         fresh = true;
-      }
-      next += take;
-      idle = __ballot_sync(full, !have);
-      if (next == cnt) {
-        tile += warps;
-        cnt = tile < ntiles ? A.xcount[tile] : 0;
-        next = 0;
       }
     }
     if (!__any_sync(full, have)) break;
@@ -3032,13 +3047,12 @@ struct fempic_env {
   int32_t* estart = nullptr;        // edge -> (tet, local edge) slots, CSR [ne + 1]
   int32_t* eslot = nullptr;         // [6 nt], slot = 6 tet + local edge
   int32_t* fslot = nullptr;         // face -> (tet, local face) slots [nf][2], 4 tet + local face or -1
-  CrossRec* xrec = nullptr;         // mixed form crossing queue [xtiles * 256]
-  CrossRec64* xrec64 = nullptr;     // FP64 form crossing queue [xtiles * 256]
-  int32_t* xcount = nullptr;        // [xtiles]
-  int64_t xtiles = 0;
+  CrossRec* xrec = nullptr;         // mixed forms: crossing queue [xslots]
+  CrossRec64* xrec64 = nullptr;     // FP64 form: crossing queue [xslots]
+  int32_t* xcount = nullptr;        // [xregions]
+  int64_t xslots = 0, xregions = 0;
   int num_sms = 1;
-  int tma_blocks_per_sm[2] = {0, 0}; // resident CTAs of the staged kernels (contract, 24-bit)
-  int cross_blocks_per_sm[3] = {0, 0, 0};   // resident CTAs of the mixed crossing passes (-, contract, 24-bit)
+  int push_blocks_per_sm[4] = {0, 0, 0, 0};   // resident CTAs of the mixed common path: [24-bit] + 2 [staged]
   int64_t steps = 0;
   // per-kernel event timing (measurement support)
   struct Rec {
@@ -3362,12 +3376,13 @@ extern "C" int fempic_locate(fempic_env* env, const fempic_particles* p, void* s
   return FEMPIC_OK;
 }
 
-// Crossing queue of the mixed form: a 256-record region per tile of 256
-// particles plus a count per tile, grown on demand (every tile count is
-// rewritten by the common path each step, so nothing needs clearing).
-static int ensure_xqueue(fempic_env* env, int64_t n, cudaStream_t st) {
-  const int64_t tiles = (n + kThreads - 1) / kThreads;
-  if (env->xtiles >= tiles) return FEMPIC_OK;
+// Crossing queue: `slots` records in `regions` regions with a count each,
+// grown on demand (every region's count is rewritten by the common path each
+// step, so nothing needs clearing).
+static int ensure_xqueue(fempic_env* env, int64_t slots, int64_t regions, cudaStream_t st) {
+  if (env->xslots >= slots && env->xregions >= regions) return FEMPIC_OK;
+  slots = std::max(slots, env->xslots);
+  regions = std::max(regions, env->xregions);
   if (env->xcount) {
     FEMPIC_CUDA(cudaStreamSynchronize(st));
     cudaFree(env->xrec);
@@ -3376,14 +3391,15 @@ static int ensure_xqueue(fempic_env* env, int64_t n, cudaStream_t st) {
     env->xrec = nullptr;
     env->xrec64 = nullptr;
     env->xcount = nullptr;
-    env->xtiles = 0;
+    env->xslots = env->xregions = 0;
   }
   if (env->opt.precision != FEMPIC_FP64)
-    FEMPIC_CUDA(dalloc(&env->xrec, tiles * kThreads));
+    FEMPIC_CUDA(dalloc(&env->xrec, slots));
   else
-    FEMPIC_CUDA(dalloc(&env->xrec64, tiles * kThreads));
-  FEMPIC_CUDA(dalloc(&env->xcount, tiles));
-  env->xtiles = tiles;
+    FEMPIC_CUDA(dalloc(&env->xrec64, slots));
+  FEMPIC_CUDA(dalloc(&env->xcount, regions));
+  env->xslots = slots;
+  env->xregions = regions;
   return FEMPIC_OK;
 }
 
@@ -3445,24 +3461,6 @@ static int validate_step(const fempic_particles* p, const HostLevels& H, double 
   for (int k = 0; k < H.nl; k++)
     if (!std::isfinite(H.w[k])) return fail(FEMPIC_EINVAL, "push_step: non-finite level weight");
   return fill_species(p, dt, sp);
-}
-
-// Resident CTAs per SM of a mixed crossing pass (1 contract, 2 24-bit),
-// cached per env: the passes hand records out along per-warp streams, so
-// one wave of resident CTAs (no second partial wave) measured fastest
-// (contract pass 0.200 -> 0.186 ms per step at 10M particles).
-static int cross_resident(fempic_env* env, int which, int* out) {
-  int& bps = env->cross_blocks_per_sm[which];
-  if (bps == 0) {
-    int nb = 0;
-    if (which == 1)
-      FEMPIC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_cross_df, kThreads, 0));
-    else
-      FEMPIC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_cross_q24, kThreads, 0));
-    bps = nb > 0 ? nb : 1;
-  }
-  *out = bps;
-  return FEMPIC_OK;
 }
 
 static int push_step_impl(fempic_env* env, const fempic_particles* p, const HostLevels& H, double omega0,
@@ -3555,7 +3553,28 @@ static int push_step_impl(fempic_env* env, const fempic_particles* p, const Host
   A.momlo = env->momlo;
   A.tetdf = env->tetdf;
   A.stats = env->stats;
-  rc = ensure_xqueue(env, p->n, st);
+  // the mixed common path's launch: persistent CTAs, staged when every
+  // particle array allows bulk copies (16-byte aligned sources) and there is
+  // a full tile
+  const int64_t all_tiles = (p->n + kTile - 1) / kTile;
+  int64_t nfull = 0, regions = all_tiles, slots = all_tiles * kTile;
+  if (mixed) {
+    const uintptr_t align = (uintptr_t)p->x | (uintptr_t)p->y | (uintptr_t)p->z | (uintptr_t)p->vx |
+                            (uintptr_t)p->vy | (uintptr_t)p->vz | (uintptr_t)p->tet;
+    nfull = (FEMPIC_USE_TMA && !(align & 15u)) ? p->n / kTile : 0;
+    int& bps = env->push_blocks_per_sm[(q24 ? 1 : 0) + (nfull > 0 ? 2 : 0)];
+    if (bps == 0) {
+      const void* k = nfull > 0 ? (q24 ? (const void*)k_push_mixed_tma<true> : (const void*)k_push_mixed_tma<false>)
+                                : (q24 ? (const void*)k_push_mixed<true> : (const void*)k_push_mixed<false>);
+      int nb = 0;
+      FEMPIC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, kThreads, 0));
+      bps = nb > 0 ? nb : 1;
+    }
+    regions = std::min<int64_t>(all_tiles, (int64_t)env->num_sms * bps);
+    A.xcap = (all_tiles + regions - 1) / regions * kTile;
+    slots = regions * A.xcap;
+  }
+  rc = ensure_xqueue(env, slots, regions, st);
   if (rc) return rc;
   A.xrec = env->xrec;
   A.xrec64 = env->xrec64;
@@ -3566,53 +3585,30 @@ static int push_step_impl(fempic_env* env, const fempic_particles* p, const Host
   {
     LaunchTimer lt(env, st, FEMPIC_K_PUSH);
     if (mixed) {
-      // bulk copies need 16-byte aligned sources: stage full tiles when every
-      // particle array allows it; the ragged tail (or everything) goes plain
-      const uintptr_t align = (uintptr_t)p->x | (uintptr_t)p->y | (uintptr_t)p->z | (uintptr_t)p->vx |
-                              (uintptr_t)p->vy | (uintptr_t)p->vz | (uintptr_t)p->tet;
-      const int64_t ntiles = (FEMPIC_USE_TMA && !(align & 15u)) ? p->n / kTile : 0;
-      if (ntiles > 0) {
-        int& bps = env->tma_blocks_per_sm[q24 ? 1 : 0];
-        if (bps == 0) {
-          int nb = 0;
-          if (q24)
-            FEMPIC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_push_mixed_tma<true>, kThreads, 0));
-          else
-            FEMPIC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_push_mixed_tma<false>, kThreads, 0));
-          bps = nb > 0 ? nb : 1;
-        }
-        const unsigned grid = (unsigned)std::min<int64_t>(ntiles, (int64_t)env->num_sms * bps);
+      const unsigned grid = (unsigned)regions;
+      if (nfull > 0) {
         if (q24)
-          k_push_mixed_tma<true><<<grid, kThreads, 0, st>>>(A, ntiles);
+          k_push_mixed_tma<true><<<grid, kThreads, 0, st>>>(A, nfull);
         else
-          k_push_mixed_tma<false><<<grid, kThreads, 0, st>>>(A, ntiles);
-        lt.kernels++;
-      }
-      const int64_t rest = p->n - ntiles * kTile;
-      if (rest > 0) {
+          k_push_mixed_tma<false><<<grid, kThreads, 0, st>>>(A, nfull);
+      } else {
         if (q24)
-          k_push_mixed<true><<<blocks_for(rest), kThreads, 0, st>>>(A, ntiles * kTile);
+          k_push_mixed<true><<<grid, kThreads, 0, st>>>(A, all_tiles);
         else
-          k_push_mixed<false><<<blocks_for(rest), kThreads, 0, st>>>(A, ntiles * kTile);
-        lt.kernels++;
+          k_push_mixed<false><<<grid, kThreads, 0, st>>>(A, all_tiles);
       }
-      const int64_t all_tiles = (p->n + kTile - 1) / kTile;
-      int cb = 0;
-      rc = cross_resident(env, q24 ? 2 : 1, &cb);
-      if (rc) return rc;
-      const unsigned cross_blocks = (unsigned)std::min<int64_t>((all_tiles + 7) / 8, (int64_t)env->num_sms * cb);
+      lt.kernels = 1;
       LaunchTimer lc(env, st, FEMPIC_K_CROSS);   // nested: also inside the push bracket
       if (q24)
-        k_cross_q24<<<cross_blocks, kThreads, 0, st>>>(A, all_tiles);
+        k_cross_q24<<<grid, kCrossThreadsQ24, 0, st>>>(A);
       else
-        k_cross_df<<<cross_blocks, kThreads, 0, st>>>(A, all_tiles);
+        k_cross_df<<<grid, kCrossThreadsDF, 0, st>>>(A);
       lc.kernels = 1;
     } else {
       k_push_fp64<<<blocks_for(p->n), kThreads, 0, st>>>(A);
       lt.kernels = 1;
       // the FP64 walk is FP64-pipe bound: 8 CTAs per SM queued (about three
       // resident waves) measured faster than one resident wave
-      const int64_t all_tiles = (p->n + kThreads - 1) / kThreads;
       const unsigned cross_blocks = (unsigned)std::min<int64_t>((all_tiles + 7) / 8, (int64_t)env->num_sms * 8);
       LaunchTimer lc(env, st, FEMPIC_K_CROSS);   // nested: also inside the push bracket
       k_cross_fp64<<<cross_blocks, kThreads, 0, st>>>(A, all_tiles);
