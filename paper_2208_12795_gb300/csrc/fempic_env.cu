@@ -81,13 +81,10 @@ struct __align__(16) CrossRec {
   int32_t p;
 };
 
-// FP64-form record of a leaving particle: start point and new velocity in
-// FP64.
+// FP64-form record of a leaving particle: start point (3), new velocity (3),
+// (particle, tet) as the two words of one double, unused.
 struct __align__(16) CrossRec64 {
-  double a[3];
-  double v[3];
-  int32_t T;
-  int32_t p;
+  double2 w[4];
 };
 
 struct PushArgs {
@@ -114,18 +111,17 @@ struct PushArgs {
   const int4* nb;
   const int4* te;
   const void* field;
-  double* dG;                   // FP64 form accumulator [Ne]
   unsigned long long* dGq;      // 24-bit form: per (species, tet) slots of the 6 local edges,
                                 // [ns][nt][8] int64 in units of 2^-48 (q w)
-  double* mom;                  // contract form: per (species, tet) moment slots [ns][nt][6]:
-                                // sum of D (3), sum of u x D (3), FP64
+  double* mom;                  // moment slots: sum of D (3), sum of u x D (3), FP64; contract form
+                                // per (species, tet) [ns][nt][6], FP64 form per tet [nt][6], times q w
   float* momlo;                 // low FP32 parts of the crossing pass's moments [ns][nt][8]
   const float4* tetdf;          // contract form: low FP32 parts of grad lambda_1..3, [nt][4] float4
   unsigned long long* stats;    // [0] crossings, [1] frozen, [2] staging wait timeouts
-  CrossRec* xrec;               // mixed forms: crossing records, one region per common-path CTA
-  CrossRec64* xrec64;           // FP64 form: FP64 records, 256-slot region per tile
+  CrossRec* xrec;               // crossing records, one region per common-path CTA (mixed forms)
+  CrossRec64* xrec64;           // FP64 form: the same, FP64 records
   int32_t* xcount;              // records per region
-  int64_t xcap;                 // mixed forms: slots of a CTA's region (its tiles times 256)
+  int64_t xcap;                 // slots of a CTA's region (its tiles times 256)
   unsigned long long wait_ns;   // limit of each bounded wait of the staged kernel
   int32_t stall_cta;            // test support: this CTA waits on a barrier nothing completes (-1: none)
 };
@@ -385,301 +381,7 @@ __device__ __forceinline__ bool negative_bits(double r) {   // r < 0 for finite 
   return hi < 0 && (((unsigned)hi & 0x7fffffffu) | (unsigned)__double2loint(r)) != 0u;
 }
 
-__device__ __forceinline__ void deposit64(const PushArgs& A, int32_t T, const double la[4], const double lb[4],
-                                          double qw) {
-  if (!A.dG) return;   // deposits off
-  const int4 e0 = __ldg(&A.te[2 * (int64_t)T]), e1 = __ldg(&A.te[2 * (int64_t)T + 1]);
-  const int32_t eid[6] = {e0.x, e0.y, e0.z, e0.w, e1.x, e1.y};
-#pragma unroll
-  for (int e = 0; e < 6; e++) {
-    const int i = le0(e), j = le1(e);
-    const double g = qw * fma(la[i], lb[j], -(la[j] * lb[i]));
-    if (idx_in(eid[e], A.ne, A.stats)) atomicAdd(A.dG + eid[e], g);
-  }
-}
-
 __device__ __forceinline__ int4 ldg_int4(const int4* p) { return __ldg(p); }
-
-// FP64 form, common path: one particle per thread (a block is one 256-particle
-// tile).  Gather, Boris, position update and the barycentrics of both ends
-// in the home tet; a particle that stays deposits its segment and is done; a
-// particle that leaves stores its new state provisionally and a record for
-// the crossing pass, so the face walk does not run here with most lanes idle.
-__global__ void __launch_bounds__(kThreads) k_push_fp64(PushArgs A) {
-  __shared__ int32_t total;
-  const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const int lane = threadIdx.x & 31;
-  const unsigned full = 0xffffffffu;
-  if (threadIdx.x == 0) total = 0;
-  __syncthreads();
-  unsigned nfrz = 0;
-  bool leave = false;
-  double a[3] = {0.0, 0.0, 0.0}, vn[3] = {0.0, 0.0, 0.0};
-  int32_t T = -1;
-  if (p < A.n) {
-    T = A.tet[p];
-    if (T >= A.nt) {
-      A.tet[p] = -1;
-      A.status[p] = FEMPIC_P_LOST;
-      nfrz = 1;
-    } else if (T >= 0) {
-      const int s = species_of(A.sp, p);
-      const double kq = A.sp.kq[s], qw = A.sp.qw[s];
-      double* vxp = static_cast<double*>(A.vx);
-      double* vyp = static_cast<double*>(A.vy);
-      double* vzp = static_cast<double*>(A.vz);
-      a[0] = A.x[p];
-      a[1] = A.y[p];
-      a[2] = A.z[p];
-      const double v[3] = {vxp[p], vyp[p], vzp[p]};
-      const double* G = A.geom64 + 12 * (int64_t)T;
-      const double2* F = reinterpret_cast<const double2*>(static_cast<const double*>(A.field) + 10 * (int64_t)T);
-      const double2 f0 = __ldg(F), f1 = __ldg(F + 1), f2 = __ldg(F + 2), f3 = __ldg(F + 3), f4 = __ldg(F + 4);
-      const double dx = a[0] - __ldg(G), dy = a[1] - __ldg(G + 1), dz = a[2] - __ldg(G + 2);
-      // (b)+(c) gather with the carrier already restored per tet
-      const double Wx = f1.y, Wy = f2.x, Wz = f2.y;
-      const double Ex = f0.x + (dy * Wz - dz * Wy);
-      const double Ey = f0.y + (dz * Wx - dx * Wz);
-      const double Ez = f1.x + (dx * Wy - dy * Wx);
-      const double beta = f4.y;
-      const double Bx = f3.x + beta * dx, By = f3.y + beta * dy, Bz = f4.x + beta * dz;
-      // (d) Boris
-      const double vmx = v[0] + kq * Ex, vmy = v[1] + kq * Ey, vmz = v[2] + kq * Ez;
-      const double tx = kq * Bx, ty = kq * By, tz = kq * Bz;
-      const double t2 = tx * tx + ty * ty + tz * tz;
-      const double f = 2.0 / (1.0 + t2);
-      const double sx = f * tx, sy = f * ty, sz = f * tz;
-      const double vpx = vmx + (vmy * tz - vmz * ty);
-      const double vpy = vmy + (vmz * tx - vmx * tz);
-      const double vpz = vmz + (vmx * ty - vmy * tx);
-      vn[0] = vmx + (vpy * sz - vpz * sy) + kq * Ex;
-      vn[1] = vmy + (vpz * sx - vpx * sz) + kq * Ey;
-      vn[2] = vmz + (vpx * sy - vpy * sx) + kq * Ez;
-      const double b[3] = {fma(A.dt, vn[0], a[0]), fma(A.dt, vn[1], a[1]), fma(A.dt, vn[2], a[2])};
-      if (!(finite_bits(vn[0]) && finite_bits(vn[1]) && finite_bits(vn[2]) && finite_bits(b[0]) &&
-            finite_bits(b[1]) && finite_bits(b[2]))) {
-        A.status[p] = FEMPIC_P_NONFINITE;
-        A.tet[p] = -2 - T;
-        nfrz = 1;
-      } else {
-        double la[4], lb[4];
-        bary64_d(G, dx, dy, dz, la);
-        bary64(G, b, lb);
-        A.x[p] = b[0];
-        A.y[p] = b[1];
-        A.z[p] = b[2];
-        vxp[p] = vn[0];
-        vyp[p] = vn[1];
-        vzp[p] = vn[2];
-        leave = negative_bits(lb[0]) || negative_bits(lb[1]) || negative_bits(lb[2]) || negative_bits(lb[3]);
-        if (!leave) deposit64(A, T, la, lb, qw);   // (f) the whole segment is in the home tet
-      }
-    }
-  }
-  // (e) leaving particles: records for the crossing pass, in the block's region
-  const unsigned qmask = __ballot_sync(full, leave);
-  if (qmask) {
-    int base = 0;
-    if (lane == 0) base = atomicAdd(&total, __popc(qmask));
-    base = __shfl_sync(full, base, 0);
-    if (leave) {
-      CrossRec64& r = A.xrec64[blockIdx.x * (int64_t)kThreads + base + __popc(qmask & ((1u << lane) - 1u))];
-      r.a[0] = a[0];
-      r.a[1] = a[1];
-      r.a[2] = a[2];
-      r.v[0] = vn[0];
-      r.v[1] = vn[1];
-      r.v[2] = vn[2];
-      r.T = T;
-      r.p = (int32_t)p;
-    }
-  }
-  nfrz = __reduce_add_sync(full, nfrz);
-  if (lane == 0 && nfrz) atomicAdd(A.stats + 1, (unsigned long long)nfrz);
-  __syncthreads();
-  if (threadIdx.x == 0) A.xcount[blockIdx.x] = total;
-}
-
-// FP64 form, crossing pass: the walk of one leaving particle, one face per
-// call, in FP64 (the paper's exit parameter s_k = la_k / (la_k - lb_k), the
-// crossing point a + s (b - a), barycentrics carried exactly onto the
-// neighbour's shared nodes).
-struct CrossState64 {
-  double a[3], b[3], vn[3];
-  double la[4], lb[4];
-  int32_t T, p;
-  int entry, nc, s;
-  uint8_t st;
-  bool reflected;
-};
-
-__device__ __forceinline__ void cross64_begin(const PushArgs& A, const CrossRec64& r, CrossState64& c) {
-  c.p = r.p;
-  c.T = r.T;
-  c.s = species_of(A.sp, r.p);
-#pragma unroll
-  for (int k = 0; k < 3; k++) {
-    c.a[k] = r.a[k];
-    c.vn[k] = r.v[k];
-    c.b[k] = fma(A.dt, r.v[k], r.a[k]);
-  }
-  const double* G = A.geom64 + 12 * (int64_t)c.T;
-  bary64(G, c.a, c.la);
-  bary64(G, c.b, c.lb);
-  c.entry = -1;
-  c.nc = 0;
-  c.st = FEMPIC_P_OK;
-  c.reflected = false;
-}
-
-__device__ __forceinline__ bool cross64_advance(const PushArgs& A, CrossState64& c) {
-  const double qw = A.sp.qw[c.s];
-  int kx = -1;
-  double smin = INFINITY;
-#pragma unroll
-  for (int k = 0; k < 4; k++) {
-    if (k == c.entry || !negative_bits(c.lb[k])) continue;
-    double sk = c.la[k] / (c.la[k] - c.lb[k]);
-    if (sk < 0.0) sk = 0.0;
-    if (sk < smin) {
-      smin = sk;
-      kx = k;
-    }
-  }
-  if (kx < 0) {
-    deposit64(A, c.T, c.la, c.lb, qw);
-#pragma unroll
-    for (int k = 0; k < 3; k++) c.a[k] = c.b[k];
-    return true;
-  }
-  double lp[4];
-#pragma unroll
-  for (int i = 0; i < 4; i++) lp[i] = (i == kx) ? 0.0 : fma(smin, c.lb[i] - c.la[i], c.la[i]);
-  deposit64(A, c.T, c.la, lp, qw);
-  c.nc++;
-#pragma unroll
-  for (int k = 0; k < 3; k++) c.a[k] = fma(smin, c.b[k] - c.a[k], c.a[k]);
-  if (c.nc > A.max_cross) {
-    c.st = FEMPIC_P_CAP;
-    return true;
-  }
-  const int4 nbv = ldg_int4(&A.nb[c.T]);
-  const int32_t nbt = kx == 0 ? nbv.x : kx == 1 ? nbv.y : kx == 2 ? nbv.z : nbv.w;
-  if (nbt >= 0 && !idx_in(nbt, A.nt, A.stats)) {
-    c.st = FEMPIC_P_LOST;
-    return true;
-  }
-  if (nbt >= 0) {
-    const int4 o4 = ldg_int4(&A.tn[c.T]), n4 = ldg_int4(&A.tn[nbt]);
-    const int32_t on[4] = {o4.x, o4.y, o4.z, o4.w}, nn[4] = {n4.x, n4.y, n4.z, n4.w};
-    int ent = 0;
-#pragma unroll
-    for (int i2 = 0; i2 < 4; i2++) {
-      int hit = -1;
-#pragma unroll
-      for (int i = 0; i < 4; i++)
-        if (on[i] == nn[i2]) hit = i;
-      double val = 0.0;
-#pragma unroll
-      for (int i = 0; i < 4; i++)
-        if (i == hit) val = lp[i];
-      c.la[i2] = val;
-      if (hit < 0) ent = i2;
-    }
-    c.T = nbt;
-    c.entry = ent;
-  } else if (nbt <= -1 && nbt >= -6 && A.wall_mode == FEMPIC_WALL_REFLECT) {
-    const int code = -1 - nbt, ax = code >> 1, side = code & 1;
-#pragma unroll
-    for (int k = 0; k < 3; k++)
-      if (k == ax) {
-        const double L = side ? A.hi[k] : A.lo[k];
-        c.b[k] = 2.0 * L - c.b[k];
-        c.vn[k] = -c.vn[k];
-      }
-    c.reflected = true;
-#pragma unroll
-    for (int i = 0; i < 4; i++) c.la[i] = lp[i];
-    c.entry = kx;
-  } else {
-    c.st = FEMPIC_P_ABSORBED;
-    return true;
-  }
-  bary64(A.geom64 + 12 * (int64_t)c.T, c.b, c.lb);
-  return false;
-}
-
-__device__ __forceinline__ void cross64_finish(const PushArgs& A, const CrossState64& c, unsigned& ncr,
-                                               unsigned& nfrz) {
-  const int64_t p = c.p;
-  if (c.st != FEMPIC_P_OK || c.reflected) {   // otherwise a = b, already stored
-    A.x[p] = c.a[0];
-    A.y[p] = c.a[1];
-    A.z[p] = c.a[2];
-  }
-  if (c.reflected) {
-    static_cast<double*>(A.vx)[p] = c.vn[0];
-    static_cast<double*>(A.vy)[p] = c.vn[1];
-    static_cast<double*>(A.vz)[p] = c.vn[2];
-  }
-  int32_t T = c.T;
-  if (c.st != FEMPIC_P_OK) {
-    A.status[p] = c.st;
-    T = -2 - T;
-    nfrz++;
-  }
-  A.tet[p] = T;
-  if (A.ncross) A.ncross[p] += c.nc;
-  ncr += (unsigned)c.nc;
-}
-
-// One warp per group of tile regions (grid stride): the warp's tiles form one
-// record stream, and lanes take the next record, across tile boundaries,
-// when their particle is done.  The FP64 walk is FP64-pipe bound, so lanes
-// left idle at the end of a tile would cost pipe cycles (the latency-bound
-// mixed pass keeps the per-tile loop, which measured faster there).
-__global__ void __launch_bounds__(kThreads) k_cross_fp64(PushArgs A, int64_t ntiles) {
-  const unsigned full = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
-  const unsigned lt = (1u << lane) - 1u;
-  unsigned ncr = 0, nfrz = 0;
-  const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  int64_t tile = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  int32_t cnt = tile < ntiles ? A.xcount[tile] : 0, next = 0;
-  bool have = false;
-  CrossState64 c;
-  for (;;) {
-    unsigned idle = __ballot_sync(full, !have);
-    while (idle && tile < ntiles) {   // warp-uniform: assigns records or advances a tile
-      const int32_t avail = cnt - next;
-      const int32_t want = __popc(idle);
-      const int32_t take = avail < want ? avail : want;
-      const int r = __popc(idle & lt);
-      if (!have && r < take) {
-        cross64_begin(A, A.xrec64[tile * kThreads + next + r], c);
-        have = true;
-      }
-      next += take;
-      idle = __ballot_sync(full, !have);
-      if (next == cnt) {
-        tile += warps;
-        cnt = tile < ntiles ? A.xcount[tile] : 0;
-        next = 0;
-      }
-    }
-    if (!__any_sync(full, have)) break;
-    if (have && cross64_advance(A, c)) {
-      cross64_finish(A, c, ncr, nfrz);
-      have = false;
-    }
-  }
-  ncr = __reduce_add_sync(full, ncr);
-  nfrz = __reduce_add_sync(full, nfrz);
-  if (lane == 0) {
-    if (ncr) atomicAdd(A.stats, (unsigned long long)ncr);
-    if (nfrz) atomicAdd(A.stats + 1, (unsigned long long)nfrz);
-  }
-}
 
 // ------------------------------------------------------------ mixed push
 // Two FP32-mixed forms share the per-tet record, the gather, the carrier
@@ -1957,6 +1659,397 @@ __global__ void __launch_bounds__(kCrossThreadsDF, 4) k_cross_df(PushArgs A) {
   }
 }
 
+// ------------------------------------------------------------ FP64 form
+// The FP64 pipe (1/64 of the FP32 rate) is the bound, so the common path
+// spends FP64 operations only where a result needs them, about 60 lane
+// operations per particle: gather and Boris as chained multiply-adds, one
+// reciprocal refined from an FP32 seed, the deposit in moment form (D = b -
+// a and u x D: 15 operations against 39 for two sets of barycentrics and six
+// edge products), and the inside test in FP32 against the tet's error bound.
+// A particle that test cannot place goes to the crossing pass, which decides
+// in FP64, so tets are those of the FP64 barycentrics.  Against barycentrics
+// of both ends and six edge products per particle (116 operations): 0.390 ->
+// 0.219 ms at 2M particles (the crossing pass 0.125 -> 0.067); four steps and
+// a sort of 6M electrons on 40^3 x 6 tets 6.88 -> 4.31 ms.  Rounding of the
+// moment form against 80-bit sums over such tets: 3e-16 of the edge values'
+// norm (1.8e-15 for the barycentric form).
+
+// Leading 24 bits of an FP64 value as a float (truncated, so at most 2^-23
+// relative below it in magnitude): 0 below 2^-126, infinite from 2^128 on.
+__device__ __forceinline__ float trunc32(double r) {
+  const unsigned hi = (unsigned)__double2hiint(r), lo = (unsigned)__double2loint(r);
+  const unsigned e = (hi >> 20) & 0x7ffu, sign = hi & 0x80000000u;
+  if (e < 897u) return 0.f;
+  if (e > 1150u) return __uint_as_float(sign | 0x7f800000u);
+  return __uint_as_float(sign | ((e - 896u) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29));
+}
+
+// 1 / w for w >= 1 to about one ulp: an FP32 reciprocal (relative error e
+// below 2^-21) and one step r (1 + e + e^2) of the residual series, whose
+// remainder e^3 lies below an FP64 ulp.  Past the FP32 range (and for a
+// non-finite w) the division.
+__device__ __forceinline__ double recip_ge1(double w) {
+  if ((unsigned)__double2hiint(w) >= (1143u << 20)) return 1.0 / w;
+  const double r = f32_to_f64(__fdividef(1.0f, trunc32(w)));
+  const double e = fma(-w, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+
+// Moment-form deposit of the straight piece a -> a + D inside tet T, u = a -
+// x0: q w D and q w (u x D) into the tet's slot (six adjacent FP64
+// reductions); k_tet_finalize64 turns them into the six edges' values.
+__device__ __forceinline__ void deposit64(const PushArgs& A, int32_t T, const double u[3], const double D[3],
+                                          double qw) {
+  if (!A.mom) return;   // deposits off
+  const double d[3] = {qw * D[0], qw * D[1], qw * D[2]};
+  double* ms = A.mom + 6 * (int64_t)T;
+#pragma unroll
+  for (int k = 0; k < 3; k++) {
+    const int i = (k + 1) % 3, j = (k + 2) % 3;
+    atomicAdd(ms + k, d[k]);
+    atomicAdd(ms + 3 + k, fma(u[i], d[j], -(u[j] * d[i])));
+  }
+}
+
+__device__ __forceinline__ CrossRec64* xregion64(const PushArgs& A) { return A.xrec64 + blockIdx.x * A.xcap; }
+
+// FP64 form, common path: persistent CTAs walk 256-particle tiles, one
+// particle per thread.  A particle surely inside its home tet deposits its
+// segment and is done; any other stores its new state provisionally and a
+// record for the crossing pass.
+__global__ void __launch_bounds__(kThreads) k_push_fp64(PushArgs A, int64_t ntiles) {
+  __shared__ int32_t total;
+  const int lane = threadIdx.x & 31;
+  const unsigned full = 0xffffffffu;
+  if (threadIdx.x == 0) total = 0;
+  __syncthreads();
+  unsigned nfrz = 0;
+  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const int64_t p = tile * kTile + threadIdx.x;
+    bool leave = false;
+    double a[3] = {0.0, 0.0, 0.0}, vn[3] = {0.0, 0.0, 0.0};
+    int32_t T = -1;
+    if (p < A.n) {
+      T = A.tet[p];
+      if (T >= A.nt) {
+        A.tet[p] = -1;
+        A.status[p] = FEMPIC_P_LOST;
+        nfrz++;
+      } else if (T >= 0) {
+        const int s = species_of(A.sp, p);
+        const double kq = A.sp.kq[s];
+        double* vxp = static_cast<double*>(A.vx);
+        double* vyp = static_cast<double*>(A.vy);
+        double* vzp = static_cast<double*>(A.vz);
+        a[0] = A.x[p];
+        a[1] = A.y[p];
+        a[2] = A.z[p];
+        const double v[3] = {vxp[p], vyp[p], vzp[p]};
+        const Geo32 G = ld_geo(A.tetrec, T);   // x0 exact; FP32 gradients and error bound for the inside test
+        const double2* F = reinterpret_cast<const double2*>(static_cast<const double*>(A.field) + 10 * (int64_t)T);
+        const double2 f0 = __ldg(F), f1 = __ldg(F + 1), f2 = __ldg(F + 2), f3 = __ldg(F + 3), f4 = __ldg(F + 4);
+        const double d[3] = {a[0] - G.x0[0], a[1] - G.x0[1], a[2] - G.x0[2]};
+        // (b)+(c) gather with the carrier already restored per tet
+        const double Wx = f1.y, Wy = f2.x, Wz = f2.y, beta = f4.y;
+        const double Ex = fma(d[1], Wz, fma(-d[2], Wy, f0.x));
+        const double Ey = fma(d[2], Wx, fma(-d[0], Wz, f0.y));
+        const double Ez = fma(d[0], Wy, fma(-d[1], Wx, f1.x));
+        // (d) Boris
+        const double vmx = fma(kq, Ex, v[0]), vmy = fma(kq, Ey, v[1]), vmz = fma(kq, Ez, v[2]);
+        const double tx = kq * fma(beta, d[0], f3.x), ty = kq * fma(beta, d[1], f3.y), tz = kq * fma(beta, d[2], f4.x);
+        const double f = 2.0 * recip_ge1(fma(tx, tx, fma(ty, ty, fma(tz, tz, 1.0))));
+        const double sx = f * tx, sy = f * ty, sz = f * tz;
+        const double vpx = fma(vmy, tz, fma(-vmz, ty, vmx));
+        const double vpy = fma(vmz, tx, fma(-vmx, tz, vmy));
+        const double vpz = fma(vmx, ty, fma(-vmy, tx, vmz));
+        vn[0] = fma(kq, Ex, fma(vpy, sz, fma(-vpz, sy, vmx)));
+        vn[1] = fma(kq, Ey, fma(vpz, sx, fma(-vpx, sz, vmy)));
+        vn[2] = fma(kq, Ez, fma(vpx, sy, fma(-vpy, sx, vmz)));
+        const double b[3] = {fma(A.dt, vn[0], a[0]), fma(A.dt, vn[1], a[1]), fma(A.dt, vn[2], a[2])};
+        if (!(finite_bits(vn[0]) && finite_bits(vn[1]) && finite_bits(vn[2]) && finite_bits(b[0]) &&
+              finite_bits(b[1]) && finite_bits(b[2]))) {
+          A.status[p] = FEMPIC_P_NONFINITE;
+          A.tet[p] = -2 - T;
+          nfrz++;
+        } else {
+          A.x[p] = b[0];
+          A.y[p] = b[1];
+          A.z[p] = b[2];
+          vxp[p] = vn[0];
+          vyp[p] = vn[1];
+          vzp[p] = vn[2];
+          const double D[3] = {b[0] - a[0], b[1] - a[1], b[2] - a[2]};
+          // inside when all four FP32 barycentrics of b reach kappa, the
+          // bound on their error for a start in the tet (|lambda(a)| is
+          // checked too: a start far outside would void the bound)
+          float lo = INFINITY, la = INFINITY;
+          {
+            const float d32[3] = {trunc32(d[0]), trunc32(d[1]), trunc32(d[2])};
+            const float e32[3] = {d32[0] + trunc32(D[0]), d32[1] + trunc32(D[1]), d32[2] + trunc32(D[2])};
+            float sb = 1.0f, sa = 1.0f;
+#pragma unroll
+            for (int k = 0; k < 3; k++) {
+              const float lb = G.g[3 * k] * e32[0] + G.g[3 * k + 1] * e32[1] + G.g[3 * k + 2] * e32[2];
+              const float l0 = G.g[3 * k] * d32[0] + G.g[3 * k + 1] * d32[1] + G.g[3 * k + 2] * d32[2];
+              sb -= lb;
+              sa -= l0;
+              lo = fminf(lo, lb);
+              la = fminf(la, l0);
+            }
+            leave = !(fminf(lo, sb) >= G.kappa && fminf(la, sa) >= -1.0f);
+          }
+          if (!leave) deposit64(A, T, d, D, A.sp.qw[s]);   // (f) the whole segment is in the home tet
+        }
+      }
+    }
+    // (e) the others: records for the crossing pass, in the CTA's region
+    const unsigned qmask = __ballot_sync(full, leave);
+    if (qmask) {
+      int base = 0;
+      if (lane == 0) base = atomicAdd(&total, __popc(qmask));
+      base = __shfl_sync(full, base, 0);
+      if (leave) {
+        double2* r = xregion64(A)[base + __popc(qmask & ((1u << lane) - 1u))].w;
+        r[0] = make_double2(a[0], a[1]);
+        r[1] = make_double2(a[2], vn[0]);
+        r[2] = make_double2(vn[1], vn[2]);
+        r[3] = make_double2(__hiloint2double((int32_t)p, T), 0.0);
+      }
+    }
+  }
+  nfrz = __reduce_add_sync(full, nfrz);
+  if (lane == 0 && nfrz) atomicAdd(A.stats + 1, (unsigned long long)nfrz);
+  __syncthreads();
+  if (threadIdx.x == 0) A.xcount[blockIdx.x] = total;
+}
+
+// FP64 form, crossing pass: the walk of one leaving particle, one face per
+// call, in FP64 (the paper's exit parameter s_k = la_k / (la_k - lb_k), the
+// crossing point a + s (b - a), barycentrics carried exactly onto the
+// neighbour's shared nodes).
+struct CrossState64 {
+  double a[3], b[3], vn[3];
+  double la[4], lb[4];
+  int32_t T, p;
+  int entry, nc, s;
+  uint8_t st;
+  bool reflected;
+};
+
+__device__ __forceinline__ void cross64_begin(const PushArgs& A, const CrossRec64& rec, CrossState64& c) {
+  const double2 r0 = rec.w[0], r1 = rec.w[1], r2 = rec.w[2], r3 = rec.w[3];
+  c.p = __double2hiint(r3.x);
+  c.T = __double2loint(r3.x);
+  c.s = species_of(A.sp, c.p);
+  c.a[0] = r0.x;
+  c.a[1] = r0.y;
+  c.a[2] = r1.x;
+  c.vn[0] = r1.y;
+  c.vn[1] = r2.x;
+  c.vn[2] = r2.y;
+#pragma unroll
+  for (int k = 0; k < 3; k++) c.b[k] = fma(A.dt, c.vn[k], c.a[k]);
+  c.entry = -1;
+  c.nc = 0;
+  c.st = FEMPIC_P_OK;
+  c.reflected = false;
+}
+
+// Exit face of the piece with end barycentrics la -> lb (entry face
+// excluded): the smallest s_k = la_k / (la_k - lb_k) clamped at 0, the lowest
+// face on ties, -1 when the piece stays inside.  FP32 quotients order the
+// faces (relative error below 2^-20: la >= 0 > lb, so la - lb does not
+// cancel) and one FP64 division serves the winner; where two faces come
+// within 2^-17, a start lies outside (la < 0) or a quotient is not finite,
+// every face is divided in FP64.
+__device__ __forceinline__ int exit_face64(const double la[4], const double lb[4], int entry, double& smin) {
+  float q1 = INFINITY, q2 = INFINITY;
+  bool close = false;
+  int kx = -1;
+  double a = 0.0, b = 0.0;
+#pragma unroll
+  for (int k = 0; k < 4; k++) {
+    if (k == entry || !negative_bits(lb[k])) continue;
+    const float x = trunc32(la[k]), y = trunc32(lb[k]);
+    const float q = __fdividef(x, x - y);
+    close = close || !(q >= 0.f && q < INFINITY) || negative_bits(la[k]);
+    if (q < q1) {
+      q2 = q1;
+      q1 = q;
+      kx = k;
+      a = la[k];
+      b = lb[k];
+    } else {
+      q2 = fminf(q2, q);
+    }
+  }
+  smin = INFINITY;
+  if (close || (kx >= 0 && q2 <= q1 + q1 * 0x1p-17f)) {
+    kx = -1;
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+      if (k == entry || !negative_bits(lb[k])) continue;
+      double sk = la[k] / (la[k] - lb[k]);
+      if (sk < 0.0) sk = 0.0;
+      if (sk < smin) {
+        smin = sk;
+        kx = k;
+      }
+    }
+  } else if (kx >= 0) {
+    smin = a / (a - b);
+  }
+  return kx;
+}
+
+__device__ __forceinline__ bool cross64_advance(const PushArgs& A, CrossState64& c, bool fresh) {
+  const double qw = A.sp.qw[c.s];
+  double u[3];   // piece start - x0 of this tet
+  {
+    const double* g = A.geom64 + 12 * (int64_t)c.T;
+    const double x0[3] = {__ldg(g), __ldg(g + 1), __ldg(g + 2)};
+#pragma unroll
+    for (int k = 0; k < 3; k++) u[k] = c.a[k] - x0[k];
+    if (fresh) bary64_d(g, u[0], u[1], u[2], c.la);
+    bary64_d(g, c.b[0] - x0[0], c.b[1] - x0[1], c.b[2] - x0[2], c.lb);
+  }
+  double smin;
+  const int kx = exit_face64(c.la, c.lb, c.entry, smin);
+  double D[3];
+#pragma unroll
+  for (int k = 0; k < 3; k++) D[k] = c.b[k] - c.a[k];
+  if (kx < 0) {
+    deposit64(A, c.T, u, D, qw);
+#pragma unroll
+    for (int k = 0; k < 3; k++) c.a[k] = c.b[k];
+    return true;
+  }
+  double lp[4];
+#pragma unroll
+  for (int i = 0; i < 4; i++) lp[i] = (i == kx) ? 0.0 : fma(smin, c.lb[i] - c.la[i], c.la[i]);
+#pragma unroll
+  for (int k = 0; k < 3; k++) {
+    const double q = fma(smin, D[k], c.a[k]);
+    D[k] = q - c.a[k];
+    c.a[k] = q;
+  }
+  deposit64(A, c.T, u, D, qw);
+  c.nc++;
+  if (c.nc > A.max_cross) {
+    c.st = FEMPIC_P_CAP;
+    return true;
+  }
+  const int4 nbv = ldg_int4(&A.nb[c.T]);
+  const int32_t nbt = kx == 0 ? nbv.x : kx == 1 ? nbv.y : kx == 2 ? nbv.z : nbv.w;
+  if (nbt >= 0 && !idx_in(nbt, A.nt, A.stats)) {
+    c.st = FEMPIC_P_LOST;
+    return true;
+  }
+  if (nbt >= 0) {
+    const int4 o4 = ldg_int4(&A.tn[c.T]), n4 = ldg_int4(&A.tn[nbt]);
+    const int32_t on[4] = {o4.x, o4.y, o4.z, o4.w}, nn[4] = {n4.x, n4.y, n4.z, n4.w};
+    int ent = 0;
+#pragma unroll
+    for (int i2 = 0; i2 < 4; i2++) {
+      int hit = -1;
+#pragma unroll
+      for (int i = 0; i < 4; i++)
+        if (on[i] == nn[i2]) hit = i;
+      double val = 0.0;
+#pragma unroll
+      for (int i = 0; i < 4; i++)
+        if (i == hit) val = lp[i];
+      c.la[i2] = val;
+      if (hit < 0) ent = i2;
+    }
+    c.T = nbt;
+    c.entry = ent;
+  } else if (nbt <= -1 && nbt >= -6 && A.wall_mode == FEMPIC_WALL_REFLECT) {
+    const int code = -1 - nbt, ax = code >> 1, side = code & 1;
+#pragma unroll
+    for (int k = 0; k < 3; k++)
+      if (k == ax) {
+        const double L = side ? A.hi[k] : A.lo[k];
+        c.b[k] = 2.0 * L - c.b[k];
+        c.vn[k] = -c.vn[k];
+      }
+    c.reflected = true;
+#pragma unroll
+    for (int i = 0; i < 4; i++) c.la[i] = lp[i];
+    c.entry = kx;
+  } else {
+    c.st = FEMPIC_P_ABSORBED;
+    return true;
+  }
+  return false;
+}
+
+__device__ __forceinline__ void cross64_finish(const PushArgs& A, const CrossState64& c, unsigned& ncr,
+                                               unsigned& nfrz) {
+  const int64_t p = c.p;
+  if (c.st != FEMPIC_P_OK || c.reflected) {   // otherwise a = b, already stored
+    A.x[p] = c.a[0];
+    A.y[p] = c.a[1];
+    A.z[p] = c.a[2];
+  }
+  if (c.reflected) {
+    static_cast<double*>(A.vx)[p] = c.vn[0];
+    static_cast<double*>(A.vy)[p] = c.vn[1];
+    static_cast<double*>(A.vz)[p] = c.vn[2];
+  }
+  int32_t T = c.T;
+  if (c.st != FEMPIC_P_OK) {
+    A.status[p] = c.st;
+    T = -2 - T;
+    nfrz++;
+  }
+  A.tet[p] = T;
+  if (A.ncross) A.ncross[p] += c.nc;
+  ncr += (unsigned)c.nc;
+}
+
+// One CTA per record region, records drawn from a shared cursor (as the mixed
+// passes).
+constexpr int kCrossThreads64 = 192;
+__global__ void __launch_bounds__(kCrossThreads64) k_cross_fp64(PushArgs A) {
+  __shared__ int32_t cursor;
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const CrossRec64* rec = xregion64(A);
+  const int32_t cnt = A.xcount[blockIdx.x];
+  if (threadIdx.x == 0) cursor = 0;
+  __syncthreads();
+  unsigned ncr = 0, nfrz = 0;
+  bool have = false, fresh = false, more = cnt > 0;
+  CrossState64 c;
+  for (;;) {
+    const unsigned idle = __ballot_sync(full, !have);
+    if (more && __popc(idle) >= kRefill) {
+      const int32_t k = draw_record(idle, lane, have, cnt, &cursor, more);
+      if (k >= 0) {
+        cross64_begin(A, rec[k], c);
+        have = true;
+        fresh = true;
+      }
+    }
+    if (!__any_sync(full, have)) break;
+    if (have) {
+      const bool done = cross64_advance(A, c, fresh);
+      fresh = false;
+      if (done) {
+        cross64_finish(A, c, ncr, nfrz);
+        have = false;
+      }
+    }
+  }
+  ncr = __reduce_add_sync(full, ncr);
+  nfrz = __reduce_add_sync(full, nfrz);
+  if (lane == 0) {
+    if (ncr) atomicAdd(A.stats, (unsigned long long)ncr);
+    if (nfrz) atomicAdd(A.stats + 1, (unsigned long long)nfrz);
+  }
+}
+
 // ------------------------------------------------------- deposit finalize
 // Contract form, per tet: the moment slots (sum of D, sum of u x D, FP64)
 // become the 6 local-edge values through the tet's gradients,
@@ -2041,17 +2134,44 @@ __global__ void __launch_bounds__(kThreads) k_tet_finalize(TetFinalizeArgs A) {
   o[2] = make_float4(g[4].h, g[4].l, g[5].h, g[5].l);
 }
 
+// FP64 form, per tet: the same conversion in FP64 (the slots already hold
+// q w times the moments): with c_ij = G_i x G_j and G_0 = -(G_1 + G_2 + G_3),
+// three products M . c_12, M . c_13, M . c_23 give all six edges' moment
+// parts.  Slots are read and cleared once per deposit; tets without particles
+// stop at their zero slot.
+__global__ void __launch_bounds__(kThreads) k_tet_finalize64(int64_t nt, const double* __restrict__ geom64,
+                                                              double* __restrict__ mom, double* __restrict__ out) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (t >= nt) return;
+  double2* m2 = reinterpret_cast<double2*>(mom + 6 * t);
+  double2* o = reinterpret_cast<double2*>(out + 6 * t);
+  const double2 a = m2[0], b = m2[1], c = m2[2];
+  const double2 z2 = make_double2(0.0, 0.0);
+  if (a.x == 0.0 && a.y == 0.0 && b.x == 0.0 && b.y == 0.0 && c.x == 0.0 && c.y == 0.0) {
+    o[0] = o[1] = o[2] = z2;
+    return;
+  }
+  m2[0] = m2[1] = m2[2] = z2;
+  const V3<double> S = {a.x, a.y, b.x}, M = {b.y, c.x, c.y};
+  const double* G = geom64 + 12 * t;
+  const V3<double> g1 = {G[3], G[4], G[5]}, g2 = {G[6], G[7], G[8]}, g3 = {G[9], G[10], G[11]};
+  const double m12 = vdot(vcross(g1, g2), M), m13 = vdot(vcross(g1, g3), M), m23 = vdot(vcross(g2, g3), M);
+  o[0] = make_double2(vdot(g1, S) + (m12 + m13), vdot(g2, S) + (m23 - m12));
+  o[1] = make_double2(vdot(g3, S) - (m13 + m23), m12);
+  o[2] = make_double2(m13, m23);
+}
+
 struct FinalizeArgs {
   int64_t ne;
   int64_t nt;
-  const int32_t* estart;         // mixed forms: edge -> (tet, local edge) slots
+  const int32_t* estart;         // edge -> (tet, local edge) slots
   const int32_t* eslot;
-  int32_t mode;                  // 0 FP64 accumulator, 1 contract form (per-tet pairs), 2 24-bit form
+  int32_t mode;                  // 0 FP64 form (per-tet values), 1 contract form (per-tet pairs), 2 24-bit form
   int32_t ns;
   double qwscale[kMaxSpecies];   // q w 2^-48 per species (24-bit form)
-  double* dG;
   const unsigned long long* dGq;  // 24-bit form: deposit slots [ns][nt][8]
-  const float* tetout;           // contract form: [nt][12] (h, l) pairs of the 6 local edges
+  const void* tetout;            // the 6 local edges' values per tet: FP64 form [nt][6] f64, contract
+                                 // form [nt][6] (h, l) pairs
   double* Gcum;
   double* dG_out;
   double* Gcum_out;
@@ -2061,12 +2181,12 @@ struct FinalizeArgs {
   unsigned long long* stats;     // bounds checks of the debug build
 };
 
-// Deposit finalize, one thread per edge.  The mixed forms pull the edge's
-// values from its tets (adjacency built once on the host, a fixed order):
-// the 24-bit form its exact int64 sums from the integer slots, scaled by
-// q w 2^-48 (the slots are cleared afterwards by one coalesced memset); the
-// contract form its tets' double-float values from k_tet_finalize.  FP64
-// form: the edge's FP64 accumulator.  Then G_cum += dG and the requested
+// Deposit finalize, one thread per edge: pulls the edge's values from its
+// tets (adjacency built once on the host, a fixed order): the 24-bit form its
+// exact int64 sums from the integer slots, scaled by q w 2^-48 (the slots are
+// cleared afterwards by one coalesced memset); the contract form its tets'
+// double-float values from k_tet_finalize; the FP64 form its tets' FP64
+// values from k_tet_finalize64.  Then G_cum += dG and the requested
 // outputs (dG, G_cum, the envelope-frame G~).
 __global__ void __launch_bounds__(kThreads) k_deposit_finalize(FinalizeArgs A) {
   const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -2090,13 +2210,17 @@ __global__ void __launch_bounds__(kThreads) k_deposit_finalize(FinalizeArgs A) {
     for (int32_t j = j0; j < j1; j++) {
       const int32_t k = A.eslot[j];
       if (!idx_in(k, 6 * A.nt, A.stats)) continue;
-      const float2 v = reinterpret_cast<const float2*>(A.tetout)[(int64_t)(k / 6) * 6 + k % 6];
+      const float2 v = static_cast<const float2*>(A.tetout)[k];
       acc = df_add(acc, DF{v.x, v.y});
     }
     d = df_to_f64(acc);
   } else {
-    d = A.dG[e];
-    A.dG[e] = 0.0;
+    d = 0.0;
+    const int32_t j0 = A.estart[e], j1 = A.estart[e + 1];
+    for (int32_t j = j0; j < j1; j++) {
+      const int32_t k = A.eslot[j];
+      if (idx_in(k, 6 * A.nt, A.stats)) d += static_cast<const double*>(A.tetout)[k];
+    }
   }
   if (A.local) {
     A.dG_out[e] = d;
@@ -3026,13 +3150,12 @@ struct fempic_env {
   int4* te = nullptr;
   int4* tf = nullptr;
   void* field = nullptr;
-  double* dG = nullptr;
   unsigned long long* dGq = nullptr;   // 24-bit form [dGq_species][nt][8]
   int32_t dGq_species = 0;
   float4* tetdf = nullptr;             // contract form: low parts of grad lambda_1..3, [nt][4]
-  double* mom = nullptr;               // contract form: moment slots [dGq_species][nt][6]
+  double* mom = nullptr;               // moment slots: contract form [dGq_species][nt][6], FP64 form [nt][6]
   float* momlo = nullptr;              // their low FP32 parts [dGq_species][nt][8]
-  float4* tetout = nullptr;            // contract form: per-tet edge values of a step [nt][3]
+  float4* tetout = nullptr;            // contract and FP64 forms: per-tet edge values of a step, 48 B per tet
   double* Gcum = nullptr;
   unsigned long long* stats = nullptr;
   int64_t* gstart = nullptr;
@@ -3052,7 +3175,7 @@ struct fempic_env {
   int32_t* xcount = nullptr;        // [xregions]
   int64_t xslots = 0, xregions = 0;
   int num_sms = 1;
-  int push_blocks_per_sm[4] = {0, 0, 0, 0};   // resident CTAs of the mixed common path: [24-bit] + 2 [staged]
+  int push_blocks_per_sm[5] = {0, 0, 0, 0, 0};   // resident CTAs of the common path: mixed [24-bit] + 2 [staged], FP64 4
   int64_t steps = 0;
   // per-kernel event timing (measurement support)
   struct Rec {
@@ -3110,7 +3233,7 @@ struct LaunchTimer {
 static void free_env(fempic_env* e) {
   if (!e) return;
   for (cudaEvent_t ev : e->pool) cudaEventDestroy(ev);
-  void* ptrs[] = {e->geom64, e->tetrec, e->tn, e->nb, e->te, e->tf, e->field, e->dG, e->dGq, e->tetdf, e->mom,
+  void* ptrs[] = {e->geom64, e->tetrec, e->tn, e->nb, e->te, e->tf, e->field, e->dGq, e->tetdf, e->mom,
                   e->momlo, e->tetout,
                   e->Gcum, e->stats, e->gstart, e->gtet, e->sort_counts, e->sort_offsets, e->sort_sums, e->tetgrad, e->tetgrad32, e->tadj, e->curw, e->estart, e->eslot, e->fslot, e->xrec, e->xrec64, e->xcount,
                   nullptr};
@@ -3242,8 +3365,9 @@ static int upload(fempic_env* e) {
   }
   if (e->opt.precision == FEMPIC_FP64) {
     FEMPIC_CUDA(dalloc(reinterpret_cast<double**>(&e->field), 10 * nt));
-    FEMPIC_CUDA(dalloc(&e->dG, m.ne));
-    FEMPIC_CUDA(cudaMemset(e->dG, 0, m.ne * sizeof(double)));
+    FEMPIC_CUDA(dalloc(&e->mom, 6 * nt));
+    FEMPIC_CUDA(cudaMemset(e->mom, 0, 6 * nt * sizeof(double)));
+    FEMPIC_CUDA(dalloc(&e->tetout, 3 * nt));
   }
   FEMPIC_CUDA(dalloc(&e->Gcum, m.ne));
   FEMPIC_CUDA(cudaMemset(e->Gcum, 0, m.ne * sizeof(double)));
@@ -3547,34 +3671,30 @@ static int push_step_impl(fempic_env* env, const fempic_particles* p, const Host
   A.nb = env->nb;
   A.te = env->te;
   A.field = env->field;
-  A.dG = env->deposit_on ? env->dG : nullptr;
   A.dGq = env->deposit_on ? env->dGq : nullptr;
   A.mom = env->deposit_on ? env->mom : nullptr;
   A.momlo = env->momlo;
   A.tetdf = env->tetdf;
   A.stats = env->stats;
-  // the mixed common path's launch: persistent CTAs, staged when every
-  // particle array allows bulk copies (16-byte aligned sources) and there is
-  // a full tile
+  // the common path's launch: persistent CTAs; the mixed forms' are staged
+  // when every particle array allows bulk copies (16-byte aligned sources)
+  // and there is a full tile
   const int64_t all_tiles = (p->n + kTile - 1) / kTile;
-  int64_t nfull = 0, regions = all_tiles, slots = all_tiles * kTile;
-  if (mixed) {
-    const uintptr_t align = (uintptr_t)p->x | (uintptr_t)p->y | (uintptr_t)p->z | (uintptr_t)p->vx |
-                            (uintptr_t)p->vy | (uintptr_t)p->vz | (uintptr_t)p->tet;
-    nfull = (FEMPIC_USE_TMA && !(align & 15u)) ? p->n / kTile : 0;
-    int& bps = env->push_blocks_per_sm[(q24 ? 1 : 0) + (nfull > 0 ? 2 : 0)];
-    if (bps == 0) {
-      const void* k = nfull > 0 ? (q24 ? (const void*)k_push_mixed_tma<true> : (const void*)k_push_mixed_tma<false>)
+  const uintptr_t align = (uintptr_t)p->x | (uintptr_t)p->y | (uintptr_t)p->z | (uintptr_t)p->vx |
+                          (uintptr_t)p->vy | (uintptr_t)p->vz | (uintptr_t)p->tet;
+  const int64_t nfull = (mixed && FEMPIC_USE_TMA && !(align & 15u)) ? p->n / kTile : 0;
+  int& bps = env->push_blocks_per_sm[mixed ? (q24 ? 1 : 0) + (nfull > 0 ? 2 : 0) : 4];
+  if (bps == 0) {
+    const void* k = !mixed      ? (const void*)k_push_fp64
+                    : nfull > 0 ? (q24 ? (const void*)k_push_mixed_tma<true> : (const void*)k_push_mixed_tma<false>)
                                 : (q24 ? (const void*)k_push_mixed<true> : (const void*)k_push_mixed<false>);
-      int nb = 0;
-      FEMPIC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, kThreads, 0));
-      bps = nb > 0 ? nb : 1;
-    }
-    regions = std::min<int64_t>(all_tiles, (int64_t)env->num_sms * bps);
-    A.xcap = (all_tiles + regions - 1) / regions * kTile;
-    slots = regions * A.xcap;
+    int nb = 0;
+    FEMPIC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, kThreads, 0));
+    bps = nb > 0 ? nb : 1;
   }
-  rc = ensure_xqueue(env, slots, regions, st);
+  const int64_t regions = std::min<int64_t>(all_tiles, (int64_t)env->num_sms * bps);
+  A.xcap = (all_tiles + regions - 1) / regions * kTile;
+  rc = ensure_xqueue(env, regions * A.xcap, regions, st);
   if (rc) return rc;
   A.xrec = env->xrec;
   A.xrec64 = env->xrec64;
@@ -3584,8 +3704,8 @@ static int push_step_impl(fempic_env* env, const fempic_particles* p, const Host
   env->stall_cta = -1;   // one launch only
   {
     LaunchTimer lt(env, st, FEMPIC_K_PUSH);
+    const unsigned grid = (unsigned)regions;
     if (mixed) {
-      const unsigned grid = (unsigned)regions;
       if (nfull > 0) {
         if (q24)
           k_push_mixed_tma<true><<<grid, kThreads, 0, st>>>(A, nfull);
@@ -3605,13 +3725,10 @@ static int push_step_impl(fempic_env* env, const fempic_particles* p, const Host
         k_cross_df<<<grid, kCrossThreadsDF, 0, st>>>(A);
       lc.kernels = 1;
     } else {
-      k_push_fp64<<<blocks_for(p->n), kThreads, 0, st>>>(A);
+      k_push_fp64<<<grid, kThreads, 0, st>>>(A, all_tiles);
       lt.kernels = 1;
-      // the FP64 walk is FP64-pipe bound: 8 CTAs per SM queued (about three
-      // resident waves) measured faster than one resident wave
-      const unsigned cross_blocks = (unsigned)std::min<int64_t>((all_tiles + 7) / 8, (int64_t)env->num_sms * 8);
       LaunchTimer lc(env, st, FEMPIC_K_CROSS);   // nested: also inside the push bracket
-      k_cross_fp64<<<cross_blocks, kThreads, 0, st>>>(A, all_tiles);
+      k_cross_fp64<<<grid, kCrossThreads64, 0, st>>>(A);
       lc.kernels = 1;
     }
   }
@@ -3689,9 +3806,8 @@ static int deposit_impl(fempic_env* env, double omega0, double t_next, double* d
   A.mode = prec == FEMPIC_FP64 ? 0 : (prec == FEMPIC_MIXED ? 1 : 2);
   A.ns = env->ns_last;
   for (int s = 0; s < kMaxSpecies; s++) A.qwscale[s] = env->qw_last[s] * 0x1p-48;
-  A.dG = env->dG;
   A.dGq = env->dGq;
-  A.tetout = reinterpret_cast<const float*>(env->tetout);
+  A.tetout = env->tetout;
   A.Gcum = env->Gcum;
   A.dG_out = dG_out;
   A.Gcum_out = G_cum_out;
@@ -3706,7 +3822,7 @@ static int deposit_impl(fempic_env* env, double omega0, double t_next, double* d
   if (A.mode == 1 && !env->mom) {
     int rc = ensure_mixed_accumulators(env, 1, st);   // no step yet: the pull reads zeros
     if (rc) return rc;
-    A.tetout = reinterpret_cast<const float*>(env->tetout);
+    A.tetout = env->tetout;
     A.ns = 0;
   }
   {
@@ -3725,6 +3841,10 @@ static int deposit_impl(fempic_env* env, double omega0, double t_next, double* d
       }
       T.out = env->tetout;
       k_tet_finalize<<<blocks_for(T.nt), kThreads, 0, st>>>(T);
+      lt.kernels++;
+    } else if (A.mode == 0) {
+      k_tet_finalize64<<<blocks_for(A.nt), kThreads, 0, st>>>(A.nt, env->geom64, env->mom,
+                                                              reinterpret_cast<double*>(env->tetout));
       lt.kernels++;
     }
     k_deposit_finalize<<<blocks_for(A.ne), kThreads, 0, st>>>(A);
@@ -3773,10 +3893,11 @@ extern "C" int fempic_reset_deposit(fempic_env* env, void* stream) {
   if (!env) return fail(FEMPIC_EINVAL, "reset_deposit: NULL env");
   cudaStream_t st = (cudaStream_t)stream;
   FEMPIC_CUDA(cudaMemsetAsync(env->Gcum, 0, env->h.ne * sizeof(double), st));
-  if (env->dG) FEMPIC_CUDA(cudaMemsetAsync(env->dG, 0, env->h.ne * sizeof(double), st));
   const size_t nslot = (size_t)env->dGq_species * env->h.nt * 8;
   if (env->dGq) FEMPIC_CUDA(cudaMemsetAsync(env->dGq, 0, nslot * sizeof(unsigned long long), st));
-  if (env->mom) {
+  if (env->opt.precision == FEMPIC_FP64) {
+    FEMPIC_CUDA(cudaMemsetAsync(env->mom, 0, (size_t)env->h.nt * 6 * sizeof(double), st));
+  } else if (env->mom) {
     FEMPIC_CUDA(cudaMemsetAsync(env->mom, 0, (size_t)env->dGq_species * env->h.nt * 6 * sizeof(double), st));
     FEMPIC_CUDA(cudaMemsetAsync(env->momlo, 0, nslot * sizeof(float), st));
   }

@@ -1,0 +1,80 @@
+"""Particle counts at the edges of the common path's launches (one particle,
+one warp, a tile less or more one, several tiles per CTA with a ragged last
+one) and particle arrays off the 16-byte boundary bulk copies need, against
+the FP64 oracle.
+
+Zero field and dt = 2^-31 s, so that both sides track and deposit the same
+straight segments: tets, crossing counts, positions and velocities bit-exact,
+G within 1e-12 of its maximum (the deposit's bound of the identical-endpoint
+tests)."""
+import numpy as np
+import pytest
+
+from oracle.oracle import OracleMesh, OracleState, push_step as oracle_push
+from paper_2208_12795_gb300 import inputs as I
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+FP64, MIXED = 0, 1
+DT = 2.0 ** -31
+SIZES = (1, 32, 255, 256, 257, 1000, 152 * 4 * 256 + 77)
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_2208_12795_gb300 import build
+    build.build()
+
+
+@pytest.fixture(scope="module")
+def oracle_run():
+    mesh = I.kuhn_cube_mesh(6, jitter=0.2, rng=np.random.default_rng(31))
+    n = max(SIZES)
+    rng = np.random.default_rng(8)
+    pos = rng.uniform(0.0, 1.0, size=(n, 3))
+    v = (rng.standard_normal((n, 3)) * 1e8).astype(np.float32).astype(np.float64)
+    parts = I.Particles(pos[:, 0], pos[:, 1], pos[:, 2], v[:, 0], v[:, 1], v[:, 2],
+                        np.array([0, n], np.int64), np.array([-I.E_CHARGE]), np.array([I.M_ELECTRON]),
+                        np.array([1e3]))
+    om = OracleMesh(mesh.nodes, mesh.tets, mesh.lo, mesh.hi)
+    tet0, _ = om.locate(parts.x, parts.y, parts.z)
+    out = {}
+    for k in SIZES:
+        sub = parts.subset(k)
+        ost = OracleState(sub, tet0[:k])
+        G = np.zeros(om.n_edges)
+        z = np.zeros(om.n_edges, np.complex128), np.zeros(om.n_faces, np.complex128)
+        for s in range(2):
+            oracle_push(om, ost, *z, 0.0, 1.3e9, s * DT, DT, G)
+        out[k] = sub, ost, G
+    return mesh, out
+
+
+@pytest.mark.parametrize("n", SIZES)
+@pytest.mark.parametrize("offset", [0, 1])
+@pytest.mark.parametrize("prec", [FP64, MIXED])
+def test_counts_and_alignment(oracle_run, prec, offset, n):
+    from paper_2208_12795_gb300.env import FempicEnv, ParticleState
+    mesh, runs = oracle_run
+    parts, ost, oG = runs[n]
+    env = FempicEnv.from_mesh(mesh, precision=prec)
+    st = ParticleState.from_host(parts, prec)
+    for k in ("x", "y", "z", "vx", "vy", "vz", "tet"):   # the same values, one element past an aligned start
+        t = getattr(st, k)
+        w = torch.empty(n + offset, dtype=t.dtype, device="cuda")[offset:]
+        setattr(st, k, w.copy_(t))
+    env.locate(st)
+    e = torch.zeros(env.n_edges, dtype=env.dof_dtype, device="cuda")
+    b = torch.zeros(env.n_faces, dtype=env.dof_dtype, device="cuda")
+    G = torch.zeros(env.n_edges, dtype=torch.float64, device="cuda")
+    for s in range(2):
+        env.push_step(st, e, b, 0.0, 1.3e9, s * DT, DT)
+        env.deposit(1.3e9, (s + 1) * DT, G_cum_out=G)
+    g = st.to_numpy()
+    for k in ("tet", "n_cross", "status", "x", "y", "z"):
+        assert np.array_equal(g[k], getattr(ost, k)), k
+    for k in ("vx", "vy", "vz"):
+        assert np.array_equal(g[k].astype(np.float64), getattr(ost, k)), k
+    assert np.abs(G.cpu().numpy() - oG).max() <= 1e-12 * np.abs(oG).max()
+    assert env.error_count()[0]
