@@ -12,6 +12,7 @@
 
 #include "fempic_downshift.h"
 #include "fempic_internal.h"
+#include "fempic_tetgeo.cuh"
 
 namespace {
 
@@ -104,15 +105,60 @@ __device__ __forceinline__ void cross3(const R a[3], const R b[3], R o[3]) {
 //   W2_ijk = const + 2 det[g_i, g_j, g_k] d, so B~ = B0 + beta d with
 //     B0 = 2 sum over the faces (0, j, k) of b~_f g_j x g_k,
 //     beta = 2 sum_f b~_f det[g_i, g_j, g_k].
-// coef[20 t ..]: Re (E0, W, B0, beta), then Im (E0, W, B0, beta), times a(t).
-template <typename C2>
-__global__ void __launch_bounds__(kThreads) k_ds_field(int64_t nt, const double* __restrict__ geom,
-                                                       const int32_t* __restrict__ te,
-                                                       const int32_t* __restrict__ tf,
-                                                       const C2* __restrict__ e,
-                                                       const C2* __restrict__ b, int64_t ne, int64_t nf,
-                                                       unsigned long long* stats, double amp,
-                                                       double* __restrict__ coef, float* __restrict__ coef32) {
+// The coefficients of a step are Re (E0, W, B0, beta), then Im (E0, W, B0,
+// beta), times a(t).  Both passes are bound by the FP64 pipe, so the
+// geometry's products come from tables built once.
+
+// FP64 form: the shared table of fempic_tetgeo.cuh, about 94 operations per
+// tet (196k tets: 77 -> 39 us).
+__global__ void __launch_bounds__(kThreads) k_ds_field64(int64_t nt, const double* __restrict__ geom,
+                                                         const double* __restrict__ tgeo,
+                                                         const int32_t* __restrict__ te,
+                                                         const int32_t* __restrict__ tf,
+                                                         const double2* __restrict__ e,
+                                                         const double2* __restrict__ b, int64_t ne, int64_t nf,
+                                                         unsigned long long* stats, double amp,
+                                                         double* __restrict__ coef) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (t >= nt) return;
+  double2 ev[6], bv[4];
+#pragma unroll
+  for (int k = 0; k < 6; k++) {
+    const int32_t id = te[6 * t + k];
+    ev[k] = ds_idx_in(id, ne, stats) ? e[id] : make_double2(0.0, 0.0);
+  }
+#pragma unroll
+  for (int f = 0; f < 4; f++) {
+    const int32_t id = tf[4 * t + f];
+    bv[f] = ds_idx_in(id, nf, stats) ? b[id] : make_double2(0.0, 0.0);
+  }
+  fempic::TetGeo G;
+  fempic::ld_tet_geo(geom, tgeo, t, G);
+  const double amp2 = 2.0 * amp;
+#pragma unroll
+  for (int part = 0; part < 2; part++) {
+    double es[6], b2[4], o[10];
+#pragma unroll
+    for (int k = 0; k < 6; k++) es[k] = amp * (part ? ev[k].y : ev[k].x);
+#pragma unroll
+    for (int f = 0; f < 4; f++) b2[f] = amp2 * (part ? bv[f].y : bv[f].x);
+    fempic::whitney_affine(G, es, b2, o);
+    double2* out = reinterpret_cast<double2*>(coef + 20 * t + 10 * part);
+#pragma unroll
+    for (int c = 0; c < 5; c++) out[c] = make_double2(o[2 * c], o[2 * c + 1]);
+  }
+}
+
+// Mixed forms: the FP64 sums rounded once to FP32.  A coefficient that rounds
+// the other way moves a particle's FP32 velocity by an ulp, so the sums keep
+// one order of operations; their geometry factors (g_j x g_i per edge, g_j x
+// g_k per face at node 0, det per face) are formed once per mesh, and the
+// conversions of DoFs and results run in integer operations off the FP64 pipe
+// (663k tets: 280 -> 155 us).
+constexpr int kDsGeo = 32;   // doubles per tet: 6 x 3, 3 x 3, 4, unused
+
+__global__ void __launch_bounds__(kThreads) k_ds_geo32(int64_t nt, const double* __restrict__ geom,
+                                                       double* __restrict__ dgeo) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= nt) return;
   const double* G = geom + 12 * t;
@@ -123,60 +169,115 @@ __global__ void __launch_bounds__(kThreads) k_ds_field(int64_t nt, const double*
     for (int a = 0; a < 3; a++) g[k][a] = G[3 * k + a];
 #pragma unroll
   for (int a = 0; a < 3; a++) g[0][a] = -(g[1][a] + g[2][a] + g[3][a]);
+  double* o = dgeo + kDsGeo * t;
+#pragma unroll
+  for (int k = 0; k < 6; k++) {
+    double gji[3];
+    cross3(g[le1(k)], g[le0(k)], gji);
+#pragma unroll
+    for (int a = 0; a < 3; a++) o[3 * k + a] = gji[a];
+  }
+#pragma unroll
+  for (int f = 0; f < 4; f++) {
+    const int i = lf(f, 0), j = lf(f, 1), k = lf(f, 2);
+    double gjk[3];
+    cross3(g[j], g[k], gjk);
+    o[27 + f] = g[i][0] * gjk[0] + g[i][1] * gjk[1] + g[i][2] * gjk[2];
+    if (i == 0) {
+#pragma unroll
+      for (int a = 0; a < 3; a++) o[18 + 3 * (f - 1) + a] = gjk[a];
+    }
+  }
+  o[31] = 0.0;
+}
+
+// Exact widening with integer operations (the hardware conversion runs at the
+// FP64 rate); zero, subnormals, infinities and NaN take the hardware's.
+__device__ __forceinline__ double widen32(float f) {
+  const unsigned u = __float_as_uint(f), e = (u >> 23) & 0xffu;
+  if (e - 1u >= 0xfeu) return (double)f;
+  return __hiloint2double((int)((u & 0x80000000u) | ((e + 896u) << 20) | ((u & 0x7fffffu) >> 3)), (int)(u << 29));
+}
+
+// FP64 -> FP32, nearest even, with integer operations; values outside the
+// normal FP32 range take the hardware conversion.
+__device__ __forceinline__ float round32(double r) {
+  const unsigned hi = (unsigned)__double2hiint(r), lo = (unsigned)__double2loint(r);
+  const unsigned e = (hi >> 20) & 0x7ffu;
+  if (e - 897u >= 253u) return (float)r;   // below 2^-126 or from 2^127 on
+  const unsigned m = ((e - 896u) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
+  const unsigned rest = lo & 0x1fffffffu;
+  const unsigned up = rest > 0x10000000u || (rest == 0x10000000u && (m & 1u)) ? 1u : 0u;
+  return __uint_as_float((hi & 0x80000000u) | (m + up));   // a carry moves into the exponent
+}
+
+__global__ void __launch_bounds__(kThreads) k_ds_field32(int64_t nt, const double* __restrict__ geom,
+                                                         const double* __restrict__ dgeo,
+                                                         const int32_t* __restrict__ te,
+                                                         const int32_t* __restrict__ tf,
+                                                         const float2* __restrict__ e, const float2* __restrict__ b,
+                                                         int64_t ne, int64_t nf, unsigned long long* stats,
+                                                         double amp, float* __restrict__ coef32) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (t >= nt) return;
+  const double2* D = reinterpret_cast<const double2*>(dgeo + kDsGeo * t);
+  double w[kDsGeo];
+#pragma unroll
+  for (int c = 0; c < kDsGeo / 2; c++) {
+    const double2 v = __ldg(D + c);
+    w[2 * c] = v.x;
+    w[2 * c + 1] = v.y;
+  }
+  const double* g1 = geom + 12 * t + 3;
   double o[20];
 #pragma unroll
   for (int c = 0; c < 20; c++) o[c] = 0.0;
 #pragma unroll
   for (int k = 0; k < 6; k++) {
-    const int i = le0(k), j = le1(k);
     const int32_t id = te[6 * t + k];
     double2 c = make_double2(0.0, 0.0);
     if (ds_idx_in(id, ne, stats)) {
-      const C2 cc = e[id];
-      c = make_double2((double)cc.x, (double)cc.y);
+      const float2 cc = e[id];
+      c = make_double2(widen32(cc.x), widen32(cc.y));
     }
-    double gji[3];
-    cross3(g[j], g[i], gji);
 #pragma unroll
     for (int a = 0; a < 3; a++) {
-      if (i == 0) {
-        o[a] += c.x * g[j][a];
-        o[10 + a] += c.y * g[j][a];
+      if (le0(k) == 0) {
+        const double g = __ldg(g1 + 3 * k + a);   // le1(k) = k + 1: g_{k+1}
+        o[a] += c.x * g;
+        o[10 + a] += c.y * g;
       }
-      o[3 + a] += c.x * gji[a];
-      o[13 + a] += c.y * gji[a];
+      o[3 + a] += c.x * w[3 * k + a];
+      o[13 + a] += c.y * w[3 * k + a];
     }
   }
 #pragma unroll
   for (int f = 0; f < 4; f++) {
-    const int i = lf(f, 0), j = lf(f, 1), k = lf(f, 2);
     const int32_t id = tf[4 * t + f];
     double2 c = make_double2(0.0, 0.0);
     if (ds_idx_in(id, nf, stats)) {
-      const C2 cc = b[id];
-      c = make_double2((double)cc.x, (double)cc.y);
+      const float2 cc = b[id];
+      c = make_double2(widen32(cc.x), widen32(cc.y));
     }
-    double gjk[3];
-    cross3(g[j], g[k], gjk);
-    const double det = g[i][0] * gjk[0] + g[i][1] * gjk[1] + g[i][2] * gjk[2];
-    if (i == 0) {
+    const double bx = 2.0 * c.x, by = 2.0 * c.y;
+    if (f > 0) {
 #pragma unroll
       for (int a = 0; a < 3; a++) {
-        o[6 + a] += 2.0 * c.x * gjk[a];
-        o[16 + a] += 2.0 * c.y * gjk[a];
+        o[6 + a] += bx * w[18 + 3 * (f - 1) + a];
+        o[16 + a] += by * w[18 + 3 * (f - 1) + a];
       }
     }
-    o[9] += 2.0 * c.x * det;
-    o[19] += 2.0 * c.y * det;
+    o[9] += bx * w[27 + f];
+    o[19] += by * w[27 + f];
   }
-  double2* out = reinterpret_cast<double2*>(coef + 20 * t);
+  if (amp != 1.0) {   // a(t) = 1 (past the envelope's rise) leaves the sums as they are
 #pragma unroll
-  for (int c = 0; c < 10; c++) out[c] = make_double2(amp * o[2 * c], amp * o[2 * c + 1]);
-  if (coef32) {
-    float2* o32 = reinterpret_cast<float2*>(coef32 + 20 * t);
-#pragma unroll
-    for (int c = 0; c < 10; c++) o32[c] = make_float2((float)(amp * o[2 * c]), (float)(amp * o[2 * c + 1]));
+    for (int c = 0; c < 20; c++) o[c] = amp * o[c];
   }
+  float4* o32 = reinterpret_cast<float4*>(coef32 + 20 * t);
+#pragma unroll
+  for (int c = 0; c < 5; c++)
+    o32[c] = make_float4(round32(o[4 * c]), round32(o[4 * c + 1]), round32(o[4 * c + 2]), round32(o[4 * c + 3]));
 }
 
 // The envelope sample at r in tet T from the per-tet coefficients:
@@ -407,18 +508,22 @@ unsigned blocks_for(int64_t n) { return (unsigned)((n + kThreads - 1) / kThreads
 struct fempic_downshift {
   int64_t nn = 0, ne = 0, nf = 0, nt = 0;
   double* geom = nullptr;
+  double* tgeo = nullptr;       // [nt][kTetGeo] products of the gradients (fempic_tetgeo.cuh)
   int32_t* te = nullptr;
   int32_t* tf = nullptr;
-  double* coef = nullptr;       // [nt][20]
+  double* coef = nullptr;       // FP64 form: [nt][20]
+  double* dgeo = nullptr;       // mixed forms: [nt][kDsGeo] geometry factors (allocated on first use)
   float* coef32 = nullptr;      // mixed forms: [nt][20] in FP32 (allocated on first use)
 };
 
 static void free_ds(fempic_downshift* d) {
   if (!d) return;
   cudaFree(d->geom);
+  cudaFree(d->tgeo);
   cudaFree(d->te);
   cudaFree(d->tf);
   cudaFree(d->coef);
+  cudaFree(d->dgeo);
   cudaFree(d->coef32);
   delete d;
 }
@@ -497,6 +602,7 @@ extern "C" int fempic_downshift_create(const fempic_mesh_desc* mesh, fempic_down
                sf = sizeof(int32_t) * 4 * (size_t)m.nt;
   if (cudaMalloc(&d->geom, sg) != cudaSuccess || cudaMalloc(&d->te, se) != cudaSuccess ||
       cudaMalloc(&d->tf, sf) != cudaSuccess ||
+      cudaMalloc(&d->tgeo, sizeof(double) * fempic::kTetGeo * (size_t)m.nt) != cudaSuccess ||
       cudaMalloc(&d->coef, sizeof(double) * 20 * (size_t)m.nt) != cudaSuccess) {
     free_ds(d);
     cudaGetLastError();
@@ -507,6 +613,11 @@ extern "C" int fempic_downshift_create(const fempic_mesh_desc* mesh, fempic_down
       cudaMemcpy(d->tf, m.tf.data(), sf, cudaMemcpyHostToDevice) != cudaSuccess) {
     free_ds(d);
     return fail(FEMPIC_ECUDA, "downshift_create: upload");
+  }
+  fempic::k_tet_geo<<<blocks_for(m.nt), kThreads>>>(m.nt, d->geom, d->tgeo);
+  if (cudaGetLastError() != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) {
+    free_ds(d);
+    return fail(FEMPIC_ECUDA, "downshift_create: geometry table");
   }
   *out = d;
   return FEMPIC_OK;
@@ -572,31 +683,34 @@ extern "C" int fempic_push_step_downshift(fempic_env* env, fempic_downshift* ds,
   A.h = hist->planes;
   A.nt = ds->nt;
   A.geom = ds->geom;
-  A.coef = ds->coef;
   A.start = start;
   compute_weights(t, dt, omega0, A.w);
   for (int i = 0; i < 24; i++) A.w32[i] = (float)A.w[i];
-  if (mixed && !ds->coef32) {
-    if (cudaMalloc(&ds->coef32, sizeof(float) * 20 * (size_t)ds->nt) != cudaSuccess) {
+  if (mixed && !ds->coef32) {   // the mixed forms' coefficients and geometry factors, on first use
+    if (cudaMalloc(&ds->dgeo, sizeof(double) * kDsGeo * (size_t)ds->nt) != cudaSuccess ||
+        cudaMalloc(&ds->coef32, sizeof(float) * 20 * (size_t)ds->nt) != cudaSuccess) {
       cudaGetLastError();
+      cudaFree(ds->dgeo);
+      ds->dgeo = nullptr;
       ds->coef32 = nullptr;
       return fail(FEMPIC_ENOMEM, "push_step_downshift: device allocation");
     }
+    k_ds_geo32<<<blocks_for(ds->nt), kThreads, 0, (cudaStream_t)stream>>>(ds->nt, ds->geom, ds->dgeo);
+    DS_CUDA(cudaGetLastError());
   }
+  A.coef = ds->coef;
   A.coef32 = ds->coef32;
   cudaStream_t st = (cudaStream_t)stream;
   if (mixed) {   // complex64 DoFs; FP32 velocities, samples and history
-    k_ds_field<float2><<<blocks_for(ds->nt), kThreads, 0, st>>>(
-        ds->nt, ds->geom, ds->te, ds->tf, static_cast<const float2*>(envl->e_tilde),
-        static_cast<const float2*>(envl->b_tilde), ds->ne, ds->nf, fempic::env_stats(env), envl->amp, ds->coef,
-        ds->coef32);
+    k_ds_field32<<<blocks_for(ds->nt), kThreads, 0, st>>>(
+        ds->nt, ds->geom, ds->dgeo, ds->te, ds->tf, static_cast<const float2*>(envl->e_tilde),
+        static_cast<const float2*>(envl->b_tilde), ds->ne, ds->nf, fempic::env_stats(env), envl->amp, ds->coef32);
     DS_CUDA(cudaGetLastError());
     k_ds_pre<float><<<blocks_for(p->n), kThreads, 0, st>>>(A);
   } else {
-    k_ds_field<double2><<<blocks_for(ds->nt), kThreads, 0, st>>>(
-        ds->nt, ds->geom, ds->te, ds->tf, static_cast<const double2*>(envl->e_tilde),
-        static_cast<const double2*>(envl->b_tilde), ds->ne, ds->nf, fempic::env_stats(env), envl->amp, ds->coef,
-        nullptr);
+    k_ds_field64<<<blocks_for(ds->nt), kThreads, 0, st>>>(
+        ds->nt, ds->geom, ds->tgeo, ds->te, ds->tf, static_cast<const double2*>(envl->e_tilde),
+        static_cast<const double2*>(envl->b_tilde), ds->ne, ds->nf, fempic::env_stats(env), envl->amp, ds->coef);
     DS_CUDA(cudaGetLastError());
     k_ds_pre<double><<<blocks_for(p->n), kThreads, 0, st>>>(A);
   }
