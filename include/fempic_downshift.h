@@ -24,10 +24,10 @@
  * velocity and B~ interpolated separately) is the one implemented.
  *
  * The straight segment r^n -> r^{n+1} is tracked, reflected or absorbed at
- * the walls and deposited by the env's own FP64 step (fempic_push_step of
- * fempic_env.h run with a zero field, whose Boris update then leaves the
- * velocity unchanged).  A wall that mirrors the segment in an axis mirrors,
- * in that axis, the new velocity and every stored velocity of the history.
+ * the walls and deposited by the env's own step kernels, as fempic_push_step
+ * of fempic_env.h does under a zero field (the rule runs in the same pass).
+ * A wall that mirrors the segment in an axis mirrors, in that axis, the new
+ * velocity and every stored velocity of the history.
  *
  * Conventions: as in fempic_env.h (device / host pointers as stated, stream-
  * ordered asynchronous calls, FEMPIC_OK or a negative FEMPIC_E* code; the
@@ -52,7 +52,7 @@ typedef struct fempic_downshift fempic_downshift;   /* opaque: per-tet geometry,
  *   FEMPIC_DS_VH + 3*i + a     v^{n-1-i} along axis a, i = 0, 1, 2
  *   FEMPIC_DS_F  + 12*l + c    envelope sample of level n-1-l, l = 0, 1:
  *                              c = 0..2 Re E~, 3..5 Im E~, 6..8 Re B~, 9..11 Im B~
- *   FEMPIC_DS_VN, FEMPIC_DS_U  per-step scratch (new velocity, AB4 velocity)
+ *   FEMPIC_DS_VN, FEMPIC_DS_U  scratch of the step (contents unspecified)
  * Zero-initialised or not, it is filled by the first step (start = 1). */
 #define FEMPIC_DS_VH 0
 #define FEMPIC_DS_F 9
@@ -68,7 +68,7 @@ typedef struct {
 
 /* Build the gather tables (FP64 barycentric geometry, tet edges and faces)
  * from the same mesh description the env was created from, upload them to
- * the current device and allocate the per-tet coefficient buffer (20 f64 per
+ * the current device and allocate the per-tet coefficient buffer (22 f64 per
  * tet).  Errors: EINVAL, EMESH, ENOMEM, ECUDA.  Synchronizes the device. */
 int fempic_downshift_create(const fempic_mesh_desc* mesh, fempic_downshift** out);
 

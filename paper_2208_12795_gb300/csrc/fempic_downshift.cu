@@ -1,9 +1,10 @@
 // Downshifted particle integrator of Sec. III-D on the FP64 form and the
 // FP32-mixed forms: the velocity rule with the carrier integrated
-// analytically (M and L weights) and AB4 positions.  Per step: k_ds_field (per-tet envelope coefficients),
-// k_ds_pre (sample, velocity rule, AB4 velocity, history shift), the env's
-// own FP64 step under a zero field (tracking, walls, deposit of the AB4
-// segment), then k_ds_post (wall mirrors of the velocity history).
+// analytically (M and L weights) and AB4 positions.  Per step: the per-tet
+// envelope coefficients (k_ds_field64, k_ds_field32), then the env's step
+// kernels with the rule in place of gather and Boris (fempic_ds_rule.cuh):
+// sample, velocity rule, AB4 velocity, history shift, tracking, walls and
+// deposit of the AB4 segment.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -11,6 +12,7 @@
 #include <string>
 
 #include "fempic_downshift.h"
+#include "fempic_ds_rule.cuh"
 #include "fempic_internal.h"
 #include "fempic_tetgeo.cuh"
 
@@ -34,10 +36,6 @@ int fail(int code, const std::string& msg) {
 
 constexpr int kThreads = 256;
 
-// Fourth-order Adams-Bashforth stencil (55, -59, 37, -9) / 24, divided once
-// here: a double division per particle costs several FP64-pipe instructions.
-__device__ constexpr double kAB4[4] = {55.0 / 24.0, -59.0 / 24.0, 37.0 / 24.0, -9.0 / 24.0};
-
 // Local edge e joins sorted local nodes (le0, le1) in the order 01,02,03,12,
 // 13,23; local face f is opposite node f and its i-th node is lf(f, i).
 __host__ __device__ constexpr int le0(int e) { return e < 3 ? 0 : (e < 5 ? 1 : 2); }
@@ -60,36 +58,6 @@ __device__ __forceinline__ bool ds_idx_in(int64_t i, int64_t n, unsigned long lo
   return false;
 }
 
-struct DsArgs {
-  int64_t n;
-  const double* x;
-  const double* y;
-  const double* z;
-  void* vx;                     // f64 (FP64 form) or f32 (mixed forms) velocities
-  void* vy;
-  void* vz;
-  const int32_t* tet;
-  void* h;                      // history planes [FEMPIC_DS_PLANES][n], the velocity type
-  int64_t nt;
-  const double* geom;           // [nt][12]: x0, grad l1, grad l2, grad l3
-  const double* coef;           // [nt][20]: per-tet envelope coefficients of this step (k_ds_field)
-  const float* coef32;          // mixed forms: the same in FP32
-  int32_t ns;
-  int32_t start;
-  int64_t begin[kMaxSpecies + 1];
-  double qm[kMaxSpecies];
-  double w[24];                 // M^r[3], M^i[3], L^r[3][3], L^i[3][3]
-  float qm32[kMaxSpecies];      // mixed forms: the same rounded to FP32
-  float w32[24];
-};
-
-__device__ __forceinline__ int species_of(const DsArgs& A, int64_t p) {
-  int s = 0;
-#pragma unroll 1
-  while (s + 1 < A.ns && p >= A.begin[s + 1]) s++;
-  return s;
-}
-
 template <typename R>
 __device__ __forceinline__ void cross3(const R a[3], const R b[3], R o[3]) {
   o[0] = a[1] * b[2] - a[2] * b[1];
@@ -108,6 +76,14 @@ __device__ __forceinline__ void cross3(const R a[3], const R b[3], R o[3]) {
 // The coefficients of a step are Re (E0, W, B0, beta), then Im (E0, W, B0,
 // beta), times a(t).  Both passes are bound by the FP64 pipe, so the
 // geometry's products come from tables built once.
+
+// A tet with a DoF that is not finite is flagged: its particles freeze with
+// status NONFINITE (as under a field that is not finite), also where a later
+// sum would hide it.
+__device__ __forceinline__ bool not_finite(double x) {
+  return (((unsigned)__double2hiint(x) >> 20) & 0x7ffu) == 0x7ffu;
+}
+__device__ __forceinline__ bool not_finite(float x) { return ((__float_as_uint(x) >> 23) & 0xffu) == 0xffu; }
 
 // FP64 form: the shared table of fempic_tetgeo.cuh, about 94 operations per
 // tet (196k tets: 77 -> 39 us).
@@ -143,10 +119,16 @@ __global__ void __launch_bounds__(kThreads) k_ds_field64(int64_t nt, const doubl
 #pragma unroll
     for (int f = 0; f < 4; f++) b2[f] = amp2 * (part ? bv[f].y : bv[f].x);
     fempic::whitney_affine(G, es, b2, o);
-    double2* out = reinterpret_cast<double2*>(coef + 20 * t + 10 * part);
+    double2* out = reinterpret_cast<double2*>(coef + fempic::kDsCoef64 * t + 10 * part);
 #pragma unroll
     for (int c = 0; c < 5; c++) out[c] = make_double2(o[2 * c], o[2 * c + 1]);
   }
+  bool bad = false;
+#pragma unroll
+  for (int k = 0; k < 6; k++) bad = bad || not_finite(ev[k].x) || not_finite(ev[k].y);
+#pragma unroll
+  for (int f = 0; f < 4; f++) bad = bad || not_finite(bv[f].x) || not_finite(bv[f].y);
+  coef[fempic::kDsCoef64 * t + 20] = bad ? 1.0 : 0.0;
 }
 
 // Mixed forms: the FP64 sums rounded once to FP32.  A coefficient that rounds
@@ -229,6 +211,7 @@ __global__ void __launch_bounds__(kThreads) k_ds_field32(int64_t nt, const doubl
     w[2 * c + 1] = v.y;
   }
   const double* g1 = geom + 12 * t + 3;
+  bool bad = false;
   double o[20];
 #pragma unroll
   for (int c = 0; c < 20; c++) o[c] = 0.0;
@@ -238,6 +221,7 @@ __global__ void __launch_bounds__(kThreads) k_ds_field32(int64_t nt, const doubl
     double2 c = make_double2(0.0, 0.0);
     if (ds_idx_in(id, ne, stats)) {
       const float2 cc = e[id];
+      bad = bad || not_finite(cc.x) || not_finite(cc.y);
       c = make_double2(widen32(cc.x), widen32(cc.y));
     }
 #pragma unroll
@@ -257,6 +241,7 @@ __global__ void __launch_bounds__(kThreads) k_ds_field32(int64_t nt, const doubl
     double2 c = make_double2(0.0, 0.0);
     if (ds_idx_in(id, nf, stats)) {
       const float2 cc = b[id];
+      bad = bad || not_finite(cc.x) || not_finite(cc.y);
       c = make_double2(widen32(cc.x), widen32(cc.y));
     }
     const double bx = 2.0 * c.x, by = 2.0 * c.y;
@@ -274,169 +259,11 @@ __global__ void __launch_bounds__(kThreads) k_ds_field32(int64_t nt, const doubl
 #pragma unroll
     for (int c = 0; c < 20; c++) o[c] = amp * o[c];
   }
-  float4* o32 = reinterpret_cast<float4*>(coef32 + 20 * t);
+  float4* o32 = reinterpret_cast<float4*>(coef32 + fempic::kDsCoef32 * t);
 #pragma unroll
   for (int c = 0; c < 5; c++)
     o32[c] = make_float4(round32(o[4 * c]), round32(o[4 * c + 1]), round32(o[4 * c + 2]), round32(o[4 * c + 3]));
-}
-
-// The envelope sample at r in tet T from the per-tet coefficients:
-// out[12] = Re E~, Im E~, Re B~, Im B~.  The mixed forms take d = r - x0 from
-// one FP64 subtraction, rounded to FP32, and evaluate in FP32.
-template <typename R>
-__device__ __forceinline__ void envelope_at(const DsArgs& A, int32_t T, double rx, double ry, double rz,
-                                            R out[12]) {
-  const double* G = A.geom + 12 * (int64_t)T;
-  const R d[3] = {(R)(rx - __ldg(G)), (R)(ry - __ldg(G + 1)), (R)(rz - __ldg(G + 2))};
-  R c[20];
-  if (sizeof(R) == 8) {
-    const double2* C = reinterpret_cast<const double2*>(A.coef + 20 * (int64_t)T);
-#pragma unroll
-    for (int i = 0; i < 10; i++) {
-      const double2 v = __ldg(C + i);
-      c[2 * i] = (R)v.x;
-      c[2 * i + 1] = (R)v.y;
-    }
-  } else {
-    const float2* C = reinterpret_cast<const float2*>(A.coef32 + 20 * (int64_t)T);
-#pragma unroll
-    for (int i = 0; i < 10; i++) {
-      const float2 v = __ldg(C + i);
-      c[2 * i] = (R)v.x;
-      c[2 * i + 1] = (R)v.y;
-    }
-  }
-#pragma unroll
-  for (int part = 0; part < 2; part++) {
-    const R* q = c + 10 * part;
-    R dw[3];
-    cross3<R>(d, q + 3, dw);
-#pragma unroll
-    for (int a = 0; a < 3; a++) {
-      out[3 * part + a] = q[a] + dw[a];
-      out[6 + 3 * part + a] = q[6 + a] + q[9] * d[a];
-    }
-  }
-}
-
-// Before the env's step: the envelope sample at r^n, the velocity rule, the
-// AB4 velocity u (left in v for the env's zero-field step to track), the new
-// velocity and u kept in the scratch planes, and the history shifted.
-// The FP32 instance streams the history planes and is bound by HBM latency:
-// it is held to 80 registers so that 3 blocks of 256 stay resident per SM
-// (128 registers left 2, and the step 4% slower).  The FP64 instance is bound
-// by the FP64 pipe and keeps the compiler's allocation (a minimum of 0 leaves
-// it unconstrained; 1 let it grow to 204 registers and one block per SM).
-template <typename R>
-__global__ void __launch_bounds__(kThreads, sizeof(R) == 4 ? 3 : 0) k_ds_pre(DsArgs A) {
-  const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (p >= A.n) return;
-  const int64_t n = A.n;
-  R* H = static_cast<R*>(A.h);
-  R* vxp = static_cast<R*>(A.vx);
-  R* vyp = static_cast<R*>(A.vy);
-  R* vzp = static_cast<R*>(A.vz);
-  const R v0[3] = {vxp[p], vyp[p], vzp[p]};
-  const int32_t T = A.tet[p];
-  if (T < 0 || T >= A.nt) {   // inactive: the state is kept (the env's step flags an out-of-range tet)
-#pragma unroll
-    for (int a = 0; a < 3; a++) {
-      H[(FEMPIC_DS_VN + a) * n + p] = v0[a];
-      H[(FEMPIC_DS_U + a) * n + p] = v0[a];
-    }
-    return;
-  }
-  R cur[12];
-  envelope_at<R>(A, T, A.x[p], A.y[p], A.z[p], cur);
-  R vh[3][3], f1[12], f2[12];
-  if (A.start) {
-#pragma unroll
-    for (int i = 0; i < 3; i++)
-#pragma unroll
-      for (int a = 0; a < 3; a++) vh[i][a] = v0[a];
-#pragma unroll
-    for (int c = 0; c < 12; c++) f1[c] = f2[c] = cur[c];
-  } else {
-#pragma unroll
-    for (int i = 0; i < 3; i++)
-#pragma unroll
-      for (int a = 0; a < 3; a++) vh[i][a] = H[(FEMPIC_DS_VH + 3 * i + a) * n + p];
-#pragma unroll
-    for (int c = 0; c < 12; c++) {
-      f1[c] = H[(FEMPIC_DS_F + c) * n + p];
-      f2[c] = H[(FEMPIC_DS_F + 12 + c) * n + p];
-    }
-  }
-  const R* S[3] = {cur, f1, f2};
-  const R* V[3] = {v0, vh[0], vh[1]};
-  // weights from the kernel parameters: M^r at 0, M^i at 3, L^r at 6, L^i at 15
-  auto wt = [&](int i) -> R { return sizeof(R) == 8 ? (R)A.w[i] : (R)A.w32[i]; };
-  R dv[3] = {R(0), R(0), R(0)};
-#pragma unroll
-  for (int k = 0; k < 3; k++)
-#pragma unroll
-    for (int a = 0; a < 3; a++) dv[a] += S[k][a] * wt(k) + S[k][3 + a] * wt(3 + k);
-#pragma unroll
-  for (int j = 0; j < 3; j++) {
-    R C[3] = {R(0), R(0), R(0)};
-#pragma unroll
-    for (int k = 0; k < 3; k++)
-#pragma unroll
-      for (int a = 0; a < 3; a++) C[a] += S[k][6 + a] * wt(6 + 3 * j + k) + S[k][9 + a] * wt(15 + 3 * j + k);
-    R vc[3];
-    cross3<R>(V[j], C, vc);
-#pragma unroll
-    for (int a = 0; a < 3; a++) dv[a] += vc[a];
-  }
-  const int s = species_of(A, p);
-  const R qm = sizeof(R) == 8 ? (R)A.qm[s] : (R)A.qm32[s];
-  const R ab[4] = {(R)kAB4[0], (R)kAB4[1], (R)kAB4[2], (R)kAB4[3]};
-  R u[3];
-#pragma unroll
-  for (int a = 0; a < 3; a++) {
-    u[a] = ab[0] * v0[a] + ab[1] * vh[0][a] + ab[2] * vh[1][a] + ab[3] * vh[2][a];
-    H[(FEMPIC_DS_VN + a) * n + p] = v0[a] + qm * dv[a];
-    H[(FEMPIC_DS_U + a) * n + p] = u[a];
-    H[(FEMPIC_DS_VH + 6 + a) * n + p] = vh[1][a];
-    H[(FEMPIC_DS_VH + 3 + a) * n + p] = vh[0][a];
-    H[(FEMPIC_DS_VH + a) * n + p] = v0[a];
-  }
-#pragma unroll
-  for (int c = 0; c < 12; c++) {
-    H[(FEMPIC_DS_F + 12 + c) * n + p] = f1[c];
-    H[(FEMPIC_DS_F + c) * n + p] = cur[c];
-  }
-  vxp[p] = u[0];
-  vyp[p] = u[1];
-  vzp[p] = u[2];
-}
-
-// After the env's step: an axis in which the tracked velocity came back
-// negated was mirrored by a wall (an odd number of times; a zero component
-// cannot reach a wall), so the new velocity and the velocity history are
-// mirrored in it; then v <- v^{n+1}.
-template <typename R>
-__global__ void __launch_bounds__(kThreads) k_ds_post(DsArgs A) {
-  const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (p >= A.n) return;
-  const int64_t n = A.n;
-  R* H = static_cast<R*>(A.h);
-  R* vp[3] = {static_cast<R*>(A.vx), static_cast<R*>(A.vy), static_cast<R*>(A.vz)};
-#pragma unroll
-  for (int a = 0; a < 3; a++) {
-    const R va = vp[a][p];
-    const R u = H[(FEMPIC_DS_U + a) * n + p];
-    R vn = H[(FEMPIC_DS_VN + a) * n + p];
-    if (u != R(0) && va == -u) {
-      vn = -vn;
-#pragma unroll
-      for (int i = 0; i < 3; i++) {
-        R& h = H[(FEMPIC_DS_VH + 3 * i + a) * n + p];
-        h = -h;
-      }
-    }
-    vp[a][p] = vn;
-  }
+  o32[5] = make_float4(bad ? 1.f : 0.f, 0.f, 0.f, 0.f);
 }
 
 // int_0^1 x^m e^{j theta x} dx, m = 0..4: the power series of the exponential
@@ -511,9 +338,9 @@ struct fempic_downshift {
   double* tgeo = nullptr;       // [nt][kTetGeo] products of the gradients (fempic_tetgeo.cuh)
   int32_t* te = nullptr;
   int32_t* tf = nullptr;
-  double* coef = nullptr;       // FP64 form: [nt][20]
+  double* coef = nullptr;       // FP64 form: [nt][kDsCoef64]
   double* dgeo = nullptr;       // mixed forms: [nt][kDsGeo] geometry factors (allocated on first use)
-  float* coef32 = nullptr;      // mixed forms: [nt][20] in FP32 (allocated on first use)
+  float* coef32 = nullptr;      // mixed forms: [nt][kDsCoef32] (allocated on first use)
 };
 
 static void free_ds(fempic_downshift* d) {
@@ -603,7 +430,7 @@ extern "C" int fempic_downshift_create(const fempic_mesh_desc* mesh, fempic_down
   if (cudaMalloc(&d->geom, sg) != cudaSuccess || cudaMalloc(&d->te, se) != cudaSuccess ||
       cudaMalloc(&d->tf, sf) != cudaSuccess ||
       cudaMalloc(&d->tgeo, sizeof(double) * fempic::kTetGeo * (size_t)m.nt) != cudaSuccess ||
-      cudaMalloc(&d->coef, sizeof(double) * 20 * (size_t)m.nt) != cudaSuccess) {
+      cudaMalloc(&d->coef, sizeof(double) * fempic::kDsCoef64 * (size_t)m.nt) != cudaSuccess) {
     free_ds(d);
     cudaGetLastError();
     return fail(FEMPIC_ENOMEM, "downshift_create: device allocation");
@@ -661,34 +488,22 @@ extern "C" int fempic_push_step_downshift(fempic_env* env, fempic_downshift* ds,
     return fail(FEMPIC_EINVAL, "push_step_downshift: species table (1..8 ranges, q, m)");
   if (p->species_begin[0] != 0 || p->species_begin[p->n_species] != p->n)
     return fail(FEMPIC_EINVAL, "push_step_downshift: species ranges must cover [0, n)");
-  DsArgs A{};
-  A.ns = p->n_species;
-  for (int s = 0; s <= kMaxSpecies; s++) A.begin[s] = s <= p->n_species ? p->species_begin[s] : p->n;
+  fempic::DsRule A{};
   for (int s = 0; s < p->n_species; s++) {
-    if (s > 0 && A.begin[s] < A.begin[s - 1]) return fail(FEMPIC_EINVAL, "push_step_downshift: species ranges decrease");
+    if (p->species_begin[s + 1] < p->species_begin[s])
+      return fail(FEMPIC_EINVAL, "push_step_downshift: species ranges decrease");
     if (!(p->m[s] > 0.0) || !std::isfinite(p->q[s])) return fail(FEMPIC_EINVAL, "push_step_downshift: q, m");
     A.qm[s] = p->q[s] / p->m[s];
     A.qm32[s] = (float)A.qm[s];
   }
-  if (A.begin[p->n_species] < A.begin[p->n_species - 1])
-    return fail(FEMPIC_EINVAL, "push_step_downshift: species ranges decrease");
   A.n = p->n;
-  A.x = p->x;
-  A.y = p->y;
-  A.z = p->z;
-  A.vx = p->vx;
-  A.vy = p->vy;
-  A.vz = p->vz;
-  A.tet = p->tet;
   A.h = hist->planes;
-  A.nt = ds->nt;
-  A.geom = ds->geom;
   A.start = start;
   compute_weights(t, dt, omega0, A.w);
   for (int i = 0; i < 24; i++) A.w32[i] = (float)A.w[i];
   if (mixed && !ds->coef32) {   // the mixed forms' coefficients and geometry factors, on first use
     if (cudaMalloc(&ds->dgeo, sizeof(double) * kDsGeo * (size_t)ds->nt) != cudaSuccess ||
-        cudaMalloc(&ds->coef32, sizeof(float) * 20 * (size_t)ds->nt) != cudaSuccess) {
+        cudaMalloc(&ds->coef32, sizeof(float) * fempic::kDsCoef32 * (size_t)ds->nt) != cudaSuccess) {
       cudaGetLastError();
       cudaFree(ds->dgeo);
       ds->dgeo = nullptr;
@@ -705,26 +520,13 @@ extern "C" int fempic_push_step_downshift(fempic_env* env, fempic_downshift* ds,
     k_ds_field32<<<blocks_for(ds->nt), kThreads, 0, st>>>(
         ds->nt, ds->geom, ds->dgeo, ds->te, ds->tf, static_cast<const float2*>(envl->e_tilde),
         static_cast<const float2*>(envl->b_tilde), ds->ne, ds->nf, fempic::env_stats(env), envl->amp, ds->coef32);
-    DS_CUDA(cudaGetLastError());
-    k_ds_pre<float><<<blocks_for(p->n), kThreads, 0, st>>>(A);
   } else {
     k_ds_field64<<<blocks_for(ds->nt), kThreads, 0, st>>>(
         ds->nt, ds->geom, ds->tgeo, ds->te, ds->tf, static_cast<const double2*>(envl->e_tilde),
         static_cast<const double2*>(envl->b_tilde), ds->ne, ds->nf, fempic::env_stats(env), envl->amp, ds->coef);
-    DS_CUDA(cudaGetLastError());
-    k_ds_pre<double><<<blocks_for(p->n), kThreads, 0, st>>>(A);
   }
   DS_CUDA(cudaGetLastError());
-  // the AB4 segment: the env's own step under a zero field tracks, reflects
-  // or absorbs and deposits r^n -> r^n + dt u
-  fempic_envelope zero = *envl;
-  zero.amp = 0.0;
-  const int rc = fempic_push_step(env, p, &zero, omega0, t, dt, stream);
-  if (rc != FEMPIC_OK) return fail(rc, std::string("push_step_downshift: env step: ") + fempic_last_error());
-  if (mixed)
-    k_ds_post<float><<<blocks_for(p->n), kThreads, 0, st>>>(A);
-  else
-    k_ds_post<double><<<blocks_for(p->n), kThreads, 0, st>>>(A);
-  DS_CUDA(cudaGetLastError());
+  const int rc = fempic::push_downshift(env, p, A, dt, st);
+  if (rc != FEMPIC_OK) return fail(rc, std::string("push_step_downshift: ") + fempic_last_error());
   return FEMPIC_OK;
 }

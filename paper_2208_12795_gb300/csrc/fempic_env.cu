@@ -29,6 +29,7 @@
 #include <mutex>
 #include <string>
 
+#include "fempic_ds_rule.cuh"
 #include "fempic_internal.h"
 #include "fempic_tetgeo.cuh"
 
@@ -487,6 +488,29 @@ __device__ __forceinline__ Geo32 ld_geo(const float4* __restrict__ rec, int64_t 
   return G;
 }
 
+__device__ __forceinline__ Geo32 ld_geo_fresh(const float4* rec, int64_t T) {   // not hoisted over stores
+  Geo32 G;
+  float h[16];
+#pragma unroll
+  for (int k = 0; k < 4; k++) {
+    float4 v;
+    asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "l"(rec + 8 * T + k)
+                 : "memory");
+    h[4 * k] = v.x;
+    h[4 * k + 1] = v.y;
+    h[4 * k + 2] = v.z;
+    h[4 * k + 3] = v.w;
+  }
+#pragma unroll
+  for (int k = 0; k < 3; k++) G.x0[k] = __hiloint2double(__float_as_int(h[2 * k + 1]), __float_as_int(h[2 * k]));
+#pragma unroll
+  for (int k = 0; k < 9; k++) G.g[k] = h[6 + k];
+  G.kappa = h[15];
+  return G;
+}
+
 // d = r - x0: one FP64 subtraction (exact for points in or near the tet,
 // whose coordinates are close to x0's), split into an FP32 pair d = hi + lo
 // (lo keeps d to 2^-48 relative), and rounded to FP32 in d32.
@@ -722,7 +746,7 @@ __device__ __forceinline__ void lane_init(LaneOut& o, int lane) {
 }
 
 // Common path of one particle with its state already loaded: gather, carrier,
-// Boris, position update, then the inside test of the end point in the home
+// Boris (mixed_particle), then position update and the inside test of the end point in the home
 // tet.  A particle that stays in its tet writes its new state and keeps its
 // one-segment deposit for the warp reduction; any other hands (start point,
 // velocity, tet) to the CTA's crossing list.
@@ -731,40 +755,12 @@ __device__ __forceinline__ void lane_init(LaneOut& o, int lane) {
 //   tet's bound on their error, so that the FP64 barycentrics are >= 0 too;
 //   a particle within kappa of a face goes to the crossing pass, which
 //   decides in double-float.
+// s: species; G: the home tet's record; dd, d: r - x0 as FP32 pairs and
+// rounded; w: velocity of the segment; vs: velocity stored as the new state.
 template <bool Q24>
-__device__ __forceinline__ void mixed_particle(const PushArgs& A, int64_t p, int32_t T, double ax, double ay,
-                                               double az, float v0, float v1, float v2, LaneOut& o) {
-  if (T >= A.nt) {
-    A.tet[p] = -1;
-    A.status[p] = FEMPIC_P_LOST;
-    o.nfrz = 1;
-    return;
-  }
-  if (T < 0) return;
-  const int s = species_of(A.sp, p);
-  const float kq = A.sp.kq32[s];
-  const float4* R = A.tetrec + 8 * (int64_t)T;
-  const Geo32 G = ld_geo(A.tetrec, T);
-  const float4 f0 = __ldg(R + 4), f1 = __ldg(R + 5), f2 = __ldg(R + 6);
-  FF dd[3];
-  float d[3];
-  dpos(G, ax, ay, az, dd, d);
-  // f0 = (E0x, E0y, E0z, Wx), f1 = (Wy, Wz, B0x, B0y), f2 = (B0z, beta, -, -)
-  const float Ex = f0.x + (d[1] * f1.y - d[2] * f1.x);
-  const float Ey = f0.y + (d[2] * f0.w - d[0] * f1.y);
-  const float Ez = f0.z + (d[0] * f1.x - d[1] * f0.w);
-  const float Bx = f1.z + f2.y * d[0], By = f1.w + f2.y * d[1], Bz = f2.x + f2.y * d[2];
-  const float vmx = v0 + kq * Ex, vmy = v1 + kq * Ey, vmz = v2 + kq * Ez;
-  const float tx = kq * Bx, ty = kq * By, tz = kq * Bz;
-  const float t2 = tx * tx + ty * ty + tz * tz;
-  const float f = 2.0f / (1.0f + t2);
-  const float sx = f * tx, sy = f * ty, sz = f * tz;
-  const float vpx = vmx + (vmy * tz - vmz * ty);
-  const float vpy = vmy + (vmz * tx - vmx * tz);
-  const float vpz = vmz + (vmx * ty - vmy * tx);
-  const float vn0 = vmx + (vpy * sz - vpz * sy) + kq * Ex;
-  const float vn1 = vmy + (vpz * sx - vpx * sz) + kq * Ey;
-  const float vn2 = vmz + (vpx * sy - vpy * sx) + kq * Ez;
+__device__ __forceinline__ void mixed_drift(const PushArgs& A, int64_t p, int32_t T, int s, const Geo32& G,
+                                            const FF dd[3], const float d[3], double ax, double ay, double az,
+                                            float vn0, float vn1, float vn2, const float vs[3], LaneOut& o) {
   const float dt32 = A.dt32;
   // the FP32 displacement and the FP64 position update (advance's sequence)
   const float D0 = __fmul_rn(dt32, vn0), D1 = __fmul_rn(dt32, vn1), D2 = __fmul_rn(dt32, vn2);
@@ -796,9 +792,9 @@ __device__ __forceinline__ void mixed_particle(const PushArgs& A, int64_t p, int
   // Every lane stores its full new state, a queued particle included (its b
   // is final unless it reflects or freezes), so the warp's stores cover whole
   // sectors and the crossing kernel rarely rewrites positions.
-  static_cast<float*>(A.vx)[p] = vn0;
-  static_cast<float*>(A.vy)[p] = vn1;
-  static_cast<float*>(A.vz)[p] = vn2;
+  static_cast<float*>(A.vx)[p] = vs[0];
+  static_cast<float*>(A.vy)[p] = vs[1];
+  static_cast<float*>(A.vz)[p] = vs[2];
   A.x[p] = b0;
   A.y[p] = b1;
   A.z[p] = b2;
@@ -836,6 +832,44 @@ __device__ __forceinline__ void mixed_particle(const PushArgs& A, int64_t p, int
   o.key = T * kMaxSpecies + s;
   o.Thome = T;
   o.shome = s;
+}
+
+template <bool Q24>
+__device__ __forceinline__ void mixed_particle(const PushArgs& A, int64_t p, int32_t T, double ax, double ay,
+                                               double az, float v0, float v1, float v2, LaneOut& o) {
+  if (T >= A.nt) {
+    A.tet[p] = -1;
+    A.status[p] = FEMPIC_P_LOST;
+    o.nfrz = 1;
+    return;
+  }
+  if (T < 0) return;
+  const int s = species_of(A.sp, p);
+  const float kq = A.sp.kq32[s];
+  const float4* R = A.tetrec + 8 * (int64_t)T;
+  const Geo32 G = ld_geo(A.tetrec, T);
+  const float4 f0 = __ldg(R + 4), f1 = __ldg(R + 5), f2 = __ldg(R + 6);
+  FF dd[3];
+  float d[3];
+  dpos(G, ax, ay, az, dd, d);
+  // f0 = (E0x, E0y, E0z, Wx), f1 = (Wy, Wz, B0x, B0y), f2 = (B0z, beta, -, -)
+  const float Ex = f0.x + (d[1] * f1.y - d[2] * f1.x);
+  const float Ey = f0.y + (d[2] * f0.w - d[0] * f1.y);
+  const float Ez = f0.z + (d[0] * f1.x - d[1] * f0.w);
+  const float Bx = f1.z + f2.y * d[0], By = f1.w + f2.y * d[1], Bz = f2.x + f2.y * d[2];
+  const float vmx = v0 + kq * Ex, vmy = v1 + kq * Ey, vmz = v2 + kq * Ez;
+  const float tx = kq * Bx, ty = kq * By, tz = kq * Bz;
+  const float t2 = tx * tx + ty * ty + tz * tz;
+  const float f = 2.0f / (1.0f + t2);
+  const float sx = f * tx, sy = f * ty, sz = f * tz;
+  const float vpx = vmx + (vmy * tz - vmz * ty);
+  const float vpy = vmy + (vmz * tx - vmx * tz);
+  const float vpz = vmz + (vmx * ty - vmy * tx);
+  const float vn0 = vmx + (vpy * sz - vpz * sy) + kq * Ex;
+  const float vn1 = vmy + (vpz * sx - vpx * sz) + kq * Ey;
+  const float vn2 = vmz + (vpx * sy - vpy * sx) + kq * Ez;
+  const float vs[3] = {vn0, vn1, vn2};
+  mixed_drift<Q24>(A, p, T, s, G, dd, d, ax, ay, az, vn0, vn1, vn2, vs, o);
 }
 
 // Record regions of the mixed common path: each CTA appends the particles
@@ -994,6 +1028,112 @@ __global__ void __launch_bounds__(kThreads, 4) k_push_mixed(PushArgs A, int64_t 
     float v[3] = {0.f, 0.f, 0.f};
     load_plain(A, p, T, r, v);
     mixed_particle<Q24>(A, p, T, r[0], r[1], r[2], v[0], v[1], v[2], o);
+    mixed_warp_epilogue<Q24>(A, p, lane, o, cl);
+  }
+  publish_region(A, cl);
+}
+
+// Downshifted step on a mixed form: the velocity rule, then the AB4 segment's
+// position update, inside test and deposit in the same pass.  The tracked
+// velocity is u, the stored one v^{n+1}; walls mirror the stored velocity and
+// the history in the crossing pass.  Bound by the stream of history planes
+// (340 B per particle).  Each thread copies its own particle's values of the
+// CTA's next tile into shared memory (cp.async, 4 or 8 bytes each: history
+// planes of any n are 4-byte aligned only) as soon as the rule has used the
+// present ones, so that the copies run under the deposit; no thread reads
+// another's slots, so a thread waits for its own copies alone.  10M particles:
+// 761 us, against 547 (rule) + 431 (zero-field push) + 35 (its field) + 105
+// (mirror pass) in separate kernels and 791 with the history read into
+// registers; 66 % of the time its bytes take at the measured copy bandwidth.
+struct DsTile {
+  double r[3][kThreads];
+  float v[3][kThreads];
+  int32_t T[kThreads];
+  float h[FEMPIC_DS_VN][kThreads];   // history planes 0 .. FEMPIC_DS_VN - 1
+};
+
+__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+
+__device__ __forceinline__ void ds_fetch(const PushArgs& A, const DsRule& D, int64_t p, DsTile& S) {
+  const int t = threadIdx.x;
+  if (p < A.n) {
+    cp_async8(&S.r[0][t], A.x + p);
+    cp_async8(&S.r[1][t], A.y + p);
+    cp_async8(&S.r[2][t], A.z + p);
+    cp_async4(&S.v[0][t], static_cast<const float*>(A.vx) + p);
+    cp_async4(&S.v[1][t], static_cast<const float*>(A.vy) + p);
+    cp_async4(&S.v[2][t], static_cast<const float*>(A.vz) + p);
+    cp_async4(&S.T[t], A.tet + p);
+    if (!D.start) {
+      const float* H = static_cast<const float*>(D.h) + p;
+#pragma unroll
+      for (int k = 0; k < FEMPIC_DS_VN; k++) cp_async4(&S.h[k][t], H + k * D.n);
+    }
+  }
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+template <bool Q24>
+__global__ void __launch_bounds__(kThreads, 3) k_ds_push_mixed(PushArgs A, DsRule D, int64_t ntiles) {
+  extern __shared__ __align__(16) unsigned char ds_smem[];
+  DsTile& S = *reinterpret_cast<DsTile*>(ds_smem);
+  __shared__ CrossList cl;
+  const int tid = threadIdx.x, lane = tid & 31;
+  if (tid == 0) cl.total = 0;
+  __syncthreads();
+  ds_fetch(A, D, blockIdx.x * (int64_t)kThreads + tid, S);
+  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const int64_t p = tile * kThreads + tid;
+    LaneOut o;
+    lane_init(o, lane);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    const int32_t T = p < A.n ? S.T[tid] : -1;
+    const double r[3] = {S.r[0][tid], S.r[1][tid], S.r[2][tid]};
+    bool frozen = false;
+    int s = 0;
+    float vn[3], u[3];
+    if (T >= A.nt) {
+      A.tet[p] = -1;
+      A.status[p] = FEMPIC_P_LOST;
+      o.nfrz = 1;
+    } else if (T >= 0) {
+      s = species_of(A.sp, p);
+      const float v[3] = {S.v[0][tid], S.v[1][tid], S.v[2][tid]};
+      const double* x0 = reinterpret_cast<const double*>(A.tetrec + 8 * (int64_t)T);
+      const float d[3] = {(float)__dsub_rn(r[0], __ldg(x0)), (float)__dsub_rn(r[1], __ldg(x0 + 1)),
+                          (float)__dsub_rn(r[2], __ldg(x0 + 2))};
+      const bool bad = ds_rule32(D, p, T, s, d, v, vn, u, [&](int k) { return S.h[k][tid]; });
+      if (bad || !isfinite(A.sp.kq32[s])) {   // a field that is not finite: frozen as the zero-field step would
+        A.status[p] = FEMPIC_P_NONFINITE;
+        A.tet[p] = -2 - T;
+        o.nfrz = 1;
+      }
+      frozen = o.nfrz != 0;
+    }
+    if (tile + gridDim.x < ntiles) ds_fetch(A, D, p + (int64_t)gridDim.x * kThreads, S);
+    if (T >= 0 && T < A.nt) {
+      if (!frozen) {
+        // the record is read after the rule's stores, so that its registers
+        // are not held while the history streams through
+        const Geo32 G = ld_geo_fresh(A.tetrec, T);
+        FF dd[3];
+        float d[3];
+        dpos(G, r[0], r[1], r[2], dd, d);
+        mixed_drift<Q24>(A, p, T, s, G, dd, d, r[0], r[1], r[2], u[0], u[1], u[2], vn, o);
+      }
+      if (o.nfrz) {   // not finite: the position stays, the velocity moves on
+        static_cast<float*>(A.vx)[p] = vn[0];
+        static_cast<float*>(A.vy)[p] = vn[1];
+        static_cast<float*>(A.vz)[p] = vn[2];
+      }
+    }
     mixed_warp_epilogue<Q24>(A, p, lane, o, cl);
   }
   publish_region(A, cl);
@@ -1158,13 +1298,26 @@ __global__ void __launch_bounds__(kThreads, FEMPIC_TMA_MIN_BLOCKS) k_push_mixed_
   publish_region(A, cl);
 }
 
+// The wall mirrors of a finished walk, on the velocity the common path stored
+// (in a downshifted step v^{n+1}, whose history is mirrored with it; there an
+// axis along which the segment does not move stays as it is).
+template <typename R>
+__device__ __forceinline__ void cross_mirror(const PushArgs& A, const DsRule* H, int64_t p, unsigned flips) {
+  R* vv[3] = {static_cast<R*>(A.vx), static_cast<R*>(A.vy), static_cast<R*>(A.vz)};
+  if (H) flips &= flips >> 3;
+#pragma unroll
+  for (int k = 0; k < 3; k++)
+    if (flips & (1u << k)) vv[k][p] = -vv[k][p];
+  if (H && (flips & 7u)) ds_mirror<R>(*H, p, flips);
+}
+
 // Crossing path of a particle that leaves its home tet, one face at a time.
 // State of the walk: the current straight piece runs from a0 + sacc (b - a0)
 // to b inside tet T, with end barycentrics Qa -> Qb; `entry` is the face it
 // came in through.
 struct CrossState {
   double a0[3], b[3];
-  float vn[3];
+  unsigned flips;   // bit k: velocity component k mirrored an odd number of times; bit 3 + k: it is not zero
   int32_t Qa[4], Qb[4];
   int32_t T, p;
   int entry, nc, s;
@@ -1180,10 +1333,11 @@ __device__ __forceinline__ void cross_begin(const PushArgs& A, const CrossRec& r
   c.T = r.T;
   c.s = species_of(A.sp, r.p);
   const float dt32 = A.dt32;
+  c.flips = 0u;
 #pragma unroll
   for (int k = 0; k < 3; k++) {
     c.a0[k] = r.a[k];
-    c.vn[k] = r.v[k];
+    if (r.v[k] != 0.f) c.flips |= 8u << k;
     c.b[k] = advance(r.a[k], dt32, r.v[k]);
   }
   c.entry = -1;
@@ -1276,7 +1430,7 @@ __device__ __forceinline__ bool cross_advance(const PushArgs& A, CrossState& c, 
       if (k == ax) {
         const double L = side ? A.hi[k] : A.lo[k];
         c.b[k] = 2.0 * L - c.b[k];
-        c.vn[k] = -c.vn[k];
+        c.flips ^= 1u << k;
       }
     c.reflected = true;
 #pragma unroll
@@ -1293,7 +1447,8 @@ __device__ __forceinline__ bool cross_advance(const PushArgs& A, CrossState& c, 
 }
 
 // Final state of a finished walk.
-__device__ __forceinline__ void cross_finish(const PushArgs& A, const CrossState& c, unsigned& ncr, unsigned& nfrz) {
+__device__ __forceinline__ void cross_finish(const PushArgs& A, const DsRule* H, const CrossState& c, unsigned& ncr,
+                                             unsigned& nfrz) {
   const int64_t p = c.p;
   if (c.moved) {
     if (c.reflected) {   // otherwise b is what the common path already stored
@@ -1318,11 +1473,7 @@ __device__ __forceinline__ void cross_finish(const PushArgs& A, const CrossState
     gq(c.Qa, Qf, g);
     depositq_atomic(A, c.T, c.s, g);
   }
-  if (c.reflected) {
-    static_cast<float*>(A.vx)[p] = c.vn[0];
-    static_cast<float*>(A.vy)[p] = c.vn[1];
-    static_cast<float*>(A.vz)[p] = c.vn[2];
-  }
+  cross_mirror<float>(A, H, p, c.flips);
   int32_t T = c.T;
   if (c.st != FEMPIC_P_OK) {
     A.status[p] = c.st;
@@ -1346,8 +1497,9 @@ __device__ __forceinline__ void cross_finish(const PushArgs& A, const CrossState
 // warp with lanes refilled one by one: 1.30 -> 1.21 ms per step on that load,
 // 0.203 -> 0.185 on the 10M cavity; waiting for 1, 8, 12, 16 idle lanes:
 // 1.29, 1.24, 1.21, 1.22 ms.
-constexpr int kCrossThreadsDF = 192;    // contract pass: 4 CTAs per SM at 80 registers
-constexpr int kCrossThreadsQ24 = 256;   // 24-bit pass: 4 CTAs per SM at 64 registers
+// A pass's CTAs number as many per SM as its common path's, so their size
+// makes up the warps: 24 per SM (32 in the 24-bit pass, at 64 registers).
+constexpr int kCrossMax = 512;
 constexpr int kRefill = 12;
 
 // Hands out the region's records to idle lanes: >= 0 for a lane that takes
@@ -1363,7 +1515,7 @@ __device__ __forceinline__ int32_t draw_record(unsigned idle, int lane, bool hav
   return !have && k < cnt ? k : -1;
 }
 
-__global__ void __launch_bounds__(kCrossThreadsQ24, 4) k_cross_q24(PushArgs A) {
+__global__ void __launch_bounds__(kCrossMax, 2) k_cross_q24(PushArgs A, DsRule D) {
   __shared__ int32_t cursor;
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
@@ -1389,7 +1541,7 @@ __global__ void __launch_bounds__(kCrossThreadsQ24, 4) k_cross_q24(PushArgs A) {
       const bool done = cross_advance(A, c, fresh);
       fresh = false;
       if (done) {
-        cross_finish(A, c, ncr, nfrz);
+        cross_finish(A, D.h ? &D : nullptr, c, ncr, nfrz);
         have = false;
       }
     }
@@ -1419,7 +1571,7 @@ struct CrossStateDF {
   DF S;                 // ... and the current piece starts at a0 + S (b - a0)
   FF w[3];              // b - a0 as FP32 pairs (before a reflection: exactly dt v)
   DF la[4];             // barycentrics of the piece start in T
-  unsigned flips;       // bit k: velocity component k mirrored an odd number of times
+  unsigned flips;       // bit k: velocity component k mirrored an odd number of times; bit 3 + k: it is not zero
   int32_t T, p;
   int entry, nc, s;
   uint8_t st;
@@ -1495,13 +1647,14 @@ __device__ __forceinline__ void cross_begin_df(const PushArgs& A, const CrossRec
   c.T = r.T;
   c.s = species_of(A.sp, r.p);
   const float dt32 = A.dt32;
+  c.flips = 0u;
 #pragma unroll
   for (int k = 0; k < 3; k++) {
     c.a0[k] = r.a[k];
+    if (r.v[k] != 0.f) c.flips |= 8u << k;
     c.w[k] = FF{__fmul_rn(dt32, r.v[k]), 0.f};
     c.b[k] = __dadd_rn(r.a[k], (double)c.w[k].hi);   // advance's value (the widening is exact)
   }
-  c.flips = 0u;
   c.S = DF{0.f, 0.f};
   c.entry = -1;
   c.nc = 0;
@@ -1615,8 +1768,8 @@ __device__ __forceinline__ bool cross_advance_df(const PushArgs& A, CrossStateDF
   return false;
 }
 
-__device__ __forceinline__ void cross_finish_df(const PushArgs& A, const CrossStateDF& c, unsigned& ncr,
-                                                unsigned& nfrz) {
+__device__ __forceinline__ void cross_finish_df(const PushArgs& A, const DsRule* H, const CrossStateDF& c,
+                                                unsigned& ncr, unsigned& nfrz) {
   const int64_t p = c.p;
   if (!c.moved) {   // frozen at the last crossing point
     double r[3];
@@ -1629,11 +1782,7 @@ __device__ __forceinline__ void cross_finish_df(const PushArgs& A, const CrossSt
     A.y[p] = c.b[1];
     A.z[p] = c.b[2];
   }
-  // the common path stored the new velocity; mirror the reflected components
-  float* vv[3] = {static_cast<float*>(A.vx), static_cast<float*>(A.vy), static_cast<float*>(A.vz)};
-#pragma unroll
-  for (int k = 0; k < 3; k++)
-    if (c.flips & (1u << k)) vv[k][p] = -vv[k][p];
+  cross_mirror<float>(A, H, p, c.flips);
   int32_t T = c.T;
   if (c.st != FEMPIC_P_OK) {
     A.status[p] = c.st;
@@ -1645,7 +1794,7 @@ __device__ __forceinline__ void cross_finish_df(const PushArgs& A, const CrossSt
   ncr += (unsigned)c.nc;
 }
 
-__global__ void __launch_bounds__(kCrossThreadsDF, 4) k_cross_df(PushArgs A) {
+__global__ void __launch_bounds__(384, 2) k_cross_df(PushArgs A, DsRule D) {
   __shared__ int32_t cursor;
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
@@ -1671,7 +1820,7 @@ __global__ void __launch_bounds__(kCrossThreadsDF, 4) k_cross_df(PushArgs A) {
       const bool done = cross_advance_df(A, c, fresh);
       fresh = false;
       if (done) {
-        cross_finish_df(A, c, ncr, nfrz);
+        cross_finish_df(A, D.h ? &D : nullptr, c, ncr, nfrz);
         have = false;
       }
     }
@@ -1738,114 +1887,176 @@ __device__ __forceinline__ void deposit64(const PushArgs& A, int32_t T, const do
 
 __device__ __forceinline__ CrossRec64* xregion64(const PushArgs& A) { return A.xrec64 + blockIdx.x * A.xcap; }
 
+// One segment a -> b = a + dt w of a particle in tet T (G its record, d = a -
+// x0): position and stored velocity vs written, the deposit of a particle
+// surely inside.  Returns whether the crossing pass has to decide; counts a
+// particle that is not finite in nfrz.
+__device__ __forceinline__ bool drift64(const PushArgs& A, int64_t p, int32_t T, int s, const Geo32& G,
+                                        const double a[3], const double d[3], const double w[3], const double vs[3],
+                                        unsigned& nfrz) {
+  const double b[3] = {fma(A.dt, w[0], a[0]), fma(A.dt, w[1], a[1]), fma(A.dt, w[2], a[2])};
+  if (!(finite_bits(w[0]) && finite_bits(w[1]) && finite_bits(w[2]) && finite_bits(b[0]) && finite_bits(b[1]) &&
+        finite_bits(b[2]))) {
+    A.status[p] = FEMPIC_P_NONFINITE;
+    A.tet[p] = -2 - T;
+    nfrz++;
+    return false;
+  }
+  A.x[p] = b[0];
+  A.y[p] = b[1];
+  A.z[p] = b[2];
+  static_cast<double*>(A.vx)[p] = vs[0];
+  static_cast<double*>(A.vy)[p] = vs[1];
+  static_cast<double*>(A.vz)[p] = vs[2];
+  const double D[3] = {b[0] - a[0], b[1] - a[1], b[2] - a[2]};
+  // inside when all four FP32 barycentrics of b reach kappa, the bound on
+  // their error for a start in the tet (|lambda(a)| is checked too: a start
+  // far outside would void the bound)
+  float lo = INFINITY, la = INFINITY, sb = 1.0f, sa = 1.0f;
+  const float d32[3] = {trunc32(d[0]), trunc32(d[1]), trunc32(d[2])};
+  const float e32[3] = {d32[0] + trunc32(D[0]), d32[1] + trunc32(D[1]), d32[2] + trunc32(D[2])};
+#pragma unroll
+  for (int k = 0; k < 3; k++) {
+    const float lb = G.g[3 * k] * e32[0] + G.g[3 * k + 1] * e32[1] + G.g[3 * k + 2] * e32[2];
+    const float l0 = G.g[3 * k] * d32[0] + G.g[3 * k + 1] * d32[1] + G.g[3 * k + 2] * d32[2];
+    sb -= lb;
+    sa -= l0;
+    lo = fminf(lo, lb);
+    la = fminf(la, l0);
+  }
+  if (!(fminf(lo, sb) >= G.kappa && fminf(la, sa) >= -1.0f)) return true;
+  deposit64(A, T, d, D, A.sp.qw[s]);   // (f) the whole segment is in the home tet
+  return false;
+}
+
+// Records of a warp's undecided particles, in the CTA's region.
+__device__ __forceinline__ void queue64(const PushArgs& A, int64_t p, int32_t T, const double a[3], const double w[3],
+                                        bool leave, int32_t* total) {
+  const int lane = threadIdx.x & 31;
+  const unsigned qmask = __ballot_sync(0xffffffffu, leave);
+  if (!qmask) return;
+  int base = 0;
+  if (lane == 0) base = atomicAdd(total, __popc(qmask));
+  base = __shfl_sync(0xffffffffu, base, 0);
+  if (leave) {
+    double2* r = xregion64(A)[base + __popc(qmask & ((1u << lane) - 1u))].w;
+    r[0] = make_double2(a[0], a[1]);
+    r[1] = make_double2(a[2], w[0]);
+    r[2] = make_double2(w[1], w[2]);
+    r[3] = make_double2(__hiloint2double((int32_t)p, T), 0.0);
+  }
+}
+
+// End of a CTA's work (all threads): frozen count and record count.
+__device__ __forceinline__ void publish64(const PushArgs& A, unsigned nfrz, const int32_t& total) {
+  nfrz = __reduce_add_sync(0xffffffffu, nfrz);
+  if ((threadIdx.x & 31) == 0 && nfrz) atomicAdd(A.stats + 1, (unsigned long long)nfrz);
+  __syncthreads();
+  if (threadIdx.x == 0) A.xcount[blockIdx.x] = total;
+}
+
+// The state of this thread's particle of a tile; T = -1 where there is none.
+// An out-of-range tet is marked LOST here.
+__device__ __forceinline__ int32_t load64(const PushArgs& A, int64_t p, double a[3], double v[3], unsigned& nfrz) {
+  int32_t T = p < A.n ? A.tet[p] : -1;
+  if (T >= A.nt) {
+    A.tet[p] = -1;
+    A.status[p] = FEMPIC_P_LOST;
+    nfrz++;
+    T = -1;
+  }
+  if (T < 0) return -1;
+  a[0] = A.x[p];
+  a[1] = A.y[p];
+  a[2] = A.z[p];
+  v[0] = static_cast<const double*>(A.vx)[p];
+  v[1] = static_cast<const double*>(A.vy)[p];
+  v[2] = static_cast<const double*>(A.vz)[p];
+  return T;
+}
+
 // FP64 form, common path: persistent CTAs walk 256-particle tiles, one
 // particle per thread.  A particle surely inside its home tet deposits its
 // segment and is done; any other stores its new state provisionally and a
 // record for the crossing pass.
 __global__ void __launch_bounds__(kThreads) k_push_fp64(PushArgs A, int64_t ntiles) {
   __shared__ int32_t total;
-  const int lane = threadIdx.x & 31;
-  const unsigned full = 0xffffffffu;
   if (threadIdx.x == 0) total = 0;
   __syncthreads();
   unsigned nfrz = 0;
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const int64_t p = tile * kTile + threadIdx.x;
+    const int64_t p = tile * kThreads + threadIdx.x;
     bool leave = false;
-    double a[3] = {0.0, 0.0, 0.0}, vn[3] = {0.0, 0.0, 0.0};
-    int32_t T = -1;
-    if (p < A.n) {
-      T = A.tet[p];
-      if (T >= A.nt) {
-        A.tet[p] = -1;
-        A.status[p] = FEMPIC_P_LOST;
-        nfrz++;
-      } else if (T >= 0) {
-        const int s = species_of(A.sp, p);
-        const double kq = A.sp.kq[s];
-        double* vxp = static_cast<double*>(A.vx);
-        double* vyp = static_cast<double*>(A.vy);
-        double* vzp = static_cast<double*>(A.vz);
-        a[0] = A.x[p];
-        a[1] = A.y[p];
-        a[2] = A.z[p];
-        const double v[3] = {vxp[p], vyp[p], vzp[p]};
-        const Geo32 G = ld_geo(A.tetrec, T);   // x0 exact; FP32 gradients and error bound for the inside test
-        const double2* F = reinterpret_cast<const double2*>(static_cast<const double*>(A.field) + 10 * (int64_t)T);
-        const double2 f0 = __ldg(F), f1 = __ldg(F + 1), f2 = __ldg(F + 2), f3 = __ldg(F + 3), f4 = __ldg(F + 4);
-        const double d[3] = {a[0] - G.x0[0], a[1] - G.x0[1], a[2] - G.x0[2]};
-        // (b)+(c) gather with the carrier already restored per tet
-        const double Wx = f1.y, Wy = f2.x, Wz = f2.y, beta = f4.y;
-        const double Ex = fma(d[1], Wz, fma(-d[2], Wy, f0.x));
-        const double Ey = fma(d[2], Wx, fma(-d[0], Wz, f0.y));
-        const double Ez = fma(d[0], Wy, fma(-d[1], Wx, f1.x));
-        // (d) Boris
-        const double vmx = fma(kq, Ex, v[0]), vmy = fma(kq, Ey, v[1]), vmz = fma(kq, Ez, v[2]);
-        const double tx = kq * fma(beta, d[0], f3.x), ty = kq * fma(beta, d[1], f3.y), tz = kq * fma(beta, d[2], f4.x);
-        const double f = 2.0 * recip_ge1(fma(tx, tx, fma(ty, ty, fma(tz, tz, 1.0))));
-        const double sx = f * tx, sy = f * ty, sz = f * tz;
-        const double vpx = fma(vmy, tz, fma(-vmz, ty, vmx));
-        const double vpy = fma(vmz, tx, fma(-vmx, tz, vmy));
-        const double vpz = fma(vmx, ty, fma(-vmy, tx, vmz));
-        vn[0] = fma(kq, Ex, fma(vpy, sz, fma(-vpz, sy, vmx)));
-        vn[1] = fma(kq, Ey, fma(vpz, sx, fma(-vpx, sz, vmy)));
-        vn[2] = fma(kq, Ez, fma(vpx, sy, fma(-vpy, sx, vmz)));
-        const double b[3] = {fma(A.dt, vn[0], a[0]), fma(A.dt, vn[1], a[1]), fma(A.dt, vn[2], a[2])};
-        if (!(finite_bits(vn[0]) && finite_bits(vn[1]) && finite_bits(vn[2]) && finite_bits(b[0]) &&
-              finite_bits(b[1]) && finite_bits(b[2]))) {
-          A.status[p] = FEMPIC_P_NONFINITE;
-          A.tet[p] = -2 - T;
-          nfrz++;
-        } else {
-          A.x[p] = b[0];
-          A.y[p] = b[1];
-          A.z[p] = b[2];
-          vxp[p] = vn[0];
-          vyp[p] = vn[1];
-          vzp[p] = vn[2];
-          const double D[3] = {b[0] - a[0], b[1] - a[1], b[2] - a[2]};
-          // inside when all four FP32 barycentrics of b reach kappa, the
-          // bound on their error for a start in the tet (|lambda(a)| is
-          // checked too: a start far outside would void the bound)
-          float lo = INFINITY, la = INFINITY;
-          {
-            const float d32[3] = {trunc32(d[0]), trunc32(d[1]), trunc32(d[2])};
-            const float e32[3] = {d32[0] + trunc32(D[0]), d32[1] + trunc32(D[1]), d32[2] + trunc32(D[2])};
-            float sb = 1.0f, sa = 1.0f;
-#pragma unroll
-            for (int k = 0; k < 3; k++) {
-              const float lb = G.g[3 * k] * e32[0] + G.g[3 * k + 1] * e32[1] + G.g[3 * k + 2] * e32[2];
-              const float l0 = G.g[3 * k] * d32[0] + G.g[3 * k + 1] * d32[1] + G.g[3 * k + 2] * d32[2];
-              sb -= lb;
-              sa -= l0;
-              lo = fminf(lo, lb);
-              la = fminf(la, l0);
-            }
-            leave = !(fminf(lo, sb) >= G.kappa && fminf(la, sa) >= -1.0f);
-          }
-          if (!leave) deposit64(A, T, d, D, A.sp.qw[s]);   // (f) the whole segment is in the home tet
-        }
-      }
+    double a[3] = {0.0, 0.0, 0.0}, v[3] = {0.0, 0.0, 0.0}, vn[3] = {0.0, 0.0, 0.0};
+    const int32_t T = load64(A, p, a, v, nfrz);
+    if (T >= 0) {
+      const int s = species_of(A.sp, p);
+      const double kq = A.sp.kq[s];
+      const Geo32 G = ld_geo(A.tetrec, T);   // x0 exact; FP32 gradients and error bound for the inside test
+      const double2* F = reinterpret_cast<const double2*>(static_cast<const double*>(A.field) + 10 * (int64_t)T);
+      const double2 f0 = __ldg(F), f1 = __ldg(F + 1), f2 = __ldg(F + 2), f3 = __ldg(F + 3), f4 = __ldg(F + 4);
+      const double d[3] = {a[0] - G.x0[0], a[1] - G.x0[1], a[2] - G.x0[2]};
+      // (b)+(c) gather with the carrier already restored per tet
+      const double Wx = f1.y, Wy = f2.x, Wz = f2.y, beta = f4.y;
+      const double Ex = fma(d[1], Wz, fma(-d[2], Wy, f0.x));
+      const double Ey = fma(d[2], Wx, fma(-d[0], Wz, f0.y));
+      const double Ez = fma(d[0], Wy, fma(-d[1], Wx, f1.x));
+      // (d) Boris
+      const double vmx = fma(kq, Ex, v[0]), vmy = fma(kq, Ey, v[1]), vmz = fma(kq, Ez, v[2]);
+      const double tx = kq * fma(beta, d[0], f3.x), ty = kq * fma(beta, d[1], f3.y), tz = kq * fma(beta, d[2], f4.x);
+      const double f = 2.0 * recip_ge1(fma(tx, tx, fma(ty, ty, fma(tz, tz, 1.0))));
+      const double sx = f * tx, sy = f * ty, sz = f * tz;
+      const double vpx = fma(vmy, tz, fma(-vmz, ty, vmx));
+      const double vpy = fma(vmz, tx, fma(-vmx, tz, vmy));
+      const double vpz = fma(vmx, ty, fma(-vmy, tx, vmz));
+      vn[0] = fma(kq, Ex, fma(vpy, sz, fma(-vpz, sy, vmx)));
+      vn[1] = fma(kq, Ey, fma(vpz, sx, fma(-vpx, sz, vmy)));
+      vn[2] = fma(kq, Ez, fma(vpx, sy, fma(-vpy, sx, vmz)));
+      leave = drift64(A, p, T, s, G, a, d, vn, vn, nfrz);
     }
-    // (e) the others: records for the crossing pass, in the CTA's region
-    const unsigned qmask = __ballot_sync(full, leave);
-    if (qmask) {
-      int base = 0;
-      if (lane == 0) base = atomicAdd(&total, __popc(qmask));
-      base = __shfl_sync(full, base, 0);
-      if (leave) {
-        double2* r = xregion64(A)[base + __popc(qmask & ((1u << lane) - 1u))].w;
-        r[0] = make_double2(a[0], a[1]);
-        r[1] = make_double2(a[2], vn[0]);
-        r[2] = make_double2(vn[1], vn[2]);
-        r[3] = make_double2(__hiloint2double((int32_t)p, T), 0.0);
-      }
-    }
+    queue64(A, p, T, a, vn, leave, &total);
   }
-  nfrz = __reduce_add_sync(full, nfrz);
-  if (lane == 0 && nfrz) atomicAdd(A.stats + 1, (unsigned long long)nfrz);
+  publish64(A, nfrz, total);
+}
+
+// Downshifted step on the FP64 form: the velocity rule, then the AB4 segment
+// (tracked velocity u, stored velocity v^{n+1}; walls mirror the stored
+// velocity and the history in the crossing pass).  FP64-pipe bound: 553 us at
+// 2M particles, against 686 (rule) + 220 (zero-field push) + 30 + 34 in
+// separate kernels; 1 and 3 CTAs per SM: 597 and 575 us.
+__global__ void __launch_bounds__(kThreads, 2) k_ds_push_fp64(PushArgs A, DsRule D, int64_t ntiles) {
+  __shared__ int32_t total;
+  if (threadIdx.x == 0) total = 0;
   __syncthreads();
-  if (threadIdx.x == 0) A.xcount[blockIdx.x] = total;
+  unsigned nfrz = 0;
+  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const int64_t p = tile * kThreads + threadIdx.x;
+    bool leave = false;
+    double a[3] = {0.0, 0.0, 0.0}, v[3] = {0.0, 0.0, 0.0}, u[3] = {0.0, 0.0, 0.0};
+    const int32_t T = load64(A, p, a, v, nfrz);
+    if (T >= 0) {
+      const int s = species_of(A.sp, p);
+      const Geo32 G = ld_geo(A.tetrec, T);
+      const double d[3] = {a[0] - G.x0[0], a[1] - G.x0[1], a[2] - G.x0[2]};
+      double vn[3];
+      const bool bad = ds_rule(D, p, T, s, d, v, vn, u) || !finite_bits(A.sp.kq[s]);
+      const unsigned before = nfrz;
+      if (bad) {   // a field that is not finite: frozen as the zero-field step would
+        A.status[p] = FEMPIC_P_NONFINITE;
+        A.tet[p] = -2 - T;
+        nfrz++;
+      } else {
+        leave = drift64(A, p, T, s, G, a, d, u, vn, nfrz);
+      }
+      if (nfrz != before) {   // the position stays, the velocity moves on
+        static_cast<double*>(A.vx)[p] = vn[0];
+        static_cast<double*>(A.vy)[p] = vn[1];
+        static_cast<double*>(A.vz)[p] = vn[2];
+      }
+    }
+    queue64(A, p, T, a, u, leave, &total);
+  }
+  publish64(A, nfrz, total);
 }
 
 // FP64 form, crossing pass: the walk of one leaving particle, one face per
@@ -1853,8 +2064,9 @@ __global__ void __launch_bounds__(kThreads) k_push_fp64(PushArgs A, int64_t ntil
 // crossing point a + s (b - a), barycentrics carried exactly onto the
 // neighbour's shared nodes).
 struct CrossState64 {
-  double a[3], b[3], vn[3];
+  double a[3], b[3];
   double la[4], lb[4];
+  unsigned flips;   // bit k: velocity component k mirrored an odd number of times; bit 3 + k: it is not zero
   int32_t T, p;
   int entry, nc, s;
   uint8_t st;
@@ -1869,11 +2081,13 @@ __device__ __forceinline__ void cross64_begin(const PushArgs& A, const CrossRec6
   c.a[0] = r0.x;
   c.a[1] = r0.y;
   c.a[2] = r1.x;
-  c.vn[0] = r1.y;
-  c.vn[1] = r2.x;
-  c.vn[2] = r2.y;
+  const double v[3] = {r1.y, r2.x, r2.y};
+  c.flips = 0u;
 #pragma unroll
-  for (int k = 0; k < 3; k++) c.b[k] = fma(A.dt, c.vn[k], c.a[k]);
+  for (int k = 0; k < 3; k++) {
+    if (((unsigned)__double2hiint(v[k]) << 1 | (unsigned)__double2loint(v[k])) != 0u) c.flips |= 8u << k;
+    c.b[k] = fma(A.dt, v[k], c.a[k]);
+  }
   c.entry = -1;
   c.nc = 0;
   c.st = FEMPIC_P_OK;
@@ -1996,7 +2210,7 @@ __device__ __forceinline__ bool cross64_advance(const PushArgs& A, CrossState64&
       if (k == ax) {
         const double L = side ? A.hi[k] : A.lo[k];
         c.b[k] = 2.0 * L - c.b[k];
-        c.vn[k] = -c.vn[k];
+        c.flips ^= 1u << k;
       }
     c.reflected = true;
 #pragma unroll
@@ -2009,19 +2223,15 @@ __device__ __forceinline__ bool cross64_advance(const PushArgs& A, CrossState64&
   return false;
 }
 
-__device__ __forceinline__ void cross64_finish(const PushArgs& A, const CrossState64& c, unsigned& ncr,
-                                               unsigned& nfrz) {
+__device__ __forceinline__ void cross64_finish(const PushArgs& A, const DsRule* H, const CrossState64& c,
+                                               unsigned& ncr, unsigned& nfrz) {
   const int64_t p = c.p;
   if (c.st != FEMPIC_P_OK || c.reflected) {   // otherwise a = b, already stored
     A.x[p] = c.a[0];
     A.y[p] = c.a[1];
     A.z[p] = c.a[2];
   }
-  if (c.reflected) {
-    static_cast<double*>(A.vx)[p] = c.vn[0];
-    static_cast<double*>(A.vy)[p] = c.vn[1];
-    static_cast<double*>(A.vz)[p] = c.vn[2];
-  }
+  cross_mirror<double>(A, H, p, c.flips);
   int32_t T = c.T;
   if (c.st != FEMPIC_P_OK) {
     A.status[p] = c.st;
@@ -2035,8 +2245,7 @@ __device__ __forceinline__ void cross64_finish(const PushArgs& A, const CrossSta
 
 // One CTA per record region, records drawn from a shared cursor (as the mixed
 // passes).
-constexpr int kCrossThreads64 = 192;
-__global__ void __launch_bounds__(kCrossThreads64) k_cross_fp64(PushArgs A) {
+__global__ void __launch_bounds__(384, 2) k_cross_fp64(PushArgs A, DsRule D) {
   __shared__ int32_t cursor;
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
@@ -2062,7 +2271,7 @@ __global__ void __launch_bounds__(kCrossThreads64) k_cross_fp64(PushArgs A) {
       const bool done = cross64_advance(A, c, fresh);
       fresh = false;
       if (done) {
-        cross64_finish(A, c, ncr, nfrz);
+        cross64_finish(A, D.h ? &D : nullptr, c, ncr, nfrz);
         have = false;
       }
     }
@@ -3201,7 +3410,8 @@ struct fempic_env {
   int32_t* xcount = nullptr;        // [xregions]
   int64_t xslots = 0, xregions = 0;
   int num_sms = 1;
-  int push_blocks_per_sm[5] = {0, 0, 0, 0, 0};   // resident CTAs of the common path: mixed [24-bit] + 2 [staged], FP64 4
+  // resident CTAs of the common path: mixed [24-bit] + 2 [staged], FP64 4; downshifted: the same + 5
+  int push_blocks_per_sm[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
   int64_t steps = 0;
   // per-kernel event timing (measurement support)
   struct Rec {
@@ -3616,6 +3826,123 @@ static int validate_step(const fempic_particles* p, const HostLevels& H, double 
   return fill_species(p, dt, sp);
 }
 
+// The particle work of a step, after its per-tet fields: common path, then
+// crossing pass.  A.sp is filled; a rule with history planes makes it a
+// downshifted step.
+static int push_particles(fempic_env* env, const fempic_particles* p, PushArgs& A, double dt, const DsRule& D,
+                          cudaStream_t st) {
+  int rc = FEMPIC_OK;
+  env->ns_last = p->n_species;
+  for (int s = 0; s < kMaxSpecies; s++) env->qw_last[s] = A.sp.qw[s];
+  env->steps++;
+  if (p->n == 0) return FEMPIC_OK;
+  const bool mixed = env->opt.precision != FEMPIC_FP64;
+  const bool q24 = env->opt.precision == FEMPIC_MIXED_Q24;
+  const bool ds = D.h != nullptr;
+  A.n = p->n;
+  A.x = p->x;
+  A.y = p->y;
+  A.z = p->z;
+  A.vx = p->vx;
+  A.vy = p->vy;
+  A.vz = p->vz;
+  A.tet = p->tet;
+  A.status = p->status;
+  A.ncross = p->n_cross;
+  A.dt = dt;
+  A.dt32 = (float)dt;
+  A.max_cross = env->opt.max_crossings;
+  A.wall_mode = env->opt.wall_mode;
+  for (int a = 0; a < 3; a++) {
+    A.lo[a] = env->h.lo[a];
+    A.hi[a] = env->h.hi[a];
+  }
+  A.nt = env->h.nt;
+  A.ne = env->h.ne;
+  A.geom64 = env->geom64;
+  A.tetrec = env->tetrec;
+  A.tn = env->tn;
+  A.nb = env->nb;
+  A.te = env->te;
+  A.field = env->field;
+  A.dGq = env->deposit_on ? env->dGq : nullptr;
+  A.mom = env->deposit_on ? env->mom : nullptr;
+  A.momlo = env->momlo;
+  A.tetdf = env->tetdf;
+  A.stats = env->stats;
+  // the common path's launch: persistent CTAs; the mixed forms' are staged
+  // when every particle array allows bulk copies (16-byte aligned sources)
+  // and there is a full tile
+  const int64_t all_tiles = (p->n + kTile - 1) / kTile;
+  const uintptr_t align = (uintptr_t)p->x | (uintptr_t)p->y | (uintptr_t)p->z | (uintptr_t)p->vx |
+                          (uintptr_t)p->vy | (uintptr_t)p->vz | (uintptr_t)p->tet;
+  const int64_t nfull = (mixed && !ds && FEMPIC_USE_TMA && !(align & 15u)) ? p->n / kTile : 0;
+  int& bps = env->push_blocks_per_sm[(mixed ? (q24 ? 1 : 0) + (nfull > 0 ? 2 : 0) : 4) + (ds ? 5 : 0)];
+  if (bps == 0) {
+    const void* k = ds          ? (!mixed ? (const void*)k_ds_push_fp64
+                                   : q24  ? (const void*)k_ds_push_mixed<true>
+                                          : (const void*)k_ds_push_mixed<false>)
+                    : !mixed    ? (const void*)k_push_fp64
+                    : nfull > 0 ? (q24 ? (const void*)k_push_mixed_tma<true> : (const void*)k_push_mixed_tma<false>)
+                                : (q24 ? (const void*)k_push_mixed<true> : (const void*)k_push_mixed<false>);
+    if (ds && mixed) FEMPIC_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(DsTile)));
+    int nb = 0;
+    FEMPIC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, kThreads, ds && mixed ? sizeof(DsTile) : 0));
+    bps = nb > 0 ? nb : 1;
+  }
+  const int64_t regions = std::min<int64_t>(all_tiles, (int64_t)env->num_sms * bps);
+  A.xcap = (all_tiles + regions - 1) / regions * kTile;
+  rc = ensure_xqueue(env, regions * A.xcap, regions, st);
+  if (rc) return rc;
+  A.xrec = env->xrec;
+  A.xrec64 = env->xrec64;
+  A.xcount = env->xcount;
+  A.wait_ns = env->stall_cta >= 0 ? env->stall_ns : kWaitLimitNs;
+  A.stall_cta = env->stall_cta;
+  env->stall_cta = -1;   // one launch only
+  {
+    LaunchTimer lt(env, st, FEMPIC_K_PUSH);
+    const unsigned grid = (unsigned)regions;
+    const int cross_threads = std::min(q24 ? kCrossMax : 384, 32 * ((q24 ? 32 : 24) / std::min(bps, 8)));
+    if (mixed) {
+      if (ds) {
+        if (q24)
+          k_ds_push_mixed<true><<<grid, kThreads, sizeof(DsTile), st>>>(A, D, all_tiles);
+        else
+          k_ds_push_mixed<false><<<grid, kThreads, sizeof(DsTile), st>>>(A, D, all_tiles);
+      } else if (nfull > 0) {
+        if (q24)
+          k_push_mixed_tma<true><<<grid, kThreads, 0, st>>>(A, nfull);
+        else
+          k_push_mixed_tma<false><<<grid, kThreads, 0, st>>>(A, nfull);
+      } else {
+        if (q24)
+          k_push_mixed<true><<<grid, kThreads, 0, st>>>(A, all_tiles);
+        else
+          k_push_mixed<false><<<grid, kThreads, 0, st>>>(A, all_tiles);
+      }
+      lt.kernels = 1;
+      LaunchTimer lc(env, st, FEMPIC_K_CROSS);   // nested: also inside the push bracket
+      if (q24)
+        k_cross_q24<<<grid, cross_threads, 0, st>>>(A, D);
+      else
+        k_cross_df<<<grid, cross_threads, 0, st>>>(A, D);
+      lc.kernels = 1;
+    } else {
+      if (ds)
+        k_ds_push_fp64<<<grid, kThreads, 0, st>>>(A, D, all_tiles);
+      else
+        k_push_fp64<<<grid, kThreads, 0, st>>>(A, all_tiles);
+      lt.kernels = 1;
+      LaunchTimer lc(env, st, FEMPIC_K_CROSS);   // nested: also inside the push bracket
+      k_cross_fp64<<<grid, cross_threads, 0, st>>>(A, D);
+      lc.kernels = 1;
+    }
+  }
+  FEMPIC_CUDA(cudaGetLastError());
+  return FEMPIC_OK;
+}
+
 static int push_step_impl(fempic_env* env, const fempic_particles* p, const HostLevels& H, double omega0,
                           double t, double dt, void* stream) {
   cudaStream_t st = (cudaStream_t)stream;
@@ -3623,7 +3950,6 @@ static int push_step_impl(fempic_env* env, const fempic_particles* p, const Host
   int rc = validate_step(p, H, omega0, t, dt, &A.sp);
   if (rc) return rc;
   const bool mixed = env->opt.precision != FEMPIC_FP64;
-  const bool q24 = env->opt.precision == FEMPIC_MIXED_Q24;
   if (mixed) {
     rc = ensure_mixed_accumulators(env, p->n_species, st);
     if (rc) return rc;
@@ -3672,99 +3998,7 @@ static int push_step_impl(fempic_env* env, const fempic_particles* p, const Host
   }
   }
   FEMPIC_CUDA(cudaGetLastError());
-  env->ns_last = p->n_species;
-  for (int s = 0; s < kMaxSpecies; s++) env->qw_last[s] = A.sp.qw[s];
-  env->steps++;
-  if (p->n == 0) return FEMPIC_OK;
-  A.n = p->n;
-  A.x = p->x;
-  A.y = p->y;
-  A.z = p->z;
-  A.vx = p->vx;
-  A.vy = p->vy;
-  A.vz = p->vz;
-  A.tet = p->tet;
-  A.status = p->status;
-  A.ncross = p->n_cross;
-  A.dt = dt;
-  A.dt32 = (float)dt;
-  A.max_cross = env->opt.max_crossings;
-  A.wall_mode = env->opt.wall_mode;
-  for (int a = 0; a < 3; a++) {
-    A.lo[a] = env->h.lo[a];
-    A.hi[a] = env->h.hi[a];
-  }
-  A.nt = nt;
-  A.ne = env->h.ne;
-  A.geom64 = env->geom64;
-  A.tetrec = env->tetrec;
-  A.tn = env->tn;
-  A.nb = env->nb;
-  A.te = env->te;
-  A.field = env->field;
-  A.dGq = env->deposit_on ? env->dGq : nullptr;
-  A.mom = env->deposit_on ? env->mom : nullptr;
-  A.momlo = env->momlo;
-  A.tetdf = env->tetdf;
-  A.stats = env->stats;
-  // the common path's launch: persistent CTAs; the mixed forms' are staged
-  // when every particle array allows bulk copies (16-byte aligned sources)
-  // and there is a full tile
-  const int64_t all_tiles = (p->n + kTile - 1) / kTile;
-  const uintptr_t align = (uintptr_t)p->x | (uintptr_t)p->y | (uintptr_t)p->z | (uintptr_t)p->vx |
-                          (uintptr_t)p->vy | (uintptr_t)p->vz | (uintptr_t)p->tet;
-  const int64_t nfull = (mixed && FEMPIC_USE_TMA && !(align & 15u)) ? p->n / kTile : 0;
-  int& bps = env->push_blocks_per_sm[mixed ? (q24 ? 1 : 0) + (nfull > 0 ? 2 : 0) : 4];
-  if (bps == 0) {
-    const void* k = !mixed      ? (const void*)k_push_fp64
-                    : nfull > 0 ? (q24 ? (const void*)k_push_mixed_tma<true> : (const void*)k_push_mixed_tma<false>)
-                                : (q24 ? (const void*)k_push_mixed<true> : (const void*)k_push_mixed<false>);
-    int nb = 0;
-    FEMPIC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, kThreads, 0));
-    bps = nb > 0 ? nb : 1;
-  }
-  const int64_t regions = std::min<int64_t>(all_tiles, (int64_t)env->num_sms * bps);
-  A.xcap = (all_tiles + regions - 1) / regions * kTile;
-  rc = ensure_xqueue(env, regions * A.xcap, regions, st);
-  if (rc) return rc;
-  A.xrec = env->xrec;
-  A.xrec64 = env->xrec64;
-  A.xcount = env->xcount;
-  A.wait_ns = env->stall_cta >= 0 ? env->stall_ns : kWaitLimitNs;
-  A.stall_cta = env->stall_cta;
-  env->stall_cta = -1;   // one launch only
-  {
-    LaunchTimer lt(env, st, FEMPIC_K_PUSH);
-    const unsigned grid = (unsigned)regions;
-    if (mixed) {
-      if (nfull > 0) {
-        if (q24)
-          k_push_mixed_tma<true><<<grid, kThreads, 0, st>>>(A, nfull);
-        else
-          k_push_mixed_tma<false><<<grid, kThreads, 0, st>>>(A, nfull);
-      } else {
-        if (q24)
-          k_push_mixed<true><<<grid, kThreads, 0, st>>>(A, all_tiles);
-        else
-          k_push_mixed<false><<<grid, kThreads, 0, st>>>(A, all_tiles);
-      }
-      lt.kernels = 1;
-      LaunchTimer lc(env, st, FEMPIC_K_CROSS);   // nested: also inside the push bracket
-      if (q24)
-        k_cross_q24<<<grid, kCrossThreadsQ24, 0, st>>>(A);
-      else
-        k_cross_df<<<grid, kCrossThreadsDF, 0, st>>>(A);
-      lc.kernels = 1;
-    } else {
-      k_push_fp64<<<grid, kThreads, 0, st>>>(A, all_tiles);
-      lt.kernels = 1;
-      LaunchTimer lc(env, st, FEMPIC_K_CROSS);   // nested: also inside the push bracket
-      k_cross_fp64<<<grid, kCrossThreads64, 0, st>>>(A);
-      lc.kernels = 1;
-    }
-  }
-  FEMPIC_CUDA(cudaGetLastError());
-  return FEMPIC_OK;
+  return push_particles(env, p, A, dt, DsRule{}, st);
 }
 
 extern "C" int fempic_push_step(fempic_env* env, const fempic_particles* p, const fempic_envelope* envl,
@@ -3794,6 +4028,17 @@ extern "C" int fempic_push_step3(fempic_env* env, const fempic_particles* p, con
 }
 
 namespace fempic {
+int push_downshift(fempic_env* env, const fempic_particles* p, const DsRule& rule, double dt, cudaStream_t st) {
+  PushArgs A{};
+  int rc = fill_species(p, dt, &A.sp);
+  if (rc) return rc;
+  if (env->opt.precision != FEMPIC_FP64) {
+    rc = ensure_mixed_accumulators(env, p->n_species, st);
+    if (rc) return rc;
+  }
+  return push_particles(env, p, A, dt, rule, st);
+}
+
 int env_precision(const fempic_env* env) { return env->opt.precision; }
 
 unsigned long long* env_stats(fempic_env* env) { return env->stats; }
