@@ -246,8 +246,9 @@ int fempic_nodal_charge(fempic_env* env, const fempic_particles* p, double* rho,
 /* Host-side counters accumulated by push_step since create:
  * out4 = {face crossings, particles frozen (any non-OK status), steps,
  * staging waits that gave up}.  The last one counts CTAs of the staged push
- * kernel whose bounded wait (about 1 s) for a bulk copy expired; they stop
- * early, so any non-zero value means that step's results are incomplete.
+ * kernel whose bounded wait expired (fempic_debug_stall; its copies' own
+ * completion is a hardware wait); they stop early, so any non-zero value
+ * means that step's results are incomplete.
  * Synchronizes the stream.  Errors: EINVAL, ECUDA. */
 int fempic_stats(fempic_env* env, int64_t* out4, void* stream);
 
@@ -256,9 +257,9 @@ int fempic_stats(fempic_env* env, int64_t* out4, void* stream);
  * has no error path).  Synchronizes `stream`, then sets *n_bad to the number
  * of particles those steps froze (status CAP, ABSORBED, NONFINITE or LOST)
  * and returns FEMPIC_OK, or FEMPIC_EINCOMPLETE when, in one of those steps, a
- * CTA of the staged mixed push gave up its bounded wait (about 1 s) for a
- * bulk copy: the particles of its remaining tiles were then not advanced and
- * their deposit is missing, so the step must be redone from a saved state.
+ * CTA of the staged mixed push gave up its bounded wait: the particles of its
+ * tiles were then not advanced and their deposit is missing, so the step must
+ * be redone from a saved state.
  * In the debug build it returns FEMPIC_EBOUNDS when a mesh-table index out of
  * range was skipped (fempic_debug_set_table; the downshifted step's own
  * tables, fempic_downshift_debug_set_table, count here too).  fempic_stats keeps the
@@ -267,11 +268,10 @@ int fempic_error_count(fempic_env* env, int64_t* n_bad, void* stream);
 
 /* Test support for the bounded waits (no counterpart in the paper): in the
  * next push step only, CTA `cta` of the staged mixed push kernel (if that
- * launch has such a CTA) waits, after its first tile's copies have landed, on
- * a barrier that no copy completes, with every bounded wait of that launch
- * limited to limit_ns (1e3 .. 1e9).  The wait runs out, the CTA drains its
- * copies in flight and stops, and fempic_error_count reports
- * FEMPIC_EINCOMPLETE: the give-up path runs without any device fault.
+ * launch has such a CTA) waits, its first tile's copies in flight, on a
+ * barrier that nothing completes, limited to limit_ns (1e3 .. 1e9).  The wait
+ * runs out, the CTA waits for its copies and stops, and fempic_error_count
+ * reports FEMPIC_EINCOMPLETE: the give-up path runs without any device fault.
  * Host only.  Errors: EINVAL. */
 int fempic_debug_stall(fempic_env* env, int32_t cta, int64_t limit_ns);
 

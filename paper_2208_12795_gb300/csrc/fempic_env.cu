@@ -124,7 +124,7 @@ struct PushArgs {
   CrossRec64* xrec64;           // FP64 form: the same, FP64 records
   int32_t* xcount;              // records per region
   int64_t xcap;                 // slots of a CTA's region (its tiles times 256)
-  unsigned long long wait_ns;   // limit of each bounded wait of the staged kernel
+  unsigned long long wait_ns;   // test support: limit of the stalled CTA's wait
   int32_t stall_cta;            // test support: this CTA waits on a barrier nothing completes (-1: none)
 };
 
@@ -729,8 +729,8 @@ struct LaneOut {
 
 struct CrossList {
   int32_t total;     // records this CTA has written
-  long long sums[kThreads / 32][32 * 6];   // per warp: run sums of the deposit, by head lane
-  int32_t keys[kThreads / 32][32];         // per warp: run keys, by head lane
+  long long sums[kThreads / 32][32 * 6];   // per warp: run sums of the deposit, by run
+  int32_t keys[kThreads / 32][32];         // per warp: run keys, by run
 };
 
 __device__ __forceinline__ void lane_init(LaneOut& o, int lane) {
@@ -963,22 +963,22 @@ __device__ __forceinline__ void mixed_warp_epilogue(const PushArgs& A, int64_t p
     const int w = threadIdx.x >> 5;
     long long* row = cl.sums[w];
     const bool dep = o.key >= 0;
+    const unsigned dheads = heads & __ballot_sync(full, dep);
     if (head && dep) {
+      const int r = __popc(dheads & ((1u << lane) - 1u));   // the run's rank: rows lie densely by run
 #pragma unroll
       for (int e = 0; e < 6; e++)
-        row[6 * lane + e] = Q24 ? o.gh[e] : (long long)o.lh[e] * 33554432ll + (long long)o.ll[e];
-      cl.keys[w][lane] = o.key;
+        row[6 * r + e] = Q24 ? o.gh[e] : (long long)o.lh[e] * 33554432ll + (long long)o.ll[e];
+      cl.keys[w][r] = o.key;
     }
-    const unsigned dheads = heads & __ballot_sync(full, dep);
     __syncwarp();
     const int npairs = 6 * __popc(dheads);
 #pragma unroll 1
     for (int j = lane; j < npairs; j += 32) {
       const int r = j / 6, c = j - 6 * r;
-      const int start = (int)__fns(dheads, 0, r + 1);
-      const long long v = row[6 * start + c];
+      const long long v = row[j];
       if (v == 0) continue;
-      const int32_t key = cl.keys[w][start];
+      const int32_t key = cl.keys[w][r];
       const int64_t slot = (int64_t)(key & (kMaxSpecies - 1)) * A.nt + (key / kMaxSpecies);
       if (Q24)
         atomicAdd(A.dGq + slot * 8 + c, (unsigned long long)v);
@@ -998,38 +998,111 @@ __device__ __forceinline__ void publish_region(const PushArgs& A, const CrossLis
   if (threadIdx.x == 0) A.xcount[blockIdx.x] = cl.total;
 }
 
-// One tile's particle of this thread, state read straight from global memory.
-__device__ __forceinline__ void load_plain(const PushArgs& A, int64_t p, int32_t& T, double r[3], float v[3]) {
-  T = p < A.n ? A.tet[p] : -1;
-  if (T < 0) return;
-  r[0] = A.x[p];
-  r[1] = A.y[p];
-  r[2] = A.z[p];
-  v[0] = static_cast<const float*>(A.vx)[p];
-  v[1] = static_cast<const float*>(A.vy)[p];
-  v[2] = static_cast<const float*>(A.vz)[p];
+// ------------------------------------------------- staged common path
+// Persistent CTAs walk the 256-particle tiles.  Each thread copies its own
+// particle's state of the CTA's next tile into shared memory (cp.async of 4
+// and 8 bytes: any array alignment, a ragged last tile included) once it has
+// read the present one, so HBM latency runs under the arithmetic.  No thread
+// reads another's slots, so a thread waits for its own copies only
+// (cp.async.wait_all, no spin) and warps never wait for each other.
+// Against bulk copies by one thread into a CTA-wide ring of three stages, whose
+// refills needed a CTA barrier per tile: 0.351 -> 0.318 ms at 10M particles
+// (1.55 -> 1.41 at 48M); two stages here 0.321; completion on a per-warp
+// mbarrier instead of wait_all 0.331 (0.324 with the rest of this kernel).
+constexpr int kTile = kThreads;
+constexpr unsigned long long kWaitLimitNs = 1000000000ull;
+
+__device__ __forceinline__ uint32_t smem_addr(const void* p) {
+  return (uint32_t)__cvta_generic_to_shared(p);
 }
 
-// Common path for particle arrays that are not 16-byte aligned (bulk copies
-// cannot stage them) and for sets below one tile: CTAs walk the tiles, each
-// thread reads its particle from global memory.
-template <bool Q24>
+__device__ __forceinline__ unsigned long long global_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+
+__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count) : "memory");
+}
+
+__device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(smem_addr(bar)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+
+// Bounded wait for phase `parity` of `bar`; false after limit_ns.
+__device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity, unsigned long long limit_ns) {
+  if (mbar_test(bar, parity)) return true;
+  const unsigned long long t0 = global_ns();
+  while (!mbar_test(bar, parity)) {
+    if (global_ns() - t0 > limit_ns) return false;
+  }
+  return true;
+}
+
+__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+}
+
+struct MixedTile {
+  double r[3][kTile];
+  float v[3][kTile];
+  int32_t T[kTile];
+};
+
+__device__ __forceinline__ void fetch_state(const PushArgs& A, int64_t p, MixedTile& S) {
+  const int t = threadIdx.x;
+  cp_async8(&S.r[0][t], A.x + p);
+  cp_async8(&S.r[1][t], A.y + p);
+  cp_async8(&S.r[2][t], A.z + p);
+  cp_async4(&S.v[0][t], static_cast<const float*>(A.vx) + p);
+  cp_async4(&S.v[1][t], static_cast<const float*>(A.vy) + p);
+  cp_async4(&S.v[2][t], static_cast<const float*>(A.vz) + p);
+  cp_async4(&S.T[t], A.tet + p);
+}
+
+// STALL: test support, the launch after fempic_debug_stall (the named CTA
+// waits on a barrier nothing completes, gives up and stops).
+template <bool Q24, bool STALL>
 __global__ void __launch_bounds__(kThreads, 4) k_push_mixed(PushArgs A, int64_t ntiles) {
+  __shared__ MixedTile S;
   __shared__ CrossList cl;
-  const int lane = threadIdx.x & 31;
-  if (threadIdx.x == 0) cl.total = 0;
+  const int tid = threadIdx.x, lane = tid & 31;
+  if (tid == 0) cl.total = 0;
   __syncthreads();
-  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const int64_t p = tile * kThreads + threadIdx.x;
+  const int64_t stride = (int64_t)gridDim.x * kTile;
+  int64_t p = blockIdx.x * (int64_t)kTile + tid;
+  if (p < A.n) fetch_state(A, p, S);
+  if (STALL) {
+    __shared__ __align__(8) uint64_t stall;
+    if (tid == 0) mbar_init(&stall, 1);
+    __syncthreads();
+    if ((int)blockIdx.x == A.stall_cta && !mbar_wait_bounded(&stall, 0u, A.wait_ns)) {
+      if (tid == 0) atomicAdd(A.stats + 2, 1ull);
+      ntiles = 0;
+    }
+  }
+  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, p += stride) {
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    const int32_t T = p < A.n ? S.T[tid] : -1;
+    const double r[3] = {S.r[0][tid], S.r[1][tid], S.r[2][tid]};
+    const float v[3] = {S.v[0][tid], S.v[1][tid], S.v[2][tid]};
+    if (p + stride < A.n) fetch_state(A, p + stride, S);
     LaneOut o;
     lane_init(o, lane);
-    int32_t T;
-    double r[3] = {0.0, 0.0, 0.0};
-    float v[3] = {0.f, 0.f, 0.f};
-    load_plain(A, p, T, r, v);
     mixed_particle<Q24>(A, p, T, r[0], r[1], r[2], v[0], v[1], v[2], o);
     mixed_warp_epilogue<Q24>(A, p, lane, o, cl);
   }
+  if (STALL) asm volatile("cp.async.wait_all;" ::: "memory");   // a CTA that gave up has copies in flight
   publish_region(A, cl);
 }
 
@@ -1046,38 +1119,20 @@ __global__ void __launch_bounds__(kThreads, 4) k_push_mixed(PushArgs A, int64_t 
 // (mirror pass) in separate kernels and 791 with the history read into
 // registers; 66 % of the time its bytes take at the measured copy bandwidth.
 struct DsTile {
-  double r[3][kThreads];
-  float v[3][kThreads];
-  int32_t T[kThreads];
+  MixedTile m;
   float h[FEMPIC_DS_VN][kThreads];   // history planes 0 .. FEMPIC_DS_VN - 1
 };
-
-__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
-               : "memory");
-}
-__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
-               : "memory");
-}
 
 __device__ __forceinline__ void ds_fetch(const PushArgs& A, const DsRule& D, int64_t p, DsTile& S) {
   const int t = threadIdx.x;
   if (p < A.n) {
-    cp_async8(&S.r[0][t], A.x + p);
-    cp_async8(&S.r[1][t], A.y + p);
-    cp_async8(&S.r[2][t], A.z + p);
-    cp_async4(&S.v[0][t], static_cast<const float*>(A.vx) + p);
-    cp_async4(&S.v[1][t], static_cast<const float*>(A.vy) + p);
-    cp_async4(&S.v[2][t], static_cast<const float*>(A.vz) + p);
-    cp_async4(&S.T[t], A.tet + p);
+    fetch_state(A, p, S.m);
     if (!D.start) {
       const float* H = static_cast<const float*>(D.h) + p;
 #pragma unroll
       for (int k = 0; k < FEMPIC_DS_VN; k++) cp_async4(&S.h[k][t], H + k * D.n);
     }
   }
-  asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
 template <bool Q24>
@@ -1094,8 +1149,8 @@ __global__ void __launch_bounds__(kThreads, 3) k_ds_push_mixed(PushArgs A, DsRul
     LaneOut o;
     lane_init(o, lane);
     asm volatile("cp.async.wait_all;" ::: "memory");
-    const int32_t T = p < A.n ? S.T[tid] : -1;
-    const double r[3] = {S.r[0][tid], S.r[1][tid], S.r[2][tid]};
+    const int32_t T = p < A.n ? S.m.T[tid] : -1;
+    const double r[3] = {S.m.r[0][tid], S.m.r[1][tid], S.m.r[2][tid]};
     bool frozen = false;
     int s = 0;
     float vn[3], u[3];
@@ -1105,7 +1160,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_ds_push_mixed(PushArgs A, DsRul
       o.nfrz = 1;
     } else if (T >= 0) {
       s = species_of(A.sp, p);
-      const float v[3] = {S.v[0][tid], S.v[1][tid], S.v[2][tid]};
+      const float v[3] = {S.m.v[0][tid], S.m.v[1][tid], S.m.v[2][tid]};
       const double* x0 = reinterpret_cast<const double*>(A.tetrec + 8 * (int64_t)T);
       const float d[3] = {(float)__dsub_rn(r[0], __ldg(x0)), (float)__dsub_rn(r[1], __ldg(x0 + 1)),
                           (float)__dsub_rn(r[2], __ldg(x0 + 2))};
@@ -1135,165 +1190,6 @@ __global__ void __launch_bounds__(kThreads, 3) k_ds_push_mixed(PushArgs A, DsRul
       }
     }
     mixed_warp_epilogue<Q24>(A, p, lane, o, cl);
-  }
-  publish_region(A, cl);
-}
-
-// ------------------------------------------------- staged common path (TMA)
-// Persistent CTAs walk the 256-particle tiles (the last one, if ragged, is
-// read straight from global memory by the CTA whose turn it is: a launch of
-// its own for it cost 5 us, a 100k-particle step 73 -> 55 us).  Each full
-// tile's slices of the seven particle arrays (x, y, z f64; vx, vy, vz f32; tet i32; 10 KB) are
-// brought into shared memory by cp.async.bulk copies completing on an
-// mbarrier, in a ring of three stages filled two tiles ahead, so HBM latency
-// overlaps the arithmetic.  A stage is refilled only after the iteration
-// that read it has finished on every thread.
-// Every wait is bounded by the global timer (about 1 s by default); a CTA
-// that times out records it in stats[2], drains the copies it issued, and
-// stops.
-constexpr int kTile = kThreads;
-constexpr int kStageBytes = kTile * (3 * 8 + 3 * 4 + 4);   // 10240
-constexpr int kStages = 3;
-constexpr unsigned long long kWaitLimitNs = 1000000000ull;
-
-__device__ __forceinline__ uint32_t smem_addr(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-
-__device__ __forceinline__ unsigned long long global_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ void mbar_fence_init() {
-  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes)
-               : "memory");
-}
-
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-          smem_addr(dst)),
-      "l"(src), "r"(bytes), "r"(smem_addr(bar))
-      : "memory");
-}
-
-__device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(smem_addr(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-
-// Bounded wait for phase `parity` of `bar`; false after limit_ns.
-__device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity, unsigned long long limit_ns) {
-  if (mbar_test(bar, parity)) return true;
-  const unsigned long long t0 = global_ns();
-  while (!mbar_test(bar, parity)) {
-    if (global_ns() - t0 > limit_ns) return false;
-  }
-  return true;
-}
-
-__device__ __forceinline__ void stage_tile(const PushArgs& A, unsigned char* stage, int64_t tile, uint64_t* bar) {
-  const int64_t p0 = tile * kTile;
-  mbar_expect_tx(bar, kStageBytes);
-  bulk_g2s(stage, A.x + p0, kTile * 8, bar);
-  bulk_g2s(stage + kTile * 8, A.y + p0, kTile * 8, bar);
-  bulk_g2s(stage + kTile * 16, A.z + p0, kTile * 8, bar);
-  bulk_g2s(stage + kTile * 24, static_cast<const float*>(A.vx) + p0, kTile * 4, bar);
-  bulk_g2s(stage + kTile * 28, static_cast<const float*>(A.vy) + p0, kTile * 4, bar);
-  bulk_g2s(stage + kTile * 32, static_cast<const float*>(A.vz) + p0, kTile * 4, bar);
-  bulk_g2s(stage + kTile * 36, A.tet + p0, kTile * 4, bar);
-}
-
-#ifndef FEMPIC_USE_TMA
-#define FEMPIC_USE_TMA 1
-#endif
-#ifndef FEMPIC_TMA_MIN_BLOCKS
-#define FEMPIC_TMA_MIN_BLOCKS 4
-#endif
-template <bool Q24>
-__global__ void __launch_bounds__(kThreads, FEMPIC_TMA_MIN_BLOCKS) k_push_mixed_tma(PushArgs A, int64_t nfull) {
-  __shared__ __align__(128) unsigned char smem[kStages][kStageBytes];
-  // bar[kStages] is test support: a barrier no copy ever completes, for the
-  // CTA that fempic_debug_stall names
-  __shared__ __align__(8) uint64_t bar[kStages + 1];
-  __shared__ CrossList cl;
-  const int tid = threadIdx.x, lane = tid & 31;
-  if (tid == 0) {
-    for (int k = 0; k <= kStages; k++) mbar_init(&bar[k], 1);
-    mbar_fence_init();
-    cl.total = 0;
-  }
-  __syncthreads();
-  const int64_t stride = gridDim.x;
-  const int64_t t0 = blockIdx.x;
-  const int64_t ntiles = nfull + (A.n > nfull * kTile ? 1 : 0);
-  if (tid == 0)
-    for (int k = 0; k < kStages; k++)
-      if (t0 + k * stride < nfull) stage_tile(A, smem[k], t0 + k * stride, &bar[k]);
-  uint32_t phase = 0u;   // bit k = parity of the next wait on stage k
-  int st = 0;
-  for (int64_t it = 0, tile = t0; tile < ntiles; tile += stride, it++) {
-    // Every thread finished iteration it-1 (which used stage st-1) before
-    // this barrier; the proxy fence orders those shared-memory reads before
-    // the bulk copy that refills that stage below.
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    bool ok = tile >= nfull || mbar_wait_bounded(&bar[st], (phase >> st) & 1u, A.wait_ns);
-    if (it == 0 && (int)blockIdx.x == A.stall_cta) ok = ok && mbar_wait_bounded(&bar[kStages], 0u, A.wait_ns);
-    if (__syncthreads_or(!ok)) {
-      // give up: record it, wait (bounded) for this CTA's copies still in
-      // flight (stages of tiles it .. it+kStages-1 not yet consumed), stop
-      if (tid == 0) {
-        atomicAdd(A.stats + 2, 1ull);
-        A.xcount[blockIdx.x] = cl.total;   // the records of the tiles done so far
-        for (int k = 0; k < kStages; k++) {
-          const int sk = (st + k) % kStages;
-          if (tile + k * stride < nfull) mbar_wait_bounded(&bar[sk], (phase >> sk) & 1u, A.wait_ns);
-        }
-      }
-      return;
-    }
-    phase ^= 1u << st;
-    if (tid == 0 && it > 0) {
-      const int prev = (st + kStages - 1) % kStages;
-      const int64_t next = tile + (kStages - 1) * stride;
-      if (next < nfull) stage_tile(A, smem[prev], next, &bar[prev]);
-    }
-    const int64_t p = tile * kTile + tid;
-    int32_t T;
-    double r[3] = {0.0, 0.0, 0.0};
-    float v[3] = {0.f, 0.f, 0.f};
-    if (tile < nfull) {
-      const unsigned char* S = smem[st];
-      r[0] = reinterpret_cast<const double*>(S)[tid];
-      r[1] = reinterpret_cast<const double*>(S + kTile * 8)[tid];
-      r[2] = reinterpret_cast<const double*>(S + kTile * 16)[tid];
-      v[0] = reinterpret_cast<const float*>(S + kTile * 24)[tid];
-      v[1] = reinterpret_cast<const float*>(S + kTile * 28)[tid];
-      v[2] = reinterpret_cast<const float*>(S + kTile * 32)[tid];
-      T = reinterpret_cast<const int32_t*>(S + kTile * 36)[tid];
-    } else {
-      load_plain(A, p, T, r, v);
-    }
-    LaneOut o;
-    lane_init(o, lane);
-    mixed_particle<Q24>(A, p, T, r[0], r[1], r[2], v[0], v[1], v[2], o);
-    mixed_warp_epilogue<Q24>(A, p, lane, o, cl);
-    st = (st + 1) % kStages;
   }
   publish_region(A, cl);
 }
@@ -3410,8 +3306,7 @@ struct fempic_env {
   int32_t* xcount = nullptr;        // [xregions]
   int64_t xslots = 0, xregions = 0;
   int num_sms = 1;
-  // resident CTAs of the common path: mixed [24-bit] + 2 [staged], FP64 4; downshifted: the same + 5
-  int push_blocks_per_sm[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+  int push_blocks_per_sm[6] = {0, 0, 0, 0, 0, 0};   // resident CTAs of the common path: contract, 24-bit, FP64; downshifted + 3
   int64_t steps = 0;
   // per-kernel event timing (measurement support)
   struct Rec {
@@ -3870,21 +3765,16 @@ static int push_particles(fempic_env* env, const fempic_particles* p, PushArgs& 
   A.momlo = env->momlo;
   A.tetdf = env->tetdf;
   A.stats = env->stats;
-  // the common path's launch: persistent CTAs; the mixed forms' are staged
-  // when every particle array allows bulk copies (16-byte aligned sources)
-  // and there is a full tile
+  // the common path's launch: one resident wave of persistent CTAs
   const int64_t all_tiles = (p->n + kTile - 1) / kTile;
-  const uintptr_t align = (uintptr_t)p->x | (uintptr_t)p->y | (uintptr_t)p->z | (uintptr_t)p->vx |
-                          (uintptr_t)p->vy | (uintptr_t)p->vz | (uintptr_t)p->tet;
-  const int64_t nfull = (mixed && !ds && FEMPIC_USE_TMA && !(align & 15u)) ? p->n / kTile : 0;
-  int& bps = env->push_blocks_per_sm[(mixed ? (q24 ? 1 : 0) + (nfull > 0 ? 2 : 0) : 4) + (ds ? 5 : 0)];
+  int& bps = env->push_blocks_per_sm[(mixed ? (q24 ? 1 : 0) : 2) + (ds ? 3 : 0)];
   if (bps == 0) {
     const void* k = ds          ? (!mixed ? (const void*)k_ds_push_fp64
                                    : q24  ? (const void*)k_ds_push_mixed<true>
                                           : (const void*)k_ds_push_mixed<false>)
                     : !mixed    ? (const void*)k_push_fp64
-                    : nfull > 0 ? (q24 ? (const void*)k_push_mixed_tma<true> : (const void*)k_push_mixed_tma<false>)
-                                : (q24 ? (const void*)k_push_mixed<true> : (const void*)k_push_mixed<false>);
+                    : q24       ? (const void*)k_push_mixed<true, false>
+                                : (const void*)k_push_mixed<false, false>;
     if (ds && mixed) FEMPIC_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(DsTile)));
     int nb = 0;
     FEMPIC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, kThreads, ds && mixed ? sizeof(DsTile) : 0));
@@ -3910,16 +3800,16 @@ static int push_particles(fempic_env* env, const fempic_particles* p, PushArgs& 
           k_ds_push_mixed<true><<<grid, kThreads, sizeof(DsTile), st>>>(A, D, all_tiles);
         else
           k_ds_push_mixed<false><<<grid, kThreads, sizeof(DsTile), st>>>(A, D, all_tiles);
-      } else if (nfull > 0) {
+      } else if (A.stall_cta >= 0) {
         if (q24)
-          k_push_mixed_tma<true><<<grid, kThreads, 0, st>>>(A, nfull);
+          k_push_mixed<true, true><<<grid, kThreads, 0, st>>>(A, all_tiles);
         else
-          k_push_mixed_tma<false><<<grid, kThreads, 0, st>>>(A, nfull);
+          k_push_mixed<false, true><<<grid, kThreads, 0, st>>>(A, all_tiles);
       } else {
         if (q24)
-          k_push_mixed<true><<<grid, kThreads, 0, st>>>(A, all_tiles);
+          k_push_mixed<true, false><<<grid, kThreads, 0, st>>>(A, all_tiles);
         else
-          k_push_mixed<false><<<grid, kThreads, 0, st>>>(A, all_tiles);
+          k_push_mixed<false, false><<<grid, kThreads, 0, st>>>(A, all_tiles);
       }
       lt.kernels = 1;
       LaunchTimer lc(env, st, FEMPIC_K_CROSS);   // nested: also inside the push bracket
@@ -4239,8 +4129,8 @@ extern "C" int fempic_error_count(fempic_env* env, int64_t* n_bad, void* stream)
   env->seen_bounds = h[3];
   if (gave_up)
     return fail(FEMPIC_EINCOMPLETE, "error_count: " + std::to_string(gave_up) +
-                                        " staged push CTA(s) gave up waiting for a bulk copy; the particles of "
-                                        "their remaining tiles were not advanced and their deposit is missing");
+                                        " staged push CTA(s) gave up their wait (fempic_debug_stall); the particles of "
+                                        "their tiles were not advanced and their deposit is missing");
   if (bad_idx)
     return fail(FEMPIC_EBOUNDS, "error_count: " + std::to_string(bad_idx) +
                                     " mesh-table index(es) out of range were skipped (debug build)");
