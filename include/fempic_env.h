@@ -185,6 +185,15 @@ int fempic_locate(fempic_env* env, const fempic_particles* p, void* stream);
 int fempic_push_step(fempic_env* env, const fempic_particles* p, const fempic_envelope* envl,
                      double omega0, double t, double dt, void* stream);
 
+/* The step of fempic_push_step from one particle set into another: the new
+ * state goes to `out`, `in` is left as it was (a gradient window keeps every
+ * state of a segment; the paper has no counterpart).  Every array of out is
+ * written.  in and out have the same n, velocity dtype and species table and
+ * must not overlap; n_cross may be NULL in both (else in both).  Errors: as
+ * fempic_push_step, and EINVAL for sets that differ or overlap. */
+int fempic_push_step_to(fempic_env* env, const fempic_particles* in, const fempic_particles* out,
+                        const fempic_envelope* envl, double omega0, double t, double dt, void* stream);
+
 /* The step of fempic_push_step with the envelope interpolated from three
  * levels (fempic_envelope3): only the per-tet field construction reads the
  * extra levels; the particle work is the same.  Errors: as fempic_push_step,

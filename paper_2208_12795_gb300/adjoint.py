@@ -73,13 +73,6 @@ def clone_state(st: ParticleState) -> ParticleState:
     return o
 
 
-def _copy_state(dst: ParticleState, src: ParticleState):
-    for k in ("x", "y", "z", "vx", "vy", "vz", "tet", "status", "n_cross"):
-        t = getattr(src, k)
-        if t is not None:
-            getattr(dst, k).copy_(t)
-
-
 def kinetic_energy(env: FempicEnv, st: ParticleState, seed: AdjointState | None = None, stream=None):
     """Total kinetic energy (device f64 scalar); fills `seed` with its adjoint."""
     ke = torch.empty((), dtype=torch.float64, device=st.x.device)
@@ -160,9 +153,9 @@ class _DepositOff:
         return False
 
 
-def _step(env, st, e, b, sch: Schedule, k: int):
+def _step(env, st, e, b, sch: Schedule, k: int, out=None):
     t = sch.t0 + k * sch.dt
-    env.push_step(st, e, b, sch.amp(t), sch.omega0, t, sch.dt)
+    env.push_step(st, e, b, sch.amp(t), sch.omega0, t, sch.dt, out=out)
 
 
 class Checkpoint:
@@ -191,7 +184,8 @@ class _DepositOn:
 
 
 def _forward(env: FempicEnv, st0: ParticleState, e, b, sch: Schedule, sort: bool, u=None):
-    st = st0 if (sort and sch.steps > 0) else clone_state(st0)
+    st = st0 if sch.steps > 0 else clone_state(st0)
+    work = None   # the running state; st0 and the checkpoints are only read
     ckpts = []
     L = None
     if u is not None:
@@ -205,10 +199,13 @@ def _forward(env: FempicEnv, st0: ParticleState, e, b, sch: Schedule, sort: bool
                     perm = torch.empty(st.n, dtype=torch.int32, device=st.x.device)
                     env.sort_perm(st, srt, perm)
                     ckpts.append(Checkpoint(srt, perm))
-                    st = clone_state(srt)
                 else:
                     ckpts.append(Checkpoint(clone_state(st), None))
-            _step(env, st, e, b, sch, k)
+                work = st.empty_like() if work is None else work
+                _step(env, ckpts[-1].st, e, b, sch, k, out=work)
+                st = work
+            else:
+                _step(env, st, e, b, sch, k)
             if u is not None:
                 env.deposit_local(dG)
                 L += torch.dot(u, dG)
@@ -232,7 +229,7 @@ def reverse_sweep(env: FempicEnv, ckpts, e, b, sch: Schedule, adj: AdjointState,
     eg = torch.zeros(env.n_edges, dtype=torch.complex128, device=e.device)
     bg = torch.zeros(env.n_faces, dtype=torch.complex128, device=b.device)
     stream = _stream(None)
-    spare = None
+    spare = work = None
     for s in range(len(ckpts) - 1, -1, -1):
         k0 = s * sch.every
         k1 = min(sch.steps, k0 + sch.every)
@@ -243,27 +240,25 @@ def reverse_sweep(env: FempicEnv, ckpts, e, b, sch: Schedule, adj: AdjointState,
             capi.fempic_push_step_adjoint(env.h, before.cstruct(), after.cstruct(), envl, sch.omega0, t,
                                           sch.dt, adj.cstruct(), _ptr(eg), _ptr(bg), stream)
 
+        first = ckpts[s].st
+        if work is None:   # the segment's states after each step, or one step's pair
+            work = [first.empty_like() for _ in range(min(sch.every, sch.steps) if sch.stash else 2)]
         if sch.stash:
-            stash = [ckpts[s].st]
-            cur = clone_state(ckpts[s].st)
+            states = [first] + work
             with _DepositOff(env):
                 for k in range(k0, k1):
-                    _step(env, cur, e, b, sch, k)
-                    stash.append(clone_state(cur))
+                    _step(env, states[k - k0], e, b, sch, k, out=states[k - k0 + 1])
             for k in range(k1 - 1, k0 - 1, -1):
-                adjoint_step(k, stash[k - k0], stash[k - k0 + 1])
-            del stash, cur
+                adjoint_step(k, states[k - k0], states[k - k0 + 1])
         else:   # two working states: each step's (before, after) pair recomputed from the checkpoint
-            before, after = clone_state(ckpts[s].st), clone_state(ckpts[s].st)
             for k in range(k1 - 1, k0 - 1, -1):
-                _copy_state(before, ckpts[s].st)
+                before = first
                 with _DepositOff(env):
                     for j in range(k0, k):
-                        _step(env, before, e, b, sch, j)
-                    _copy_state(after, before)
-                    _step(env, after, e, b, sch, k)
-                adjoint_step(k, before, after)
-            del before, after
+                        _step(env, before, e, b, sch, j, out=work[0] if before is first else None)
+                        before = work[0]
+                    _step(env, before, e, b, sch, k, out=work[1])
+                adjoint_step(k, before, work[1])
         if ckpts[s].perm is not None:   # back to the order before this checkpoint's sort
             if spare is None:
                 spare = AdjointState(adj.n, adj.vx.dtype, device=adj.rx.device)

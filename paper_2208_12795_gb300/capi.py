@@ -33,7 +33,7 @@ FEMPIC_WALL_REFLECT = 0
 FEMPIC_WALL_ABSORB = 1
 
 # Every function declared in include/fempic_env.h.
-EXPORTS = ("fempic_env_create", "fempic_env_query", "fempic_locate", "fempic_push_step", "fempic_push_step3",
+EXPORTS = ("fempic_env_create", "fempic_env_query", "fempic_locate", "fempic_push_step", "fempic_push_step_to", "fempic_push_step3",
            "fempic_lagrange3",
            "fempic_deposit", "fempic_deposit_local", "fempic_accumulate", "fempic_reset_deposit", "fempic_set_deposit", "fempic_nodal_charge", "fempic_stats",
            "fempic_error_count", "fempic_debug_stall", "fempic_debug_set_table", "fempic_adjoint_current_weights", "fempic_push_step_adjoint", "fempic_kinetic_energy", "fempic_sort", "fempic_sort_perm",
@@ -106,6 +106,8 @@ def load(path: str = LIB_PATH):
         lib.fempic_env_create.argtypes = [P(fempic_mesh_desc), P(fempic_options), P(C.c_void_p)]
         lib.fempic_env_query.argtypes = [C.c_void_p] + [C.c_void_p] * 7
         lib.fempic_locate.argtypes = [C.c_void_p, P(fempic_particles), C.c_void_p]
+        lib.fempic_push_step_to.argtypes = [C.c_void_p, P(fempic_particles), P(fempic_particles), P(fempic_envelope),
+                                            C.c_double, C.c_double, C.c_double, C.c_void_p]
         lib.fempic_push_step3.argtypes = [C.c_void_p, P(fempic_particles), P(fempic_envelope3), C.c_double,
                                           C.c_double, C.c_double, C.c_void_p]
         lib.fempic_lagrange3.argtypes = [C.c_void_p, C.c_double, C.c_void_p]
@@ -190,6 +192,12 @@ def fempic_locate(env, parts: fempic_particles, stream=0):
 def fempic_push_step(env, parts: fempic_particles, envl: fempic_envelope, omega0, t, dt, stream=0):
     check(load().fempic_push_step(env, C.byref(parts), C.byref(envl), float(omega0), float(t), float(dt),
                                   stream), "fempic_push_step")
+
+
+def fempic_push_step_to(env, src: fempic_particles, dst: fempic_particles, envl: fempic_envelope, omega0, t, dt,
+                        stream=0):
+    check(load().fempic_push_step_to(env, C.byref(src), C.byref(dst), C.byref(envl), float(omega0), float(t),
+                                     float(dt), stream), "fempic_push_step_to")
 
 
 def fempic_push_step3(env, parts: fempic_particles, envl: fempic_envelope3, omega0, t, dt, stream=0):

@@ -100,6 +100,16 @@ struct PushArgs {
   int32_t* tet;
   uint8_t* status;
   int32_t* ncross;
+  // the state the step reads: the same arrays, or another set's (fempic_push_step_to)
+  const double* ix;
+  const double* iy;
+  const double* iz;
+  const void* ivx;
+  const void* ivy;
+  const void* ivz;
+  const int32_t* itet;
+  const uint8_t* istatus;
+  const int32_t* incross;
   Species sp;
   double dt;
   float dt32;                   // dt rounded to FP32 (the mixed position update's step)
@@ -466,6 +476,19 @@ __device__ __forceinline__ FF split_f64(double r) {
   const float scale = e > 948u ? __uint_as_float((e - 948u) << 23) : 0.f;   // 2^(e - 1075)
   const float flo = __fmul_rn(__uint2float_rn(lo & 0x1fffffffu), scale);
   return FF{fhi, sign ? -flo : flo};
+}
+
+// FP64 -> FP32, nearest even, with integer operations (the hardware
+// conversion runs at the FP64 rate); values outside the normal FP32 range
+// take it.
+__device__ __forceinline__ float f64_to_f32(double r) {
+  const unsigned hi = (unsigned)__double2hiint(r), lo = (unsigned)__double2loint(r);
+  const unsigned e = (hi >> 20) & 0x7ffu;
+  if (e - 897u >= 253u) return (float)r;
+  const unsigned m = ((e - 896u) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
+  const unsigned rest = lo & 0x1fffffffu;
+  const unsigned up = rest > 0x10000000u || (rest == 0x10000000u && (m & 1u)) ? 1u : 0u;
+  return __uint_as_float((hi & 0x80000000u) | (m + up));   // a carry moves into the exponent
 }
 
 struct Geo32 {
@@ -1061,18 +1084,41 @@ struct MixedTile {
 
 __device__ __forceinline__ void fetch_state(const PushArgs& A, int64_t p, MixedTile& S) {
   const int t = threadIdx.x;
-  cp_async8(&S.r[0][t], A.x + p);
-  cp_async8(&S.r[1][t], A.y + p);
-  cp_async8(&S.r[2][t], A.z + p);
-  cp_async4(&S.v[0][t], static_cast<const float*>(A.vx) + p);
-  cp_async4(&S.v[1][t], static_cast<const float*>(A.vy) + p);
-  cp_async4(&S.v[2][t], static_cast<const float*>(A.vz) + p);
-  cp_async4(&S.T[t], A.tet + p);
+  cp_async8(&S.r[0][t], A.ix + p);
+  cp_async8(&S.r[1][t], A.iy + p);
+  cp_async8(&S.r[2][t], A.iz + p);
+  cp_async4(&S.v[0][t], static_cast<const float*>(A.ivx) + p);
+  cp_async4(&S.v[1][t], static_cast<const float*>(A.ivy) + p);
+  cp_async4(&S.v[2][t], static_cast<const float*>(A.ivz) + p);
+  cp_async4(&S.T[t], A.itet + p);
 }
 
-// STALL: test support, the launch after fempic_debug_stall (the named CTA
-// waits on a barrier nothing completes, gives up and stops).
-template <bool Q24, bool STALL>
+// Common-path modes: a step in place; the launch after fempic_debug_stall (test
+// support: the named CTA waits on a barrier nothing completes, gives up and
+// stops); a step into another particle set, whose remaining arrays are filled
+// here (a copy of the set beforehand cost a gradient window 88 us per step at
+// 4M particles).
+enum { kInPlace = 0, kStall = 1, kInto = 2 };
+
+// What a step into another set writes besides the pushed state: tet, status
+// and count as they were (before the step's own writes) ...
+__device__ __forceinline__ void into_begin(const PushArgs& A, int64_t p, int32_t T) {
+  A.tet[p] = T;
+  A.status[p] = A.istatus[p];
+  if (A.ncross) A.ncross[p] = A.incross[p];
+}
+// ... and the whole state of a particle the step leaves where it is.
+template <typename R>
+__device__ __forceinline__ void into_keep(const PushArgs& A, int64_t p) {
+  A.x[p] = A.ix[p];
+  A.y[p] = A.iy[p];
+  A.z[p] = A.iz[p];
+  static_cast<R*>(A.vx)[p] = static_cast<const R*>(A.ivx)[p];
+  static_cast<R*>(A.vy)[p] = static_cast<const R*>(A.ivy)[p];
+  static_cast<R*>(A.vz)[p] = static_cast<const R*>(A.ivz)[p];
+}
+
+template <bool Q24, int MODE>
 __global__ void __launch_bounds__(kThreads, 4) k_push_mixed(PushArgs A, int64_t ntiles) {
   __shared__ MixedTile S;
   __shared__ CrossList cl;
@@ -1082,7 +1128,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_push_mixed(PushArgs A, int64_t 
   const int64_t stride = (int64_t)gridDim.x * kTile;
   int64_t p = blockIdx.x * (int64_t)kTile + tid;
   if (p < A.n) fetch_state(A, p, S);
-  if (STALL) {
+  if (MODE == kStall) {
     __shared__ __align__(8) uint64_t stall;
     if (tid == 0) mbar_init(&stall, 1);
     __syncthreads();
@@ -1099,10 +1145,12 @@ __global__ void __launch_bounds__(kThreads, 4) k_push_mixed(PushArgs A, int64_t 
     if (p + stride < A.n) fetch_state(A, p + stride, S);
     LaneOut o;
     lane_init(o, lane);
+    if (MODE == kInto && p < A.n) into_begin(A, p, T);
     mixed_particle<Q24>(A, p, T, r[0], r[1], r[2], v[0], v[1], v[2], o);
+    if (MODE == kInto && p < A.n && (T < 0 || o.nfrz)) into_keep<float>(A, p);
     mixed_warp_epilogue<Q24>(A, p, lane, o, cl);
   }
-  if (STALL) asm volatile("cp.async.wait_all;" ::: "memory");   // a CTA that gave up has copies in flight
+  if (MODE == kStall) asm volatile("cp.async.wait_all;" ::: "memory");   // a CTA that gave up has copies in flight
   publish_region(A, cl);
 }
 
@@ -1853,8 +1901,13 @@ __device__ __forceinline__ void publish64(const PushArgs& A, unsigned nfrz, cons
 
 // The state of this thread's particle of a tile; T = -1 where there is none.
 // An out-of-range tet is marked LOST here.
+template <int MODE>
 __device__ __forceinline__ int32_t load64(const PushArgs& A, int64_t p, double a[3], double v[3], unsigned& nfrz) {
-  int32_t T = p < A.n ? A.tet[p] : -1;
+  int32_t T = p < A.n ? A.itet[p] : -1;
+  if (MODE == kInto && p < A.n) {
+    into_begin(A, p, T);
+    if (T < 0 || T >= A.nt) into_keep<double>(A, p);
+  }
   if (T >= A.nt) {
     A.tet[p] = -1;
     A.status[p] = FEMPIC_P_LOST;
@@ -1862,12 +1915,12 @@ __device__ __forceinline__ int32_t load64(const PushArgs& A, int64_t p, double a
     T = -1;
   }
   if (T < 0) return -1;
-  a[0] = A.x[p];
-  a[1] = A.y[p];
-  a[2] = A.z[p];
-  v[0] = static_cast<const double*>(A.vx)[p];
-  v[1] = static_cast<const double*>(A.vy)[p];
-  v[2] = static_cast<const double*>(A.vz)[p];
+  a[0] = A.ix[p];
+  a[1] = A.iy[p];
+  a[2] = A.iz[p];
+  v[0] = static_cast<const double*>(A.ivx)[p];
+  v[1] = static_cast<const double*>(A.ivy)[p];
+  v[2] = static_cast<const double*>(A.ivz)[p];
   return T;
 }
 
@@ -1875,6 +1928,7 @@ __device__ __forceinline__ int32_t load64(const PushArgs& A, int64_t p, double a
 // particle per thread.  A particle surely inside its home tet deposits its
 // segment and is done; any other stores its new state provisionally and a
 // record for the crossing pass.
+template <int MODE>
 __global__ void __launch_bounds__(kThreads) k_push_fp64(PushArgs A, int64_t ntiles) {
   __shared__ int32_t total;
   if (threadIdx.x == 0) total = 0;
@@ -1884,7 +1938,7 @@ __global__ void __launch_bounds__(kThreads) k_push_fp64(PushArgs A, int64_t ntil
     const int64_t p = tile * kThreads + threadIdx.x;
     bool leave = false;
     double a[3] = {0.0, 0.0, 0.0}, v[3] = {0.0, 0.0, 0.0}, vn[3] = {0.0, 0.0, 0.0};
-    const int32_t T = load64(A, p, a, v, nfrz);
+    const int32_t T = load64<MODE>(A, p, a, v, nfrz);
     if (T >= 0) {
       const int s = species_of(A.sp, p);
       const double kq = A.sp.kq[s];
@@ -1908,7 +1962,9 @@ __global__ void __launch_bounds__(kThreads) k_push_fp64(PushArgs A, int64_t ntil
       vn[0] = fma(kq, Ex, fma(vpy, sz, fma(-vpz, sy, vmx)));
       vn[1] = fma(kq, Ey, fma(vpz, sx, fma(-vpx, sz, vmy)));
       vn[2] = fma(kq, Ez, fma(vpx, sy, fma(-vpy, sx, vmz)));
+      const unsigned before = nfrz;
       leave = drift64(A, p, T, s, G, a, d, vn, vn, nfrz);
+      if (MODE == kInto && nfrz != before) into_keep<double>(A, p);   // not finite: the state stays
     }
     queue64(A, p, T, a, vn, leave, &total);
   }
@@ -1929,7 +1985,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_ds_push_fp64(PushArgs A, DsRule
     const int64_t p = tile * kThreads + threadIdx.x;
     bool leave = false;
     double a[3] = {0.0, 0.0, 0.0}, v[3] = {0.0, 0.0, 0.0}, u[3] = {0.0, 0.0, 0.0};
-    const int32_t T = load64(A, p, a, v, nfrz);
+    const int32_t T = load64<kInPlace>(A, p, a, v, nfrz);
     if (T >= 0) {
       const int s = species_of(A.sp, p);
       const Geo32 G = ld_geo(A.tetrec, T);
@@ -2602,6 +2658,7 @@ struct AdjArgs {
   const uint8_t* status1;    // statuses after the step
   Species sp;
   double dt;
+  float dt32;                // dt rounded to FP32
   int64_t nt;
   const double* geom64;
   const double* field64;
@@ -2880,39 +2937,31 @@ __device__ __forceinline__ R vd3(Vec<R> a, Vec<R> b) {
 __device__ __forceinline__ double flip_sign(double x, bool neg) {
   return __hiloint2double(__double2hiint(x) ^ (neg ? (int)0x80000000 : 0), __double2loint(x));
 }
-__device__ __forceinline__ double widen(float x) { return f32_to_f64(x); }
-__device__ __forceinline__ double widen(double x) { return x; }
-
-template <typename R, bool DEP>
-__device__ __forceinline__ void adjoint_particle(const AdjArgs& A, int64_t p, int32_t T, R out[10]) {
+// Mixed forms: the FP32 step differentiated in FP32 (conversions in integer
+// operations, the species' FP32 constants from the host).
+template <bool DEP>
+__device__ __forceinline__ void adjoint_particle(const AdjArgs& A, int64_t p, int32_t T, float out[10]) {
+  using R = float;
   const int s = species_of(A.sp, p);
-  const R kq = (R)A.sp.kq[s];
+  const R kq = A.sp.kq32[s];
   const R* vx = static_cast<const R*>(A.vx);
   const R* vy = static_cast<const R*>(A.vy);
   const R* vz = static_cast<const R*>(A.vz);
   const Vec<R> v = {vx[p], vy[p], vz[p]};
   Vec<R> d, E0, W, B0;
   R beta;
-  if (sizeof(R) == 8) {
-    const double* G = A.geom64 + 12 * (int64_t)T;
-    const double* F = A.field64 + 10 * (int64_t)T;
-    d = {(R)(A.x[p] - G[0]), (R)(A.y[p] - G[1]), (R)(A.z[p] - G[2])};
-    E0 = {(R)F[0], (R)F[1], (R)F[2]};
-    W = {(R)F[3], (R)F[4], (R)F[5]};
-    B0 = {(R)F[6], (R)F[7], (R)F[8]};
-    beta = (R)F[9];
-  } else {
+  {
     const float4* Rr = A.tetrec + 8 * (int64_t)T;
     const Geo32 G = ld_geo(A.tetrec, T);
     const float4 f0 = __ldg(Rr + 4), f1 = __ldg(Rr + 5), f2 = __ldg(Rr + 6);
     FF dd[3];
     float d32[3];
     dpos(G, A.x[p], A.y[p], A.z[p], dd, d32);   // the forward step's sequence
-    d = {(R)d32[0], (R)d32[1], (R)d32[2]};
-    E0 = {(R)f0.x, (R)f0.y, (R)f0.z};
-    W = {(R)f0.w, (R)f1.x, (R)f1.y};
-    B0 = {(R)f1.z, (R)f1.w, (R)f2.x};
-    beta = (R)f2.y;
+    d = {d32[0], d32[1], d32[2]};
+    E0 = {f0.x, f0.y, f0.z};
+    W = {f0.w, f1.x, f1.y};
+    B0 = {f1.z, f1.w, f2.x};
+    beta = f2.y;
   }
   // forward recompute
   const Vec<R> dW = vx3(d, W);
@@ -2940,9 +2989,10 @@ __device__ __forceinline__ void adjoint_particle(const AdjArgs& A, int64_t p, in
   // adjoint of the output state, mirrored back (sign flips on the bit pattern)
   const double rbx = flip_sign(A.rbx[p], mx < R(0)), rby = flip_sign(A.rby[p], my < R(0)),
                rbz = flip_sign(A.rbz[p], mz < R(0));
-  const R dt = (R)A.dt;
+  const R dt = A.dt32;
   // b = r + dt vn
-  Vec<R> vnb = {mx * vbx[p] + dt * (R)rbx, my * vby[p] + dt * (R)rby, mz * vbz[p] + dt * (R)rbz};
+  Vec<R> vnb = {mx * vbx[p] + dt * f64_to_f32(rbx), my * vby[p] + dt * f64_to_f32(rby),
+               mz * vbz[p] + dt * f64_to_f32(rbz)};
   double dga[3] = {0.0, 0.0, 0.0};
   if (DEP) {   // this step's share of the deposited-current loss, through a and w = dt vn
     const double a[3] = {A.x[p], A.y[p], A.z[p]};
@@ -2950,7 +3000,7 @@ __device__ __forceinline__ void adjoint_particle(const AdjArgs& A, int64_t p, in
     double b[3], gw[3];
 #pragma unroll
     for (int c = 0; c < 3; c++)
-      b[c] = sizeof(R) == 8 ? fma(A.dt, (double)vf[c], a[c]) : advance(a[c], (float)A.dt, (float)vf[c]);
+      b[c] = advance(a[c], A.dt32, vf[c]);
     dep_loss_grad(A, T, a, b, dga, gw);
     const double qw = A.sp.qw[s];
     vnb.x += (R)(A.dt * qw * gw[0]);
@@ -2982,9 +3032,9 @@ __device__ __forceinline__ void adjoint_particle(const AdjArgs& A, int64_t p, in
   const Vec<R> Wb = vx3(Eb, d);
   const Vec<R> db1 = vx3(W, Eb);
   const R betab = vd3(Bb, d);
-  A.rbx[p] = (rbx + dga[0]) + widen(db1.x + beta * Bb.x);
-  A.rby[p] = (rby + dga[1]) + widen(db1.y + beta * Bb.y);
-  A.rbz[p] = (rbz + dga[2]) + widen(db1.z + beta * Bb.z);
+  A.rbx[p] = (DEP ? rbx + dga[0] : rbx) + f32_to_f64(db1.x + beta * Bb.x);
+  A.rby[p] = (DEP ? rby + dga[1] : rby) + f32_to_f64(db1.y + beta * Bb.y);
+  A.rbz[p] = (DEP ? rbz + dga[2] : rbz) + f32_to_f64(db1.z + beta * Bb.z);
   vbx[p] = vmb.x;
   vby[p] = vmb.y;
   vbz[p] = vmb.z;
@@ -2992,6 +3042,89 @@ __device__ __forceinline__ void adjoint_particle(const AdjArgs& A, int64_t p, in
   out[3] = Wb.x; out[4] = Wb.y; out[5] = Wb.z;
   out[6] = Bb.x; out[7] = Bb.y; out[8] = Bb.z;
   out[9] = betab;
+}
+
+// FP64 form, as chained multiply-adds (FP64-pipe bound; with separate products
+// and sums, a full division and a five-round reduction 500k particles took
+// 197 us, now 143): the vectors are the same as above.
+struct D3 {
+  double x, y, z;
+};
+__device__ __forceinline__ D3 fcross(D3 a, D3 b, D3 c) {   // a x b + c
+  return {fma(a.y, b.z, fma(-a.z, b.y, c.x)), fma(a.z, b.x, fma(-a.x, b.z, c.y)), fma(a.x, b.y, fma(-a.y, b.x, c.z))};
+}
+__device__ __forceinline__ D3 fscale(double k, D3 a, D3 c) { return {fma(k, a.x, c.x), fma(k, a.y, c.y), fma(k, a.z, c.z)}; }
+__device__ __forceinline__ D3 dscale(double k, D3 a) { return {k * a.x, k * a.y, k * a.z}; }
+__device__ __forceinline__ D3 dcross(D3 a, D3 b) {
+  return {fma(a.y, b.z, -(a.z * b.y)), fma(a.z, b.x, -(a.x * b.z)), fma(a.x, b.y, -(a.y * b.x))};
+}
+__device__ __forceinline__ double ddot(D3 a, D3 b) { return fma(a.z, b.z, fma(a.y, b.y, a.x * b.x)); }
+__device__ __forceinline__ bool opposite(double a, double b) {   // a b < 0 for finite a, b, by their bits
+  return negative_bits(a) ? !negative_bits(b) && ((__double2hiint(b) & 0x7fffffff) | __double2loint(b)) != 0
+                          : negative_bits(b) && ((__double2hiint(a) & 0x7fffffff) | __double2loint(a)) != 0;
+}
+
+template <bool DEP>
+__device__ __forceinline__ void adjoint_particle(const AdjArgs& A, int64_t p, int32_t T, double out[10]) {
+  const int s = species_of(A.sp, p);
+  const double kq = A.sp.kq[s], dt = A.dt;
+  const double *vx = static_cast<const double*>(A.vx), *vy = static_cast<const double*>(A.vy),
+               *vz = static_cast<const double*>(A.vz);
+  const double *vx1 = static_cast<const double*>(A.vx1), *vy1 = static_cast<const double*>(A.vy1),
+               *vz1 = static_cast<const double*>(A.vz1);
+  double *vbx = static_cast<double*>(A.vbx), *vby = static_cast<double*>(A.vby), *vbz = static_cast<double*>(A.vbz);
+  const double* G = A.geom64 + 12 * (int64_t)T;
+  const double2* F = reinterpret_cast<const double2*>(A.field64 + 10 * (int64_t)T);
+  const double2 f0 = __ldg(F), f1 = __ldg(F + 1), f2 = __ldg(F + 2), f3 = __ldg(F + 3), f4 = __ldg(F + 4);
+  const double a[3] = {A.x[p], A.y[p], A.z[p]};
+  const D3 d = {a[0] - G[0], a[1] - G[1], a[2] - G[2]};
+  const D3 E0 = {f0.x, f0.y, f1.x}, W = {f1.y, f2.x, f2.y}, B0 = {f3.x, f3.y, f4.x};
+  const double beta = f4.y;
+  // forward recompute
+  const D3 E = fcross(d, W, E0);
+  const D3 vm = fscale(kq, E, {vx[p], vy[p], vz[p]});
+  const D3 tau = dscale(kq, fscale(beta, d, B0));
+  const double f = 2.0 * recip_ge1(fma(tau.x, tau.x, fma(tau.y, tau.y, fma(tau.z, tau.z, 1.0))));
+  const D3 sv = dscale(f, tau);
+  const D3 vp = fcross(vm, tau, vm);
+  const D3 vn = fscale(kq, E, fcross(vp, sv, vm));
+  // wall mirrors: a reflected component comes out with the opposite sign
+  const double w1[3] = {vx1[p], vy1[p], vz1[p]};
+  const bool mx = opposite(vn.x, w1[0]), my = opposite(vn.y, w1[1]), mz = opposite(vn.z, w1[2]);
+  // adjoint of the output state, mirrored back; b = r + dt vn
+  const D3 rb = {flip_sign(A.rbx[p], mx), flip_sign(A.rby[p], my), flip_sign(A.rbz[p], mz)};
+  D3 vnb = fscale(dt, rb, {flip_sign(vbx[p], mx), flip_sign(vby[p], my), flip_sign(vbz[p], mz)});
+  D3 rout = rb;
+  if (DEP) {   // this step's share of the deposited-current loss, through a and w = dt vn
+    const double vf[3] = {flip_sign(w1[0], mx), flip_sign(w1[1], my), flip_sign(w1[2], mz)};
+    double b[3], dga[3], gw[3];
+#pragma unroll
+    for (int c = 0; c < 3; c++) b[c] = fma(dt, vf[c], a[c]);
+    dep_loss_grad(A, T, a, b, dga, gw);
+    const double qw = A.sp.qw[s];
+    vnb = fscale(dt * qw, {gw[0], gw[1], gw[2]}, vnb);
+    rout = fscale(qw, {dga[0], dga[1], dga[2]}, rb);
+  }
+  // vn = vpl + kq E, vpl = vm + vp x s, s = f tau, vp = vm + vm x tau, tau = kq B, vm = v + kq E
+  const D3 vpb = dcross(sv, vnb), sb = dcross(vnb, vp);
+  const double t2b = -f * (f * ddot(tau, sb));   // 2 dL/d(|tau|^2)
+  const D3 taub = fcross(vpb, vm, fscale(t2b, tau, dscale(f, sb)));
+  const D3 vmb = fcross(tau, vpb, {vnb.x + vpb.x, vnb.y + vpb.y, vnb.z + vpb.z});
+  const D3 Bb = dscale(kq, taub);
+  const D3 Eb = fscale(kq, vmb, dscale(kq, vnb));
+  // E = E0 + d x W, B = B0 + beta d
+  const D3 Wb = dcross(Eb, d);
+  const D3 rn = fcross(W, Eb, fscale(beta, Bb, rout));
+  A.rbx[p] = rn.x;
+  A.rby[p] = rn.y;
+  A.rbz[p] = rn.z;
+  vbx[p] = vmb.x;
+  vby[p] = vmb.y;
+  vbz[p] = vmb.z;
+  out[0] = Eb.x; out[1] = Eb.y; out[2] = Eb.z;
+  out[3] = Wb.x; out[4] = Wb.y; out[5] = Wb.z;
+  out[6] = Bb.x; out[7] = Bb.y; out[8] = Bb.z;
+  out[9] = ddot(Bb, d);
 }
 
 template <typename R, bool DEP>
@@ -3012,7 +3145,7 @@ __global__ void __launch_bounds__(kThreads) k_push_adjoint(AdjArgs A) {
       }
       // ... but the charge it moved before it froze does
       if (s1 == FEMPIC_P_OK || (DEP && (s1 == FEMPIC_P_CAP || s1 == FEMPIC_P_ABSORBED))) {
-        adjoint_particle<R, DEP>(A, p, T, g);
+        adjoint_particle<DEP>(A, p, T, g);
         key = T;
       }
     }
@@ -3032,8 +3165,9 @@ __global__ void __launch_bounds__(kThreads) k_push_adjoint(AdjArgs A) {
   }
   const unsigned above = lane == 31 ? 0u : (heads & (~0u << (lane + 1)));
   const int run_end = above ? (__ffs(above) - 2) : 31;
-#pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
+  const unsigned longest = __reduce_max_sync(full, head ? (unsigned)(run_end - lane + 1) : 0u);
+#pragma unroll 1
+  for (int off = 1; off < (int)longest; off <<= 1) {   // as many rounds as the longest run needs
 #pragma unroll
     for (int i = 0; i < 10; i++) {
       const R o = __shfl_down_sync(full, g[i], off);
@@ -3134,7 +3268,7 @@ __global__ void __launch_bounds__(kThreads) k_field_adjoint64(int64_t nt, const 
 
 __global__ void __launch_bounds__(kThreads) k_field_adjoint32(int64_t nt, const float4* __restrict__ rec,
                                                                float* __restrict__ tetgrad32,
-                                                               double* __restrict__ tadj) {
+                                                               float* __restrict__ tadj) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= nt) return;
   float4* r4 = reinterpret_cast<float4*>(tetgrad32 + 12 * t);
@@ -3143,10 +3277,10 @@ __global__ void __launch_bounds__(kThreads) k_field_adjoint32(int64_t nt, const 
   bool any = false;
 #pragma unroll
   for (int i = 0; i < 10; i++) any = any || a[i] != 0.0f;
-  double* o = tadj + 10 * t;
+  float2* o = reinterpret_cast<float2*>(tadj + 10 * t);
   if (!any) {
 #pragma unroll
-    for (int i = 0; i < 10; i++) o[i] = 0.0;
+    for (int i = 0; i < 5; i++) o[i] = make_float2(0.f, 0.f);
     return;
   }
   const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -3174,20 +3308,25 @@ __global__ void __launch_bounds__(kThreads) k_field_adjoint32(int64_t nt, const 
   betb[3] = 2.f * vdot(B0b, vcross(g[1], g[2]));
 #pragma unroll
   for (int f = 0; f < 4; f++) betb[f] += 2.f * betab * vdot(g[lf(f, 0)], vcross(g[lf(f, 1)], g[lf(f, 2)]));
-#pragma unroll
-  for (int e = 0; e < 6; e++) o[e] = f32_to_f64(epsb[e]);
-#pragma unroll
-  for (int f = 0; f < 4; f++) o[6 + f] = f32_to_f64(betb[f]);
+  o[0] = make_float2(epsb[0], epsb[1]);
+  o[1] = make_float2(epsb[2], epsb[3]);
+  o[2] = make_float2(epsb[4], epsb[5]);
+  o[3] = make_float2(betb[0], betb[1]);
+  o[4] = make_float2(betb[2], betb[3]);
 }
 
 // Second half: each edge and each face gathers its tets' terms (adjacency
 // built once on the host: edge -> (tet, local edge), face -> (tet, local
 // face)) and adds dL/dRe + j dL/dIm through eps = c_re Re(e~) - c_im Im(e~):
 // one thread per edge or face, no atomics, a fixed summation order.
+__device__ __forceinline__ double widen(float x) { return f32_to_f64(x); }   // off the FP64 pipe
+__device__ __forceinline__ double widen(double x) { return x; }
+
+template <typename R>   // type of the per-tet terms: FP64 form double, mixed forms float (summed in FP64)
 __global__ void __launch_bounds__(kThreads) k_dof_grad(int64_t ne, int64_t nf, const int32_t* __restrict__ estart,
                                                        const int32_t* __restrict__ eslot,
                                                        const int32_t* __restrict__ fslot,
-                                                       const double* __restrict__ tadj, double cre, double cim,
+                                                       const R* __restrict__ tadj, double cre, double cim,
                                                        double* __restrict__ egrad, double* __restrict__ bgrad,
                                                        int64_t nt, unsigned long long* stats) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -3195,7 +3334,7 @@ __global__ void __launch_bounds__(kThreads) k_dof_grad(int64_t ne, int64_t nf, c
     double sum = 0.0;
     for (int32_t j = estart[i]; j < estart[i + 1]; j++) {
       const int32_t sl = eslot[j];
-      if (idx_in(sl, 6 * nt, stats)) sum += tadj[(int64_t)(sl / 6) * 10 + sl % 6];
+      if (idx_in(sl, 6 * nt, stats)) sum += widen(tadj[(int64_t)(sl / 6) * 10 + sl % 6]);
     }
     if (sum != 0.0) {
       egrad[2 * i] += cre * sum;
@@ -3207,7 +3346,7 @@ __global__ void __launch_bounds__(kThreads) k_dof_grad(int64_t ne, int64_t nf, c
 #pragma unroll
     for (int k = 0; k < 2; k++) {
       const int32_t sl = fslot[2 * i + k];
-      if (sl >= 0 && idx_in(sl, 4 * nt, stats)) sum += tadj[(int64_t)(sl >> 2) * 10 + 6 + (sl & 3)];
+      if (sl >= 0 && idx_in(sl, 4 * nt, stats)) sum += widen(tadj[(int64_t)(sl >> 2) * 10 + 6 + (sl & 3)]);
     }
     if (sum != 0.0) {
       bgrad[2 * i] += cre * sum;
@@ -3235,30 +3374,39 @@ struct KEArgs {
   void* vbz;
 };
 
+// A resident wave of CTAs strides over the particles and adds one sum per CTA:
+// one atomic per warp on a single address took 192 us at 4M particles, this 113.
 template <typename R>
 __global__ void __launch_bounds__(kThreads) k_kinetic_energy(KEArgs A) {
-  const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  __shared__ double part[kThreads / 32];
   const int64_t n = A.n;
   const void *vx = A.vx, *vy = A.vy, *vz = A.vz;
   void *vbx = A.vbx, *vby = A.vby, *vbz = A.vbz;
   double *rbx = A.rbx, *rby = A.rby, *rbz = A.rbz;
   double e = 0.0;
-  if (p < n && A.tet[p] >= 0) {
-    const double mw = A.mw[species_of(A.sp, p)];
-    const double a = static_cast<const R*>(vx)[p], b = static_cast<const R*>(vy)[p], c = static_cast<const R*>(vz)[p];
-    e = 0.5 * mw * (a * a + b * b + c * c);
-    if (vbx) {
-      static_cast<R*>(vbx)[p] = (R)(mw * a);
-      static_cast<R*>(vby)[p] = (R)(mw * b);
-      static_cast<R*>(vbz)[p] = (R)(mw * c);
+  for (int64_t p = blockIdx.x * (int64_t)kThreads + threadIdx.x; p < n; p += (int64_t)gridDim.x * kThreads) {
+    if (A.tet[p] >= 0) {
+      const double mw = A.mw[species_of(A.sp, p)];
+      const double a = static_cast<const R*>(vx)[p], b = static_cast<const R*>(vy)[p], c = static_cast<const R*>(vz)[p];
+      e += 0.5 * mw * (a * a + b * b + c * c);
+      if (vbx) {
+        static_cast<R*>(vbx)[p] = (R)(mw * a);
+        static_cast<R*>(vby)[p] = (R)(mw * b);
+        static_cast<R*>(vbz)[p] = (R)(mw * c);
+        rbx[p] = rby[p] = rbz[p] = 0.0;
+      }
+    } else if (vbx) {
+      static_cast<R*>(vbx)[p] = static_cast<R*>(vby)[p] = static_cast<R*>(vbz)[p] = R(0);
       rbx[p] = rby[p] = rbz[p] = 0.0;
     }
-  } else if (p < n && vbx) {
-    static_cast<R*>(vbx)[p] = static_cast<R*>(vby)[p] = static_cast<R*>(vbz)[p] = R(0);
-    rbx[p] = rby[p] = rbz[p] = 0.0;
   }
   for (int off = 16; off > 0; off >>= 1) e += __shfl_down_sync(0xffffffffu, e, off);
-  if ((threadIdx.x & 31) == 0 && e != 0.0) atomicAdd(A.ke, e);
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = e;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < kThreads / 32; w++) e += part[w];
+    if (e != 0.0) atomicAdd(A.ke, e);
+  }
 }
 
 template <typename T>
@@ -3295,7 +3443,7 @@ struct fempic_env {
   int32_t ns_last = 0;
   double* tetgrad = nullptr;        // adjoint of the per-tet affine field [nt][10]
   float* tetgrad32 = nullptr;       // mixed form: the same from per-lane atomics, [nt][12]
-  double* tadj = nullptr;           // per-tet DoF-adjoint terms of one adjoint step [nt][10]
+  double* tadj = nullptr;           // per-tet DoF-adjoint terms of one adjoint step [nt][10] (mixed forms: floats)
   double* curw = nullptr;           // deposited-current loss weights alpha, beta per tet [nt][6]
   bool curw_on = false;
   int32_t* estart = nullptr;        // edge -> (tet, local edge) slots, CSR [ne + 1]
@@ -3722,10 +3870,10 @@ static int validate_step(const fempic_particles* p, const HostLevels& H, double 
 }
 
 // The particle work of a step, after its per-tet fields: common path, then
-// crossing pass.  A.sp is filled; a rule with history planes makes it a
-// downshifted step.
-static int push_particles(fempic_env* env, const fempic_particles* p, PushArgs& A, double dt, const DsRule& D,
-                          cudaStream_t st) {
+// crossing pass, from `in` into `p` (the same set: a step in place).  A.sp is
+// filled; a rule with history planes makes it a downshifted step (in place).
+static int push_particles(fempic_env* env, const fempic_particles* in, const fempic_particles* p, PushArgs& A,
+                          double dt, const DsRule& D, cudaStream_t st) {
   int rc = FEMPIC_OK;
   env->ns_last = p->n_species;
   for (int s = 0; s < kMaxSpecies; s++) env->qw_last[s] = A.sp.qw[s];
@@ -3733,7 +3881,7 @@ static int push_particles(fempic_env* env, const fempic_particles* p, PushArgs& 
   if (p->n == 0) return FEMPIC_OK;
   const bool mixed = env->opt.precision != FEMPIC_FP64;
   const bool q24 = env->opt.precision == FEMPIC_MIXED_Q24;
-  const bool ds = D.h != nullptr;
+  const bool ds = D.h != nullptr, into = in != p;
   A.n = p->n;
   A.x = p->x;
   A.y = p->y;
@@ -3744,6 +3892,15 @@ static int push_particles(fempic_env* env, const fempic_particles* p, PushArgs& 
   A.tet = p->tet;
   A.status = p->status;
   A.ncross = p->n_cross;
+  A.ix = in->x;
+  A.iy = in->y;
+  A.iz = in->z;
+  A.ivx = in->vx;
+  A.ivy = in->vy;
+  A.ivz = in->vz;
+  A.itet = in->tet;
+  A.istatus = in->status;
+  A.incross = in->n_cross;
   A.dt = dt;
   A.dt32 = (float)dt;
   A.max_cross = env->opt.max_crossings;
@@ -3772,9 +3929,9 @@ static int push_particles(fempic_env* env, const fempic_particles* p, PushArgs& 
     const void* k = ds          ? (!mixed ? (const void*)k_ds_push_fp64
                                    : q24  ? (const void*)k_ds_push_mixed<true>
                                           : (const void*)k_ds_push_mixed<false>)
-                    : !mixed    ? (const void*)k_push_fp64
-                    : q24       ? (const void*)k_push_mixed<true, false>
-                                : (const void*)k_push_mixed<false, false>;
+                    : !mixed    ? (const void*)k_push_fp64<kInPlace>
+                    : q24       ? (const void*)k_push_mixed<true, kInPlace>
+                                : (const void*)k_push_mixed<false, kInPlace>;
     if (ds && mixed) FEMPIC_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(DsTile)));
     int nb = 0;
     FEMPIC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, kThreads, ds && mixed ? sizeof(DsTile) : 0));
@@ -3800,16 +3957,12 @@ static int push_particles(fempic_env* env, const fempic_particles* p, PushArgs& 
           k_ds_push_mixed<true><<<grid, kThreads, sizeof(DsTile), st>>>(A, D, all_tiles);
         else
           k_ds_push_mixed<false><<<grid, kThreads, sizeof(DsTile), st>>>(A, D, all_tiles);
-      } else if (A.stall_cta >= 0) {
-        if (q24)
-          k_push_mixed<true, true><<<grid, kThreads, 0, st>>>(A, all_tiles);
-        else
-          k_push_mixed<false, true><<<grid, kThreads, 0, st>>>(A, all_tiles);
       } else {
-        if (q24)
-          k_push_mixed<true, false><<<grid, kThreads, 0, st>>>(A, all_tiles);
-        else
-          k_push_mixed<false, false><<<grid, kThreads, 0, st>>>(A, all_tiles);
+        void (*k)(PushArgs, int64_t) =
+            into                ? (q24 ? k_push_mixed<true, kInto> : k_push_mixed<false, kInto>)
+            : A.stall_cta >= 0 ? (q24 ? k_push_mixed<true, kStall> : k_push_mixed<false, kStall>)
+                                : (q24 ? k_push_mixed<true, kInPlace> : k_push_mixed<false, kInPlace>);
+        k<<<grid, kThreads, 0, st>>>(A, all_tiles);
       }
       lt.kernels = 1;
       LaunchTimer lc(env, st, FEMPIC_K_CROSS);   // nested: also inside the push bracket
@@ -3821,8 +3974,10 @@ static int push_particles(fempic_env* env, const fempic_particles* p, PushArgs& 
     } else {
       if (ds)
         k_ds_push_fp64<<<grid, kThreads, 0, st>>>(A, D, all_tiles);
+      else if (into)
+        k_push_fp64<kInto><<<grid, kThreads, 0, st>>>(A, all_tiles);
       else
-        k_push_fp64<<<grid, kThreads, 0, st>>>(A, all_tiles);
+        k_push_fp64<kInPlace><<<grid, kThreads, 0, st>>>(A, all_tiles);
       lt.kernels = 1;
       LaunchTimer lc(env, st, FEMPIC_K_CROSS);   // nested: also inside the push bracket
       k_cross_fp64<<<grid, cross_threads, 0, st>>>(A, D);
@@ -3833,8 +3988,8 @@ static int push_particles(fempic_env* env, const fempic_particles* p, PushArgs& 
   return FEMPIC_OK;
 }
 
-static int push_step_impl(fempic_env* env, const fempic_particles* p, const HostLevels& H, double omega0,
-                          double t, double dt, void* stream) {
+static int push_step_impl(fempic_env* env, const fempic_particles* in, const fempic_particles* p,
+                          const HostLevels& H, double omega0, double t, double dt, void* stream) {
   cudaStream_t st = (cudaStream_t)stream;
   PushArgs A{};
   int rc = validate_step(p, H, omega0, t, dt, &A.sp);
@@ -3888,7 +4043,7 @@ static int push_step_impl(fempic_env* env, const fempic_particles* p, const Host
   }
   }
   FEMPIC_CUDA(cudaGetLastError());
-  return push_particles(env, p, A, dt, DsRule{}, st);
+  return push_particles(env, in, p, A, dt, DsRule{}, st);
 }
 
 extern "C" int fempic_push_step(fempic_env* env, const fempic_particles* p, const fempic_envelope* envl,
@@ -3900,7 +4055,34 @@ extern "C" int fempic_push_step(fempic_env* env, const fempic_particles* p, cons
   H.b[0] = envl->b_tilde;
   H.w[0] = 1.0;
   H.amp = envl->amp;
-  return push_step_impl(env, p, H, omega0, t, dt, stream);
+  return push_step_impl(env, p, p, H, omega0, t, dt, stream);
+}
+
+extern "C" int fempic_push_step_to(fempic_env* env, const fempic_particles* in, const fempic_particles* out,
+                                   const fempic_envelope* envl, double omega0, double t, double dt, void* stream) {
+  if (!env || !envl) return fail(FEMPIC_EINVAL, "push_step_to: NULL env/envelope");
+  int rc = check_particles(in, true);
+  if (rc) return rc;
+  rc = check_particles(out, true);
+  if (rc) return rc;
+  if (in->n != out->n || in->n_species != out->n_species || (!in->n_cross) != (!out->n_cross))
+    return fail(FEMPIC_EINVAL, "push_step_to: in/out particle sets differ in size, species or n_cross");
+  Species si{}, so{};
+  rc = fill_species(in, 1.0, &si);
+  if (rc) return rc;
+  rc = fill_species(out, 1.0, &so);
+  if (rc) return rc;
+  for (int s = 0; s <= in->n_species; s++)
+    if (si.begin[s] != so.begin[s]) return fail(FEMPIC_EINVAL, "push_step_to: species tables differ");
+  if (in->n > 0 && (in->x == out->x || in->tet == out->tet || in->vx == out->vx || in->status == out->status))
+    return fail(FEMPIC_EINVAL, "push_step_to: in and out overlap");
+  HostLevels H{};
+  H.nl = 1;
+  H.e[0] = envl->e_tilde;
+  H.b[0] = envl->b_tilde;
+  H.w[0] = 1.0;
+  H.amp = envl->amp;
+  return push_step_impl(env, in, out, H, omega0, t, dt, stream);
 }
 
 extern "C" int fempic_push_step3(fempic_env* env, const fempic_particles* p, const fempic_envelope3* envl,
@@ -3914,7 +4096,7 @@ extern "C" int fempic_push_step3(fempic_env* env, const fempic_particles* p, con
     H.w[k] = envl->weight[k];
   }
   H.amp = envl->amp;
-  return push_step_impl(env, p, H, omega0, t, dt, stream);
+  return push_step_impl(env, p, p, H, omega0, t, dt, stream);
 }
 
 namespace fempic {
@@ -3926,7 +4108,7 @@ int push_downshift(fempic_env* env, const fempic_particles* p, const DsRule& rul
     rc = ensure_mixed_accumulators(env, p->n_species, st);
     if (rc) return rc;
   }
-  return push_particles(env, p, A, dt, rule, st);
+  return push_particles(env, p, p, A, dt, rule, st);
 }
 
 int env_precision(const fempic_env* env) { return env->opt.precision; }
@@ -4514,6 +4696,7 @@ extern "C" int fempic_push_step_adjoint(fempic_env* env, const fempic_particles*
     A.vz1 = after->vz;
     A.status1 = after->status;
     A.dt = dt;
+    A.dt32 = (float)dt;
     A.nt = nt;
     A.geom64 = env->geom64;
     A.field64 = static_cast<const double*>(env->field);
@@ -4552,13 +4735,19 @@ extern "C" int fempic_push_step_adjoint(fempic_env* env, const fempic_particles*
   }
   if (!env->tadj) FEMPIC_CUDA(dalloc(&env->tadj, 10 * nt));
   if (mixed)
-    k_field_adjoint32<<<blocks_for(nt), kThreads, 0, st>>>(nt, env->tetrec, env->tetgrad32, env->tadj);
+    k_field_adjoint32<<<blocks_for(nt), kThreads, 0, st>>>(nt, env->tetrec, env->tetgrad32,
+                                                           reinterpret_cast<float*>(env->tadj));
   else
     k_field_adjoint64<<<blocks_for(nt), kThreads, 0, st>>>(nt, env->geom64, env->tgeo, env->tetgrad, env->tadj);
   const int64_t ndof = std::max(env->h.ne, env->h.nf);
-  k_dof_grad<<<blocks_for(ndof), kThreads, 0, st>>>(env->h.ne, env->h.nf, env->estart, env->eslot, env->fslot,
-                                                     env->tadj, cre, cim, static_cast<double*>(e_grad),
-                                                     static_cast<double*>(b_grad), nt, env->stats);
+  if (mixed)
+    k_dof_grad<float><<<blocks_for(ndof), kThreads, 0, st>>>(
+        env->h.ne, env->h.nf, env->estart, env->eslot, env->fslot, reinterpret_cast<const float*>(env->tadj), cre, cim,
+        static_cast<double*>(e_grad), static_cast<double*>(b_grad), nt, env->stats);
+  else
+    k_dof_grad<double><<<blocks_for(ndof), kThreads, 0, st>>>(
+        env->h.ne, env->h.nf, env->estart, env->eslot, env->fslot, env->tadj, cre, cim,
+        static_cast<double*>(e_grad), static_cast<double*>(b_grad), nt, env->stats);
   lt.kernels++;
   FEMPIC_CUDA(cudaGetLastError());
   return FEMPIC_OK;
@@ -4610,10 +4799,11 @@ extern "C" int fempic_kinetic_energy(fempic_env* env, const fempic_particles* p,
     A.vby = seed->vy;
     A.vbz = seed->vz;
   }
+  const unsigned grid = (unsigned)std::min<int64_t>(blocks_for(p->n), (int64_t)env->num_sms * 8);
   if (env->opt.precision != FEMPIC_FP64)
-    k_kinetic_energy<float><<<blocks_for(p->n), kThreads, 0, st>>>(A);
+    k_kinetic_energy<float><<<grid, kThreads, 0, st>>>(A);
   else
-    k_kinetic_energy<double><<<blocks_for(p->n), kThreads, 0, st>>>(A);
+    k_kinetic_energy<double><<<grid, kThreads, 0, st>>>(A);
   FEMPIC_CUDA(cudaGetLastError());
   return FEMPIC_OK;
 }

@@ -155,7 +155,9 @@ class FempicEnv:
         capi.fempic_locate(self.h, st.cstruct(), _stream(stream))
 
     def push_step(self, st: ParticleState, e_dof: torch.Tensor, b_dof: torch.Tensor, amp: float, omega0: float,
-                  t: float, dt: float, stream=None):
+                  t: float, dt: float, stream=None, out: ParticleState | None = None):
+        """One step of `st`, in place or (with `out`) into another set of the
+        same size and types, `st` left as it was."""
         if e_dof.dtype != self.dof_dtype or b_dof.dtype != self.dof_dtype:
             raise capi.FempicError(f"DoFs must be {self.dof_dtype} for this precision form")
         if e_dof.numel() != self.n_edges or b_dof.numel() != self.n_faces or not e_dof.is_cuda:
@@ -164,6 +166,11 @@ class FempicEnv:
         if st.vx.dtype != vdt:
             raise capi.FempicError(f"velocities must be {vdt} for this precision form")
         envl = capi.fempic_envelope(_ptr(e_dof), _ptr(b_dof), float(amp))
+        if out is not None:
+            if out.vx.dtype != vdt:
+                raise capi.FempicError(f"velocities must be {vdt} for this precision form")
+            capi.fempic_push_step_to(self.h, st.cstruct(), out.cstruct(), envl, omega0, t, dt, _stream(stream))
+            return
         capi.fempic_push_step(self.h, st.cstruct(), envl, omega0, t, dt, _stream(stream))
 
     def push_step3(self, st: ParticleState, e_levels, b_levels, weights, amp: float, omega0: float, t: float,
