@@ -1831,6 +1831,25 @@ __device__ __forceinline__ void deposit64(const PushArgs& A, int32_t T, const do
 
 __device__ __forceinline__ CrossRec64* xregion64(const PushArgs& A) { return A.xrec64 + blockIdx.x * A.xcap; }
 
+// Inside when all four FP32 barycentrics of the end d + D (both from x0)
+// reach kappa, the bound on their error for a start in the tet (|lambda| of
+// the start is checked too: a start far outside would void the bound).
+__device__ __forceinline__ bool surely_inside(const Geo32& G, const double d[3], const double D[3]) {
+  float lo = INFINITY, la = INFINITY, sb = 1.0f, sa = 1.0f;
+  const float d32[3] = {trunc32(d[0]), trunc32(d[1]), trunc32(d[2])};
+  const float e32[3] = {d32[0] + trunc32(D[0]), d32[1] + trunc32(D[1]), d32[2] + trunc32(D[2])};
+#pragma unroll
+  for (int k = 0; k < 3; k++) {
+    const float lb = G.g[3 * k] * e32[0] + G.g[3 * k + 1] * e32[1] + G.g[3 * k + 2] * e32[2];
+    const float l0 = G.g[3 * k] * d32[0] + G.g[3 * k + 1] * d32[1] + G.g[3 * k + 2] * d32[2];
+    sb -= lb;
+    sa -= l0;
+    lo = fminf(lo, lb);
+    la = fminf(la, l0);
+  }
+  return fminf(lo, sb) >= G.kappa && fminf(la, sa) >= -1.0f;
+}
+
 // One segment a -> b = a + dt w of a particle in tet T (G its record, d = a -
 // x0): position and stored velocity vs written, the deposit of a particle
 // surely inside.  Returns whether the crossing pass has to decide; counts a
@@ -1853,22 +1872,7 @@ __device__ __forceinline__ bool drift64(const PushArgs& A, int64_t p, int32_t T,
   static_cast<double*>(A.vy)[p] = vs[1];
   static_cast<double*>(A.vz)[p] = vs[2];
   const double D[3] = {b[0] - a[0], b[1] - a[1], b[2] - a[2]};
-  // inside when all four FP32 barycentrics of b reach kappa, the bound on
-  // their error for a start in the tet (|lambda(a)| is checked too: a start
-  // far outside would void the bound)
-  float lo = INFINITY, la = INFINITY, sb = 1.0f, sa = 1.0f;
-  const float d32[3] = {trunc32(d[0]), trunc32(d[1]), trunc32(d[2])};
-  const float e32[3] = {d32[0] + trunc32(D[0]), d32[1] + trunc32(D[1]), d32[2] + trunc32(D[2])};
-#pragma unroll
-  for (int k = 0; k < 3; k++) {
-    const float lb = G.g[3 * k] * e32[0] + G.g[3 * k + 1] * e32[1] + G.g[3 * k + 2] * e32[2];
-    const float l0 = G.g[3 * k] * d32[0] + G.g[3 * k + 1] * d32[1] + G.g[3 * k + 2] * d32[2];
-    sb -= lb;
-    sa -= l0;
-    lo = fminf(lo, lb);
-    la = fminf(la, l0);
-  }
-  if (!(fminf(lo, sb) >= G.kappa && fminf(la, sa) >= -1.0f)) return true;
+  if (!surely_inside(G, d, D)) return true;
   deposit64(A, T, d, D, A.sp.qw[s]);   // (f) the whole segment is in the home tet
   return false;
 }
@@ -2739,18 +2743,8 @@ __device__ __noinline__ void dep_loss_grad(const AdjArgs& A, int32_t T0, const d
   bary64(A.geom64 + 12 * (int64_t)T, pnt, la);
   for (;;) {
     bary64(A.geom64 + 12 * (int64_t)T, b, lb);
-    int kx = -1;
-    double smin = INFINITY;
-#pragma unroll
-    for (int k = 0; k < 4; k++) {
-      if (k == entry || !negative_bits(lb[k])) continue;
-      double sk = la[k] / (la[k] - lb[k]);
-      if (sk < 0.0) sk = 0.0;
-      if (sk < smin) {
-        smin = sk;
-        kx = k;
-      }
-    }
+    double smin;
+    const int kx = exit_face64(la, lb, entry, smin);
     double G[4][3];
     grads64(A.geom64, T, G);
     const double* cw = A.curw + 6 * (int64_t)T;
@@ -2921,6 +2915,67 @@ __device__ __noinline__ void dep_loss_grad(const AdjArgs& A, int32_t T0, const d
   }
 }
 
+// The gradients of a CTA's particles (all threads; `want`: this thread has
+// one).  A segment surely inside its home tet (the FP32 test of the FP64
+// common path) has them in closed form, d/da = w x beta and d/dw = alpha +
+// beta x (a - x0).  The others, about one in seven on the cavity, are walked
+// from a list in shared memory by the CTA's first threads, so that the FP64
+// walk runs with full warps: with every warp walking its own few, 300k
+// particles took 225 us, now DEPNOW.
+struct DepQueue {
+  int32_t n;
+  int32_t T[kThreads];
+  double a[3][kThreads], b[3][kThreads];   // start and end; after the walk d/da and d/dw
+};
+
+__device__ __forceinline__ void dep_block(const AdjArgs& A, DepQueue& Q, bool want, int32_t T, const double a[3],
+                                          const double b[3], double ga[3], double gw[3]) {
+  int at = -1;
+  if (want) {
+    const Geo32 G = ld_geo(A.tetrec, T);
+    const double u[3] = {a[0] - G.x0[0], a[1] - G.x0[1], a[2] - G.x0[2]};
+    const double w[3] = {b[0] - a[0], b[1] - a[1], b[2] - a[2]};
+    if (surely_inside(G, u, w)) {
+      const double* cw = A.curw + 6 * (int64_t)T;
+      const double al[3] = {cw[0], cw[1], cw[2]}, be[3] = {cw[3], cw[4], cw[5]};
+#pragma unroll
+      for (int k = 0; k < 3; k++) {
+        const int i = (k + 1) % 3, j = (k + 2) % 3;
+        ga[k] = fma(w[i], be[j], -(w[j] * be[i]));
+        gw[k] = fma(be[i], u[j], fma(-be[j], u[i], al[k]));
+      }
+    } else {
+      at = atomicAdd(&Q.n, 1);
+      Q.T[at] = T;
+#pragma unroll
+      for (int k = 0; k < 3; k++) {
+        Q.a[k][at] = a[k];
+        Q.b[k][at] = b[k];
+      }
+    }
+  }
+  __syncthreads();
+  const int m = Q.n;
+  for (int i = threadIdx.x; i < m; i += kThreads) {
+    const double sa[3] = {Q.a[0][i], Q.a[1][i], Q.a[2][i]}, sb[3] = {Q.b[0][i], Q.b[1][i], Q.b[2][i]};
+    double da[3], dw[3];
+    dep_loss_grad(A, Q.T[i], sa, sb, da, dw);
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+      Q.a[k][i] = da[k];
+      Q.b[k][i] = dw[k];
+    }
+  }
+  __syncthreads();
+  if (at >= 0) {
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+      ga[k] = Q.a[k][at];
+      gw[k] = Q.b[k][at];
+    }
+  }
+}
+
 template <typename R>
 struct Vec {
   R x, y, z;
@@ -2937,17 +2992,41 @@ __device__ __forceinline__ R vd3(Vec<R> a, Vec<R> b) {
 __device__ __forceinline__ double flip_sign(double x, bool neg) {
   return __hiloint2double(__double2hiint(x) ^ (neg ? (int)0x80000000 : 0), __double2loint(x));
 }
+// A particle's arrays of one adjoint step, loaded before its tet is looked at,
+// so that one HBM latency covers them all (4M particles mixed: 151 -> 142 us).
+template <typename R>
+struct AdjLoad {
+  double r[3], rb[3];
+  R v[3], v1[3], vb[3];
+};
+template <typename R>
+__device__ __forceinline__ void adj_load(const AdjArgs& A, int64_t p, AdjLoad<R>& L) {
+  L.r[0] = A.x[p];
+  L.r[1] = A.y[p];
+  L.r[2] = A.z[p];
+  L.v[0] = static_cast<const R*>(A.vx)[p];
+  L.v[1] = static_cast<const R*>(A.vy)[p];
+  L.v[2] = static_cast<const R*>(A.vz)[p];
+  L.v1[0] = static_cast<const R*>(A.vx1)[p];
+  L.v1[1] = static_cast<const R*>(A.vy1)[p];
+  L.v1[2] = static_cast<const R*>(A.vz1)[p];
+  L.rb[0] = A.rbx[p];
+  L.rb[1] = A.rby[p];
+  L.rb[2] = A.rbz[p];
+  L.vb[0] = static_cast<const R*>(A.vbx)[p];
+  L.vb[1] = static_cast<const R*>(A.vby)[p];
+  L.vb[2] = static_cast<const R*>(A.vbz)[p];
+}
+
 // Mixed forms: the FP32 step differentiated in FP32 (conversions in integer
 // operations, the species' FP32 constants from the host).
 template <bool DEP>
-__device__ __forceinline__ void adjoint_particle(const AdjArgs& A, int64_t p, int32_t T, float out[10]) {
+__device__ __forceinline__ void adjoint_particle(const AdjArgs& A, int64_t p, int32_t T, const AdjLoad<float>& L,
+                                                 float out[10], bool act, DepQueue* Q) {
   using R = float;
   const int s = species_of(A.sp, p);
   const R kq = A.sp.kq32[s];
-  const R* vx = static_cast<const R*>(A.vx);
-  const R* vy = static_cast<const R*>(A.vy);
-  const R* vz = static_cast<const R*>(A.vz);
-  const Vec<R> v = {vx[p], vy[p], vz[p]};
+  const Vec<R> v = {L.v[0], L.v[1], L.v[2]};
   Vec<R> d, E0, W, B0;
   R beta;
   {
@@ -2956,7 +3035,7 @@ __device__ __forceinline__ void adjoint_particle(const AdjArgs& A, int64_t p, in
     const float4 f0 = __ldg(Rr + 4), f1 = __ldg(Rr + 5), f2 = __ldg(Rr + 6);
     FF dd[3];
     float d32[3];
-    dpos(G, A.x[p], A.y[p], A.z[p], dd, d32);   // the forward step's sequence
+    dpos(G, L.r[0], L.r[1], L.r[2], dd, d32);   // the forward step's sequence
     d = {d32[0], d32[1], d32[2]};
     E0 = {f0.x, f0.y, f0.z};
     W = {f0.w, f1.x, f1.y};
@@ -2977,31 +3056,29 @@ __device__ __forceinline__ void adjoint_particle(const AdjArgs& A, int64_t p, in
   const Vec<R> c2 = vx3(vp, sv);
   const Vec<R> vn = {vm.x + c2.x + kq * E.x, vm.y + c2.y + kq * E.y, vm.z + c2.z + kq * E.z};
   // wall mirrors: a reflected component comes out with the opposite sign
-  const R* vx1 = static_cast<const R*>(A.vx1);
-  const R* vy1 = static_cast<const R*>(A.vy1);
-  const R* vz1 = static_cast<const R*>(A.vz1);
-  const R mx = vn.x * vx1[p] < R(0) ? R(-1) : R(1);
-  const R my = vn.y * vy1[p] < R(0) ? R(-1) : R(1);
-  const R mz = vn.z * vz1[p] < R(0) ? R(-1) : R(1);
+  const R mx = vn.x * L.v1[0] < R(0) ? R(-1) : R(1);
+  const R my = vn.y * L.v1[1] < R(0) ? R(-1) : R(1);
+  const R mz = vn.z * L.v1[2] < R(0) ? R(-1) : R(1);
   R* vbx = static_cast<R*>(A.vbx);
   R* vby = static_cast<R*>(A.vby);
   R* vbz = static_cast<R*>(A.vbz);
   // adjoint of the output state, mirrored back (sign flips on the bit pattern)
-  const double rbx = flip_sign(A.rbx[p], mx < R(0)), rby = flip_sign(A.rby[p], my < R(0)),
-               rbz = flip_sign(A.rbz[p], mz < R(0));
+  const double rbx = flip_sign(L.rb[0], mx < R(0)), rby = flip_sign(L.rb[1], my < R(0)),
+               rbz = flip_sign(L.rb[2], mz < R(0));
   const R dt = A.dt32;
   // b = r + dt vn
-  Vec<R> vnb = {mx * vbx[p] + dt * f64_to_f32(rbx), my * vby[p] + dt * f64_to_f32(rby),
-               mz * vbz[p] + dt * f64_to_f32(rbz)};
+  Vec<R> vnb = {mx * L.vb[0] + dt * f64_to_f32(rbx), my * L.vb[1] + dt * f64_to_f32(rby),
+               mz * L.vb[2] + dt * f64_to_f32(rbz)};
   double dga[3] = {0.0, 0.0, 0.0};
   if (DEP) {   // this step's share of the deposited-current loss, through a and w = dt vn
-    const double a[3] = {A.x[p], A.y[p], A.z[p]};
-    const R vf[3] = {mx * vx1[p], my * vy1[p], mz * vz1[p]};   // the forward's vn, exactly
+    const double* a = L.r;
+    const R vf[3] = {mx * L.v1[0], my * L.v1[1], mz * L.v1[2]};   // the forward's vn, exactly
     double b[3], gw[3];
 #pragma unroll
     for (int c = 0; c < 3; c++)
       b[c] = advance(a[c], A.dt32, vf[c]);
-    dep_loss_grad(A, T, a, b, dga, gw);
+    dep_block(A, *Q, act, T, a, b, dga, gw);
+    if (!act) return;
     const double qw = A.sp.qw[s];
     vnb.x += (R)(A.dt * qw * gw[0]);
     vnb.y += (R)(A.dt * qw * gw[1]);
@@ -3065,42 +3142,40 @@ __device__ __forceinline__ bool opposite(double a, double b) {   // a b < 0 for 
 }
 
 template <bool DEP>
-__device__ __forceinline__ void adjoint_particle(const AdjArgs& A, int64_t p, int32_t T, double out[10]) {
+__device__ __forceinline__ void adjoint_particle(const AdjArgs& A, int64_t p, int32_t T, const AdjLoad<double>& L,
+                                                 double out[10], bool act, DepQueue* Q) {
   const int s = species_of(A.sp, p);
   const double kq = A.sp.kq[s], dt = A.dt;
-  const double *vx = static_cast<const double*>(A.vx), *vy = static_cast<const double*>(A.vy),
-               *vz = static_cast<const double*>(A.vz);
-  const double *vx1 = static_cast<const double*>(A.vx1), *vy1 = static_cast<const double*>(A.vy1),
-               *vz1 = static_cast<const double*>(A.vz1);
   double *vbx = static_cast<double*>(A.vbx), *vby = static_cast<double*>(A.vby), *vbz = static_cast<double*>(A.vbz);
   const double* G = A.geom64 + 12 * (int64_t)T;
   const double2* F = reinterpret_cast<const double2*>(A.field64 + 10 * (int64_t)T);
   const double2 f0 = __ldg(F), f1 = __ldg(F + 1), f2 = __ldg(F + 2), f3 = __ldg(F + 3), f4 = __ldg(F + 4);
-  const double a[3] = {A.x[p], A.y[p], A.z[p]};
+  const double* a = L.r;
   const D3 d = {a[0] - G[0], a[1] - G[1], a[2] - G[2]};
   const D3 E0 = {f0.x, f0.y, f1.x}, W = {f1.y, f2.x, f2.y}, B0 = {f3.x, f3.y, f4.x};
   const double beta = f4.y;
   // forward recompute
   const D3 E = fcross(d, W, E0);
-  const D3 vm = fscale(kq, E, {vx[p], vy[p], vz[p]});
+  const D3 vm = fscale(kq, E, {L.v[0], L.v[1], L.v[2]});
   const D3 tau = dscale(kq, fscale(beta, d, B0));
   const double f = 2.0 * recip_ge1(fma(tau.x, tau.x, fma(tau.y, tau.y, fma(tau.z, tau.z, 1.0))));
   const D3 sv = dscale(f, tau);
   const D3 vp = fcross(vm, tau, vm);
   const D3 vn = fscale(kq, E, fcross(vp, sv, vm));
   // wall mirrors: a reflected component comes out with the opposite sign
-  const double w1[3] = {vx1[p], vy1[p], vz1[p]};
+  const double* w1 = L.v1;
   const bool mx = opposite(vn.x, w1[0]), my = opposite(vn.y, w1[1]), mz = opposite(vn.z, w1[2]);
   // adjoint of the output state, mirrored back; b = r + dt vn
-  const D3 rb = {flip_sign(A.rbx[p], mx), flip_sign(A.rby[p], my), flip_sign(A.rbz[p], mz)};
-  D3 vnb = fscale(dt, rb, {flip_sign(vbx[p], mx), flip_sign(vby[p], my), flip_sign(vbz[p], mz)});
+  const D3 rb = {flip_sign(L.rb[0], mx), flip_sign(L.rb[1], my), flip_sign(L.rb[2], mz)};
+  D3 vnb = fscale(dt, rb, {flip_sign(L.vb[0], mx), flip_sign(L.vb[1], my), flip_sign(L.vb[2], mz)});
   D3 rout = rb;
   if (DEP) {   // this step's share of the deposited-current loss, through a and w = dt vn
     const double vf[3] = {flip_sign(w1[0], mx), flip_sign(w1[1], my), flip_sign(w1[2], mz)};
     double b[3], dga[3], gw[3];
 #pragma unroll
     for (int c = 0; c < 3; c++) b[c] = fma(dt, vf[c], a[c]);
-    dep_loss_grad(A, T, a, b, dga, gw);
+    dep_block(A, *Q, act, T, a, b, dga, gw);
+    if (!act) return;
     const double qw = A.sp.qw[s];
     vnb = fscale(dt * qw, {gw[0], gw[1], gw[2]}, vnb);
     rout = fscale(qw, {dga[0], dga[1], dga[2]}, rb);
@@ -3135,20 +3210,36 @@ __global__ void __launch_bounds__(kThreads) k_push_adjoint(AdjArgs A) {
 #pragma unroll
   for (int i = 0; i < 10; i++) g[i] = R(0);
   int32_t key = -1 - lane;
+  extern __shared__ __align__(8) unsigned char dep_smem[];   // DEP: the CTA's DepQueue
+  DepQueue* Q = reinterpret_cast<DepQueue*>(dep_smem);
+  bool act = false;
+  int32_t T = 0;
+  AdjLoad<R> L{};
   if (p < A.n) {
-    const int32_t T = A.tet[p];
+    T = A.tet[p];
+    const uint8_t s1 = A.status1[p];
+    adj_load(A, p, L);
     if (T >= 0 && T < A.nt) {
-      const uint8_t s1 = A.status1[p];
       if (s1 != FEMPIC_P_OK) {   // frozen during the step: its later state does not enter the loss
         A.rbx[p] = A.rby[p] = A.rbz[p] = 0.0;
         static_cast<R*>(A.vbx)[p] = static_cast<R*>(A.vby)[p] = static_cast<R*>(A.vbz)[p] = R(0);
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+          L.rb[k] = 0.0;
+          L.vb[k] = R(0);
+        }
       }
       // ... but the charge it moved before it froze does
-      if (s1 == FEMPIC_P_OK || (DEP && (s1 == FEMPIC_P_CAP || s1 == FEMPIC_P_ABSORBED))) {
-        adjoint_particle<DEP>(A, p, T, g);
-        key = T;
-      }
+      act = s1 == FEMPIC_P_OK || (DEP && (s1 == FEMPIC_P_CAP || s1 == FEMPIC_P_ABSORBED));
+      if (act) key = T;
     }
+  }
+  if (DEP) {   // every thread goes through the CTA's list of walks
+    if (threadIdx.x == 0) Q->n = 0;
+    __syncthreads();
+    adjoint_particle<DEP>(A, p, act ? T : 0, L, g, act, Q);
+  } else if (act) {
+    adjoint_particle<DEP>(A, p, T, L, g, true, nullptr);
   }
   const unsigned full = 0xffffffffu;
   const int32_t prev = __shfl_up_sync(full, key, 1);
@@ -4721,12 +4812,12 @@ extern "C" int fempic_push_step_adjoint(fempic_env* env, const fempic_particles*
     }
     if (mixed) {
       if (A.curw)
-        k_push_adjoint<float, true><<<blocks_for(A.n), kThreads, 0, st>>>(A);
+        k_push_adjoint<float, true><<<blocks_for(A.n), kThreads, sizeof(DepQueue), st>>>(A);
       else
         k_push_adjoint<float, false><<<blocks_for(A.n), kThreads, 0, st>>>(A);
     } else {
       if (A.curw)
-        k_push_adjoint<double, true><<<blocks_for(A.n), kThreads, 0, st>>>(A);
+        k_push_adjoint<double, true><<<blocks_for(A.n), kThreads, sizeof(DepQueue), st>>>(A);
       else
         k_push_adjoint<double, false><<<blocks_for(A.n), kThreads, 0, st>>>(A);
     }

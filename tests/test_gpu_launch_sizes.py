@@ -78,3 +78,35 @@ def test_counts_and_alignment(oracle_run, prec, offset, n):
         assert np.array_equal(g[k].astype(np.float64), getattr(ost, k)), k
     assert np.abs(G.cpu().numpy() - oG).max() <= 1e-12 * np.abs(oG).max()
     assert env.error_count()[0]
+
+
+@pytest.mark.parametrize("n", [1, 257, 5000])
+@pytest.mark.parametrize("prec", [FP64, MIXED, 2])
+def test_step_into_another_set_equals_the_step_in_place(prec, n):
+    """Walls that absorb, a crossing cap, a NaN velocity, an out-of-range and a
+    missing tet: every array of the other set comes out as the step in place
+    leaves it, and the set stepped from is unchanged."""
+    from paper_2208_12795_gb300 import capi
+    from paper_2208_12795_gb300.env import FempicEnv, ParticleState
+    wl = I.workload_hot_small(n_particles=5000, wall_mode=1)
+    env = FempicEnv.from_mesh(wl.mesh, precision=prec, wall_mode=1, max_crossings=2)
+    st = ParticleState.from_host(wl.particles.subset(n), prec)
+    env.locate(st)
+    if n > 100:
+        st.vy[7] = float("nan")
+        st.tet[11] = env.n_tets + 3
+        st.tet[12] = -1
+    e = torch.from_numpy(wl.e_tilde).to(env.dof_dtype).cuda()
+    b = torch.from_numpy(wl.b_tilde).to(env.dof_dtype).cuda()
+    env.push_step(st, e, b, 1.0, wl.omega0, 0.0, wl.dt)   # some particles are frozen already
+    src, dst = st.to_numpy(), st.empty_like()
+    env.push_step(st, e, b, 1.0, wl.omega0, wl.dt, wl.dt, out=dst)
+    for k, v in st.to_numpy().items():
+        assert np.array_equal(v, src[k], equal_nan=True), k
+    env.push_step(st, e, b, 1.0, wl.omega0, wl.dt, wl.dt)
+    got = dst.to_numpy()
+    assert n < 100 or (got["status"] != 0).sum() > 100
+    for k, v in st.to_numpy().items():
+        assert np.array_equal(v, got[k], equal_nan=True), k
+    with pytest.raises(capi.FempicError, match="overlap"):
+        env.push_step(st, e, b, 1.0, wl.omega0, 0.0, wl.dt, out=st)
