@@ -14,12 +14,15 @@
 #include "fempic_downshift.h"
 #include "fempic_ds_rule.cuh"
 #include "fempic_internal.h"
+#include "fempic_launch.cuh"
 #include "fempic_tetgeo.cuh"
 
 namespace {
 
 using fempic::HostMesh;
 using fempic::kMaxSpecies;
+using fempic::grid_wait;
+using fempic::launch;
 
 thread_local std::string g_ds_error;
 
@@ -95,6 +98,7 @@ __global__ void __launch_bounds__(kThreads) k_ds_field64(int64_t nt, const doubl
                                                          const double2* __restrict__ b, int64_t ne, int64_t nf,
                                                          unsigned long long* stats, double amp,
                                                          double* __restrict__ coef) {
+  grid_wait();
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= nt) return;
   double2 ev[6], bv[4];
@@ -200,6 +204,7 @@ __global__ void __launch_bounds__(kThreads) k_ds_field32(int64_t nt, const doubl
                                                          const float2* __restrict__ e, const float2* __restrict__ b,
                                                          int64_t ne, int64_t nf, unsigned long long* stats,
                                                          double amp, float* __restrict__ coef32) {
+  grid_wait();
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= nt) return;
   const double2* D = reinterpret_cast<const double2*>(dgeo + kDsGeo * t);
@@ -517,11 +522,11 @@ extern "C" int fempic_push_step_downshift(fempic_env* env, fempic_downshift* ds,
   A.coef32 = ds->coef32;
   cudaStream_t st = (cudaStream_t)stream;
   if (mixed) {   // complex64 DoFs; FP32 velocities, samples and history
-    k_ds_field32<<<blocks_for(ds->nt), kThreads, 0, st>>>(
+    launch(k_ds_field32, blocks_for(ds->nt), kThreads, 0, st, 
         ds->nt, ds->geom, ds->dgeo, ds->te, ds->tf, static_cast<const float2*>(envl->e_tilde),
         static_cast<const float2*>(envl->b_tilde), ds->ne, ds->nf, fempic::env_stats(env), envl->amp, ds->coef32);
   } else {
-    k_ds_field64<<<blocks_for(ds->nt), kThreads, 0, st>>>(
+    launch(k_ds_field64, blocks_for(ds->nt), kThreads, 0, st, 
         ds->nt, ds->geom, ds->tgeo, ds->te, ds->tf, static_cast<const double2*>(envl->e_tilde),
         static_cast<const double2*>(envl->b_tilde), ds->ne, ds->nf, fempic::env_stats(env), envl->amp, ds->coef);
   }

@@ -31,6 +31,7 @@
 
 #include "fempic_ds_rule.cuh"
 #include "fempic_internal.h"
+#include "fempic_launch.cuh"
 #include "fempic_tetgeo.cuh"
 
 using namespace fempic;
@@ -332,6 +333,7 @@ __global__ void __launch_bounds__(kThreads) k_field_fp64(int64_t nt, const doubl
                                                           const double* __restrict__ tgeo,
                                                           const int4* __restrict__ te, const int4* __restrict__ tf,
                                                           Levels<double2, double> L, double* __restrict__ field) {
+  grid_wait();
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= nt) return;
   const int4 e0 = te[2 * t], e1 = te[2 * t + 1], f = tf[t];
@@ -373,6 +375,7 @@ template <int NL>
 __global__ void __launch_bounds__(kThreads) k_field_f32(int64_t nt, float4* __restrict__ rec,
                                                          const int4* __restrict__ te, const int4* __restrict__ tf,
                                                          Levels<float2, float> L) {
+  grid_wait();
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= nt) return;
   const float4 a = rec[8 * t + 1], b = rec[8 * t + 2], c = rec[8 * t + 3];
@@ -1120,13 +1123,14 @@ __device__ __forceinline__ void into_keep(const PushArgs& A, int64_t p) {
 
 template <bool Q24, int MODE>
 __global__ void __launch_bounds__(kThreads, 4) k_push_mixed(PushArgs A, int64_t ntiles) {
+  grid_wait();
   __shared__ MixedTile S;
   __shared__ CrossList cl;
   const int tid = threadIdx.x, lane = tid & 31;
   if (tid == 0) cl.total = 0;
   __syncthreads();
-  const int64_t stride = (int64_t)gridDim.x * kTile;
-  int64_t p = blockIdx.x * (int64_t)kTile + tid;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  int64_t p = blockIdx.x * (int64_t)blockDim.x + tid;
   if (p < A.n) fetch_state(A, p, S);
   if (MODE == kStall) {
     __shared__ __align__(8) uint64_t stall;
@@ -1185,15 +1189,16 @@ __device__ __forceinline__ void ds_fetch(const PushArgs& A, const DsRule& D, int
 
 template <bool Q24>
 __global__ void __launch_bounds__(kThreads, 3) k_ds_push_mixed(PushArgs A, DsRule D, int64_t ntiles) {
+  grid_wait();
   extern __shared__ __align__(16) unsigned char ds_smem[];
   DsTile& S = *reinterpret_cast<DsTile*>(ds_smem);
   __shared__ CrossList cl;
   const int tid = threadIdx.x, lane = tid & 31;
   if (tid == 0) cl.total = 0;
   __syncthreads();
-  ds_fetch(A, D, blockIdx.x * (int64_t)kThreads + tid, S);
+  ds_fetch(A, D, blockIdx.x * (int64_t)blockDim.x + tid, S);
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const int64_t p = tile * kThreads + tid;
+    const int64_t p = tile * blockDim.x + tid;
     LaneOut o;
     lane_init(o, lane);
     asm volatile("cp.async.wait_all;" ::: "memory");
@@ -1220,7 +1225,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_ds_push_mixed(PushArgs A, DsRul
       }
       frozen = o.nfrz != 0;
     }
-    if (tile + gridDim.x < ntiles) ds_fetch(A, D, p + (int64_t)gridDim.x * kThreads, S);
+    if (tile + gridDim.x < ntiles) ds_fetch(A, D, p + (int64_t)gridDim.x * blockDim.x, S);
     if (T >= 0 && T < A.nt) {
       if (!frozen) {
         // the record is read after the rule's stores, so that its registers
@@ -1460,6 +1465,7 @@ __device__ __forceinline__ int32_t draw_record(unsigned idle, int lane, bool hav
 }
 
 __global__ void __launch_bounds__(kCrossMax, 2) k_cross_q24(PushArgs A, DsRule D) {
+  grid_wait();
   __shared__ int32_t cursor;
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
@@ -1739,6 +1745,7 @@ __device__ __forceinline__ void cross_finish_df(const PushArgs& A, const DsRule*
 }
 
 __global__ void __launch_bounds__(384, 2) k_cross_df(PushArgs A, DsRule D) {
+  grid_wait();
   __shared__ int32_t cursor;
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
@@ -1934,12 +1941,13 @@ __device__ __forceinline__ int32_t load64(const PushArgs& A, int64_t p, double a
 // record for the crossing pass.
 template <int MODE>
 __global__ void __launch_bounds__(kThreads) k_push_fp64(PushArgs A, int64_t ntiles) {
+  grid_wait();
   __shared__ int32_t total;
   if (threadIdx.x == 0) total = 0;
   __syncthreads();
   unsigned nfrz = 0;
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const int64_t p = tile * kThreads + threadIdx.x;
+    const int64_t p = tile * blockDim.x + threadIdx.x;
     bool leave = false;
     double a[3] = {0.0, 0.0, 0.0}, v[3] = {0.0, 0.0, 0.0}, vn[3] = {0.0, 0.0, 0.0};
     const int32_t T = load64<MODE>(A, p, a, v, nfrz);
@@ -1981,12 +1989,13 @@ __global__ void __launch_bounds__(kThreads) k_push_fp64(PushArgs A, int64_t ntil
 // 2M particles, against 686 (rule) + 220 (zero-field push) + 30 + 34 in
 // separate kernels; 1 and 3 CTAs per SM: 597 and 575 us.
 __global__ void __launch_bounds__(kThreads, 2) k_ds_push_fp64(PushArgs A, DsRule D, int64_t ntiles) {
+  grid_wait();
   __shared__ int32_t total;
   if (threadIdx.x == 0) total = 0;
   __syncthreads();
   unsigned nfrz = 0;
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const int64_t p = tile * kThreads + threadIdx.x;
+    const int64_t p = tile * blockDim.x + threadIdx.x;
     bool leave = false;
     double a[3] = {0.0, 0.0, 0.0}, v[3] = {0.0, 0.0, 0.0}, u[3] = {0.0, 0.0, 0.0};
     const int32_t T = load64<kInPlace>(A, p, a, v, nfrz);
@@ -2202,6 +2211,7 @@ __device__ __forceinline__ void cross64_finish(const PushArgs& A, const DsRule* 
 // One CTA per record region, records drawn from a shared cursor (as the mixed
 // passes).
 __global__ void __launch_bounds__(384, 2) k_cross_fp64(PushArgs A, DsRule D) {
+  grid_wait();
   __shared__ int32_t cursor;
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
@@ -2265,6 +2275,7 @@ __device__ __forceinline__ void df_cross(const DF a[3], const DF b[3], DF c[3]) 
 }
 
 __global__ void __launch_bounds__(kThreads) k_tet_finalize(TetFinalizeArgs A) {
+  grid_wait();
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= A.nt) return;
   // the slots' sums, as FP32 pairs, scaled by q w and summed over species
@@ -2332,6 +2343,7 @@ __global__ void __launch_bounds__(kThreads) k_tet_finalize(TetFinalizeArgs A) {
 __global__ void __launch_bounds__(kThreads) k_tet_finalize64(int64_t nt, const double* __restrict__ geom64,
                                                               const double* __restrict__ tgeo,
                                                               double* __restrict__ mom, double* __restrict__ out) {
+  grid_wait();
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= nt) return;
   double2* m2 = reinterpret_cast<double2*>(mom + 6 * t);
@@ -2380,6 +2392,7 @@ struct FinalizeArgs {
 // values from k_tet_finalize64.  Then G_cum += dG and the requested
 // outputs (dG, G_cum, the envelope-frame G~).
 __global__ void __launch_bounds__(kThreads) k_deposit_finalize(FinalizeArgs A) {
+  grid_wait();
   const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (e >= A.ne) return;
   double d;
@@ -2429,6 +2442,7 @@ __global__ void __launch_bounds__(kThreads) k_deposit_finalize(FinalizeArgs A) {
 __global__ void __launch_bounds__(kThreads) k_accumulate(int64_t ne, const double* __restrict__ dG,
                                                          double* __restrict__ Gcum, double* Gcum_out,
                                                          double2* Genv_out, double c, double s) {
+  grid_wait();
   const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (e >= ne) return;
   const double g = Gcum[e] + dG[e];
@@ -2921,7 +2935,7 @@ __device__ __noinline__ void dep_loss_grad(const AdjArgs& A, int32_t T0, const d
 // beta x (a - x0).  The others, about one in seven on the cavity, are walked
 // from a list in shared memory by the CTA's first threads, so that the FP64
 // walk runs with full warps: with every warp walking its own few, 300k
-// particles took 225 us, now DEPNOW.
+// particles took 225 us, now 161.
 struct DepQueue {
   int32_t n;
   int32_t T[kThreads];
@@ -3204,6 +3218,7 @@ __device__ __forceinline__ void adjoint_particle(const AdjArgs& A, int64_t p, in
 
 template <typename R, bool DEP>
 __global__ void __launch_bounds__(kThreads) k_push_adjoint(AdjArgs A) {
+  grid_wait();
   const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int lane = threadIdx.x & 31;
   R g[10];
@@ -3327,6 +3342,7 @@ __global__ void __launch_bounds__(kThreads) k_field_adjoint64(int64_t nt, const 
                                                                const double* __restrict__ tgeo,
                                                                double* __restrict__ tetgrad,
                                                                double* __restrict__ tadj) {
+  grid_wait();
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= nt) return;
   double2* tg = reinterpret_cast<double2*>(tetgrad + 10 * t);
@@ -3360,6 +3376,7 @@ __global__ void __launch_bounds__(kThreads) k_field_adjoint64(int64_t nt, const 
 __global__ void __launch_bounds__(kThreads) k_field_adjoint32(int64_t nt, const float4* __restrict__ rec,
                                                                float* __restrict__ tetgrad32,
                                                                float* __restrict__ tadj) {
+  grid_wait();
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= nt) return;
   float4* r4 = reinterpret_cast<float4*>(tetgrad32 + 12 * t);
@@ -3420,6 +3437,7 @@ __global__ void __launch_bounds__(kThreads) k_dof_grad(int64_t ne, int64_t nf, c
                                                        const R* __restrict__ tadj, double cre, double cim,
                                                        double* __restrict__ egrad, double* __restrict__ bgrad,
                                                        int64_t nt, unsigned long long* stats) {
+  grid_wait();
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i < ne) {
     double sum = 0.0;
@@ -4013,8 +4031,13 @@ static int push_particles(fempic_env* env, const fempic_particles* in, const fem
   A.momlo = env->momlo;
   A.tetdf = env->tetdf;
   A.stats = env->stats;
-  // the common path's launch: one resident wave of persistent CTAs
-  const int64_t all_tiles = (p->n + kTile - 1) / kTile;
+  // the common path's launch: one resident wave of persistent CTAs, a tile of
+  // one particle per thread at a time.  Small sets take smaller CTAs, down to
+  // a warp, so that they reach every SM (2000 particles: 8 CTAs of 256 left 144
+  // SMs idle; FP64 step and deposit 39 -> 33 us with the overlapped launches).
+  int block = kThreads;
+  while (block > 32 && (p->n + block - 1) / block < 2 * (int64_t)env->num_sms) block /= 2;
+  const int64_t all_tiles = (p->n + block - 1) / block;
   int& bps = env->push_blocks_per_sm[(mixed ? (q24 ? 1 : 0) : 2) + (ds ? 3 : 0)];
   if (bps == 0) {
     const void* k = ds          ? (!mixed ? (const void*)k_ds_push_fp64
@@ -4029,7 +4052,7 @@ static int push_particles(fempic_env* env, const fempic_particles* in, const fem
     bps = nb > 0 ? nb : 1;
   }
   const int64_t regions = std::min<int64_t>(all_tiles, (int64_t)env->num_sms * bps);
-  A.xcap = (all_tiles + regions - 1) / regions * kTile;
+  A.xcap = (all_tiles + regions - 1) / regions * block;
   rc = ensure_xqueue(env, regions * A.xcap, regions, st);
   if (rc) return rc;
   A.xrec = env->xrec;
@@ -4045,33 +4068,33 @@ static int push_particles(fempic_env* env, const fempic_particles* in, const fem
     if (mixed) {
       if (ds) {
         if (q24)
-          k_ds_push_mixed<true><<<grid, kThreads, sizeof(DsTile), st>>>(A, D, all_tiles);
+          launch(k_ds_push_mixed<true>, grid, block, sizeof(DsTile), st, A, D, all_tiles);
         else
-          k_ds_push_mixed<false><<<grid, kThreads, sizeof(DsTile), st>>>(A, D, all_tiles);
+          launch(k_ds_push_mixed<false>, grid, block, sizeof(DsTile), st, A, D, all_tiles);
       } else {
         void (*k)(PushArgs, int64_t) =
             into                ? (q24 ? k_push_mixed<true, kInto> : k_push_mixed<false, kInto>)
             : A.stall_cta >= 0 ? (q24 ? k_push_mixed<true, kStall> : k_push_mixed<false, kStall>)
                                 : (q24 ? k_push_mixed<true, kInPlace> : k_push_mixed<false, kInPlace>);
-        k<<<grid, kThreads, 0, st>>>(A, all_tiles);
+        launch(k, grid, block, 0, st, A, all_tiles);
       }
       lt.kernels = 1;
       LaunchTimer lc(env, st, FEMPIC_K_CROSS);   // nested: also inside the push bracket
       if (q24)
-        k_cross_q24<<<grid, cross_threads, 0, st>>>(A, D);
+        launch(k_cross_q24, grid, cross_threads, 0, st, A, D);
       else
-        k_cross_df<<<grid, cross_threads, 0, st>>>(A, D);
+        launch(k_cross_df, grid, cross_threads, 0, st, A, D);
       lc.kernels = 1;
     } else {
       if (ds)
-        k_ds_push_fp64<<<grid, kThreads, 0, st>>>(A, D, all_tiles);
+        launch(k_ds_push_fp64, grid, block, 0, st, A, D, all_tiles);
       else if (into)
-        k_push_fp64<kInto><<<grid, kThreads, 0, st>>>(A, all_tiles);
+        launch(k_push_fp64<kInto>, grid, block, 0, st, A, all_tiles);
       else
-        k_push_fp64<kInPlace><<<grid, kThreads, 0, st>>>(A, all_tiles);
+        launch(k_push_fp64<kInPlace>, grid, block, 0, st, A, all_tiles);
       lt.kernels = 1;
       LaunchTimer lc(env, st, FEMPIC_K_CROSS);   // nested: also inside the push bracket
-      k_cross_fp64<<<grid, cross_threads, 0, st>>>(A, D);
+      launch(k_cross_fp64, grid, cross_threads, 0, st, A, D);
       lc.kernels = 1;
     }
   }
@@ -4109,9 +4132,9 @@ static int push_step_impl(fempic_env* env, const fempic_particles* in, const fem
       L.cim[k] = (float)(cim * H.w[k]);
     }
     if (H.nl == 1)
-      k_field_f32<1><<<blocks_for(nt), kThreads, 0, st>>>(nt, env->tetrec, env->te, env->tf, L);
+      launch(k_field_f32<1>, blocks_for(nt), kThreads, 0, st, nt, env->tetrec, env->te, env->tf, L);
     else
-      k_field_f32<3><<<blocks_for(nt), kThreads, 0, st>>>(nt, env->tetrec, env->te, env->tf, L);
+      launch(k_field_f32<3>, blocks_for(nt), kThreads, 0, st, nt, env->tetrec, env->te, env->tf, L);
   } else {
     Levels<double2, double> L{};
     L.ne = env->h.ne;
@@ -4126,10 +4149,10 @@ static int push_step_impl(fempic_env* env, const fempic_particles* in, const fem
       L.cim2[k] = 2.0 * L.cim[k];
     }
     if (H.nl == 1)
-      k_field_fp64<1><<<blocks_for(nt), kThreads, 0, st>>>(nt, env->geom64, env->tgeo, env->te, env->tf, L,
+      launch(k_field_fp64<1>, blocks_for(nt), kThreads, 0, st, nt, env->geom64, env->tgeo, env->te, env->tf, L,
                                                             static_cast<double*>(env->field));
     else
-      k_field_fp64<3><<<blocks_for(nt), kThreads, 0, st>>>(nt, env->geom64, env->tgeo, env->te, env->tf, L,
+      launch(k_field_fp64<3>, blocks_for(nt), kThreads, 0, st, nt, env->geom64, env->tgeo, env->te, env->tf, L,
                                                             static_cast<double*>(env->field));
   }
   }
@@ -4279,14 +4302,14 @@ static int deposit_impl(fempic_env* env, double omega0, double t_next, double* d
         T.qwl[s] = (float)(env->qw_last[s] - (double)T.qwh[s]);
       }
       T.out = env->tetout;
-      k_tet_finalize<<<blocks_for(T.nt), kThreads, 0, st>>>(T);
+      launch(k_tet_finalize, blocks_for(T.nt), kThreads, 0, st, T);
       lt.kernels++;
     } else if (A.mode == 0) {
-      k_tet_finalize64<<<blocks_for(A.nt), kThreads, 0, st>>>(A.nt, env->geom64, env->tgeo, env->mom,
+      launch(k_tet_finalize64, blocks_for(A.nt), kThreads, 0, st, A.nt, env->geom64, env->tgeo, env->mom,
                                                               reinterpret_cast<double*>(env->tetout));
       lt.kernels++;
     }
-    k_deposit_finalize<<<blocks_for(A.ne), kThreads, 0, st>>>(A);
+    launch(k_deposit_finalize, blocks_for(A.ne), kThreads, 0, st, A);
     lt.kernels++;
     if (A.mode == 2 && A.ns > 0)
       FEMPIC_CUDA(cudaMemsetAsync(env->dGq, 0, (size_t)A.ns * env->h.nt * 8 * sizeof(unsigned long long), st));
@@ -4314,7 +4337,7 @@ extern "C" int fempic_accumulate(fempic_env* env, double omega0, double t_next, 
   const double phi = omega0 * t_next;
   {
     LaunchTimer lt(env, (cudaStream_t)stream, FEMPIC_K_FINALIZE);
-    k_accumulate<<<blocks_for(env->h.ne), kThreads, 0, (cudaStream_t)stream>>>(
+    launch(k_accumulate, blocks_for(env->h.ne), kThreads, 0, (cudaStream_t)stream, 
         env->h.ne, dG, env->Gcum, G_cum_out, static_cast<double2*>(G_env_out), std::cos(phi), std::sin(phi));
     lt.kernels = 1;
   }
@@ -4755,7 +4778,7 @@ extern "C" int fempic_push_step_adjoint(fempic_env* env, const fempic_particles*
     L.b[0] = static_cast<const float2*>(envl->b_tilde);
     L.cre[0] = (float)cre;
     L.cim[0] = (float)cim;
-    k_field_f32<1><<<blocks_for(nt), kThreads, 0, st>>>(nt, env->tetrec, env->te, env->tf, L);
+    launch(k_field_f32<1>, blocks_for(nt), kThreads, 0, st, nt, env->tetrec, env->te, env->tf, L);
     cre = (double)(float)cre;
     cim = (double)(float)cim;
   } else {
@@ -4769,7 +4792,7 @@ extern "C" int fempic_push_step_adjoint(fempic_env* env, const fempic_particles*
     L.cim[0] = cim;
     L.cre2[0] = 2.0 * cre;
     L.cim2[0] = 2.0 * cim;
-    k_field_fp64<1><<<blocks_for(nt), kThreads, 0, st>>>(nt, env->geom64, env->tgeo, env->te, env->tf, L,
+    launch(k_field_fp64<1>, blocks_for(nt), kThreads, 0, st, nt, env->geom64, env->tgeo, env->te, env->tf, L,
                                                           static_cast<double*>(env->field));
   }
   FEMPIC_CUDA(cudaGetLastError());
@@ -4812,31 +4835,31 @@ extern "C" int fempic_push_step_adjoint(fempic_env* env, const fempic_particles*
     }
     if (mixed) {
       if (A.curw)
-        k_push_adjoint<float, true><<<blocks_for(A.n), kThreads, sizeof(DepQueue), st>>>(A);
+        launch(k_push_adjoint<float, true>, blocks_for(A.n), kThreads, sizeof(DepQueue), st, A);
       else
-        k_push_adjoint<float, false><<<blocks_for(A.n), kThreads, 0, st>>>(A);
+        launch(k_push_adjoint<float, false>, blocks_for(A.n), kThreads, 0, st, A);
     } else {
       if (A.curw)
-        k_push_adjoint<double, true><<<blocks_for(A.n), kThreads, sizeof(DepQueue), st>>>(A);
+        launch(k_push_adjoint<double, true>, blocks_for(A.n), kThreads, sizeof(DepQueue), st, A);
       else
-        k_push_adjoint<double, false><<<blocks_for(A.n), kThreads, 0, st>>>(A);
+        launch(k_push_adjoint<double, false>, blocks_for(A.n), kThreads, 0, st, A);
     }
     lt.kernels++;
     FEMPIC_CUDA(cudaGetLastError());
   }
   if (!env->tadj) FEMPIC_CUDA(dalloc(&env->tadj, 10 * nt));
   if (mixed)
-    k_field_adjoint32<<<blocks_for(nt), kThreads, 0, st>>>(nt, env->tetrec, env->tetgrad32,
+    launch(k_field_adjoint32, blocks_for(nt), kThreads, 0, st, nt, env->tetrec, env->tetgrad32,
                                                            reinterpret_cast<float*>(env->tadj));
   else
-    k_field_adjoint64<<<blocks_for(nt), kThreads, 0, st>>>(nt, env->geom64, env->tgeo, env->tetgrad, env->tadj);
+    launch(k_field_adjoint64, blocks_for(nt), kThreads, 0, st, nt, env->geom64, env->tgeo, env->tetgrad, env->tadj);
   const int64_t ndof = std::max(env->h.ne, env->h.nf);
   if (mixed)
-    k_dof_grad<float><<<blocks_for(ndof), kThreads, 0, st>>>(
+    launch(k_dof_grad<float>, blocks_for(ndof), kThreads, 0, st, 
         env->h.ne, env->h.nf, env->estart, env->eslot, env->fslot, reinterpret_cast<const float*>(env->tadj), cre, cim,
         static_cast<double*>(e_grad), static_cast<double*>(b_grad), nt, env->stats);
   else
-    k_dof_grad<double><<<blocks_for(ndof), kThreads, 0, st>>>(
+    launch(k_dof_grad<double>, blocks_for(ndof), kThreads, 0, st, 
         env->h.ne, env->h.nf, env->estart, env->eslot, env->fslot, env->tadj, cre, cim,
         static_cast<double*>(e_grad), static_cast<double*>(b_grad), nt, env->stats);
   lt.kernels++;

@@ -110,3 +110,42 @@ def test_step_into_another_set_equals_the_step_in_place(prec, n):
         assert np.array_equal(v, got[k], equal_nan=True), k
     with pytest.raises(capi.FempicError, match="overlap"):
         env.push_step(st, e, b, 1.0, wl.omega0, 0.0, wl.dt, out=st)
+
+
+@pytest.mark.parametrize("prec", [FP64, MIXED, 2])
+def test_captured_steps_replay(prec):
+    """Two steps with their deposits captured in a CUDA graph (the launches
+    overlap their set-up) and replayed: the state and G_cum of the same steps
+    launched one by one."""
+    from paper_2208_12795_gb300.env import FempicEnv, ParticleState
+    wl = I.workload_hot_small(n_particles=3000)
+    got = []
+    for captured in (False, True):
+        env = FempicEnv.from_mesh(wl.mesh, precision=prec)
+        st = ParticleState.from_host(wl.particles, prec)
+        env.locate(st)
+        e = torch.from_numpy(wl.e_tilde).to(env.dof_dtype).cuda()
+        b = torch.from_numpy(wl.b_tilde).to(env.dof_dtype).cuda()
+        G = torch.zeros(env.n_edges, dtype=torch.float64, device="cuda")
+
+        def steps():
+            for k in range(2):
+                env.push_step(st, e, b, 1.0, wl.omega0, k * wl.dt, wl.dt)
+                env.deposit(wl.omega0, (k + 1) * wl.dt, G_cum_out=G)
+
+        steps()   # the first calls allocate
+        torch.cuda.synchronize()
+        if captured:
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph):
+                steps()
+            for _ in range(3):
+                graph.replay()
+        else:
+            for _ in range(3):
+                steps()
+        got.append((st.to_numpy(), G.cpu().numpy()))
+    (a, Ga), (c, Gc) = got
+    for k in a:
+        assert np.array_equal(a[k], c[k]), k
+    assert np.abs(Ga - Gc).max() <= 1e-13 * np.abs(Ga).max()
