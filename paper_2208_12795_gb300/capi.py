@@ -96,6 +96,8 @@ _lib = None
 def load(path: str = LIB_PATH):
     """Load the CUDA library (raises if it has not been built)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib

@@ -16,15 +16,15 @@ from .capi import FEMPIC_FP64, FEMPIC_MIXED, FEMPIC_MIXED_Q24  # noqa: F401
 
 
 def _stream(stream) -> int:
-    if stream is None:
-        return torch.cuda.current_stream().cuda_stream
+    if stream is None:   # the handle alone: current_stream() builds a Stream object around it (2.9 us against 0.3)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     if isinstance(stream, torch.cuda.Stream):
         return stream.cuda_stream
     return int(stream)
 
 
 def _ptr(t) -> int:
-    return 0 if t is None else int(t.data_ptr())
+    return 0 if t is None else t.data_ptr()
 
 
 def _mesh_desc(nodes: np.ndarray, tets: np.ndarray, lo, hi) -> capi.fempic_mesh_desc:
@@ -54,6 +54,21 @@ class ParticleState:
         self.m = np.ascontiguousarray(m, dtype=np.float64)
         self.w = np.ascontiguousarray(w, dtype=np.float64)
 
+    def __setattr__(self, name, value):
+        """The species arrays' addresses are taken when they are set (numpy
+        builds an object around an array's address each time it is asked, 1 us
+        for each of the four; an array keeps its memory while it is held)."""
+        object.__setattr__(self, name, value)
+        if name in ("species_begin", "q", "m", "w"):
+            object.__setattr__(self, "_at_" + name, value.ctypes.data)
+
+    def __getstate__(self):   # a copy takes the addresses of its own arrays
+        return {k: v for k, v in self.__dict__.items() if not k.startswith("_at_")}
+
+    def __setstate__(self, state):
+        for k, v in state.items():
+            setattr(self, k, v)
+
     @classmethod
     def from_host(cls, parts, precision: int, device="cuda", track_crossings=True, pin=False):
         vdt = torch.float64 if precision == FEMPIC_FP64 else torch.float32
@@ -73,15 +88,12 @@ class ParticleState:
         return int(self.x.shape[0])
 
     def cstruct(self) -> capi.fempic_particles:
-        p = capi.fempic_particles()
-        p.n = self.n
-        p.x, p.y, p.z = _ptr(self.x), _ptr(self.y), _ptr(self.z)
-        p.vx, p.vy, p.vz = _ptr(self.vx), _ptr(self.vy), _ptr(self.vz)
-        p.tet, p.status, p.n_cross = _ptr(self.tet), _ptr(self.status), _ptr(self.n_cross)
-        p.n_species = len(self.q)
-        p.species_begin = self.species_begin.ctypes.data
-        p.q, p.m, p.w = self.q.ctypes.data, self.m.ctypes.data, self.w.ctypes.data
-        return p
+        nc = self.n_cross
+        return capi.fempic_particles(self.x.shape[0], self.x.data_ptr(), self.y.data_ptr(), self.z.data_ptr(),
+                                     self.vx.data_ptr(), self.vy.data_ptr(), self.vz.data_ptr(),
+                                     self.tet.data_ptr(), self.status.data_ptr(),
+                                     0 if nc is None else nc.data_ptr(), len(self.q), self._at_species_begin,
+                                     self._at_q, self._at_m, self._at_w)
 
     def empty_like(self) -> "ParticleState":
         """Second buffer of the same shape and dtypes (the sort's output)."""
@@ -158,14 +170,14 @@ class FempicEnv:
                   t: float, dt: float, stream=None, out: ParticleState | None = None):
         """One step of `st`, in place or (with `out`) into another set of the
         same size and types, `st` left as it was."""
-        if e_dof.dtype != self.dof_dtype or b_dof.dtype != self.dof_dtype:
-            raise capi.FempicError(f"DoFs must be {self.dof_dtype} for this precision form")
+        cdt, vdt = self.dof_dtype, torch.float64 if self.precision == FEMPIC_FP64 else torch.float32
+        if e_dof.dtype != cdt or b_dof.dtype != cdt:
+            raise capi.FempicError(f"DoFs must be {cdt} for this precision form")
         if e_dof.numel() != self.n_edges or b_dof.numel() != self.n_faces or not e_dof.is_cuda:
             raise capi.FempicError("DoF arrays must be device tensors of length n_edges / n_faces")
-        vdt = torch.float64 if self.precision == FEMPIC_FP64 else torch.float32
         if st.vx.dtype != vdt:
             raise capi.FempicError(f"velocities must be {vdt} for this precision form")
-        envl = capi.fempic_envelope(_ptr(e_dof), _ptr(b_dof), float(amp))
+        envl = capi.fempic_envelope(e_dof.data_ptr(), b_dof.data_ptr(), float(amp))
         if out is not None:
             if out.vx.dtype != vdt:
                 raise capi.FempicError(f"velocities must be {vdt} for this precision form")
