@@ -3,16 +3,18 @@
 //
 // Data layout on the device (per tet, indexed by tet id):
 //   geom64  double[12]  x0, grad l1, grad l2, grad l3        (96 B, FP64 form + location)
-//   tetrec  float4 x8   mixed form, one 128 B line per tet: x0 as an FP32 pair
-//                       and grad l1..l3 (64 B), the per-step affine field
-//                       (48 B, written by k_field_f32), neighbours (16 B)
+//   tetrec  float4 x8   one 128 B line per tet: x0, FP32 grad l1..l3 and the
+//                       inside test's bound (64 B, the common path), the low
+//                       parts of the gradients, face maps and neighbours (64
+//                       B, with the first half the crossing passes')
+//   grad32  float4 x3   mixed forms: grad l1..l3 alone, for the per-tet passes
 //   tn      int4        sorted global node ids
 //   nb      int4        neighbour across local face k, or wall code
 //   te      int4 x 2    6 global edge ids, padded to 8
 //   tf      int4        4 global face ids
 //   field   per step: the affine envelope field of the tet after the carrier
 //           is restored, E(r) = E0 + (r - x0) x W, B(r) = B0 + beta (r - x0):
-//           double[10] (FP64 form) or float[12] (mixed form).
+//           double[10] (FP64 form) or float[12] (mixed forms).
 // Whitney-1 fields are affine with an antisymmetric gradient and Whitney-2
 // fields are affine with an isotropic gradient, so these 10 numbers carry the
 // whole gather of Sec. III-A for every particle in the tet; they are built
@@ -129,7 +131,6 @@ struct PushArgs {
   double* mom;                  // moment slots: sum of D (3), sum of u x D (3), FP64; contract form
                                 // per (species, tet) [ns][nt][6], FP64 form per tet [nt][6], times q w
   float* momlo;                 // low FP32 parts of the crossing pass's moments [ns][nt][8]
-  const float4* tetdf;          // contract form: low FP32 parts of grad lambda_1..3, [nt][4] float4
   unsigned long long* stats;    // [0] crossings, [1] frozen, [2] staging wait timeouts
   CrossRec* xrec;               // crossing records, one region per common-path CTA (mixed forms)
   CrossRec64* xrec64;           // FP64 form: the same, FP64 records
@@ -371,27 +372,31 @@ __global__ void __launch_bounds__(kThreads) k_field_fp64(int64_t nt, const doubl
   for (int i = 0; i < 5; i++) o[i] = make_double2(out[2 * i], out[2 * i + 1]);
 }
 
+// Bound by L1 wavefronts (a thread per tet: every access of a warp touches as
+// many lines as its stride makes it), so gradients and field are dense arrays
+// of 48 B: with both in the 128 B records 663k tets took 31 us, now 25.
 template <int NL>
-__global__ void __launch_bounds__(kThreads) k_field_f32(int64_t nt, float4* __restrict__ rec,
+__global__ void __launch_bounds__(kThreads) k_field_f32(int64_t nt, const float4* __restrict__ grad32,
+                                                         float4* __restrict__ field,
                                                          const int4* __restrict__ te, const int4* __restrict__ tf,
                                                          Levels<float2, float> L) {
   grid_wait();
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= nt) return;
-  const float4 a = rec[8 * t + 1], b = rec[8 * t + 2], c = rec[8 * t + 3];
+  const float4 a = __ldg(grad32 + 3 * t), b = __ldg(grad32 + 3 * t + 1), c = __ldg(grad32 + 3 * t + 2);
   V3<float> g[4];
-  g[1] = {a.z, a.w, b.x};
-  g[2] = {b.y, b.z, b.w};
-  g[3] = {c.x, c.y, c.z};
+  g[1] = {a.x, a.y, a.z};
+  g[2] = {a.w, b.x, b.y};
+  g[3] = {b.z, b.w, c.x};
   g[0] = {-(g[1].x + g[2].x + g[3].x), -(g[1].y + g[2].y + g[3].y), -(g[1].z + g[2].z + g[3].z)};
   const int4 e0 = te[2 * t], e1 = te[2 * t + 1], f = tf[t];
   const int32_t eid[6] = {e0.x, e0.y, e0.z, e0.w, e1.x, e1.y};
   const int32_t fid[4] = {f.x, f.y, f.z, f.w};
   float out[10];
   field_coeffs<float, float2, NL>(g, L, eid, fid, out);
-  rec[8 * t + 4] = make_float4(out[0], out[1], out[2], out[3]);
-  rec[8 * t + 5] = make_float4(out[4], out[5], out[6], out[7]);
-  reinterpret_cast<float2*>(rec + 8 * t + 6)[0] = make_float2(out[8], out[9]);   // z, w: face maps
+  field[3 * t] = make_float4(out[0], out[1], out[2], out[3]);
+  field[3 * t + 1] = make_float4(out[4], out[5], out[6], out[7]);
+  field[3 * t + 2] = make_float4(out[8], out[9], 0.f, 0.f);
 }
 
 // ------------------------------------------------------------ FP64 push
@@ -445,8 +450,10 @@ __device__ __forceinline__ int4 ldg_int4(const int4* p) { return __ldg(p); }
 //   bytes   0-23  x0 (node 0 of the tet) as 3 x f64, exact
 //   bytes  24-59  grad lambda_1..3 in FP32 (9 floats)
 //   bytes  60-63  kappa: error bound of the FP32 inside test (contract form)
-//   bytes  64-103 the step's affine field (10 floats, k_field_f32)
-//   bytes 104-111 four 16-bit face maps;  bytes 112-127 neighbour ids
+//   bytes  64-99  low FP32 parts of grad lambda_1..3
+//   bytes 100-107 four 16-bit face maps;  bytes 112-127 neighbour ids
+// The step's affine field lies apart (48 B per tet), so that the per-tet pass
+// that writes it does so in whole lines.
 struct FF {
   float hi, lo;
 };
@@ -872,9 +879,9 @@ __device__ __forceinline__ void mixed_particle(const PushArgs& A, int64_t p, int
   if (T < 0) return;
   const int s = species_of(A.sp, p);
   const float kq = A.sp.kq32[s];
-  const float4* R = A.tetrec + 8 * (int64_t)T;
+  const float4* F = static_cast<const float4*>(A.field) + 3 * (int64_t)T;
   const Geo32 G = ld_geo(A.tetrec, T);
-  const float4 f0 = __ldg(R + 4), f1 = __ldg(R + 5), f2 = __ldg(R + 6);
+  const float4 f0 = __ldg(F), f1 = __ldg(F + 1), f2 = __ldg(F + 2);
   FF dd[3];
   float d[3];
   dpos(G, ax, ay, az, dd, d);
@@ -1353,8 +1360,8 @@ __device__ __forceinline__ bool cross_advance(const PushArgs& A, CrossState& c, 
   if (nbt >= 0) {
     // the face map (same record line) says which of this tet's nodes each of
     // the neighbour's nodes is, and which one it enters through
-    const float2 fm2 = __ldg(reinterpret_cast<const float2*>(A.tetrec + 8 * (int64_t)c.T + 6) + 1);
-    const uint32_t fm = ((kx < 2 ? __float_as_uint(fm2.x) : __float_as_uint(fm2.y)) >> (16 * (kx & 1))) & 0xffffu;
+    const float4 fm4 = __ldg(A.tetrec + 8 * (int64_t)c.T + 6);
+    const uint32_t fm = ((kx < 2 ? __float_as_uint(fm4.y) : __float_as_uint(fm4.z)) >> (16 * (kx & 1))) & 0xffffu;
     const int ent = (int)(fm & 3u);
 #pragma unroll
     for (int i2 = 0; i2 < 4; i2++) {
@@ -1550,8 +1557,8 @@ __device__ __forceinline__ void lambda_df(const Geo32& G, const float glo[9], co
   lam[0] = df_sub(DF{1.0f, 0.0f}, df_add(df_add(lam[1], lam[2]), lam[3]));
 }
 
-__device__ __forceinline__ void ld_glo(const float4* __restrict__ tetdf, int64_t T, float glo[9]) {
-  const float4 a = __ldg(tetdf + 4 * T), b = __ldg(tetdf + 4 * T + 1), c = __ldg(tetdf + 4 * T + 2);
+__device__ __forceinline__ void ld_glo(const float4* __restrict__ rec, int64_t T, float glo[9]) {
+  const float4 a = __ldg(rec + 8 * T + 4), b = __ldg(rec + 8 * T + 5), c = __ldg(rec + 8 * T + 6);
   glo[0] = a.x; glo[1] = a.y; glo[2] = a.z; glo[3] = a.w;
   glo[4] = b.x; glo[5] = b.y; glo[6] = b.z; glo[7] = b.w;
   glo[8] = c.x;
@@ -1628,7 +1635,7 @@ __device__ __forceinline__ bool cross_advance_df(const PushArgs& A, CrossStateDF
   {
     const Geo32 G = ld_geo(A.tetrec, c.T);
     float glo[9];
-    ld_glo(A.tetdf, c.T, glo);
+    ld_glo(A.tetrec, c.T, glo);
     if (fresh) lambda_df(G, glo, c.a0, c.la, db);
     lambda_df(G, glo, c.b, lb, db);
   }
@@ -1675,8 +1682,8 @@ __device__ __forceinline__ bool cross_advance_df(const PushArgs& A, CrossStateDF
   if (nbt >= 0) {
     // the face map says which of this tet's nodes each of the neighbour's
     // nodes is, and which one it enters through
-    const float2 fm2 = __ldg(reinterpret_cast<const float2*>(A.tetrec + 8 * (int64_t)c.T + 6) + 1);
-    const uint32_t fm = ((kx < 2 ? __float_as_uint(fm2.x) : __float_as_uint(fm2.y)) >> (16 * (kx & 1))) & 0xffffu;
+    const float4 fm4 = __ldg(A.tetrec + 8 * (int64_t)c.T + 6);
+    const uint32_t fm = ((kx < 2 ? __float_as_uint(fm4.y) : __float_as_uint(fm4.z)) >> (16 * (kx & 1))) & 0xffffu;
     const int ent = (int)(fm & 3u);
 #pragma unroll
     for (int i2 = 0; i2 < 4; i2++) {
@@ -2261,7 +2268,6 @@ struct TetFinalizeArgs {
   int64_t nt;
   int32_t ns;
   const float4* tetrec;
-  const float4* tetdf;
   double* mom;
   float* momlo;
   float qwh[kMaxSpecies], qwl[kMaxSpecies];   // q w per species as FP32 pairs
@@ -2311,7 +2317,7 @@ __global__ void __launch_bounds__(kThreads) k_tet_finalize(TetFinalizeArgs A) {
   }
   // gradients G_1..3 as FP32 pairs, G_0 = -(G_1 + G_2 + G_3)
   const float4 a = __ldg(A.tetrec + 8 * t + 1), b = __ldg(A.tetrec + 8 * t + 2), c = __ldg(A.tetrec + 8 * t + 3);
-  const float4 p = __ldg(A.tetdf + 4 * t), q = __ldg(A.tetdf + 4 * t + 1), r = __ldg(A.tetdf + 4 * t + 2);
+  const float4 p = __ldg(A.tetrec + 8 * t + 4), q = __ldg(A.tetrec + 8 * t + 5), r = __ldg(A.tetrec + 8 * t + 6);
   const float gh[9] = {a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y, c.z};
   const float gl[9] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w, r.x};
   DF G[4][3];
@@ -2680,6 +2686,7 @@ struct AdjArgs {
   int64_t nt;
   const double* geom64;
   const double* field64;
+  const float4* field32;
   const float4* tetrec;
   double* rbx;
   double* rby;
@@ -3044,9 +3051,9 @@ __device__ __forceinline__ void adjoint_particle(const AdjArgs& A, int64_t p, in
   Vec<R> d, E0, W, B0;
   R beta;
   {
-    const float4* Rr = A.tetrec + 8 * (int64_t)T;
+    const float4* F = A.field32 + 3 * (int64_t)T;
     const Geo32 G = ld_geo(A.tetrec, T);
-    const float4 f0 = __ldg(Rr + 4), f1 = __ldg(Rr + 5), f2 = __ldg(Rr + 6);
+    const float4 f0 = __ldg(F), f1 = __ldg(F + 1), f2 = __ldg(F + 2);
     FF dd[3];
     float d32[3];
     dpos(G, L.r[0], L.r[1], L.r[2], dd, d32);   // the forward step's sequence
@@ -3373,7 +3380,7 @@ __global__ void __launch_bounds__(kThreads) k_field_adjoint64(int64_t nt, const 
   }
 }
 
-__global__ void __launch_bounds__(kThreads) k_field_adjoint32(int64_t nt, const float4* __restrict__ rec,
+__global__ void __launch_bounds__(kThreads) k_field_adjoint32(int64_t nt, const float4* __restrict__ grad32,
                                                                float* __restrict__ tetgrad32,
                                                                float* __restrict__ tadj) {
   grid_wait();
@@ -3395,11 +3402,11 @@ __global__ void __launch_bounds__(kThreads) k_field_adjoint32(int64_t nt, const 
   r4[0] = z;
   r4[1] = z;
   r4[2] = z;
-  const float4 q = rec[8 * t + 1], r = rec[8 * t + 2], c = rec[8 * t + 3];
+  const float4 q = __ldg(grad32 + 3 * t), r = __ldg(grad32 + 3 * t + 1), c = __ldg(grad32 + 3 * t + 2);
   V3<float> g[4];
-  g[1] = {q.z, q.w, r.x};
-  g[2] = {r.y, r.z, r.w};
-  g[3] = {c.x, c.y, c.z};
+  g[1] = {q.x, q.y, q.z};
+  g[2] = {q.w, r.x, r.y};
+  g[3] = {r.z, r.w, c.x};
   // g_0 formed as in the forward pre-pass
   g[0] = {-(g[1].x + g[2].x + g[3].x), -(g[1].y + g[2].y + g[3].y), -(g[1].z + g[2].z + g[3].z)};
   const V3<float> E0b = {a[0], a[1], a[2]}, Wb = {a[3], a[4], a[5]}, B0b = {a[6], a[7], a[8]};
@@ -3540,7 +3547,7 @@ struct fempic_env {
   void* field = nullptr;
   unsigned long long* dGq = nullptr;   // 24-bit form [dGq_species][nt][8]
   int32_t dGq_species = 0;
-  float4* tetdf = nullptr;             // contract form: low parts of grad lambda_1..3, [nt][4]
+  float4* grad32 = nullptr;            // mixed forms: FP32 grad lambda_1..3, [nt][3]
   double* mom = nullptr;               // moment slots: contract form [dGq_species][nt][6], FP64 form [nt][6]
   float* momlo = nullptr;              // their low FP32 parts [dGq_species][nt][8]
   float4* tetout = nullptr;            // contract and FP64 forms: per-tet edge values of a step, 48 B per tet
@@ -3621,7 +3628,7 @@ struct LaunchTimer {
 static void free_env(fempic_env* e) {
   if (!e) return;
   for (cudaEvent_t ev : e->pool) cudaEventDestroy(ev);
-  void* ptrs[] = {e->geom64, e->tgeo, e->tetrec, e->tn, e->nb, e->te, e->tf, e->field, e->dGq, e->tetdf, e->mom,
+  void* ptrs[] = {e->geom64, e->tgeo, e->tetrec, e->tn, e->nb, e->te, e->tf, e->field, e->dGq, e->grad32, e->mom,
                   e->momlo, e->tetout,
                   e->Gcum, e->stats, e->gstart, e->gtet, e->sort_counts, e->sort_offsets, e->sort_sums, e->tetgrad, e->tetgrad32, e->tadj, e->curw, e->estart, e->eslot, e->fslot, e->xrec, e->xrec64, e->xcount,
                   nullptr};
@@ -3637,7 +3644,7 @@ extern "C" void fempic_env_destroy(fempic_env* env) { free_env(env); }
 static int upload(fempic_env* e) {
   const HostMesh& m = e->h;
   const int64_t nt = m.nt;
-  std::vector<float4> geo(8 * nt), gdf(4 * nt);
+  std::vector<float4> geo(8 * nt), grd(3 * nt);
   std::vector<int4> tn(nt), nb(nt), te(2 * nt), tf(nt);
   double max_coord = 0.0;
   for (int64_t i = 0; i < m.nn * 3; i++) max_coord = std::max(max_coord, std::fabs(m.xyz[i]));
@@ -3645,7 +3652,7 @@ static int upload(fempic_env* e) {
     const double* G = &m.geom[12 * t];
     // mixed-form record: x0 exactly (3 x f64), FP32 gradients, the error
     // bound kappa of the FP32 inside test; the low FP32 parts of the
-    // gradients go to tetdf (contract form)
+    // gradients and the crossing passes' tables fill its second half
     float g[9], glo[9];
     for (int i = 0; i < 9; i++) {
       g[i] = (float)G[3 + i];
@@ -3675,11 +3682,12 @@ static int upload(fempic_env* e) {
     std::memcpy(head + 6, g, sizeof(g));
     head[15] = kappa;
     std::memcpy(&geo[8 * t], head, sizeof(head));
-    for (int k = 4; k < 7; k++) geo[8 * t + k] = make_float4(0.f, 0.f, 0.f, 0.f);
-    gdf[4 * t] = make_float4(glo[0], glo[1], glo[2], glo[3]);
-    gdf[4 * t + 1] = make_float4(glo[4], glo[5], glo[6], glo[7]);
-    gdf[4 * t + 2] = make_float4(glo[8], 0.f, 0.f, 0.f);
-    gdf[4 * t + 3] = make_float4(0.f, 0.f, 0.f, 0.f);
+    geo[8 * t + 4] = make_float4(glo[0], glo[1], glo[2], glo[3]);
+    geo[8 * t + 5] = make_float4(glo[4], glo[5], glo[6], glo[7]);
+    geo[8 * t + 6] = make_float4(glo[8], 0.f, 0.f, 0.f);
+    grd[3 * t] = make_float4(g[0], g[1], g[2], g[3]);
+    grd[3 * t + 1] = make_float4(g[4], g[5], g[6], g[7]);
+    grd[3 * t + 2] = make_float4(g[8], 0.f, 0.f, 0.f);
     {
       // face maps of the mixed crossing walk, 16 bits per local face k with a
       // neighbour: bits 0-1 the neighbour's local node that is not in this
@@ -3701,8 +3709,8 @@ static int upload(fempic_env* e) {
         }
         fmap[k >> 1] |= code << (16 * (k & 1));
       }
-      std::memcpy(&geo[8 * t + 6].z, &fmap[0], 4);
-      std::memcpy(&geo[8 * t + 6].w, &fmap[1], 4);
+      std::memcpy(&geo[8 * t + 6].y, &fmap[0], 4);
+      std::memcpy(&geo[8 * t + 6].z, &fmap[1], 4);
     }
     int32_t nbk[4] = {m.nb[4 * t], m.nb[4 * t + 1], m.nb[4 * t + 2], m.nb[4 * t + 3]};
     float4 nbf;
@@ -3722,9 +3730,10 @@ static int upload(fempic_env* e) {
   FEMPIC_CUDA(dalloc(&e->tf, nt));
   FEMPIC_CUDA(cudaMemcpy(e->geom64, m.geom.data(), 12 * nt * sizeof(double), cudaMemcpyHostToDevice));
   FEMPIC_CUDA(cudaMemcpy(e->tetrec, geo.data(), 8 * nt * sizeof(float4), cudaMemcpyHostToDevice));
-  if (e->opt.precision == FEMPIC_MIXED) {
-    FEMPIC_CUDA(dalloc(&e->tetdf, 4 * nt));
-    FEMPIC_CUDA(cudaMemcpy(e->tetdf, gdf.data(), 4 * nt * sizeof(float4), cudaMemcpyHostToDevice));
+  if (e->opt.precision != FEMPIC_FP64) {
+    FEMPIC_CUDA(dalloc(&e->grad32, 3 * nt));
+    FEMPIC_CUDA(cudaMemcpy(e->grad32, grd.data(), 3 * nt * sizeof(float4), cudaMemcpyHostToDevice));
+    FEMPIC_CUDA(dalloc(reinterpret_cast<float4**>(&e->field), 3 * nt));
   }
   FEMPIC_CUDA(cudaMemcpy(e->tn, tn.data(), nt * sizeof(int4), cudaMemcpyHostToDevice));
   FEMPIC_CUDA(cudaMemcpy(e->nb, nb.data(), nt * sizeof(int4), cudaMemcpyHostToDevice));
@@ -4029,7 +4038,6 @@ static int push_particles(fempic_env* env, const fempic_particles* in, const fem
   A.dGq = env->deposit_on ? env->dGq : nullptr;
   A.mom = env->deposit_on ? env->mom : nullptr;
   A.momlo = env->momlo;
-  A.tetdf = env->tetdf;
   A.stats = env->stats;
   // the common path's launch: one resident wave of persistent CTAs, a tile of
   // one particle per thread at a time.  Small sets take smaller CTAs, down to
@@ -4132,9 +4140,9 @@ static int push_step_impl(fempic_env* env, const fempic_particles* in, const fem
       L.cim[k] = (float)(cim * H.w[k]);
     }
     if (H.nl == 1)
-      launch(k_field_f32<1>, blocks_for(nt), kThreads, 0, st, nt, env->tetrec, env->te, env->tf, L);
+      launch(k_field_f32<1>, blocks_for(nt), kThreads, 0, st, nt, env->grad32, static_cast<float4*>(env->field), env->te, env->tf, L);
     else
-      launch(k_field_f32<3>, blocks_for(nt), kThreads, 0, st, nt, env->tetrec, env->te, env->tf, L);
+      launch(k_field_f32<3>, blocks_for(nt), kThreads, 0, st, nt, env->grad32, static_cast<float4*>(env->field), env->te, env->tf, L);
   } else {
     Levels<double2, double> L{};
     L.ne = env->h.ne;
@@ -4294,7 +4302,6 @@ static int deposit_impl(fempic_env* env, double omega0, double t_next, double* d
       T.nt = env->h.nt;
       T.ns = A.ns;
       T.tetrec = env->tetrec;
-      T.tetdf = env->tetdf;
       T.mom = env->mom;
       T.momlo = env->momlo;
       for (int s = 0; s < kMaxSpecies; s++) {
@@ -4778,7 +4785,7 @@ extern "C" int fempic_push_step_adjoint(fempic_env* env, const fempic_particles*
     L.b[0] = static_cast<const float2*>(envl->b_tilde);
     L.cre[0] = (float)cre;
     L.cim[0] = (float)cim;
-    launch(k_field_f32<1>, blocks_for(nt), kThreads, 0, st, nt, env->tetrec, env->te, env->tf, L);
+    launch(k_field_f32<1>, blocks_for(nt), kThreads, 0, st, nt, env->grad32, static_cast<float4*>(env->field), env->te, env->tf, L);
     cre = (double)(float)cre;
     cim = (double)(float)cim;
   } else {
@@ -4814,6 +4821,7 @@ extern "C" int fempic_push_step_adjoint(fempic_env* env, const fempic_particles*
     A.nt = nt;
     A.geom64 = env->geom64;
     A.field64 = static_cast<const double*>(env->field);
+    A.field32 = static_cast<const float4*>(env->field);
     A.tetrec = env->tetrec;
     A.rbx = adj->rx;
     A.rby = adj->ry;
@@ -4849,7 +4857,7 @@ extern "C" int fempic_push_step_adjoint(fempic_env* env, const fempic_particles*
   }
   if (!env->tadj) FEMPIC_CUDA(dalloc(&env->tadj, 10 * nt));
   if (mixed)
-    launch(k_field_adjoint32, blocks_for(nt), kThreads, 0, st, nt, env->tetrec, env->tetgrad32,
+    launch(k_field_adjoint32, blocks_for(nt), kThreads, 0, st, nt, env->grad32, env->tetgrad32,
                                                            reinterpret_cast<float*>(env->tadj));
   else
     launch(k_field_adjoint64, blocks_for(nt), kThreads, 0, st, nt, env->geom64, env->tgeo, env->tetgrad, env->tadj);
