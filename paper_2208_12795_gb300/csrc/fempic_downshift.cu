@@ -463,6 +463,36 @@ extern "C" int fempic_downshift_weights(double t, double dt, double omega0, doub
   return FEMPIC_OK;
 }
 
+// The mixed forms' coefficients and geometry factors, on first use.  Built on a
+// stream of its own that is waited for: later steps may be on any stream, and a
+// first step that is being captured must not defer the table to its replay.
+static int make_mixed_tables(fempic_downshift* ds) {
+  double* dgeo = nullptr;
+  float* coef32 = nullptr;
+  if (cudaMalloc(&dgeo, sizeof(double) * kDsGeo * (size_t)ds->nt) != cudaSuccess ||
+      cudaMalloc(&coef32, sizeof(float) * fempic::kDsCoef32 * (size_t)ds->nt) != cudaSuccess) {
+    cudaGetLastError();
+    cudaFree(dgeo);
+    return fail(FEMPIC_ENOMEM, "push_step_downshift: device allocation");
+  }
+  cudaStream_t own = nullptr;
+  cudaError_t rc = cudaStreamCreateWithFlags(&own, cudaStreamNonBlocking);
+  if (rc == cudaSuccess) {
+    k_ds_geo32<<<blocks_for(ds->nt), kThreads, 0, own>>>(ds->nt, ds->geom, dgeo);
+    rc = cudaGetLastError();
+    if (rc == cudaSuccess) rc = cudaStreamSynchronize(own);
+    cudaStreamDestroy(own);
+  }
+  if (rc != cudaSuccess) {
+    cudaFree(dgeo);
+    cudaFree(coef32);
+  }
+  DS_CUDA(rc);
+  ds->dgeo = dgeo;
+  ds->coef32 = coef32;
+  return FEMPIC_OK;
+}
+
 extern "C" int fempic_push_step_downshift(fempic_env* env, fempic_downshift* ds, const fempic_particles* p,
                                           const fempic_downshift_history* hist, const fempic_envelope* envl,
                                           double omega0, double t, double dt, int32_t start, void* stream) {
@@ -506,17 +536,9 @@ extern "C" int fempic_push_step_downshift(fempic_env* env, fempic_downshift* ds,
   A.start = start;
   compute_weights(t, dt, omega0, A.w);
   for (int i = 0; i < 24; i++) A.w32[i] = (float)A.w[i];
-  if (mixed && !ds->coef32) {   // the mixed forms' coefficients and geometry factors, on first use
-    if (cudaMalloc(&ds->dgeo, sizeof(double) * kDsGeo * (size_t)ds->nt) != cudaSuccess ||
-        cudaMalloc(&ds->coef32, sizeof(float) * fempic::kDsCoef32 * (size_t)ds->nt) != cudaSuccess) {
-      cudaGetLastError();
-      cudaFree(ds->dgeo);
-      ds->dgeo = nullptr;
-      ds->coef32 = nullptr;
-      return fail(FEMPIC_ENOMEM, "push_step_downshift: device allocation");
-    }
-    k_ds_geo32<<<blocks_for(ds->nt), kThreads, 0, (cudaStream_t)stream>>>(ds->nt, ds->geom, ds->dgeo);
-    DS_CUDA(cudaGetLastError());
+  if (mixed && !ds->coef32) {
+    const int rc = make_mixed_tables(ds);
+    if (rc != FEMPIC_OK) return rc;
   }
   A.coef = ds->coef;
   A.coef32 = ds->coef32;

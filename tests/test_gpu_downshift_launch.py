@@ -70,3 +70,28 @@ def test_dof_not_finite_freezes_its_tets(prec):
     assert np.array_equal(bad["x"][hit], good["x0"][hit])
     for k in ("x", "vx", "tet", "status"):
         assert np.array_equal(bad[k][~hit], good[k][~hit]), k
+
+
+def test_first_step_captured_leaves_nothing_to_the_replay():
+    """A first step that is only captured (its graph never replayed) and the
+    same steps launched after it: the run of a new integrator."""
+    from paper_2208_12795_gb300.env import Downshift, FempicEnv, ParticleState
+    n = 2000
+    wl = I.te101_cavity(5, MOST, 200.0, 1e4, 1, 21, dt=2e-9, ramp_sigma=0.0, jitter=0.2)
+    env = FempicEnv.from_mesh(wl.mesh, precision=MIXED)
+    st = ParticleState.from_host(wl.particles.subset(n), MIXED)
+    env.locate(st)
+    e = torch.from_numpy(wl.e_tilde).to(env.dof_dtype).cuda()
+    b = torch.from_numpy(wl.b_tilde).to(env.dof_dtype).cuda()
+    env.push_step(st, e, b, 0.0, wl.omega0, 0.0, wl.dt, out=st.empty_like())   # the env's own scratch
+    env.deposit(wl.omega0, wl.dt)
+    ds = Downshift(env, n)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, capture_error_mode="relaxed"):
+        ds.step(st, e, b, 1.0, wl.omega0, 0.0, wl.dt)
+    ds.started = False
+    for k in range(3):
+        ds.step(st, e, b, 1.0, wl.omega0, k * wl.dt, wl.dt)
+    want, got = _run(MIXED, n), st.to_numpy()
+    for k in got:
+        assert np.array_equal(got[k], want[k]), k
