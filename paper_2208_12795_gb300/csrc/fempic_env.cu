@@ -586,7 +586,7 @@ __device__ __forceinline__ void gq(const int32_t a[4], const int32_t b[4], long 
   }
 }
 
-// The mixed form deposits into one 64-byte slot per (species, tet): the 6
+// The 24-bit form deposits into one 64-byte slot per (species, tet): the 6
 // local edges of the tet, contiguous, so a run head touches 2 sectors instead
 // of 6 scattered edge entries; k_deposit_finalize pulls each edge's sum from
 // the slots of its incident tets.
@@ -1497,8 +1497,8 @@ __device__ __forceinline__ void cross_finish(const PushArgs& A, const DsRule* H,
 // where some tiles hold many long walks (a 10 keV beam leaves its tet every
 // step and crosses about eight faces).  Against a fixed stream of tiles per
 // warp with lanes refilled one by one: 1.30 -> 1.21 ms per step on that load,
-// 0.203 -> 0.185 on the 10M cavity; waiting for 1, 8, 12, 16 idle lanes:
-// 1.29, 1.24, 1.21, 1.22 ms.
+// 0.203 -> 0.185 on the 10M cavity (0.168 since a piece reads one line of the
+// tet record); waiting for 1, 8, 12, 16 idle lanes: 1.29, 1.24, 1.21, 1.22 ms.
 // A pass's CTAs number as many per SM as its common path's, so their size
 // makes up the warps: 24 per SM (32 in the 24-bit pass, at 64 registers).
 constexpr int kCrossMax = 512;
@@ -1848,9 +1848,10 @@ __global__ void __launch_bounds__(384, 2) k_cross_df(PushArgs A, DsRule D) {
 // in FP64, so tets are those of the FP64 barycentrics.  Against barycentrics
 // of both ends and six edge products per particle (116 operations): 0.390 ->
 // 0.219 ms at 2M particles (the crossing pass 0.125 -> 0.067); four steps and
-// a sort of 6M electrons on 40^3 x 6 tets 6.88 -> 4.31 ms.  Rounding of the
-// moment form against 80-bit sums over such tets: 3e-16 of the edge values'
-// norm (1.8e-15 for the barycentric form).
+// a sort of 6M electrons on 40^3 x 6 tets 6.88 -> 4.31 ms (now 4.04: the field
+// pass from tables, overlapped launches).  Rounding of the moment form against
+// 80-bit sums over such tets: 3e-16 of the edge values' norm (1.8e-15 for the
+// barycentric form).
 
 // Leading 24 bits of an FP64 value as a float (truncated, so at most 2^-23
 // relative below it in magnitude): 0 below 2^-126, infinite from 2^128 on.
@@ -2307,9 +2308,10 @@ __global__ void __launch_bounds__(384, 2) k_cross_fp64(PushArgs A, DsRule D) {
 // Contract form, per tet: the moment slots (sum of D, sum of u x D, FP64)
 // become the 6 local-edge values through the tet's gradients,
 //   g_0j = G_j . sum D + (G_0 x G_j) . sum(u x D),  g_ij = (G_i x G_j) . sum(u x D),
-// in double-float from the FP64 gradients' FP32 pairs; the crossing pass's
-// edge-form deposits are added, each species scaled by its q w, and the sum
-// is written as FP32 pairs for the per-edge pull.  The slots are cleared.
+// in double-float from the FP64 gradients' FP32 pairs, each species scaled by
+// its q w (the crossing pass's pieces are in the same slots, their low parts
+// in the FP32 companion slots).  The sum is written as FP32 pairs for the
+// per-edge pull.  The slots are cleared.
 struct TetFinalizeArgs {
   int64_t nt;
   int32_t ns;
@@ -3611,10 +3613,10 @@ struct fempic_env {
   int32_t* estart = nullptr;        // edge -> (tet, local edge) slots, CSR [ne + 1]
   int32_t* eslot = nullptr;         // [6 nt], slot = 6 tet + local edge
   int32_t* fslot = nullptr;         // face -> (tet, local face) slots [nf][2], 4 tet + local face or -1
-  CrossRec* xrec = nullptr;         // mixed forms: crossing queue [xslots]
-  CrossRec64* xrec64 = nullptr;     // FP64 form: crossing queue [xslots]
-  int32_t* xcount = nullptr;        // [xregions]
-  int64_t xslots = 0, xregions = 0;
+  CrossRec* xrec = nullptr;         // mixed forms: crossing queue [xqueue_slots]
+  CrossRec64* xrec64 = nullptr;     // FP64 form: crossing queue [xqueue_slots]
+  int32_t* xcount = nullptr;        // per record region
+  int64_t xn = 0;                   // particles these hold the records of (xqueue_slots)
   int num_sms = 1;
   int push_blocks_per_sm[6] = {0, 0, 0, 0, 0, 0};   // resident CTAs of the common path: contract, 24-bit, FP64; downshifted + 3
   int64_t steps = 0;
@@ -3946,13 +3948,23 @@ extern "C" int fempic_locate(fempic_env* env, const fempic_particles* p, void* s
   return FEMPIC_OK;
 }
 
-// Crossing queue: `slots` records in `regions` regions with a count each,
-// grown on demand (every region's count is rewritten by the common path each
-// step, so nothing needs clearing).
-static int ensure_xqueue(fempic_env* env, int64_t slots, int64_t regions, cudaStream_t st) {
-  if (env->xslots >= slots && env->xregions >= regions) return FEMPIC_OK;
-  slots = std::max(slots, env->xslots);
-  regions = std::max(regions, env->xregions);
+// Crossing queue: record regions with a count each, grown on demand (every
+// region's count is rewritten by the common path each step, so nothing needs
+// clearing).
+// Slots that hold the record regions of every launch on n particles or fewer:
+// R <= min(tiles, SMs x kMaxRegionsPerSm) regions of ceil(tiles / R) tiles of
+// at most kThreads particles take at most n + min(n, R x kThreads) slots and a
+// tile.  Sized so, a step on fewer particles, or of the other integrator,
+// never allocates (one may be captured into a graph once a larger set has
+// stepped).
+constexpr int kMaxRegionsPerSm = 2048 / kThreads;   // resident CTAs of kThreads
+
+static int64_t xqueue_slots(const fempic_env* env, int64_t n) {
+  return n + std::min<int64_t>(n, (int64_t)env->num_sms * kMaxRegionsPerSm * kThreads) + 2 * kThreads;
+}
+
+static int ensure_xqueue(fempic_env* env, int64_t n, cudaStream_t st) {
+  if (env->xcount && env->xn >= n) return FEMPIC_OK;
   if (env->xcount) {
     FEMPIC_CUDA(cudaStreamSynchronize(st));
     cudaFree(env->xrec);
@@ -3961,15 +3973,15 @@ static int ensure_xqueue(fempic_env* env, int64_t slots, int64_t regions, cudaSt
     env->xrec = nullptr;
     env->xrec64 = nullptr;
     env->xcount = nullptr;
-    env->xslots = env->xregions = 0;
+    env->xn = 0;
   }
+  const int64_t slots = xqueue_slots(env, n);
   if (env->opt.precision != FEMPIC_FP64)
     FEMPIC_CUDA(dalloc(&env->xrec, slots));
   else
     FEMPIC_CUDA(dalloc(&env->xrec64, slots));
-  FEMPIC_CUDA(dalloc(&env->xcount, regions));
-  env->xslots = slots;
-  env->xregions = regions;
+  FEMPIC_CUDA(dalloc(&env->xcount, std::min<int64_t>(n / 32 + 1, (int64_t)env->num_sms * kMaxRegionsPerSm)));
+  env->xn = n;
   return FEMPIC_OK;
 }
 
@@ -4116,11 +4128,11 @@ static int push_particles(fempic_env* env, const fempic_particles* in, const fem
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(DsTile)));
     int nb = 0;
     FEMPIC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, kThreads, ds && mixed ? sizeof(DsTile) : 0));
-    bps = nb > 0 ? nb : 1;
+    bps = nb > 0 ? std::min(nb, kMaxRegionsPerSm) : 1;
   }
   const int64_t regions = std::min<int64_t>(all_tiles, (int64_t)env->num_sms * bps);
   A.xcap = (all_tiles + regions - 1) / regions * block;
-  rc = ensure_xqueue(env, regions * A.xcap, regions, st);
+  rc = ensure_xqueue(env, p->n, st);
   if (rc) return rc;
   A.xrec = env->xrec;
   A.xrec64 = env->xrec64;
@@ -4131,7 +4143,7 @@ static int push_particles(fempic_env* env, const fempic_particles* in, const fem
   {
     LaunchTimer lt(env, st, FEMPIC_K_PUSH);
     const unsigned grid = (unsigned)regions;
-    const int cross_threads = std::min(q24 ? kCrossMax : 384, 32 * ((q24 ? 32 : 24) / std::min(bps, 8)));
+    const int cross_threads = std::min(q24 ? kCrossMax : 384, 32 * ((q24 ? 32 : 24) / bps));
     if (mixed) {
       if (ds) {
         const bool vec = vec_state(p) && !(((uintptr_t)D.h) & 15u) && p->n % 4 == 0;

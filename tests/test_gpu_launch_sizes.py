@@ -149,3 +149,32 @@ def test_captured_steps_replay(prec):
     for k in a:
         assert np.array_equal(a[k], c[k]), k
     assert np.abs(Ga - Gc).max() <= 1e-13 * np.abs(Ga).max()
+
+
+@pytest.mark.parametrize("prec", [FP64, MIXED, 2])
+def test_fewer_particles_never_allocate(prec):
+    """After a step on a set, steps on smaller ones (whose launches take other
+    tiles and more regions) can be captured: their scratch is the larger set's."""
+    from paper_2208_12795_gb300.env import FempicEnv, ParticleState
+    sizes = (152 * 2 * 256 - 256, 152 * 2 * 128 - 1, 5000, 33)
+    wl = I.workload_hot_small(n_particles=sizes[0] + 1)
+    env = FempicEnv.from_mesh(wl.mesh, precision=prec)
+    e = torch.from_numpy(wl.e_tilde).to(env.dof_dtype).cuda()
+    b = torch.from_numpy(wl.b_tilde).to(env.dof_dtype).cuda()
+
+    def load(n):
+        st = ParticleState.from_host(wl.particles.subset(n), prec)
+        env.locate(st)
+        return st
+
+    env.push_step(load(sizes[0] + 1), e, b, 1.0, wl.omega0, 0.0, wl.dt)
+    for n in sizes:
+        want, got = load(n), load(n)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            env.push_step(got, e, b, 1.0, wl.omega0, 0.0, wl.dt)
+        graph.replay()
+        env.push_step(want, e, b, 1.0, wl.omega0, 0.0, wl.dt)
+        w, g = want.to_numpy(), got.to_numpy()
+        for k in w:
+            assert np.array_equal(w[k], g[k]), (n, k)
