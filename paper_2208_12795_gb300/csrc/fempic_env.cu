@@ -2765,16 +2765,12 @@ struct AdjArgs {
 // w) follows the FP64 walk again: a crossing point q = a0 + S w on face f
 // moves in the face plane, dq = P (da0 + S dw) with P = I - w G_f^T / (G_f .
 // w); a wall reflection starts a new run a0' = q, w' = M (1 - S) w (M the
-// mirror), whose Jacobian is folded into the running 6 x 6 one.
+// mirror).
 __device__ __forceinline__ void cross3d(const double a[3], const double b[3], double c[3]) {
   c[0] = a[1] * b[2] - a[2] * b[1];
   c[1] = a[2] * b[0] - a[0] * b[2];
   c[2] = a[0] * b[1] - a[1] * b[0];
 }
-__device__ __forceinline__ double dot3d(const double a[3], const double b[3]) {
-  return a[0] * b[0] + a[1] * b[1] + a[2] * b[2];
-}
-
 // Gradient rows of tet T (FP64): G[k] = grad lambda_k, G_0 = -(G_1 + G_2 + G_3).
 __device__ __forceinline__ void grads64(const double* geom64, int32_t T, double G[4][3]) {
   const double* g = geom64 + 12 * (int64_t)T;
@@ -2786,200 +2782,298 @@ __device__ __forceinline__ void grads64(const double* geom64, int32_t T, double 
   for (int c = 0; c < 3; c++) G[0][c] = -((G[1][c] + G[2][c]) + G[3][c]);
 }
 
-// d(loss)/d(a), d(loss)/d(w) of one particle-step whose run starts at a with
-// end b (= a + w as the forward step formed it), tet T0 at the start.
-// The 6 x 6 Jacobian lives in local memory (loops not unrolled): only
-// particles that reflected in this step touch it.
-__device__ __noinline__ void dep_loss_grad(const AdjArgs& A, int32_t T0, const double a[3], const double b_in[3],
-                                           double ga[3], double gw[3]) {
-  double a0[3], b[3], w[3], pnt[3];
+struct DepQueue {
+  int32_t n, next;
+  int32_t T[kThreads];
+  double a[3][kThreads], b[3][kThreads];   // start and end; after the walk d/da and d/dw
+};
+
+// One reflection of a run a0 + S w at its point q (S) on a wall of axis `ax`
+// with face gradient g: the new run is a0' = q, w' = M (1 - S) w.
+struct DepWall {
+  double w[3], gr[3], S;   // gr = g / (g . w)
+  int ax;
+};
+
+// Gradients (ca, cw) with respect to the run after a reflection -> to the run
+// before it: dq = P (da0 + S dw) with P = I - w gr^T, dw' = M ((1 - S) dw +
+// w gr^T (da0 + S dw)).
+__device__ __forceinline__ void dep_unreflect(const DepWall& W, const double ca[3], const double cw[3], double a[3],
+                                              double w[3]) {
+  double mw[3];
+#pragma unroll
+  for (int c = 0; c < 3; c++) mw[c] = c == W.ax ? -cw[c] : cw[c];
+  const double f = tet_dot(W.w, mw) - tet_dot(W.w, ca);
 #pragma unroll
   for (int c = 0; c < 3; c++) {
-    a0[c] = a[c];
-    b[c] = b_in[c];
-    w[c] = b[c] - a[c];
-    pnt[c] = a[c];
-    ga[c] = gw[c] = 0.0;
+    a[c] = fma(W.gr[c], f, ca[c]);
+    w[c] = fma(W.S, a[c], (1.0 - W.S) * mw[c]);
   }
-  double J[6][6];          // d(a0, w of the current run) / d(a, w of the step), once a wall reflected it
-  bool refl = false;
-  double gprev[3] = {0.0, 0.0, 0.0}, Sprev = 0.0;
-  bool on_face = false;    // the piece start is a crossing point of this run (face gradient gprev)
-  double S = 0.0;
-  int32_t T = T0;
-  int entry = -1, nc = 0;
-  double la[4], lb[4];
-  bary64(A.geom64 + 12 * (int64_t)T, pnt, la);
-  for (;;) {
-    bary64(A.geom64 + 12 * (int64_t)T, b, lb);
-    double smin;
-    const int kx = exit_face64(la, lb, entry, smin);
-    double G[4][3];
-    grads64(A.geom64, T, G);
-    const double* cw = A.curw + 6 * (int64_t)T;
-    const double al[3] = {cw[0], cw[1], cw[2]}, be[3] = {cw[3], cw[4], cw[5]};
-    const double* x0 = A.geom64 + 12 * (int64_t)T;
-    double q[3], Sq = 1.0;
-    if (kx < 0) {
-#pragma unroll
-      for (int c = 0; c < 3; c++) q[c] = b[c];
-    } else {
-#pragma unroll
-      for (int c = 0; c < 3; c++) q[c] = fma(smin, b[c] - pnt[c], pnt[c]);
-      Sq = S + smin * (1.0 - S);
-    }
-    // this piece's gradients at its ends
-    double u[3], d[3], bu[3], db_[3], gp[3], gq[3];
-#pragma unroll
-    for (int c = 0; c < 3; c++) {
-      u[c] = pnt[c] - x0[c];
-      d[c] = q[c] - pnt[c];
-    }
-    cross3d(be, u, bu);
-    cross3d(d, be, db_);
-#pragma unroll
-    for (int c = 0; c < 3; c++) {
-      gp[c] = -al[c] - bu[c] + db_[c];
-      gq[c] = al[c] + bu[c];
-    }
-    // ... through the ends' dependence on (a0, w) of this run
-    double ca[3], cwv[3];
-    {
-      double tp[3];
-      if (on_face) {
-        const double f = dot3d(w, gp) / dot3d(gprev, w);
-#pragma unroll
-        for (int c = 0; c < 3; c++) tp[c] = gp[c] - gprev[c] * f;
-      } else {
-#pragma unroll
-        for (int c = 0; c < 3; c++) tp[c] = gp[c];
-      }
-#pragma unroll
-      for (int c = 0; c < 3; c++) {
-        ca[c] = tp[c];
-        cwv[c] = on_face ? Sprev * tp[c] : 0.0;
-      }
-      if (kx < 0) {
-#pragma unroll
-        for (int c = 0; c < 3; c++) {
-          ca[c] += gq[c];
-          cwv[c] += gq[c];
-        }
-      } else {
-        const double f = dot3d(w, gq) / dot3d(G[kx], w);
-#pragma unroll
-        for (int c = 0; c < 3; c++) {
-          const double t = gq[c] - G[kx][c] * f;
-          ca[c] += t;
-          cwv[c] += Sq * t;
-        }
-      }
-    }
-    // ... and through the run's dependence on the step's (a, w)
-    if (refl) {
+}
+
+// Adds (ca, cw) of a run after several reflections through the Jacobian J
+// (columns: the step's a, w) of the reflections before the last, which is W.
+__device__ __noinline__ void dep_through(const double* J, const DepWall& W, const double* c6, double* g6) {
+  double a[3], w[3];
+  dep_unreflect(W, c6, c6 + 3, a, w);
 #pragma unroll 1
-      for (int i = 0; i < 3; i++) {
-        double sa = 0.0, sw = 0.0;
+  for (int i = 0; i < 6; i++) {
+    double acc = 0.0;
 #pragma unroll
-        for (int r = 0; r < 3; r++) {
-          sa += J[r][i] * ca[r] + J[3 + r][i] * cwv[r];
-          sw += J[r][3 + i] * ca[r] + J[3 + r][3 + i] * cwv[r];
+    for (int r = 0; r < 3; r++) acc += J[6 * r + i] * a[r] + J[6 * (3 + r) + i] * w[r];
+    g6[i] += acc;
+  }
+}
+
+// Folds reflection W into J (6 x 6; the identity before the first): row r of
+// the new Jacobian is the gradient of component r of the run after W.
+__device__ __noinline__ void dep_fold(double* J, const DepWall& W, bool first) {
+  double Jn[36];
+#pragma unroll 1
+  for (int r = 0; r < 6; r++) {
+    double c[6], a[3], w[3];
+#pragma unroll
+    for (int k = 0; k < 6; k++) c[k] = k == r ? 1.0 : 0.0;
+    dep_unreflect(W, c, c + 3, a, w);
+#pragma unroll 1
+    for (int i = 0; i < 6; i++) {
+      double acc = 0.0;
+      if (first) {
+        acc = i < 3 ? (i == 0 ? a[0] : i == 1 ? a[1] : a[2]) : (i == 3 ? w[0] : i == 4 ? w[1] : w[2]);
+      } else {
+#pragma unroll
+        for (int k = 0; k < 3; k++) acc += a[k] * J[6 * k + i] + w[k] * J[6 * (3 + k) + i];
+      }
+      Jn[6 * r + i] = acc;
+    }
+  }
+#pragma unroll 1
+  for (int i = 0; i < 36; i++) J[i] = Jn[i];
+}
+
+// t = g - G (w . g) r: a gradient with respect to a crossing point, moved onto
+// the face of gradient G, r = 1 / (G . w).
+__device__ __forceinline__ void onto_face(const double g[3], const double G[3], const double w[3], double r,
+                                          double t[3]) {
+  const double f = tet_dot(w, g) * r;
+#pragma unroll
+  for (int c = 0; c < 3; c++) t[c] = fma(-f, G[c], g[c]);
+}
+
+// The walks of a CTA's list, by its first warps: each loop iteration advances
+// a busy lane by one piece, and a lane that is done takes the list's next
+// walk.  A piece p -> q of a run has the gradients gp = -alpha - beta x u + d x
+// beta and gq = alpha + beta x u at its ends; at a crossing the ended piece's
+// gq and the next one's gp meet, and their sum is moved onto the face once.  A
+// run's own start and end enter as they are.  The rest of the CTA waits for
+// its walks, a chain of FP64 operations and tet records, so what counts is
+// their operations (one projection a crossing instead of two: 161 -> 127 us at
+// 300k particles), their reflections (mapped back as vectors, a Jacobian only
+// from the second on: 18 us less) and the CTAs per SM (2, 3, 4: 116, 101, 95
+// us).  Without any walk the kernel takes 32 us.
+__device__ __noinline__ void dep_walk(const AdjArgs& A, DepQueue& Q) {
+  const int m = Q.n, lane = threadIdx.x & 31;
+  const unsigned full = 0xffffffffu;
+  double J[36];            // Jacobian of the reflections before the last one, once there are two
+  DepWall W;               // the last reflection
+  double b[3], w[3], pnt[3], la[4], lb[4];
+  double ga[3], gw[3];     // of the step, from runs that ended
+  double ca[3], cw[3];     // of the current run
+  double gm[3], gf[3], rf = 0.0;   // at a crossing: the ended piece's gq; the face's gradient and 1 / (gf . w)
+  double S = 0.0;
+  int32_t T = 0, at = -1;
+  int entry = -1, nc = 0;
+  int refl = 0;            // reflections of the walk so far
+  bool on_face = false, more = true;
+  for (;;) {
+    const unsigned idle = __ballot_sync(full, at < 0);
+    bool fresh = false;
+    if (idle && more) {
+      const int32_t k = draw_record(idle, lane, at >= 0, m, &Q.next, more);
+      if (k >= 0) {
+        at = k;
+        fresh = true;
+        T = Q.T[k];
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+          pnt[c] = Q.a[c][k];
+          b[c] = Q.b[c][k];
+          w[c] = b[c] - pnt[c];
+          ga[c] = gw[c] = ca[c] = cw[c] = 0.0;
         }
-        ga[i] += sa;
-        gw[i] += sw;
+        S = 0.0;
+        entry = -1;
+        nc = 0;
+        refl = 0;
+        on_face = false;
+      }
+    }
+    if (!__any_sync(full, at >= 0)) return;
+    if (at < 0) continue;
+    const double* g = A.geom64 + 12 * (int64_t)T;
+    const double* wt = A.curw + 6 * (int64_t)T;
+    const int4 nbv = ldg_int4(&A.nb[T]), o4 = ldg_int4(&A.tn[T]);
+    double u[3], gp[3], gq[3], q[3], gk[3], smin, Sq = 1.0;
+    int kx;
+    {
+      double G[9];
+#pragma unroll
+      for (int i = 0; i < 9; i++) G[i] = g[3 + i];
+      double ub[3];
+#pragma unroll
+      for (int c = 0; c < 3; c++) {
+        u[c] = pnt[c] - g[c];
+        ub[c] = b[c] - g[c];
+      }
+      if (fresh) bary64_d(g, u[0], u[1], u[2], la);
+      bary64_d(g, ub[0], ub[1], ub[2], lb);
+      kx = exit_face64(la, lb, entry, smin);
+#pragma unroll
+      for (int c = 0; c < 3; c++) {   // the exit face's gradient, G_0 = -(G_1 + G_2 + G_3)
+        gk[c] = kx == 1 ? G[c] : kx == 2 ? G[3 + c] : G[6 + c];
+        if (kx == 0) gk[c] = -((G[c] + G[3 + c]) + G[6 + c]);
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < 3; c++) q[c] = kx < 0 ? b[c] : fma(smin, b[c] - pnt[c], pnt[c]);
+    if (kx >= 0) Sq = fma(smin, 1.0 - S, S);
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+      const int i = (c + 1) % 3, j = (c + 2) % 3;
+      const double di = q[i] - pnt[i], dj = q[j] - pnt[j];
+      gq[c] = fma(wt[3 + i], u[j], fma(-wt[3 + j], u[i], wt[c]));
+      gp[c] = fma(di, wt[3 + j], fma(-dj, wt[3 + i], -gq[c]));
+    }
+    if (on_face) {   // with the piece before, moved onto the face between
+#pragma unroll
+      for (int c = 0; c < 3; c++) gp[c] += gm[c];
+      double t[3];
+      onto_face(gp, gf, w, rf, t);
+#pragma unroll
+      for (int c = 0; c < 3; c++) {
+        ca[c] += t[c];
+        cw[c] = fma(S, t[c], cw[c]);
+      }
+    } else {
+#pragma unroll
+      for (int c = 0; c < 3; c++) ca[c] += gp[c];
+    }
+    // what the piece ends at: b (0), a face it crosses (1), a wall it reflects
+    // from (2), the point where the particle froze or was absorbed (3)
+    int end = 0;
+    int32_t nbt = 0;
+    if (kx >= 0) {
+      end = 3;
+      rf = 1.0 / tet_dot(gk, w);
+      nc++;
+      if (nc <= A.max_cross) {
+        nbt = kx == 0 ? nbv.x : kx == 1 ? nbv.y : kx == 2 ? nbv.z : nbv.w;
+        if (nbt >= 0) {
+          if (idx_in(nbt, A.nt, A.stats)) end = 1;
+        } else if (nbt >= -6 && A.wall_mode == FEMPIC_WALL_REFLECT) {
+          end = 2;
+        }
+      }
+      if (end == 1) {
+#pragma unroll
+        for (int c = 0; c < 3; c++) gm[c] = gq[c];
+      } else {
+        double t[3];
+        onto_face(gq, gk, w, rf, t);
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+          ca[c] += t[c];
+          cw[c] = fma(Sq, t[c], cw[c]);
+        }
       }
     } else {
 #pragma unroll
       for (int c = 0; c < 3; c++) {
-        ga[c] += ca[c];
-        gw[c] += cwv[c];
+        ca[c] += gq[c];
+        cw[c] += gq[c];
       }
     }
-    if (kx < 0) break;
+    if (end != 1) {   // the run is over
+      if (refl > 1) {
+        double c6[6], g6[6];
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+          c6[c] = ca[c];
+          c6[3 + c] = cw[c];
+          g6[c] = ga[c];
+          g6[3 + c] = gw[c];
+        }
+        dep_through(J, W, c6, g6);
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+          ga[c] = g6[c];
+          gw[c] = g6[3 + c];
+        }
+      } else {
+        if (refl) dep_unreflect(W, ca, cw, ca, cw);
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+          ga[c] += ca[c];
+          gw[c] += cw[c];
+        }
+      }
+    }
+    if (end == 0 || end == 3) {
+#pragma unroll
+      for (int c = 0; c < 3; c++) {
+        Q.a[c][at] = ga[c];
+        Q.b[c][at] = gw[c];
+      }
+      at = -1;
+      continue;
+    }
     double lp[4];
 #pragma unroll
     for (int i = 0; i < 4; i++) lp[i] = (i == kx) ? 0.0 : fma(smin, lb[i] - la[i], la[i]);
-    nc++;
-    if (nc > A.max_cross) break;   // frozen at q: the deposit ended there
-    const int4 nbv = ldg_int4(&A.nb[T]);
-    const int32_t nbt = kx == 0 ? nbv.x : kx == 1 ? nbv.y : kx == 2 ? nbv.z : nbv.w;
-    if (nbt >= 0 && !idx_in(nbt, A.nt, A.stats)) break;
-    if (nbt >= 0) {
-      const int4 o4 = ldg_int4(&A.tn[T]), n4 = ldg_int4(&A.tn[nbt]);
+    if (end == 1) {
+      const int4 n4 = ldg_int4(&A.tn[nbt]);
       const int32_t on[4] = {o4.x, o4.y, o4.z, o4.w}, nn[4] = {n4.x, n4.y, n4.z, n4.w};
-      int ent = 0;
 #pragma unroll
       for (int i2 = 0; i2 < 4; i2++) {
-        int hit = -1;
-#pragma unroll
-        for (int i = 0; i < 4; i++)
-          if (on[i] == nn[i2]) hit = i;
         double val = 0.0;
+        bool hit = false;
 #pragma unroll
         for (int i = 0; i < 4; i++)
-          if (i == hit) val = lp[i];
+          if (on[i] == nn[i2]) {
+            val = lp[i];
+            hit = true;
+          }
         la[i2] = val;
-        if (hit < 0) ent = i2;
+        if (!hit) entry = i2;
       }
 #pragma unroll
       for (int c = 0; c < 3; c++) {
-        gprev[c] = G[kx][c];
+        gf[c] = gk[c];
         pnt[c] = q[c];
       }
-      Sprev = Sq;
       S = Sq;
       on_face = true;
       T = nbt;
-      entry = ent;
-    } else if (nbt <= -1 && nbt >= -6 && A.wall_mode == FEMPIC_WALL_REFLECT) {
-      // new run a0' = q, w' = M (1 - Sq) w: its Jacobian with respect to this run
+    } else {
       const int code = -1 - nbt, ax = code >> 1, side = code & 1;
-      const double gfw = dot3d(G[kx], w);
-      double Jr[6][6];
-#pragma unroll 1
-      for (int i = 0; i < 3; i++)
-#pragma unroll 1
-        for (int j = 0; j < 3; j++) {
-          const double pij = (i == j ? 1.0 : 0.0) - w[i] * G[kx][j] / gfw;   // P = I - w G_f^T / (G_f . w)
-          const double mi = (i == ax) ? -1.0 : 1.0;
-          Jr[i][j] = pij;
-          Jr[i][3 + j] = Sq * pij;
-          Jr[3 + i][j] = mi * w[i] * G[kx][j] / gfw;
-          Jr[3 + i][3 + j] = mi * ((i == j ? 1.0 - Sq : 0.0) + Sq * w[i] * G[kx][j] / gfw);
-        }
-      if (refl) {
-        double Jn[6][6];
-#pragma unroll 1
-        for (int i = 0; i < 6; i++)
-#pragma unroll 1
-          for (int j = 0; j < 6; j++) {
-            double acc = 0.0;
-#pragma unroll 1
-            for (int k = 0; k < 6; k++) acc += Jr[i][k] * J[k][j];
-            Jn[i][j] = acc;
-          }
-#pragma unroll 1
-        for (int i = 0; i < 36; i++) J[i / 6][i % 6] = Jn[i / 6][i % 6];
-      } else {
-#pragma unroll 1
-        for (int i = 0; i < 36; i++) J[i / 6][i % 6] = Jr[i / 6][i % 6];
-        refl = true;
-      }
-      const double L = side ? A.hi[ax] : A.lo[ax];
-      b[ax] = 2.0 * L - b[ax];
+      if (refl) dep_fold(J, W, refl == 1);
+      refl++;
+      W.ax = ax;
+      W.S = Sq;
 #pragma unroll
       for (int c = 0; c < 3; c++) {
-        a0[c] = q[c];
+        W.w[c] = w[c];
+        W.gr[c] = gk[c] * rf;
+        if (c == ax) b[c] = 2.0 * (side ? A.hi[c] : A.lo[c]) - b[c];
         pnt[c] = q[c];
-        w[c] = b[c] - a0[c];
+        w[c] = b[c] - q[c];
+        ca[c] = cw[c] = 0.0;
       }
 #pragma unroll
       for (int i = 0; i < 4; i++) la[i] = lp[i];
       entry = kx;
       S = 0.0;
       on_face = false;
-    } else {
-      break;   // absorbed at q
     }
   }
 }
@@ -2990,13 +3084,7 @@ __device__ __noinline__ void dep_loss_grad(const AdjArgs& A, int32_t T0, const d
 // beta x (a - x0).  The others, about one in seven on the cavity, are walked
 // from a list in shared memory by the CTA's first threads, so that the FP64
 // walk runs with full warps: with every warp walking its own few, 300k
-// particles took 225 us, now 161.
-struct DepQueue {
-  int32_t n;
-  int32_t T[kThreads];
-  double a[3][kThreads], b[3][kThreads];   // start and end; after the walk d/da and d/dw
-};
-
+// particles took 225 us, from a list 161, and 95 by the walk above.
 __device__ __forceinline__ void dep_block(const AdjArgs& A, DepQueue& Q, bool want, int32_t T, const double a[3],
                                           const double b[3], double ga[3], double gw[3]) {
   int at = -1;
@@ -3024,17 +3112,7 @@ __device__ __forceinline__ void dep_block(const AdjArgs& A, DepQueue& Q, bool wa
     }
   }
   __syncthreads();
-  const int m = Q.n;
-  for (int i = threadIdx.x; i < m; i += kThreads) {
-    const double sa[3] = {Q.a[0][i], Q.a[1][i], Q.a[2][i]}, sb[3] = {Q.b[0][i], Q.b[1][i], Q.b[2][i]};
-    double da[3], dw[3];
-    dep_loss_grad(A, Q.T[i], sa, sb, da, dw);
-#pragma unroll
-    for (int k = 0; k < 3; k++) {
-      Q.a[k][i] = da[k];
-      Q.b[k][i] = dw[k];
-    }
-  }
+  if ((int)(threadIdx.x & ~31u) < Q.n) dep_walk(A, Q);   // a warp per 32 walks
   __syncthreads();
   if (at >= 0) {
 #pragma unroll
@@ -3272,7 +3350,7 @@ __device__ __forceinline__ void adjoint_particle(const AdjArgs& A, int64_t p, in
 }
 
 template <typename R, bool DEP>
-__global__ void __launch_bounds__(kThreads) k_push_adjoint(AdjArgs A) {
+__global__ void __launch_bounds__(kThreads, DEP ? 4 : 0) k_push_adjoint(AdjArgs A) {
   grid_wait();
   const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int lane = threadIdx.x & 31;
@@ -3305,7 +3383,7 @@ __global__ void __launch_bounds__(kThreads) k_push_adjoint(AdjArgs A) {
     }
   }
   if (DEP) {   // every thread goes through the CTA's list of walks
-    if (threadIdx.x == 0) Q->n = 0;
+    if (threadIdx.x == 0) Q->n = Q->next = 0;
     __syncthreads();
     adjoint_particle<DEP>(A, p, act ? T : 0, L, g, act, Q);
   } else if (act) {
