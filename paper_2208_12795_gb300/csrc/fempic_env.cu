@@ -1848,8 +1848,8 @@ __global__ void __launch_bounds__(384, 2) k_cross_df(PushArgs A, DsRule D) {
 // in FP64, so tets are those of the FP64 barycentrics.  Against barycentrics
 // of both ends and six edge products per particle (116 operations): 0.390 ->
 // 0.219 ms at 2M particles (the crossing pass 0.125 -> 0.067); four steps and
-// a sort of 6M electrons on 40^3 x 6 tets 6.88 -> 4.31 ms (now 4.04: the field
-// pass from tables, overlapped launches).  Rounding of the moment form against
+// a sort of 6M electrons on 40^3 x 6 tets 6.88 -> 4.31 ms (now 4.16: the field
+// pass from tables, overlapped launches, crossing pieces as edge values).  Rounding of the moment form against
 // 80-bit sums over such tets: 3e-16 of the edge values' norm (1.8e-15 for the
 // barycentric form).
 
@@ -1874,19 +1874,41 @@ __device__ __forceinline__ double recip_ge1(double w) {
   return fma(r, fma(e, e, e), r);
 }
 
-// Moment-form deposit of the straight piece a -> a + D inside tet T, u = a -
+// FP64 form's deposit slot of a tet: six moments of the segments that stay in
+// it, then the six edges' values of the pieces the crossing pass adds.
+constexpr int kSlot64 = 12;
+
+// Moment-form deposit of the straight segment a -> a + D inside tet T, u = a -
 // x0: q w D and q w (u x D) into the tet's slot (six adjacent FP64
 // reductions); k_tet_finalize64 turns them into the six edges' values.
 __device__ __forceinline__ void deposit64(const PushArgs& A, int32_t T, const double u[3], const double D[3],
                                           double qw) {
   if (!A.mom) return;   // deposits off
   const double d[3] = {qw * D[0], qw * D[1], qw * D[2]};
-  double* ms = A.mom + 6 * (int64_t)T;
+  double* ms = A.mom + kSlot64 * (int64_t)T;
 #pragma unroll
   for (int k = 0; k < 3; k++) {
     const int i = (k + 1) % 3, j = (k + 2) % 3;
     atomicAdd(ms + k, d[k]);
     atomicAdd(ms + 3 + k, fma(u[i], d[j], -(u[j] * d[i])));
+  }
+}
+
+// The same of a crossing particle's piece between barycentrics la and lb, as
+// edge values: the pieces of a path share their crossing points' barycentrics
+// (0 on the face), so its charge telescopes over them whatever the rounding of
+// the points.  In moment form (no fewer operations here, 48 B of slot less) a
+// 100-step run on the 48^3 cube conserved charge to 9e-15, so to 8e-16; four
+// steps and a sort of 6M electrons 4.04 -> 4.16 ms.
+__device__ __forceinline__ void deposit64_piece(const PushArgs& A, int32_t T, const double la[4], const double lb[4],
+                                                double qw) {
+  if (!A.mom) return;   // deposits off
+  const double l[4] = {qw * la[0], qw * la[1], qw * la[2], qw * la[3]};
+  double* es = A.mom + kSlot64 * (int64_t)T + 6;
+#pragma unroll
+  for (int e = 0; e < 6; e++) {
+    const int i = le0(e), j = le1(e);
+    atomicAdd(es + e, fma(l[i], lb[j], -(l[j] * lb[i])));
   }
 }
 
@@ -2162,22 +2184,16 @@ __device__ __forceinline__ int exit_face64(const double la[4], const double lb[4
 
 __device__ __forceinline__ bool cross64_advance(const PushArgs& A, CrossState64& c, bool fresh) {
   const double qw = A.sp.qw[c.s];
-  double u[3];   // piece start - x0 of this tet
   {
     const double* g = A.geom64 + 12 * (int64_t)c.T;
     const double x0[3] = {__ldg(g), __ldg(g + 1), __ldg(g + 2)};
-#pragma unroll
-    for (int k = 0; k < 3; k++) u[k] = c.a[k] - x0[k];
-    if (fresh) bary64_d(g, u[0], u[1], u[2], c.la);
+    if (fresh) bary64_d(g, c.a[0] - x0[0], c.a[1] - x0[1], c.a[2] - x0[2], c.la);
     bary64_d(g, c.b[0] - x0[0], c.b[1] - x0[1], c.b[2] - x0[2], c.lb);
   }
   double smin;
   const int kx = exit_face64(c.la, c.lb, c.entry, smin);
-  double D[3];
-#pragma unroll
-  for (int k = 0; k < 3; k++) D[k] = c.b[k] - c.a[k];
   if (kx < 0) {
-    deposit64(A, c.T, u, D, qw);
+    deposit64_piece(A, c.T, c.la, c.lb, qw);
 #pragma unroll
     for (int k = 0; k < 3; k++) c.a[k] = c.b[k];
     return true;
@@ -2186,12 +2202,8 @@ __device__ __forceinline__ bool cross64_advance(const PushArgs& A, CrossState64&
 #pragma unroll
   for (int i = 0; i < 4; i++) lp[i] = (i == kx) ? 0.0 : fma(smin, c.lb[i] - c.la[i], c.la[i]);
 #pragma unroll
-  for (int k = 0; k < 3; k++) {
-    const double q = fma(smin, D[k], c.a[k]);
-    D[k] = q - c.a[k];
-    c.a[k] = q;
-  }
-  deposit64(A, c.T, u, D, qw);
+  for (int k = 0; k < 3; k++) c.a[k] = fma(smin, c.b[k] - c.a[k], c.a[k]);
+  deposit64_piece(A, c.T, c.la, lp, qw);
   c.nc++;
   if (c.nc > A.max_cross) {
     c.st = FEMPIC_P_CAP;
@@ -2390,7 +2402,7 @@ __global__ void __launch_bounds__(kThreads) k_tet_finalize(TetFinalizeArgs A) {
 }
 
 // FP64 form, per tet: the same conversion in FP64 (the slots already hold
-// q w times the moments): with c_ij = G_i x G_j and G_0 = -(G_1 + G_2 + G_3),
+// q w times the moments), plus the crossing pass's edge values: with c_ij = G_i x G_j and G_0 = -(G_1 + G_2 + G_3),
 // three products M . c_12, M . c_13, M . c_23 give all six edges' moment
 // parts.  Slots are read and cleared once per deposit; tets without particles
 // stop at their zero slot.
@@ -2400,22 +2412,29 @@ __global__ void __launch_bounds__(kThreads) k_tet_finalize64(int64_t nt, const d
   grid_wait();
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= nt) return;
-  double2* m2 = reinterpret_cast<double2*>(mom + 6 * t);
+  double2* m2 = reinterpret_cast<double2*>(mom + kSlot64 * t);
   double2* o = reinterpret_cast<double2*>(out + 6 * t);
-  const double2 a = m2[0], b = m2[1], c = m2[2];
+  double2 v[6];
+  bool any = false;
+#pragma unroll
+  for (int k = 0; k < 6; k++) {
+    v[k] = m2[k];
+    any = any || v[k].x != 0.0 || v[k].y != 0.0;
+  }
   const double2 z2 = make_double2(0.0, 0.0);
-  if (a.x == 0.0 && a.y == 0.0 && b.x == 0.0 && b.y == 0.0 && c.x == 0.0 && c.y == 0.0) {
+  if (!any) {
     o[0] = o[1] = o[2] = z2;
     return;
   }
-  m2[0] = m2[1] = m2[2] = z2;
-  const double S[3] = {a.x, a.y, b.x}, M[3] = {b.y, c.x, c.y};
+#pragma unroll
+  for (int k = 0; k < 6; k++) m2[k] = z2;
+  const double S[3] = {v[0].x, v[0].y, v[1].x}, M[3] = {v[1].y, v[2].x, v[2].y};
   TetGeo G;
   ld_tet_geo(geom64, tgeo, t, G);
   const double m12 = tet_dot(G.c, M), m13 = tet_dot(G.c + 3, M), m23 = tet_dot(G.c + 6, M);
-  o[0] = make_double2(tet_dot(G.g, S) + (m12 + m13), tet_dot(G.g + 3, S) + (m23 - m12));
-  o[1] = make_double2(tet_dot(G.g + 6, S) - (m13 + m23), m12);
-  o[2] = make_double2(m13, m23);
+  o[0] = make_double2(tet_dot(G.g, S) + (m12 + m13) + v[3].x, tet_dot(G.g + 3, S) + (m23 - m12) + v[3].y);
+  o[1] = make_double2(tet_dot(G.g + 6, S) - (m13 + m23) + v[4].x, m12 + v[4].y);
+  o[2] = make_double2(m13 + v[5].x, m23 + v[5].y);
 }
 
 struct FinalizeArgs {
@@ -3674,7 +3693,7 @@ struct fempic_env {
   unsigned long long* dGq = nullptr;   // 24-bit form [dGq_species][nt][8]
   int32_t dGq_species = 0;
   float4* grad32 = nullptr;            // mixed forms: FP32 grad lambda_1..3, [nt][3]
-  double* mom = nullptr;               // moment slots: contract form [dGq_species][nt][6], FP64 form [nt][6]
+  double* mom = nullptr;               // moment slots: contract form [dGq_species][nt][6], FP64 form [nt][kSlot64]
   float* momlo = nullptr;              // their low FP32 parts [dGq_species][nt][8]
   float4* tetout = nullptr;            // contract and FP64 forms: per-tet edge values of a step, 48 B per tet
   double* Gcum = nullptr;
@@ -3891,8 +3910,8 @@ static int upload(fempic_env* e) {
     k_tet_geo<<<(unsigned)((nt + kThreads - 1) / kThreads), kThreads>>>(nt, e->geom64, e->tgeo);
     FEMPIC_CUDA(cudaGetLastError());
     FEMPIC_CUDA(dalloc(reinterpret_cast<double**>(&e->field), 10 * nt));
-    FEMPIC_CUDA(dalloc(&e->mom, 6 * nt));
-    FEMPIC_CUDA(cudaMemset(e->mom, 0, 6 * nt * sizeof(double)));
+    FEMPIC_CUDA(dalloc(&e->mom, kSlot64 * nt));
+    FEMPIC_CUDA(cudaMemset(e->mom, 0, kSlot64 * nt * sizeof(double)));
     FEMPIC_CUDA(dalloc(&e->tetout, 3 * nt));
   }
   FEMPIC_CUDA(dalloc(&e->Gcum, m.ne));
@@ -4512,7 +4531,7 @@ extern "C" int fempic_reset_deposit(fempic_env* env, void* stream) {
   const size_t nslot = (size_t)env->dGq_species * env->h.nt * 8;
   if (env->dGq) FEMPIC_CUDA(cudaMemsetAsync(env->dGq, 0, nslot * sizeof(unsigned long long), st));
   if (env->opt.precision == FEMPIC_FP64) {
-    FEMPIC_CUDA(cudaMemsetAsync(env->mom, 0, (size_t)env->h.nt * 6 * sizeof(double), st));
+    FEMPIC_CUDA(cudaMemsetAsync(env->mom, 0, (size_t)env->h.nt * kSlot64 * sizeof(double), st));
   } else if (env->mom) {
     FEMPIC_CUDA(cudaMemsetAsync(env->mom, 0, (size_t)env->dGq_species * env->h.nt * 6 * sizeof(double), st));
     FEMPIC_CUDA(cudaMemsetAsync(env->momlo, 0, nslot * sizeof(float), st));
