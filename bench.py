@@ -53,7 +53,8 @@ NOMINAL_HBM_GBS = 7900.0   # GB300 HBM3e nominal, for context next to the measur
 PROFILE_SUMMARY = os.path.join(ROOT, "profiles", "push_mixed_cube48_10M.txt")
 FP64_SUMMARY = os.path.join(ROOT, "profiles", "fp64_ops_cube48_4M.txt")
 KERNEL_SOURCES = [os.path.join(ROOT, "paper_2208_12795_gb300", "csrc", f)
-                  for f in ("fempic_env.cu", "fempic_internal.h")]
+                  for f in ("fempic_env.cu", "fempic_internal.h", "fempic_ds_rule.cuh", "fempic_tetgeo.cuh",
+                            "fempic_launch.cuh")]
 
 
 def parse():
@@ -167,18 +168,18 @@ def profiled_traffic(n_p):
 
 
 def issue_roofline(n_p, t_launch_s, sm_mhz):
-    """Issue-slot roofline of the staged common path k_push_mixed_tma: its
+    """Issue-slot roofline of the staged common path k_push_mixed: its
     warp instructions per launch (ncu count per particle, scaled to n_p) over
     the launch time, against 4 warp instructions per clock on each of the
     GPU's SMs at the sampled SM clock."""
-    ipp = _profile_value("tma_warp_instructions_per_particle")
+    ipp = _profile_value("push_warp_instructions_per_particle")
     if ipp is None or t_launch_s <= 0:
         return None
     import torch
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     peak = sms * 4 * sm_mhz * 1e6
     achieved = ipp * n_p / t_launch_s
-    return {"kernel": "k_push_mixed_tma", "bound": "issue", "achieved": achieved, "peak": peak,
+    return {"kernel": "k_push_mixed", "bound": "issue", "achieved": achieved, "peak": peak,
             "unit": "warp instructions/s", "frac": achieved / peak, "warp_instructions_per_launch": ipp * n_p,
             "avg_launch_ms": t_launch_s * 1e3,
             "peak_source": f"{sms} SMs x 4 schedulers x {sm_mhz:.0f} MHz (median SM clock sampled in the timed region)"}
@@ -687,8 +688,8 @@ def run_ours(args):
             "algorithmic_bytes_per_step": b_ds,
             "hbm_frac_of_step": b_ds / t_step / 1e9 / measured_peaks()[0],
             "what": f"fempic_push_step_downshift ({'FP64' if prec == 0 else 'contract mixed form: FP32 rule, samples and history'}): "
-                    "envelope samples + M/L velocity rule + AB4 (k_ds_pre), the env's step under a zero field "
-                    "for tracking/deposit, wall mirrors of the history (k_ds_post); re-sorted with the history "
+                    "one pass for the envelope samples, M/L velocity rule, AB4 and the env's inside test and "
+                    "deposit, then its crossing pass, which mirrors the history at walls; re-sorted with the history "
                     "carried along (sort_ms_per_step: the particle sort; the plane gather is in the step time)"}
         ds.close()
         env_d.close()
@@ -942,12 +943,12 @@ def report(args, world, n_p, out, cpu, adj=None):
             "form": "mixed",
             "particles_per_gpu": n_p,
             "n_tets": m["counts"][3],
-            "sort_every": 4 * args.sort_every,
+            "sort_every": args.sort_every,
             "l2": f"inputs larger than L2 (particle SoA {n_p * 41 / 1e6:.0f} MB per GPU per step)",
             "parallelism": f"particles sharded by tet range over {world} GPUs, dG all-reduced" if world > 1 else "1 GPU",
         },
         "roofline": {
-            "kernel": "push step group: k_push_mixed_tma (+ k_push_mixed ragged tail) + k_cross_df",
+            "kernel": "push step group: k_push_mixed + k_cross_df",
             "bound": "hbm",
             "achieved": achieved,
             "peak": peak,
