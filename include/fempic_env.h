@@ -188,9 +188,10 @@ int fempic_push_step(fempic_env* env, const fempic_particles* p, const fempic_en
 /* The step of fempic_push_step from one particle set into another: the new
  * state goes to `out`, `in` is left as it was (a gradient window keeps every
  * state of a segment; the paper has no counterpart).  Every array of out is
- * written.  in and out have the same n, velocity dtype and species table and
- * must not overlap; n_cross may be NULL in both (else in both).  Errors: as
- * fempic_push_step, and EINVAL for sets that differ or overlap. */
+ * written.  in and out have the same n, velocity dtype and species table
+ * (ranges, q, m, w), and no array of out shares memory with one of in; n_cross
+ * may be NULL in both (else in neither).  Errors: as fempic_push_step, and
+ * EINVAL for sets that differ or overlap. */
 int fempic_push_step_to(fempic_env* env, const fempic_particles* in, const fempic_particles* out,
                         const fempic_envelope* envl, double omega0, double t, double dt, void* stream);
 

@@ -4346,6 +4346,39 @@ extern "C" int fempic_push_step(fempic_env* env, const fempic_particles* p, cons
   return push_step_impl(env, p, p, H, omega0, t, dt, stream);
 }
 
+// Whether any array of one set shares memory with any array of the other (a
+// step from one set into the other would then read what it has written).
+static bool sets_overlap(const fempic_particles* a, const fempic_particles* b, size_t vbytes) {
+  struct Range {
+    uintptr_t at;
+    size_t bytes;
+  };
+  auto ranges = [vbytes](const fempic_particles* p, Range r[9]) {
+    const void* at[9] = {p->x, p->y, p->z, p->vx, p->vy, p->vz, p->tet, p->status, p->n_cross};
+    const size_t size[9] = {8, 8, 8, vbytes, vbytes, vbytes, 4, 1, 4};
+    for (int k = 0; k < 9; k++) r[k] = Range{(uintptr_t)at[k], at[k] ? size[k] * (size_t)p->n : 0};
+  };
+  Range ra[9], rb[9];
+  ranges(a, ra);
+  ranges(b, rb);
+  for (const Range& u : ra)
+    for (const Range& v : rb)
+      if (u.at < v.at + v.bytes && v.at < u.at + u.bytes) return true;
+  return false;
+}
+
+// Whether two species tables hold the same ranges, charges, masses and weights
+// (a NaN equals a NaN).
+static bool species_equal(const fempic_particles* a, const fempic_particles* b) {
+  auto same = [](double u, double v) { return u == v || (std::isnan(u) && std::isnan(v)); };
+  if (a->n_species != b->n_species) return false;
+  for (int s = 0; s <= a->n_species; s++)
+    if (a->species_begin[s] != b->species_begin[s]) return false;
+  for (int s = 0; s < a->n_species; s++)
+    if (!same(a->q[s], b->q[s]) || !same(a->m[s], b->m[s]) || !same(a->w[s], b->w[s])) return false;
+  return true;
+}
+
 extern "C" int fempic_push_step_to(fempic_env* env, const fempic_particles* in, const fempic_particles* out,
                                    const fempic_envelope* envl, double omega0, double t, double dt, void* stream) {
   if (!env || !envl) return fail(FEMPIC_EINVAL, "push_step_to: NULL env/envelope");
@@ -4360,9 +4393,8 @@ extern "C" int fempic_push_step_to(fempic_env* env, const fempic_particles* in, 
   if (rc) return rc;
   rc = fill_species(out, 1.0, &so);
   if (rc) return rc;
-  for (int s = 0; s <= in->n_species; s++)
-    if (si.begin[s] != so.begin[s]) return fail(FEMPIC_EINVAL, "push_step_to: species tables differ");
-  if (in->n > 0 && (in->x == out->x || in->tet == out->tet || in->vx == out->vx || in->status == out->status))
+  if (!species_equal(in, out)) return fail(FEMPIC_EINVAL, "push_step_to: species tables differ");
+  if (sets_overlap(in, out, env->opt.precision == FEMPIC_FP64 ? 8 : 4))
     return fail(FEMPIC_EINVAL, "push_step_to: in and out overlap");
   HostLevels H{};
   H.nl = 1;
