@@ -94,8 +94,7 @@ __global__ void __launch_bounds__(kThreads) k_ds_field64(int64_t nt, const doubl
                                                          const double* __restrict__ tgeo,
                                                          const int32_t* __restrict__ te,
                                                          const int32_t* __restrict__ tf,
-                                                         const double2* __restrict__ e,
-                                                         const double2* __restrict__ b, int64_t ne, int64_t nf,
+                                                         const double2* e, const double2* b, int64_t ne, int64_t nf,
                                                          unsigned long long* stats, double amp,
                                                          double* __restrict__ coef) {
   grid_wait();
@@ -201,7 +200,7 @@ __global__ void __launch_bounds__(kThreads) k_ds_field32(int64_t nt, const doubl
                                                          const double* __restrict__ dgeo,
                                                          const int32_t* __restrict__ te,
                                                          const int32_t* __restrict__ tf,
-                                                         const float2* __restrict__ e, const float2* __restrict__ b,
+                                                         const float2* e, const float2* b,
                                                          int64_t ne, int64_t nf, unsigned long long* stats,
                                                          double amp, float* __restrict__ coef32) {
   grid_wait();

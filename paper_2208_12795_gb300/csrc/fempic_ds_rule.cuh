@@ -113,7 +113,7 @@ __device__ __forceinline__ bool ds_rule32(const DsRule& A, int64_t p, int32_t T,
   float c[kDsCoef32];
 #pragma unroll
   for (int i = 0; i < kDsCoef32 / 4; i++) {
-    const float4 v = __ldg(C + i);
+    const float4 v = C[i];
     c[4 * i] = v.x;
     c[4 * i + 1] = v.y;
     c[4 * i + 2] = v.z;
@@ -195,7 +195,7 @@ __device__ __forceinline__ bool ds_rule(const DsRule& A, int64_t p, int32_t T, i
     double q[10];
 #pragma unroll
     for (int i = 0; i < 5; i++) {
-      const double2 v = __ldg(C + 5 * part + i);
+      const double2 v = C[5 * part + i];
       q[2 * i] = v.x;
       q[2 * i + 1] = v.y;
     }
@@ -206,7 +206,7 @@ __device__ __forceinline__ bool ds_rule(const DsRule& A, int64_t p, int32_t T, i
       cur[6 + 3 * part + a] = fma(q[9], d[a], q[6 + a]);
     }
   }
-  const bool bad = __ldg(reinterpret_cast<const double*>(C) + 20) != 0.0;
+  const bool bad = reinterpret_cast<const double*>(C)[20] != 0.0;
   ds_fill(A, v0, cur, h);
   const double* S[3] = {cur, h.f1, h.f2};
   const double* V[3] = {v0, h.vh[0], h.vh[1]};

@@ -881,7 +881,7 @@ __device__ __forceinline__ void mixed_particle(const PushArgs& A, int64_t p, int
   const float kq = A.sp.kq32[s];
   const float4* F = static_cast<const float4*>(A.field) + 3 * (int64_t)T;
   const Geo32 G = ld_geo(A.tetrec, T);
-  const float4 f0 = __ldg(F), f1 = __ldg(F + 1), f2 = __ldg(F + 2);
+  const float4 f0 = F[0], f1 = F[1], f2 = F[2];
   FF dd[3];
   float d[3];
   dpos(G, ax, ay, az, dd, d);
@@ -2032,7 +2032,7 @@ __global__ void __launch_bounds__(kThreads) k_push_fp64(PushArgs A, int64_t ntil
       const double kq = A.sp.kq[s];
       const Geo32 G = ld_geo(A.tetrec, T);   // x0 exact; FP32 gradients and error bound for the inside test
       const double2* F = reinterpret_cast<const double2*>(static_cast<const double*>(A.field) + 10 * (int64_t)T);
-      const double2 f0 = __ldg(F), f1 = __ldg(F + 1), f2 = __ldg(F + 2), f3 = __ldg(F + 3), f4 = __ldg(F + 4);
+      const double2 f0 = F[0], f1 = F[1], f2 = F[2], f3 = F[3], f4 = F[4];
       const double d[3] = {a[0] - G.x0[0], a[1] - G.x0[1], a[2] - G.x0[2]};
       // (b)+(c) gather with the carrier already restored per tet
       const double Wx = f1.y, Wy = f2.x, Wz = f2.y, beta = f4.y;
@@ -2512,7 +2512,7 @@ __global__ void __launch_bounds__(kThreads) k_deposit_finalize(FinalizeArgs A) {
 
 // G_cum += dG for a step deposit reduced outside the library (a sharded run
 // all-reduces each rank's dG), then the requested outputs.
-__global__ void __launch_bounds__(kThreads) k_accumulate(int64_t ne, const double* __restrict__ dG,
+__global__ void __launch_bounds__(kThreads) k_accumulate(int64_t ne, const double* dG,
                                                          double* __restrict__ Gcum, double* Gcum_out,
                                                          double2* Genv_out, double c, double s) {
   grid_wait();
@@ -3198,7 +3198,7 @@ __device__ __forceinline__ void adjoint_particle(const AdjArgs& A, int64_t p, in
   {
     const float4* F = A.field32 + 3 * (int64_t)T;
     const Geo32 G = ld_geo(A.tetrec, T);
-    const float4 f0 = __ldg(F), f1 = __ldg(F + 1), f2 = __ldg(F + 2);
+    const float4 f0 = F[0], f1 = F[1], f2 = F[2];
     FF dd[3];
     float d32[3];
     dpos(G, L.r[0], L.r[1], L.r[2], dd, d32);   // the forward step's sequence
@@ -3315,7 +3315,7 @@ __device__ __forceinline__ void adjoint_particle(const AdjArgs& A, int64_t p, in
   double *vbx = static_cast<double*>(A.vbx), *vby = static_cast<double*>(A.vby), *vbz = static_cast<double*>(A.vbz);
   const double* G = A.geom64 + 12 * (int64_t)T;
   const double2* F = reinterpret_cast<const double2*>(A.field64 + 10 * (int64_t)T);
-  const double2 f0 = __ldg(F), f1 = __ldg(F + 1), f2 = __ldg(F + 2), f3 = __ldg(F + 3), f4 = __ldg(F + 4);
+  const double2 f0 = F[0], f1 = F[1], f2 = F[2], f3 = F[3], f4 = F[4];
   const double* a = L.r;
   const D3 d = {a[0] - G[0], a[1] - G[1], a[2] - G[2]};
   const D3 E0 = {f0.x, f0.y, f1.x}, W = {f1.y, f2.x, f2.y}, B0 = {f3.x, f3.y, f4.x};
@@ -3586,7 +3586,7 @@ template <typename R>   // type of the per-tet terms: FP64 form double, mixed fo
 __global__ void __launch_bounds__(kThreads) k_dof_grad(int64_t ne, int64_t nf, const int32_t* __restrict__ estart,
                                                        const int32_t* __restrict__ eslot,
                                                        const int32_t* __restrict__ fslot,
-                                                       const R* __restrict__ tadj, double cre, double cim,
+                                                       const R* tadj, double cre, double cim,
                                                        double* __restrict__ egrad, double* __restrict__ bgrad,
                                                        int64_t nt, unsigned long long* stats) {
   grid_wait();

@@ -2,7 +2,10 @@
 // be set up while the one before it still runs (programmatic stream
 // serialization) and waits for that one's end before its first access to
 // memory.  What follows a step (another library's kernel, a copy, an event)
-// is ordered as after any kernel.
+// is ordered as after any kernel.  A kernel is resident while the ones before it
+// still write, so what they write (fields, coefficients, per-tet terms, a
+// caller's DoFs) is read with plain loads; the non-coherent path (__ldg, const
+// __restrict__) is for the tables that are fixed once per mesh.
 #pragma once
 #include <cuda_runtime.h>
 
