@@ -267,21 +267,24 @@ int fempic_stats(fempic_env* env, int64_t* out4, void* stream);
  * has no error path).  Synchronizes `stream`, then sets *n_bad to the number
  * of particles those steps froze (status CAP, ABSORBED, NONFINITE or LOST)
  * and returns FEMPIC_OK, or FEMPIC_EINCOMPLETE when, in one of those steps, a
- * CTA of the staged mixed push gave up its bounded wait: the particles of its
- * tiles were then not advanced and their deposit is missing, so the step must
- * be redone from a saved state.
+ * CTA of the staged mixed push gave up a wait (only fempic_debug_stall makes
+ * one wait): the particles of its tiles were then not advanced and their
+ * deposit is missing, so the step must be redone from a saved state.
  * In the debug build it returns FEMPIC_EBOUNDS when a mesh-table index out of
  * range was skipped (fempic_debug_set_table; the downshifted step's own
  * tables, fempic_downshift_debug_set_table, count here too).  fempic_stats keeps the
  * cumulative counters.  Errors: EINVAL, ECUDA, EINCOMPLETE, EBOUNDS. */
 int fempic_error_count(fempic_env* env, int64_t* n_bad, void* stream);
 
-/* Test support for the bounded waits (no counterpart in the paper): in the
- * next push step only, CTA `cta` of the staged mixed push kernel (if that
- * launch has such a CTA) waits, its first tile's copies in flight, on a
- * barrier that nothing completes, limited to limit_ns (1e3 .. 1e9).  The wait
- * runs out, the CTA waits for its copies and stops, and fempic_error_count
- * reports FEMPIC_EINCOMPLETE: the give-up path runs without any device fault.
+/* Test support for FEMPIC_EINCOMPLETE (no counterpart in the paper): in the
+ * next fempic_push_step or fempic_push_step3 of a mixed form, and in that one
+ * only, CTA `cta` of the staged push kernel (if that launch has such a CTA)
+ * waits, its first tile's copies in flight, on a barrier that nothing
+ * completes, limited to limit_ns (1e3 .. 1e9).  The wait runs out, the CTA
+ * waits for its copies and stops, and fempic_error_count reports
+ * FEMPIC_EINCOMPLETE: the give-up path runs without any device fault.  Steps
+ * into another set and downshifted steps have no such kernel and leave the
+ * call in force; without it no step waits in software.
  * Host only.  Errors: EINVAL. */
 int fempic_debug_stall(fempic_env* env, int32_t cta, int64_t limit_ns);
 

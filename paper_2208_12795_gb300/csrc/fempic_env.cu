@@ -4254,9 +4254,9 @@ static int push_particles(fempic_env* env, const fempic_particles* in, const fem
   A.xrec = env->xrec;
   A.xrec64 = env->xrec64;
   A.xcount = env->xcount;
-  A.wait_ns = env->stall_cta >= 0 ? env->stall_ns : kWaitLimitNs;
-  A.stall_cta = env->stall_cta;
-  env->stall_cta = -1;   // one launch only
+  A.wait_ns = env->stall_ns;
+  A.stall_cta = mixed && !ds && !into ? env->stall_cta : -1;
+  if (A.stall_cta >= 0) env->stall_cta = -1;   // one launch only; a step that has no such kernel leaves it armed
   {
     LaunchTimer lt(env, st, FEMPIC_K_PUSH);
     const unsigned grid = (unsigned)regions;
