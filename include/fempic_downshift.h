@@ -68,9 +68,17 @@ typedef struct {
 
 /* Build the gather tables (FP64 barycentric geometry, tet edges and faces)
  * from the same mesh description the env was created from, upload them to
- * the current device and allocate the per-tet coefficient buffer (22 f64 per
- * tet).  Errors: EINVAL, EMESH, ENOMEM, ECUDA.  Synchronizes the device. */
+ * the current device and make the FP64 form's per-tet tables (32 f64 per tet).
+ * The mixed forms' (352 bytes per tet) are made by the first step on an env of
+ * such a form.  Errors: EINVAL, EMESH, ENOMEM, ECUDA.  Synchronizes the
+ * device. */
 int fempic_downshift_create(const fempic_mesh_desc* mesh, fempic_downshift** out);
+
+/* The same for envs of one precision form (fempic_options.precision): the
+ * FP64 form's tables are left out where the form is a mixed one.  A step on an
+ * env of the other kind still works and makes what it needs first.  Errors: as
+ * fempic_downshift_create, and EINVAL for an unknown form. */
+int fempic_downshift_create_form(const fempic_mesh_desc* mesh, int32_t precision, fempic_downshift** out);
 
 /* Host only, no GPU work: the weights of the step [t, t + dt] at carrier
  * frequency omega0, w_out[24] = {M^r[3], M^i[3], L^r[3][3], L^i[3][3]}

@@ -40,7 +40,7 @@ EXPORTS = ("fempic_env_create", "fempic_env_query", "fempic_locate", "fempic_pus
            "fempic_adjoint_unpermute", "fempic_sort_noalloc", "fempic_profile_enable", "fempic_profile_read",
            "fempic_measure_fp64_rate", "fempic_last_error", "fempic_env_destroy")
 # Every function declared in include/fempic_downshift.h.
-DS_EXPORTS = ("fempic_downshift_create", "fempic_downshift_weights", "fempic_push_step_downshift",
+DS_EXPORTS = ("fempic_downshift_create", "fempic_downshift_create_form", "fempic_downshift_weights", "fempic_push_step_downshift",
               "fempic_downshift_permute", "fempic_downshift_last_error", "fempic_downshift_destroy",
               "fempic_downshift_debug_set_table")
 FEMPIC_DS_VH, FEMPIC_DS_F, FEMPIC_DS_VN, FEMPIC_DS_U, FEMPIC_DS_PLANES = 0, 9, 33, 36, 39
@@ -143,6 +143,7 @@ def load(path: str = LIB_PATH):
         lib.fempic_profile_read.argtypes = [C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p]
         lib.fempic_measure_fp64_rate.argtypes = [C.c_void_p, C.c_void_p]
         lib.fempic_downshift_create.argtypes = [P(fempic_mesh_desc), P(C.c_void_p)]
+        lib.fempic_downshift_create_form.argtypes = [P(fempic_mesh_desc), C.c_int32, P(C.c_void_p)]
         lib.fempic_downshift_weights.argtypes = [C.c_double, C.c_double, C.c_double, C.c_void_p]
         lib.fempic_push_step_downshift.argtypes = [C.c_void_p, C.c_void_p, P(fempic_particles),
                                                    P(fempic_downshift_history), P(fempic_envelope), C.c_double,
@@ -154,7 +155,7 @@ def load(path: str = LIB_PATH):
         lib.fempic_downshift_destroy.argtypes = [C.c_void_p]
         lib.fempic_downshift_destroy.restype = None
         lib.fempic_downshift_debug_set_table.argtypes = [C.c_void_p, C.c_int32, C.c_int64, C.c_int32]
-        for name in ("fempic_downshift_create", "fempic_downshift_weights", "fempic_push_step_downshift",
+        for name in ("fempic_downshift_create", "fempic_downshift_create_form", "fempic_downshift_weights", "fempic_push_step_downshift",
                      "fempic_downshift_permute", "fempic_downshift_debug_set_table"):
             getattr(lib, name).restype = C.c_int
         lib.fempic_last_error.restype = C.c_char_p
@@ -335,6 +336,13 @@ def check_ds(rc: int, what: str):
 def fempic_downshift_create(mesh: fempic_mesh_desc) -> int:
     h = C.c_void_p()
     check_ds(load().fempic_downshift_create(C.byref(mesh), C.byref(h)), "fempic_downshift_create")
+    return h.value
+
+
+def fempic_downshift_create_form(mesh: fempic_mesh_desc, precision: int) -> int:
+    h = C.c_void_p()
+    check_ds(load().fempic_downshift_create_form(C.byref(mesh), int(precision), C.byref(h)),
+             "fempic_downshift_create_form")
     return h.value
 
 

@@ -339,12 +339,12 @@ unsigned blocks_for(int64_t n) { return (unsigned)((n + kThreads - 1) / kThreads
 struct fempic_downshift {
   int64_t nn = 0, ne = 0, nf = 0, nt = 0;
   double* geom = nullptr;
-  double* tgeo = nullptr;       // [nt][kTetGeo] products of the gradients (fempic_tetgeo.cuh)
+  double* tgeo = nullptr;       // FP64 form: [nt][kTetGeo] products of the gradients (fempic_tetgeo.cuh)
   int32_t* te = nullptr;
   int32_t* tf = nullptr;
   double* coef = nullptr;       // FP64 form: [nt][kDsCoef64]
-  double* dgeo = nullptr;       // mixed forms: [nt][kDsGeo] geometry factors (allocated on first use)
-  float* coef32 = nullptr;      // mixed forms: [nt][kDsCoef32] (allocated on first use)
+  double* dgeo = nullptr;       // mixed forms: [nt][kDsGeo] geometry factors
+  float* coef32 = nullptr;      // mixed forms: [nt][kDsCoef32]
 };
 
 static void free_ds(fempic_downshift* d) {
@@ -416,12 +416,68 @@ extern "C" int fempic_downshift_debug_set_table(fempic_downshift* ds, int32_t ta
   return FEMPIC_OK;
 }
 
-extern "C" int fempic_downshift_create(const fempic_mesh_desc* mesh, fempic_downshift** out) {
-  if (!mesh || !out) return fail(FEMPIC_EINVAL, "downshift_create: NULL argument");
+extern "C" int fempic_downshift_weights(double t, double dt, double omega0, double* w_out) {
+  if (!w_out) return fail(FEMPIC_EINVAL, "downshift_weights: NULL output");
+  if (!std::isfinite(t) || !std::isfinite(dt) || !std::isfinite(omega0) || !(dt > 0.0))
+    return fail(FEMPIC_EINVAL, "downshift_weights: non-finite scalar or dt <= 0");
+  compute_weights(t, dt, omega0, w_out);
+  return FEMPIC_OK;
+}
+
+// A table of the mesh's geometry, filled by `fill` on a stream of its own that
+// is waited for: later steps may be on any stream, and a first step that is
+// being captured must not defer the table to its replay.
+template <typename F>
+static cudaError_t fill_table(F fill) {
+  cudaStream_t own = nullptr;
+  cudaError_t rc = cudaStreamCreateWithFlags(&own, cudaStreamNonBlocking);
+  if (rc != cudaSuccess) return rc;
+  fill(own);
+  rc = cudaGetLastError();
+  if (rc == cudaSuccess) rc = cudaStreamSynchronize(own);
+  cudaStreamDestroy(own);
+  return rc;
+}
+
+// A form's coefficients and geometry products, when the handle is made for that
+// form (FP64) or on first use: nothing is held for a form that never steps.
+// The handle is left unchanged by an error.
+template <typename C>
+static int make_tables(fempic_downshift* ds, int per_tet, int coef_per_tet, double** geo, C** coef,
+                       void (*kernel)(int64_t, const double*, double*)) {
+  double* g = nullptr;
+  C* c = nullptr;
+  if (cudaMalloc(&g, sizeof(double) * per_tet * (size_t)ds->nt) != cudaSuccess ||
+      cudaMalloc(&c, sizeof(C) * coef_per_tet * (size_t)ds->nt) != cudaSuccess) {
+    cudaGetLastError();
+    cudaFree(g);
+    return fail(FEMPIC_ENOMEM, "downshift: device allocation");
+  }
+  const cudaError_t rc =
+      fill_table([&](cudaStream_t st) { kernel<<<blocks_for(ds->nt), kThreads, 0, st>>>(ds->nt, ds->geom, g); });
+  if (rc != cudaSuccess) {
+    cudaFree(g);
+    cudaFree(c);
+  }
+  DS_CUDA(rc);
+  *geo = g;
+  *coef = c;
+  return FEMPIC_OK;
+}
+
+static int make_form_tables(fempic_downshift* ds, bool mixed) {
+  if (mixed)
+    return ds->coef32 ? FEMPIC_OK
+                      : make_tables(ds, kDsGeo, fempic::kDsCoef32, &ds->dgeo, &ds->coef32, k_ds_geo32);
+  return ds->coef ? FEMPIC_OK
+                  : make_tables(ds, fempic::kTetGeo, fempic::kDsCoef64, &ds->tgeo, &ds->coef, fempic::k_tet_geo);
+}
+
+static int create_impl(const fempic_mesh_desc* mesh, bool fp64_tables, fempic_downshift** out) {
   *out = nullptr;
   HostMesh m;
   std::string err;
-  const int rc = fempic::build_host_mesh(*mesh, &m, &err);
+  int rc = fempic::build_host_mesh(*mesh, &m, &err);
   if (rc != FEMPIC_OK) return fail(rc, "downshift_create: " + err);
   fempic_downshift* d = new (std::nothrow) fempic_downshift();
   if (!d) return fail(FEMPIC_ENOMEM, "downshift_create: host allocation");
@@ -432,64 +488,38 @@ extern "C" int fempic_downshift_create(const fempic_mesh_desc* mesh, fempic_down
   const size_t sg = sizeof(double) * 12 * (size_t)m.nt, se = sizeof(int32_t) * 6 * (size_t)m.nt,
                sf = sizeof(int32_t) * 4 * (size_t)m.nt;
   if (cudaMalloc(&d->geom, sg) != cudaSuccess || cudaMalloc(&d->te, se) != cudaSuccess ||
-      cudaMalloc(&d->tf, sf) != cudaSuccess ||
-      cudaMalloc(&d->tgeo, sizeof(double) * fempic::kTetGeo * (size_t)m.nt) != cudaSuccess ||
-      cudaMalloc(&d->coef, sizeof(double) * fempic::kDsCoef64 * (size_t)m.nt) != cudaSuccess) {
+      cudaMalloc(&d->tf, sf) != cudaSuccess) {
     free_ds(d);
     cudaGetLastError();
     return fail(FEMPIC_ENOMEM, "downshift_create: device allocation");
   }
   if (cudaMemcpy(d->geom, m.geom.data(), sg, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(d->te, m.te.data(), se, cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(d->tf, m.tf.data(), sf, cudaMemcpyHostToDevice) != cudaSuccess) {
+      cudaMemcpy(d->tf, m.tf.data(), sf, cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaDeviceSynchronize() != cudaSuccess) {
     free_ds(d);
     return fail(FEMPIC_ECUDA, "downshift_create: upload");
   }
-  fempic::k_tet_geo<<<blocks_for(m.nt), kThreads>>>(m.nt, d->geom, d->tgeo);
-  if (cudaGetLastError() != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) {
+  rc = fp64_tables ? make_form_tables(d, false) : FEMPIC_OK;
+  if (rc != FEMPIC_OK) {
     free_ds(d);
-    return fail(FEMPIC_ECUDA, "downshift_create: geometry table");
+    return rc;
   }
   *out = d;
   return FEMPIC_OK;
 }
 
-extern "C" int fempic_downshift_weights(double t, double dt, double omega0, double* w_out) {
-  if (!w_out) return fail(FEMPIC_EINVAL, "downshift_weights: NULL output");
-  if (!std::isfinite(t) || !std::isfinite(dt) || !std::isfinite(omega0) || !(dt > 0.0))
-    return fail(FEMPIC_EINVAL, "downshift_weights: non-finite scalar or dt <= 0");
-  compute_weights(t, dt, omega0, w_out);
-  return FEMPIC_OK;
+extern "C" int fempic_downshift_create(const fempic_mesh_desc* mesh, fempic_downshift** out) {
+  if (!mesh || !out) return fail(FEMPIC_EINVAL, "downshift_create: NULL argument");
+  return create_impl(mesh, true, out);
 }
 
-// The mixed forms' coefficients and geometry factors, on first use.  Built on a
-// stream of its own that is waited for: later steps may be on any stream, and a
-// first step that is being captured must not defer the table to its replay.
-static int make_mixed_tables(fempic_downshift* ds) {
-  double* dgeo = nullptr;
-  float* coef32 = nullptr;
-  if (cudaMalloc(&dgeo, sizeof(double) * kDsGeo * (size_t)ds->nt) != cudaSuccess ||
-      cudaMalloc(&coef32, sizeof(float) * fempic::kDsCoef32 * (size_t)ds->nt) != cudaSuccess) {
-    cudaGetLastError();
-    cudaFree(dgeo);
-    return fail(FEMPIC_ENOMEM, "push_step_downshift: device allocation");
-  }
-  cudaStream_t own = nullptr;
-  cudaError_t rc = cudaStreamCreateWithFlags(&own, cudaStreamNonBlocking);
-  if (rc == cudaSuccess) {
-    k_ds_geo32<<<blocks_for(ds->nt), kThreads, 0, own>>>(ds->nt, ds->geom, dgeo);
-    rc = cudaGetLastError();
-    if (rc == cudaSuccess) rc = cudaStreamSynchronize(own);
-    cudaStreamDestroy(own);
-  }
-  if (rc != cudaSuccess) {
-    cudaFree(dgeo);
-    cudaFree(coef32);
-  }
-  DS_CUDA(rc);
-  ds->dgeo = dgeo;
-  ds->coef32 = coef32;
-  return FEMPIC_OK;
+extern "C" int fempic_downshift_create_form(const fempic_mesh_desc* mesh, int32_t precision,
+                                            fempic_downshift** out) {
+  if (!mesh || !out) return fail(FEMPIC_EINVAL, "downshift_create: NULL argument");
+  if (precision != FEMPIC_FP64 && precision != FEMPIC_MIXED && precision != FEMPIC_MIXED_Q24)
+    return fail(FEMPIC_EINVAL, "downshift_create: unknown precision form");
+  return create_impl(mesh, precision == FEMPIC_FP64, out);
 }
 
 extern "C" int fempic_push_step_downshift(fempic_env* env, fempic_downshift* ds, const fempic_particles* p,
@@ -535,10 +565,8 @@ extern "C" int fempic_push_step_downshift(fempic_env* env, fempic_downshift* ds,
   A.start = start;
   compute_weights(t, dt, omega0, A.w);
   for (int i = 0; i < 24; i++) A.w32[i] = (float)A.w[i];
-  if (mixed && !ds->coef32) {
-    const int rc = make_mixed_tables(ds);
-    if (rc != FEMPIC_OK) return rc;
-  }
+  int rc = make_form_tables(ds, mixed);
+  if (rc != FEMPIC_OK) return rc;
   A.coef = ds->coef;
   A.coef32 = ds->coef32;
   cudaStream_t st = (cudaStream_t)stream;
@@ -552,7 +580,7 @@ extern "C" int fempic_push_step_downshift(fempic_env* env, fempic_downshift* ds,
         static_cast<const double2*>(envl->b_tilde), ds->ne, ds->nf, fempic::env_stats(env), envl->amp, ds->coef);
   }
   DS_CUDA(cudaGetLastError());
-  const int rc = fempic::push_downshift(env, p, A, dt, st);
+  rc = fempic::push_downshift(env, p, A, dt, st);
   if (rc != FEMPIC_OK) return fail(rc, std::string("push_step_downshift: ") + fempic_last_error());
   return FEMPIC_OK;
 }

@@ -292,7 +292,7 @@ class Downshift:
     def __init__(self, env: FempicEnv, n: int, device="cuda"):
         self.env = env
         self.f32 = env.precision != FEMPIC_FP64   # mixed forms: f32 velocities, samples and history
-        self.h = capi.fempic_downshift_create(_mesh_desc(*env._mesh))
+        self.h = capi.fempic_downshift_create_form(_mesh_desc(*env._mesh), env.precision)
         dt = torch.float32 if self.f32 else torch.float64
         self.planes = torch.zeros((capi.FEMPIC_DS_PLANES, n), dtype=dt, device=device)
         self.started = False
