@@ -24,7 +24,7 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 SOURCES_CU = ["fempic_env.cu", "fempic_downshift.cu"]
 SOURCES_CPP = ["fempic_mesh.cpp"]
 HEADERS = [os.path.join(CSRC, "fempic_internal.h"), os.path.join(CSRC, "fempic_tetgeo.cuh"), os.path.join(CSRC, "fempic_ds_rule.cuh"),
-           os.path.join(CSRC, "fempic_launch.cuh"),
+           os.path.join(CSRC, "fempic_launch.cuh"), os.path.join(CSRC, "fempic_bits.cuh"),
            os.path.join(INCLUDE, "fempic_env.h"),
            os.path.join(INCLUDE, "fempic_downshift.h")]
 

@@ -12,6 +12,7 @@
 #include <string>
 
 #include "fempic_downshift.h"
+#include "fempic_bits.cuh"
 #include "fempic_ds_rule.cuh"
 #include "fempic_internal.h"
 #include "fempic_launch.cuh"
@@ -176,26 +177,6 @@ __global__ void __launch_bounds__(kThreads) k_ds_geo32(int64_t nt, const double*
   o[31] = 0.0;
 }
 
-// Exact widening with integer operations (the hardware conversion runs at the
-// FP64 rate); zero, subnormals, infinities and NaN take the hardware's.
-__device__ __forceinline__ double widen32(float f) {
-  const unsigned u = __float_as_uint(f), e = (u >> 23) & 0xffu;
-  if (e - 1u >= 0xfeu) return (double)f;
-  return __hiloint2double((int)((u & 0x80000000u) | ((e + 896u) << 20) | ((u & 0x7fffffu) >> 3)), (int)(u << 29));
-}
-
-// FP64 -> FP32, nearest even, with integer operations; values outside the
-// normal FP32 range take the hardware conversion.
-__device__ __forceinline__ float round32(double r) {
-  const unsigned hi = (unsigned)__double2hiint(r), lo = (unsigned)__double2loint(r);
-  const unsigned e = (hi >> 20) & 0x7ffu;
-  if (e - 897u >= 253u) return (float)r;   // below 2^-126 or from 2^127 on
-  const unsigned m = ((e - 896u) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
-  const unsigned rest = lo & 0x1fffffffu;
-  const unsigned up = rest > 0x10000000u || (rest == 0x10000000u && (m & 1u)) ? 1u : 0u;
-  return __uint_as_float((hi & 0x80000000u) | (m + up));   // a carry moves into the exponent
-}
-
 __global__ void __launch_bounds__(kThreads) k_ds_field32(int64_t nt, const double* __restrict__ geom,
                                                          const double* __restrict__ dgeo,
                                                          const int32_t* __restrict__ te,
@@ -226,7 +207,7 @@ __global__ void __launch_bounds__(kThreads) k_ds_field32(int64_t nt, const doubl
     if (ds_idx_in(id, ne, stats)) {
       const float2 cc = e[id];
       bad = bad || not_finite(cc.x) || not_finite(cc.y);
-      c = make_double2(widen32(cc.x), widen32(cc.y));
+      c = make_double2(fempic::widen32(cc.x), fempic::widen32(cc.y));
     }
 #pragma unroll
     for (int a = 0; a < 3; a++) {
@@ -246,7 +227,7 @@ __global__ void __launch_bounds__(kThreads) k_ds_field32(int64_t nt, const doubl
     if (ds_idx_in(id, nf, stats)) {
       const float2 cc = b[id];
       bad = bad || not_finite(cc.x) || not_finite(cc.y);
-      c = make_double2(widen32(cc.x), widen32(cc.y));
+      c = make_double2(fempic::widen32(cc.x), fempic::widen32(cc.y));
     }
     const double bx = 2.0 * c.x, by = 2.0 * c.y;
     if (f > 0) {
@@ -266,7 +247,7 @@ __global__ void __launch_bounds__(kThreads) k_ds_field32(int64_t nt, const doubl
   float4* o32 = reinterpret_cast<float4*>(coef32 + fempic::kDsCoef32 * t);
 #pragma unroll
   for (int c = 0; c < 5; c++)
-    o32[c] = make_float4(round32(o[4 * c]), round32(o[4 * c + 1]), round32(o[4 * c + 2]), round32(o[4 * c + 3]));
+    o32[c] = make_float4(fempic::f64_to_f32(o[4 * c]), fempic::f64_to_f32(o[4 * c + 1]), fempic::f64_to_f32(o[4 * c + 2]), fempic::f64_to_f32(o[4 * c + 3]));
   o32[5] = make_float4(bad ? 1.f : 0.f, 0.f, 0.f, 0.f);
 }
 

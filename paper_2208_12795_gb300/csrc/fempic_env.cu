@@ -31,6 +31,7 @@
 #include <mutex>
 #include <string>
 
+#include "fempic_bits.cuh"
 #include "fempic_ds_rule.cuh"
 #include "fempic_internal.h"
 #include "fempic_launch.cuh"
@@ -414,17 +415,6 @@ __device__ __forceinline__ void bary64(const double* __restrict__ g, const doubl
   bary64_d(g, r[0] - g[0], r[1] - g[1], r[2] - g[2], lam);
 }
 
-// Sign and finiteness tests of doubles on their bit patterns: integer
-// instructions instead of FP64 compares, which GB300 issues at the FP64 rate.
-__device__ __forceinline__ bool finite_bits(double r) {
-  return (((unsigned)__double2hiint(r) >> 20) & 0x7ffu) != 0x7ffu;
-}
-
-__device__ __forceinline__ bool negative_bits(double r) {   // r < 0 for finite r (-0 is not negative)
-  const int hi = __double2hiint(r);
-  return hi < 0 && (((unsigned)hi & 0x7fffffffu) | (unsigned)__double2loint(r)) != 0u;
-}
-
 __device__ __forceinline__ int4 ldg_int4(const int4* p) { return __ldg(p); }
 
 // ------------------------------------------------------------ mixed push
@@ -454,53 +444,6 @@ __device__ __forceinline__ int4 ldg_int4(const int4* p) { return __ldg(p); }
 //   bytes 100-107 four 16-bit face maps;  bytes 112-127 neighbour ids
 // The step's affine field lies apart (48 B per tet), so that the per-tet pass
 // that writes it does so in whole lines.
-struct FF {
-  float hi, lo;
-};
-
-// Exact widening of a float to double with integer operations (rebias the
-// exponent, shift the significand): GB300 runs the hardware conversion at
-// the FP64 rate, 1/64 of the FP32 rate.  Zero keeps its sign; subnormal,
-// infinite and NaN inputs take the hardware conversion, so the result is the
-// double the conversion gives for every float.
-__device__ __forceinline__ double f32_to_f64(float f) {
-  const unsigned u = __float_as_uint(f);
-  const unsigned e = (u >> 23) & 0xffu, m = u & 0x7fffffu, sign = u & 0x80000000u;
-  if (e - 1u >= 0xfeu) {
-    if ((u << 1) == 0u) return __hiloint2double((int)sign, 0);
-    return (double)f;
-  }
-  return __hiloint2double((int)(sign | ((e + 896u) << 20) | (m >> 3)), (int)(m << 29));
-}
-
-// r = hi + lo: hi keeps the leading 24 bits of the FP64 significand
-// (truncated, so exactly a float), lo the remaining 29 bits rounded to FP32.
-// |r| outside [2^-126, 2^128) maps to 0 (non-finite values are rejected
-// before this is called).
-__device__ __forceinline__ FF split_f64(double r) {
-  const unsigned hi = (unsigned)__double2hiint(r), lo = (unsigned)__double2loint(r);
-  const unsigned e = (hi >> 20) & 0x7ffu;
-  if (e < 897u || e > 1150u) return FF{0.f, 0.f};
-  const unsigned sign = hi & 0x80000000u;
-  const float fhi = __uint_as_float(sign | ((e - 896u) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29));
-  const float scale = e > 948u ? __uint_as_float((e - 948u) << 23) : 0.f;   // 2^(e - 1075)
-  const float flo = __fmul_rn(__uint2float_rn(lo & 0x1fffffffu), scale);
-  return FF{fhi, sign ? -flo : flo};
-}
-
-// FP64 -> FP32, nearest even, with integer operations (the hardware
-// conversion runs at the FP64 rate); values outside the normal FP32 range
-// take it.
-__device__ __forceinline__ float f64_to_f32(double r) {
-  const unsigned hi = (unsigned)__double2hiint(r), lo = (unsigned)__double2loint(r);
-  const unsigned e = (hi >> 20) & 0x7ffu;
-  if (e - 897u >= 253u) return (float)r;
-  const unsigned m = ((e - 896u) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
-  const unsigned rest = lo & 0x1fffffffu;
-  const unsigned up = rest > 0x10000000u || (rest == 0x10000000u && (m & 1u)) ? 1u : 0u;
-  return __uint_as_float((hi & 0x80000000u) | (m + up));   // a carry moves into the exponent
-}
-
 struct Geo32 {
   double x0[3];
   float g[9];    // grad lambda_1, _2, _3
@@ -1853,27 +1796,6 @@ __global__ void __launch_bounds__(384, 2) k_cross_df(PushArgs A, DsRule D) {
 // 80-bit sums over such tets: 3e-16 of the edge values' norm (1.8e-15 for the
 // barycentric form).
 
-// Leading 24 bits of an FP64 value as a float (truncated, so at most 2^-23
-// relative below it in magnitude): 0 below 2^-126, infinite from 2^128 on.
-__device__ __forceinline__ float trunc32(double r) {
-  const unsigned hi = (unsigned)__double2hiint(r), lo = (unsigned)__double2loint(r);
-  const unsigned e = (hi >> 20) & 0x7ffu, sign = hi & 0x80000000u;
-  if (e < 897u) return 0.f;
-  if (e > 1150u) return __uint_as_float(sign | 0x7f800000u);
-  return __uint_as_float(sign | ((e - 896u) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29));
-}
-
-// 1 / w for w >= 1 to about one ulp: an FP32 reciprocal (relative error e
-// below 2^-21) and one step r (1 + e + e^2) of the residual series, whose
-// remainder e^3 lies below an FP64 ulp.  Past the FP32 range (and for a
-// non-finite w) the division.
-__device__ __forceinline__ double recip_ge1(double w) {
-  if ((unsigned)__double2hiint(w) >= (1143u << 20)) return 1.0 / w;
-  const double r = f32_to_f64(__fdividef(1.0f, trunc32(w)));
-  const double e = fma(-w, r, 1.0);
-  return fma(r, fma(e, e, e), r);
-}
-
 // FP64 form's deposit slot of a tet: six moments of the segments that stay in
 // it, then the six edges' values of the pieces the crossing pass adds.
 constexpr int kSlot64 = 12;
@@ -2133,53 +2055,6 @@ __device__ __forceinline__ void cross64_begin(const PushArgs& A, const CrossRec6
   c.nc = 0;
   c.st = FEMPIC_P_OK;
   c.reflected = false;
-}
-
-// Exit face of the piece with end barycentrics la -> lb (entry face
-// excluded): the smallest s_k = la_k / (la_k - lb_k) clamped at 0, the lowest
-// face on ties, -1 when the piece stays inside.  FP32 quotients order the
-// faces (relative error below 2^-20: la >= 0 > lb, so la - lb does not
-// cancel) and one FP64 division serves the winner; where two faces come
-// within 2^-17, a start lies outside (la < 0) or a quotient is not finite,
-// every face is divided in FP64.
-__device__ __forceinline__ int exit_face64(const double la[4], const double lb[4], int entry, double& smin) {
-  float q1 = INFINITY, q2 = INFINITY;
-  bool close = false;
-  int kx = -1;
-  double a = 0.0, b = 0.0;
-#pragma unroll
-  for (int k = 0; k < 4; k++) {
-    if (k == entry || !negative_bits(lb[k])) continue;
-    const float x = trunc32(la[k]), y = trunc32(lb[k]);
-    const float q = __fdividef(x, x - y);
-    close = close || !(q >= 0.f && q < INFINITY) || negative_bits(la[k]);
-    if (q < q1) {
-      q2 = q1;
-      q1 = q;
-      kx = k;
-      a = la[k];
-      b = lb[k];
-    } else {
-      q2 = fminf(q2, q);
-    }
-  }
-  smin = INFINITY;
-  if (close || (kx >= 0 && q2 <= q1 + q1 * 0x1p-17f)) {
-    kx = -1;
-#pragma unroll
-    for (int k = 0; k < 4; k++) {
-      if (k == entry || !negative_bits(lb[k])) continue;
-      double sk = la[k] / (la[k] - lb[k]);
-      if (sk < 0.0) sk = 0.0;
-      if (sk < smin) {
-        smin = sk;
-        kx = k;
-      }
-    }
-  } else if (kx >= 0) {
-    smin = a / (a - b);
-  }
-  return kx;
 }
 
 __device__ __forceinline__ bool cross64_advance(const PushArgs& A, CrossState64& c, bool fresh) {
