@@ -181,8 +181,9 @@ FEMPIC_HD double recip_ge1(double w) {
 // face on ties, -1 when the piece stays inside.  FP32 quotients order the
 // faces (relative error below 2^-20: la >= 0 > lb, so la - lb does not
 // cancel) and one FP64 division serves the winner; where two faces come
-// within 2^-17, a start lies outside (la < 0) or a quotient is not finite,
-// every face is divided in FP64.
+// within 2^-17, a start lies outside (la < 0) or so near a face that FP32
+// loses bits of it (0 < la < 2^-104), or a quotient is not finite or below
+// 2^-100 without being 0, every face is divided in FP64.
 FEMPIC_HD int exit_face64(const double la[4], const double lb[4], int entry, double& smin) {
   float q1 = INFINITY, q2 = INFINITY;
   bool close = false;
@@ -193,7 +194,8 @@ FEMPIC_HD int exit_face64(const double la[4], const double lb[4], int entry, dou
     if (k == entry || !negative_bits(lb[k])) continue;
     const float x = trunc32(la[k]), y = trunc32(lb[k]);
     const float q = fast_div(x, x - y);
-    close = close || !(q >= 0.f && q < INFINITY) || negative_bits(la[k]);
+    const unsigned h = (unsigned)hi_word(la[k]);
+    close = close || !(q >= 0.f && q < INFINITY) || !(h - (919u << 20) < (1128u << 20) || (h | (unsigned)lo_word(la[k])) == 0u);
     if (q < q1) {
       q2 = q1;
       q1 = q;
@@ -205,7 +207,7 @@ FEMPIC_HD int exit_face64(const double la[4], const double lb[4], int entry, dou
     }
   }
   smin = INFINITY;
-  if (close || (kx >= 0 && q2 <= q1 + q1 * 0x1p-17f)) {
+  if (close || (kx >= 0 && (q2 <= q1 + q1 * 0x1p-17f || (q1 < 0x1p-100f && (hi_word(a) | lo_word(a)) != 0)))) {
     kx = -1;
 #pragma unroll
     for (int k = 0; k < 4; k++) {
