@@ -54,7 +54,7 @@ PROFILE_SUMMARY = os.path.join(ROOT, "profiles", "push_mixed_cube48_10M.txt")
 FP64_SUMMARY = os.path.join(ROOT, "profiles", "fp64_ops_cube48_4M.txt")
 KERNEL_SOURCES = [os.path.join(ROOT, "paper_2208_12795_gb300", "csrc", f)
                   for f in ("fempic_env.cu", "fempic_internal.h", "fempic_ds_rule.cuh", "fempic_tetgeo.cuh",
-                            "fempic_launch.cuh")]
+                            "fempic_launch.cuh", "fempic_bits.cuh")]
 
 
 def parse():

@@ -165,7 +165,7 @@ FEMPIC_HD float trunc32(double r) {
   return from_word(sign | ((e - 896u) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29));
 }
 
-// 1 / w for w >= 1 to about one ulp: an FP32 reciprocal (relative error e
+// 1 / w for w >= 1 within 0.502 ulp: an FP32 reciprocal (relative error e
 // below 2^-21) and one step r (1 + e + e^2) of the residual series, whose
 // remainder e^3 lies below an FP64 ulp.  Past the FP32 range (and for a
 // non-finite w) the division.

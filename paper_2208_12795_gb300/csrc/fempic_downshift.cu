@@ -140,7 +140,8 @@ __global__ void __launch_bounds__(kThreads) k_ds_field64(int64_t nt, const doubl
 // one order of operations; their geometry factors (g_j x g_i per edge, g_j x
 // g_k per face at node 0, det per face) are formed once per mesh, and the
 // conversions of DoFs and results run in integer operations off the FP64 pipe
-// (663k tets: 280 -> 155 us).
+// (663k tets: 280 -> 155 us with a(t) = 1, past the envelope's rise, 182 during
+// it, when the 20 sums are scaled).
 constexpr int kDsGeo = 32;   // doubles per tet: 6 x 3, 3 x 3, 4, unused
 
 __global__ void __launch_bounds__(kThreads) k_ds_geo32(int64_t nt, const double* __restrict__ geom,

@@ -78,7 +78,7 @@ struct Species {
 };
 
 // Record of a particle that leaves its home tet: written by the common path
-// into its tile's region of the crossing queue (contiguous, so the crossing
+// into its CTA's region of the crossing queue (contiguous, so the crossing
 // kernel reads it coalesced instead of re-reading the SoA sparsely).
 struct __align__(16) CrossRec {
   double a[3];
@@ -120,12 +120,11 @@ struct PushArgs {
   int32_t max_cross;
   int32_t wall_mode;
   double lo[3], hi[3];
-  int64_t nt, ne;
+  int64_t nt;
   const double* geom64;
   const float4* tetrec;
   const int4* tn;
   const int4* nb;
-  const int4* te;
   const void* field;
   unsigned long long* dGq;      // 24-bit form: per (species, tet) slots of the 6 local edges,
                                 // [ns][nt][8] int64 in units of 2^-48 (q w)
@@ -694,8 +693,6 @@ struct LaneOut {
   int lh[6];           // the six values as 32-bit limbs (hi 2^25 + lo), for the run sums
   unsigned ll[6];
   int32_t key;         // (home tet, species) run key; negative = no deposit
-  int32_t Thome;
-  int shome;
   bool queue;          // leaves its tet (or may): tracked by the crossing pass
   unsigned nfrz;
   double a[3];         // start point and new velocity of a queued particle
@@ -715,8 +712,6 @@ __device__ __forceinline__ void lane_init(LaneOut& o, int lane) {
 #pragma unroll
   for (int e = 0; e < 9; e++) o.mv[e] = 0.f;
   o.key = -1 - lane;
-  o.Thome = 0;
-  o.shome = 0;
   o.queue = false;
   o.nfrz = 0;
 }
@@ -806,8 +801,6 @@ __device__ __forceinline__ void mixed_drift(const PushArgs& A, int64_t p, int32_
     }
   }
   o.key = T * kMaxSpecies + s;
-  o.Thome = T;
-  o.shome = s;
 }
 
 template <bool Q24>
@@ -1142,26 +1135,21 @@ __device__ __forceinline__ void ds_fetch(const PushArgs& A, const DsRule& D, int
 // of 16 bytes a lane instead of 40 of 4 and 8.  Lanes read each other's
 // copies, so the warp synchronizes around them.  10M particles: 761 -> 665
 // us; the plain push, with 7 copies a lane, measured 2 % slower this way.
-__device__ __forceinline__ void cp_async16(void* dst, const void* src, int bytes) {   // the rest of the 16 is zeroed
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_addr(dst)), "l"(src), "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ int bytes_in(int64_t left, int size) {   // of a 16-byte chunk with `left` elements to the end
-  return left * size >= 16 ? 16 : left > 0 ? (int)left * size : 0;
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
 }
 __device__ __forceinline__ void fetch_state16(const PushArgs& A, int64_t w, MixedTile& S) {
   const int lane = threadIdx.x & 31, t0 = threadIdx.x & ~31;
   const int h = lane >> 4, c2 = 2 * (lane & 15), q = lane >> 3, c4 = 4 * (lane & 7);
   const double* r01 = h ? A.iy : A.ix;
-  const int b2 = bytes_in(A.n - w - c2, 8), b4 = bytes_in(A.n - w - c4, 4);
-  if (b2) {
-    cp_async16(&S.r[h][t0 + c2], r01 + w + c2, b2);
-    if (h == 0) cp_async16(&S.r[2][t0 + c2], A.iz + w + c2, b2);
+  if (w + c2 < A.n) {   // n is a multiple of 4: a chunk lies inside or outside
+    cp_async16(&S.r[h][t0 + c2], r01 + w + c2);
+    if (h == 0) cp_async16(&S.r[2][t0 + c2], A.iz + w + c2);
   }
-  if (b4) {
+  if (w + c4 < A.n) {
     const void* a = q == 0 ? A.ivx : q == 1 ? A.ivy : q == 2 ? A.ivz : (const void*)A.itet;
     void* d = q < 3 ? (void*)&S.v[q][t0 + c4] : (void*)&S.T[t0 + c4];
-    cp_async16(d, static_cast<const float*>(a) + w + c4, b4);
+    cp_async16(d, static_cast<const float*>(a) + w + c4);
   }
 }
 
@@ -1172,7 +1160,7 @@ __device__ __forceinline__ void ds_fetch16(const PushArgs& A, const DsRule& D, i
   const float* H = static_cast<const float*>(D.h) + w + c;
 #pragma unroll
   for (int k0 = 0; k0 < FEMPIC_DS_VN; k0 += 4)
-    if (k0 + q < FEMPIC_DS_VN) cp_async16(&S.h[k0 + q][t0 + c], H + (k0 + q) * D.n, 16);
+    if (k0 + q < FEMPIC_DS_VN) cp_async16(&S.h[k0 + q][t0 + c], H + (k0 + q) * D.n);
 }
 
 template <bool Q24, bool VEC>
@@ -1578,7 +1566,7 @@ __device__ __forceinline__ void deposit_piece_df(const PushArgs& A, int s, int32
     e = __fmaf_rn(-u[j].h, w[i].lo, __fmaf_rn(-u[j].l, w[i].hi, e));
     const DF m = df_mul(dS, fast_two_sum(sd.h, e));
     const DF d = df_mul(dS, DF{w[k].hi, w[k].lo});
-    atomicAdd(ms + k, (double)d.h);   // exact widening (the FP64 pipe is idle here)
+    atomicAdd(ms + k, (double)d.h);   // exact widening; in integer operations the pass took 1241 us, so 1209
     atomicAdd(ms + 3 + k, (double)m.h);
     lo[k] = d.l;
     lo[3 + k] = m.l;
@@ -2605,7 +2593,7 @@ __global__ void __launch_bounds__(kThreads) k_adjoint_unpermute(AdjPermArgs A) {
 // form) or into an FP32 row with vector atomics (mixed form, no FP64-pipe
 // work); in the mixed form a warp whose particles fall into more than 4 runs
 // (the order has drifted since the last sort) skips the reduction and adds
-// each lane's 10 values straight into the row.  The transposed pre-pass k_field_adjoint maps both
+// each lane's 10 values straight into the row.  The transposed pre-pass k_field_adjoint32/64 maps both
 // to the complex DoFs.  A
 // particle frozen during the step gets a zero adjoint (its later state no
 // longer depends on its earlier one through the step map).
@@ -4089,12 +4077,10 @@ static int push_particles(fempic_env* env, const fempic_particles* in, const fem
     A.hi[a] = env->h.hi[a];
   }
   A.nt = env->h.nt;
-  A.ne = env->h.ne;
   A.geom64 = env->geom64;
   A.tetrec = env->tetrec;
   A.tn = env->tn;
   A.nb = env->nb;
-  A.te = env->te;
   A.field = env->field;
   A.dGq = env->deposit_on ? env->dGq : nullptr;
   A.mom = env->deposit_on ? env->mom : nullptr;
