@@ -111,11 +111,14 @@ def plan_window(n: int, steps: int, state_bytes: int, adj_bytes: int, budget_byt
     """Checkpoint interval and reverse mode of a gradient window that fits in
     budget_bytes of device memory with the fewest recomputed steps (ties: the
     smaller peak).  Peak: ceil(K/every) checkpoints (a state and its sort
-    permutation each), then in the reverse sweep either every + 1 stashed
-    states of the segment (stash) or 2 (each step's pair recomputed from the
-    checkpoint, every (every + 1) / 2 steps per segment), and the adjoint
-    state with its spare for the checkpoint unpermutes.  Raises
-    MemoryError when even the leanest plan does not fit."""
+    permutation each), then in the reverse sweep either every + 1 states
+    (stash: the segment's own and the final one) or 2 (each step's pair
+    recomputed from the checkpoint, every (every + 1) / 2 steps per segment),
+    and the adjoint state with its spare for the checkpoint unpermutes.  The
+    autograd function holds the final state through its backward pass (in
+    recompute mode on top of the plan); the direct entry points have let it go
+    by then and stay one state below a plan with a stash.  Raises MemoryError
+    when even the leanest plan does not fit."""
     perm = 4 * n
     best = None
     for every in range(1, max(steps, 1) + 1):
