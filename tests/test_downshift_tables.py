@@ -30,7 +30,7 @@ def test_bad_arguments_rejected_on_host():
 
 # Bytes per tet: geometry, edge and face ids 136; then tables and coefficients
 # 32 f64 (FP64) or 32 f64 + 24 f32 (mixed).  Five allocations, each rounded up
-# to the driver's 2 MiB pages.
+# to 2 MiB.
 @pytest.mark.gpu
 @pytest.mark.parametrize("prec,per_tet", [(FP64, 136 + 256), (MIXED, 136 + 352), (Q24, 136 + 352)])
 def test_memory_of_one_form(prec, per_tet):
